@@ -10,6 +10,7 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <utility>
 
 #include "dual_attn_sm100.cuh"
 #include "jvp_bwd_sm100.cuh"
@@ -411,43 +412,94 @@ __global__ void selftest_timeout_kernel(int* status, unsigned long long limit_ns
 
 // ------------------------------------------------------------------------------------------------
 // RMSNorm QK-normalisation prologue
-static int rms_geometry(const Shape& s, int* cpr, int* gs) {
-    *cpr = s.d * (s.fp32 ? 4 : 2) / 16;
-    *gs = *cpr;   // lanes per row
-    return *gs <= 32 ? TVM_ATTN_OK : TVM_ATTN_UNSUPPORTED;
+// The rows of a side in memory order.  Dimensions of one element drop out, and two that are dense in one another
+// merge: both tensor layouts of a transformer, packed and (B, rows, H, d), end as one dimension.
+static RmsRows rms_rows(const Shape& s, const Geom& g) {
+    struct Dim { long long n, st; } dim[3] = {{g.rows, g.rs}, {s.H, g.hs}, {s.B, g.bs}};
+    for (int i = 0; i < 2; ++i)   // by stride, innermost first
+        for (int j = 0; j < 2 - i; ++j)
+            if (dim[j].n == 1 || (dim[j + 1].n > 1 && dim[j + 1].st < dim[j].st)) std::swap(dim[j], dim[j + 1]);
+    RmsRows r;
+    r.total = (unsigned)(s.BH * g.rows);
+    int n = 0;
+    Dim out[3] = {{1, s.d}, {1, 0}, {1, 0}};
+    for (int i = 0; i < 3; ++i) {
+        if (dim[i].n == 1) continue;
+        if (n > 0 && dim[i].st == out[n - 1].n * out[n - 1].st) out[n - 1].n *= dim[i].n;
+        else out[n++] = dim[i];
+    }
+    r.n0 = (unsigned)out[0].n; r.n1 = (unsigned)out[1].n;
+    r.s0 = out[0].st; r.s1 = out[1].st; r.s2 = out[2].st;
+    return r;
+}
+
+// Blocks of both sides, at most `most` of them: in proportion to the rows, at least one each.
+static void rms_blocks(long long rows_q, long long rows_k, int rows_per_block, int most, int* nbq, int* nbk) {
+    const long long need_q = (rows_q + rows_per_block - 1) / rows_per_block, need_k = (rows_k + rows_per_block - 1) / rows_per_block;
+    if (need_q + need_k <= most) { *nbq = (int)need_q; *nbk = (int)need_k; return; }
+    long long q = (most * rows_q + (rows_q + rows_k) / 2) / (rows_q + rows_k);
+    q = q < 1 ? 1 : q > most - 1 ? most - 1 : q;
+    *nbq = (int)(q < need_q ? q : need_q);
+    *nbk = (int)(most - q < need_k ? most - q : need_k);
+}
+
+template <typename T, int C>
+static int rms_fwd_c(const Shape& s, float eps, const RmsFwdSide<T>& q, const RmsFwdSide<T>& k, int P, cudaStream_t st) {
+    int nbq, nbk;
+    rms_blocks(q.rows.total, k.rows.total, (RMS_THREADS / 32) * rms_fwd_groups(C) * (32 / P), RMS_FWD_BLOCKS, &nbq, &nbk);
+    qk_rmsnorm_jvp_fwd_kernel<T, C><<<nbq + nbk, RMS_THREADS, 0, st>>>(q, k, nbq, s.d, P, eps);
+    g_launches += 1;
+    return cuda_status(cudaGetLastError());
 }
 
 template <typename T>
 static int rms_fwd(const Shape& s, float eps, const void* Q, const void* tQ, const void* K, const void* tK, const float* gQ,
                    const float* gK, void* Qn, void* tQn, void* Kn, void* tKn, cudaStream_t st) {
-    int cpr, gs;
-    const int rc = rms_geometry(s, &cpr, &gs);
-    if (rc != TVM_ATTN_OK) return rc;
-    const long long rows_q = s.BH * s.M, rows_k = s.BH * s.N, rows_per_block = (long long)(RMS_THREADS / 32) * (32 / gs);
-    const RmsFwdSide<T> q{(const T*)Q, (const T*)tQ, gQ, (T*)Qn, (T*)tQn, s.q, rows_q};
-    const RmsFwdSide<T> k{(const T*)K, (const T*)tK, gK, (T*)Kn, (T*)tKn, s.k, rows_k};
-    const long long rows = rows_q > rows_k ? rows_q : rows_k;
-    const dim3 grid((unsigned)((rows + rows_per_block - 1) / rows_per_block), 2);
-    qk_rmsnorm_jvp_fwd_kernel<T><<<grid, RMS_THREADS, 0, st>>>(q, k, s.H, s.d, cpr, gs, eps);
-    g_launches += 1;
-    return cuda_status(cudaGetLastError());
+    const RmsFwdSide<T> q{(const T*)Q, (const T*)tQ, gQ, (T*)Qn, (T*)tQn, rms_rows(s, s.q)};
+    const RmsFwdSide<T> k{(const T*)K, (const T*)tK, gK, (T*)Kn, (T*)tKn, rms_rows(s, s.k)};
+    const int cpr = s.d * (int)sizeof(T) / 16, C = rms_split(cpr, 4), P = cpr / C;
+    switch (C) {
+        case 1: return rms_fwd_c<T, 1>(s, eps, q, k, P, st);
+        case 2: return rms_fwd_c<T, 2>(s, eps, q, k, P, st);
+        case 3: return rms_fwd_c<T, 3>(s, eps, q, k, P, st);
+        default: return rms_fwd_c<T, 4>(s, eps, q, k, P, st);
+    }
+}
+
+template <typename T, int C>
+static int rms_bwd_c(const Shape& s, float eps, RmsBwdSide<T> q, RmsBwdSide<T> k, int P, float* dgQ, float* dgK, cudaStream_t st) {
+    int nbq, nbk;
+    rms_blocks(q.rows.total, k.rows.total, (RMS_BWD_THREADS / 32) * (32 / P), RMS_BWD_BLOCKS, &nbq, &nbk);
+    k.partial = q.partial + (size_t)nbq * s.d;
+    qk_rmsnorm_jvp_bwd_kernel<T, C><<<nbq + nbk, RMS_BWD_THREADS, 0, st>>>(q, k, nbq, s.d, P, eps);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return TVM_ATTN_CUDA_ERROR;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)s.d / 4, 2);
+    cfg.blockDim = dim3(RMS_REDUCE_THREADS);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, qk_rmsnorm_dg_reduce_kernel, (const float*)q.partial, (const float*)k.partial, dgQ, dgK, nbq, nbk, s.d);
+    g_launches += 2;
+    return cuda_status(e);
 }
 
 template <typename T>
 static int rms_bwd(const Shape& s, float eps, const void* Q, const void* tQ, const void* K, const void* tK, const float* gQ,
                    const float* gK, const void* dQn, const void* dtQn, const void* dKn, const void* dtKn, void* dQ, void* dtQ,
                    void* dK, void* dtK, float* dgQ, float* dgK, float* partial, cudaStream_t st) {
-    int cpr, gs;
-    const int rc = rms_geometry(s, &cpr, &gs);
-    if (rc != TVM_ATTN_OK) return rc;
-    float* pq = partial;
-    float* pk = partial + (size_t)RMS_BWD_BLOCKS * s.d;
-    const RmsBwdSide<T> q{(const T*)Q, (const T*)tQ, gQ, (const T*)dQn, (const T*)dtQn, (T*)dQ, (T*)dtQ, pq, s.q, s.BH * s.M};
-    const RmsBwdSide<T> k{(const T*)K, (const T*)tK, gK, (const T*)dKn, (const T*)dtKn, (T*)dK, (T*)dtK, pk, s.k, s.BH * s.N};
-    qk_rmsnorm_jvp_bwd_kernel<T><<<dim3(RMS_BWD_BLOCKS, 2), RMS_THREADS, 0, st>>>(q, k, s.H, s.d, cpr, gs, eps);
-    qk_rmsnorm_dg_reduce_kernel<<<2, 1024, 0, st>>>(pq, pk, dgQ, dgK, RMS_BWD_BLOCKS, s.d);
-    g_launches += 2;
-    return cuda_status(cudaGetLastError());
+    const RmsBwdSide<T> q{(const T*)Q, (const T*)tQ, gQ, (const T*)dQn, (const T*)dtQn, (T*)dQ, (T*)dtQ, partial, rms_rows(s, s.q)};
+    const RmsBwdSide<T> k{(const T*)K, (const T*)tK, gK, (const T*)dKn, (const T*)dtKn, (T*)dK, (T*)dtK, nullptr, rms_rows(s, s.k)};
+    const int cpr = s.d * (int)sizeof(T) / 16, C = rms_split(cpr, 3), P = cpr / C;
+    switch (C) {
+        case 1: return rms_bwd_c<T, 1>(s, eps, q, k, P, dgQ, dgK, st);
+        case 2: return rms_bwd_c<T, 2>(s, eps, q, k, P, dgQ, dgK, st);
+        default: return rms_bwd_c<T, 3>(s, eps, q, k, P, dgQ, dgK, st);
+    }
 }
 
 static bool rms_eps_ok(float eps) { return eps >= 0.0f && std::isfinite(eps); }
@@ -650,7 +702,7 @@ int tvm_attn_check_status(void* cuda_stream) {
 size_t tvm_qk_rmsnorm_jvp_workspace_bytes(const tvm_attn_params* p) {
     Shape s;
     if (check_params(p, &s) != TVM_ATTN_OK) return 0;
-    return (size_t)2 * RMS_BWD_BLOCKS * (size_t)s.d * sizeof(float);
+    return (size_t)RMS_PARTIAL_ROWS * (size_t)s.d * sizeof(float);
 }
 
 int tvm_qk_rmsnorm_jvp_fwd(const tvm_attn_params* p, float eps, const void* Q, const void* tQ, const void* K, const void* tK,
@@ -678,7 +730,7 @@ int tvm_qk_rmsnorm_jvp_bwd(const tvm_attn_params* p, float eps, const void* Q, c
     const void* ptrs[] = {Q, tQ, K, tK, gQ, gK, dQn, dtQn, dKn, dtKn, dQ, dtQ, dK, dtK, dgQ, dgK, workspace};
     for (const void* x : ptrs)
         if (!x || !aligned16(x)) return TVM_ATTN_INVALID_ARG;
-    if (workspace_bytes < (size_t)2 * RMS_BWD_BLOCKS * (size_t)s.d * sizeof(float)) return TVM_ATTN_WORKSPACE_TOO_SMALL;
+    if (workspace_bytes < (size_t)RMS_PARTIAL_ROWS * (size_t)s.d * sizeof(float)) return TVM_ATTN_WORKSPACE_TOO_SMALL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     float* part = static_cast<float*>(workspace);
     return s.fp32 ? rms_bwd<float>(s, eps, Q, tQ, K, tK, gQ, gK, dQn, dtQn, dKn, dtKn, dQ, dtQ, dK, dtK, dgQ, dgK, part, st)

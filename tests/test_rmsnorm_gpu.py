@@ -53,6 +53,39 @@ def test_rmsnorm_prologue_against_the_oracle(B, H, N, d, mode):
     assert not bad, (bad, errs)
 
 
+# every split of a row over lanes (1 to 4 chunks on 1 to 16 lanes), a last row group that is partly empty, more rows than
+# one sweep of the grid covers
+@pytest.mark.parametrize("B,H,N,d", [(1, 2, 37, 8), (1, 1, 131, 16), (2, 3, 77, 24), (1, 2, 99, 48), (2, 2, 61, 56), (1, 3, 45, 80), (1, 2, 51, 88),
+                                     (2, 1, 67, 96), (1, 2, 35, 104), (2, 1, 70, 112), (1, 3, 41, 120), (3, 16, 1003, 72), (3, 16, 1003, 40)])
+def test_rmsnorm_prologue_at_every_split_of_a_row(B, H, N, d):
+    errs = _case(B, H, N, d, torch.bfloat16, seed=900 + N + d, eps=1e-6)
+    bad = {k: e for k, e in errs.items() if not e <= (1e-3 if k.startswith("dg") else 1e-2)}
+    assert not bad, (bad, errs)
+
+
+@pytest.mark.parametrize("H,slots", [(3, 1), (3, 4), (1, 2)])
+def test_rmsnorm_prologue_on_strided_rows(H, slots):
+    """(B, N, slots, H, d) buffers: dense token-major rows (slots = 1) and the slices of a fused projection."""
+    B, N, d = 2, 150, 72
+    x = {k: v.to(torch.bfloat16).cuda() for k, v in inputs.make_inputs(inputs.custom(B, H, N, d, seed=12)).items()}
+    g = torch.linspace(0.5, 1.5, d, device="cuda")
+
+    def strided(t):
+        buf = torch.zeros((B, N, slots, H, d), dtype=t.dtype, device="cuda")
+        buf[:, :, slots - 1] = t.permute(0, 2, 1, 3)
+        return buf[:, :, slots - 1].permute(0, 2, 1, 3)
+
+    names = ("Q", "tQ", "K", "tK")
+    want = binding.tvm_qk_rmsnorm_jvp_fwd(*(x[k] for k in names), g, g)
+    got = binding.tvm_qk_rmsnorm_jvp_fwd(*(strided(x[k]) for k in names), g, g)
+    want += binding.tvm_qk_rmsnorm_jvp_bwd(*(x[k] for k in names), g, g, *(x[k] for k in ("dO", "dtO", "V", "tV")))
+    got += binding.tvm_qk_rmsnorm_jvp_bwd(*(strided(x[k]) for k in names), g, g, *(strided(x[k]) for k in ("dO", "dtO", "V", "tV")))
+    for a, b in zip(got[:8], want[:8]):
+        assert torch.equal(a, b)
+    for a, b in zip(got[8:], want[8:]):   # the scales' gradients are sums over the rows, in another order
+        assert torch.allclose(a, b, rtol=1e-4, atol=1e-3)
+
+
 def test_rmsnorm_prologue_with_a_large_epsilon():
     errs = _case(1, 2, 96, 48, torch.float32, seed=3, eps=0.5)
     assert max(errs.values()) <= 1e-4, errs
