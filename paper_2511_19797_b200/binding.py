@@ -1,10 +1,13 @@
-"""ctypes binding of the C-ABI library declared in include/tvm_attn.h.
+"""Python binding of the C-ABI library declared in include/tvm_attn.h.
 
 Argument marshalling only: every step of the path runs in the CUDA kernels of the library.
-PyTorch provides device memory and streams.  There is no CPU or library fallback: if the
+PyTorch provides device memory and streams.  The tensor functions go through a native module
+(csrc/torch_binding.cpp: a call on a small problem is over on the GPU before Python has compared
+its arguments' shapes), the rest through ctypes.  There is no CPU or library fallback: if a
 shared object is missing or a call fails, an exception is raised.
 """
 import ctypes
+import importlib.util
 import os
 
 import torch
@@ -33,6 +36,9 @@ class Params(ctypes.Structure):
 
 
 _lib = None
+_native = None
+_BOUND = ("tvm_attn_jvp_fwd", "tvm_attn_jvp_bwd", "tvm_attn_jvp_bwd_noalloc", "tvm_attn_jvp_workspace_bytes",
+          "tvm_qk_rmsnorm_jvp_fwd", "tvm_qk_rmsnorm_jvp_bwd", "tvm_qk_rmsnorm_jvp_workspace_bytes")
 EXPORTS = ("tvm_attn_jvp_workspace_bytes", "tvm_attn_jvp_fwd", "tvm_attn_jvp_bwd", "tvm_attn_jvp_bwd_noalloc",
            "tvm_attn_check_status", "tvm_attn_selftest_timeout",
            "tvm_qk_rmsnorm_jvp_fwd", "tvm_qk_rmsnorm_jvp_bwd", "tvm_qk_rmsnorm_jvp_workspace_bytes",
@@ -93,55 +99,18 @@ def _raise(where, code):
     raise TvmAttnError(where, code, load().tvm_attn_strerror(code).decode())
 
 
-def _strides(t):
-    """{row, head, batch} element strides of a (B, H, rows, d) tensor; zeros for the packed layout."""
-    if t.stride(3) != 1 and t.shape[3] != 1:
-        raise ValueError("the d elements of a row must be contiguous")
-    if t.is_contiguous():
-        return (0, 0, 0)
-    return (t.stride(2), t.stride(1), t.stride(0))
-
-
-def _params(q, scale, flags, k=None):
-    """Parameters from a query-side tensor q (B, H, M, d) and, for M != N or strided layouts, a key-side tensor k."""
-    if q.dim() != 4:
-        raise ValueError("expected (B, H, rows, d) tensors")
-    if q.dtype == torch.bfloat16:
-        dt = BF16
-    elif q.dtype == torch.float32:
-        dt = FP32
-    else:
-        raise ValueError("tensors must be bfloat16 or float32")
-    B, H, M, d = q.shape
-    k = q if k is None else k
-    if k.dim() != 4 or k.shape[0] != B or k.shape[1] != H or k.shape[3] != d:
-        raise ValueError("query-side and key-side tensors must agree in B, H and d")
-    N = k.shape[2]
-    p = Params(B, H, N, d, float(scale), dt, int(flags), 0 if M == N else M)
-    p.q_strides[:] = _strides(q)
-    p.k_strides[:] = _strides(k)
-    return p
-
-
-def _check_tensors(ref, tensors):
-    """Every tensor of one side shares shape, strides, dtype and device with the side's first tensor."""
-    for t in tensors:
-        if t.shape != ref.shape or t.dtype != ref.dtype or t.device != ref.device or t.stride() != ref.stride():
-            raise ValueError("all tensors of one side must share shape, strides, dtype and device")
-        if not t.is_cuda:
-            raise ValueError("tensors must be CUDA tensors")
-    if not ref.is_cuda:
-        raise ValueError("tensors must be CUDA tensors")
-
-
-def _like(t):
-    """A new tensor with the shape AND the strides of t (torch.empty_like does not keep the strides of a slice)."""
-    return torch.empty_strided(t.shape, t.stride(), dtype=t.dtype, device=t.device)
-
-
-def _ptr(t):
-    """Device address of a tensor, or a null pointer for None (an absent cotangent or an unwanted output)."""
-    return None if t is None else t.data_ptr()
+def _load_native():
+    """The native half of the binding, bound to the library's entry points.  Raises if it is not built."""
+    global _native
+    lib = load()
+    if not os.path.exists(_build.BINDING_PATH):
+        raise FileNotFoundError("%s is missing: run paper_2511_19797_b200/build.py first" % _build.BINDING_PATH)
+    spec = importlib.util.spec_from_file_location("_tvm_binding", _build.BINDING_PATH)
+    native = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(native)
+    native.bind(*[ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in _BOUND])
+    _native = native
+    return native
 
 
 def _stream_ptr(stream):
@@ -156,23 +125,10 @@ def tvm_attn_jvp_workspace_bytes(B, H, N, d, dtype=BF16, is_bwd=True, scale=0.0,
 
 def tvm_attn_jvp_fwd(Q, K, V, tQ, tK, tV, scale=0.0, flags=0, out=None, stream=None):
     """Forward: returns (O, tO, lse, mu).  `out` may hold preallocated (O, tO, lse, mu)."""
-    lib = load()
-    if out is None:
-        O, tO = _like(Q), _like(Q)
-        lse = torch.empty(Q.shape[:3], dtype=torch.float32, device=Q.device)
-        mu = torch.empty_like(lse)
-    else:
-        O, tO, lse, mu = out
-    _check_tensors(Q, (tQ, O, tO))
-    _check_tensors(K, (V, tK, tV))
-    p = _params(Q, scale, flags, K)
-    with torch.cuda.device(Q.device):
-        rc = lib.tvm_attn_jvp_fwd(ctypes.byref(p), Q.data_ptr(), K.data_ptr(), V.data_ptr(), tQ.data_ptr(),
-                                  tK.data_ptr(), tV.data_ptr(), O.data_ptr(), tO.data_ptr(), lse.data_ptr(),
-                                  mu.data_ptr(), None, 0, _stream_ptr(stream))
-    if rc != 0:
-        _raise("tvm_attn_jvp_fwd", rc)
-    return O, tO, lse, mu
+    r = (_native or _load_native()).fwd(Q, K, V, tQ, tK, tV, scale, flags, out, None if stream is None else stream.cuda_stream)
+    if r.__class__ is int:
+        _raise("tvm_attn_jvp_fwd", r)
+    return r
 
 
 def tvm_attn_jvp_bwd(Q, K, V, tQ, tK, tV, O, tO, lse, mu, dO, dtO, scale=0.0, flags=0, out=None, workspace=None,
@@ -181,22 +137,11 @@ def tvm_attn_jvp_bwd(Q, K, V, tQ, tK, tV, O, tO, lse, mu, dO, dtO, scale=0.0, fl
     tvm_attn_jvp_workspace_bytes(...) bytes; one is allocated with torch when not given.
     dO or dtO may be None (a zero cotangent; dtO=None is the "detach JVP" setting).  With dtO=None the entries
     dtQ, dtK, dtV of `out` may be None too; tensors given there come back zero."""
-    lib = load()
-    p = _params(Q, scale, flags, K)
-    need = int(lib.tvm_attn_jvp_workspace_bytes(ctypes.byref(p), 1))
-    if workspace is None:
-        workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=Q.device)
-    outs = out if out is not None else (_like(Q), _like(K), _like(K), _like(Q), _like(K), _like(K))
-    _check_tensors(Q, tuple(t for t in (tQ, O, tO, dO, dtO, outs[0], outs[3]) if t is not None))
-    _check_tensors(K, tuple(t for t in (V, tK, tV, outs[1], outs[2], outs[4], outs[5]) if t is not None))
-    with torch.cuda.device(Q.device):
-        rc = lib.tvm_attn_jvp_bwd(ctypes.byref(p), Q.data_ptr(), K.data_ptr(), V.data_ptr(), tQ.data_ptr(),
-                                  tK.data_ptr(), tV.data_ptr(), O.data_ptr(), tO.data_ptr(), lse.data_ptr(),
-                                  mu.data_ptr(), _ptr(dO), _ptr(dtO), *[_ptr(o) for o in outs],
-                                  workspace.data_ptr(), workspace.numel(), _stream_ptr(stream))
-    if rc != 0:
-        _raise("tvm_attn_jvp_bwd", rc)
-    return outs
+    r = (_native or _load_native()).bwd(Q, K, V, tQ, tK, tV, O, tO, lse, mu, dO, dtO, scale, flags, out, workspace,
+                                        None if stream is None else stream.cuda_stream, False)
+    if r.__class__ is int:
+        _raise("tvm_attn_jvp_bwd", r)
+    return r
 
 
 def tvm_attn_jvp_bwd_noalloc(Q, K, V, tQ, tK, tV, O, tO, lse, mu, dO, dtO, out, scale=0.0, flags=0, stream=None):
@@ -205,63 +150,28 @@ def tvm_attn_jvp_bwd_noalloc(Q, K, V, tQ, tK, tV, O, tO, lse, mu, dO, dtO, out, 
     `out` must hold the six preallocated gradient tensors (dQ, dK, dV, dtQ, dtK, dtV): this wrapper, like the
     C entry point behind it, allocates nothing.  B*H*N may not exceed NOALLOC_MAX_ROWS.  Calls that may overlap
     on the GPU race on the shared scratch; the first call on a device should come before any stream capture."""
-    lib = load()
-    _check_tensors(Q, tuple(t for t in (tQ, O, tO, dO, dtO, out[0], out[3]) if t is not None))
-    _check_tensors(K, tuple(t for t in (V, tK, tV, out[1], out[2], out[4], out[5]) if t is not None))
-    p = _params(Q, scale, flags, K)
-    with torch.cuda.device(Q.device):
-        rc = lib.tvm_attn_jvp_bwd_noalloc(ctypes.byref(p), Q.data_ptr(), K.data_ptr(), V.data_ptr(), tQ.data_ptr(),
-                                          tK.data_ptr(), tV.data_ptr(), O.data_ptr(), tO.data_ptr(), lse.data_ptr(),
-                                          mu.data_ptr(), _ptr(dO), _ptr(dtO), *[_ptr(o) for o in out],
-                                          _stream_ptr(stream))
-    if rc != 0:
-        _raise("tvm_attn_jvp_bwd_noalloc", rc)
-    return tuple(out)
-
-
-def _check_scale(g, ref):
-    if g.dtype != torch.float32 or g.dim() != 1 or g.numel() != ref.shape[-1] or g.device != ref.device or not g.is_contiguous():
-        raise ValueError("a scale must be a contiguous float32 CUDA vector of d elements")
+    r = (_native or _load_native()).bwd(Q, K, V, tQ, tK, tV, O, tO, lse, mu, dO, dtO, scale, flags, out, None,
+                                        None if stream is None else stream.cuda_stream, True)
+    if r.__class__ is int:
+        _raise("tvm_attn_jvp_bwd_noalloc", r)
+    return r
 
 
 def tvm_qk_rmsnorm_jvp_fwd(Q, tQ, K, tK, gQ, gK, eps=1e-6, stream=None):
     """RMSNorm QK-normalisation with a tangent: returns (Qn, tQn, Kn, tKn)."""
-    lib = load()
-    _check_tensors(Q, (tQ,))
-    _check_tensors(K, (tK,))
-    _check_scale(gQ, Q)
-    _check_scale(gK, Q)
-    p = _params(Q, 0.0, 0, K)
-    outs = (_like(Q), _like(Q), _like(K), _like(K))
-    with torch.cuda.device(Q.device):
-        rc = lib.tvm_qk_rmsnorm_jvp_fwd(ctypes.byref(p), float(eps), Q.data_ptr(), tQ.data_ptr(), K.data_ptr(), tK.data_ptr(),
-                                        gQ.data_ptr(), gK.data_ptr(), *[o.data_ptr() for o in outs], _stream_ptr(stream))
-    if rc != 0:
-        _raise("tvm_qk_rmsnorm_jvp_fwd", rc)
-    return outs
+    r = (_native or _load_native()).norm_fwd(Q, tQ, K, tK, gQ, gK, eps, None if stream is None else stream.cuda_stream)
+    if r.__class__ is int:
+        _raise("tvm_qk_rmsnorm_jvp_fwd", r)
+    return r
 
 
 def tvm_qk_rmsnorm_jvp_bwd(Q, tQ, K, tK, gQ, gK, dQn, dtQn, dKn, dtKn, eps=1e-6, workspace=None, stream=None):
     """Backward of the normalisation: returns (dQ, dtQ, dK, dtK, dgQ, dgK)."""
-    lib = load()
-    _check_tensors(Q, (tQ, dQn, dtQn))
-    _check_tensors(K, (tK, dKn, dtKn))
-    _check_scale(gQ, Q)
-    _check_scale(gK, Q)
-    p = _params(Q, 0.0, 0, K)
-    need = int(lib.tvm_qk_rmsnorm_jvp_workspace_bytes(ctypes.byref(p)))
-    if workspace is None:
-        workspace = torch.empty(max(need, 16), dtype=torch.uint8, device=Q.device)
-    outs = (_like(Q), _like(Q), _like(K), _like(K))
-    dgQ, dgK = torch.empty_like(gQ), torch.empty_like(gK)
-    with torch.cuda.device(Q.device):
-        rc = lib.tvm_qk_rmsnorm_jvp_bwd(ctypes.byref(p), float(eps), Q.data_ptr(), tQ.data_ptr(), K.data_ptr(), tK.data_ptr(),
-                                        gQ.data_ptr(), gK.data_ptr(), dQn.data_ptr(), dtQn.data_ptr(), dKn.data_ptr(),
-                                        dtKn.data_ptr(), *[o.data_ptr() for o in outs], dgQ.data_ptr(), dgK.data_ptr(),
-                                        workspace.data_ptr(), workspace.numel(), _stream_ptr(stream))
-    if rc != 0:
-        _raise("tvm_qk_rmsnorm_jvp_bwd", rc)
-    return outs + (dgQ, dgK)
+    r = (_native or _load_native()).norm_bwd(Q, tQ, K, tK, gQ, gK, dQn, dtQn, dKn, dtKn, eps, workspace,
+                                             None if stream is None else stream.cuda_stream)
+    if r.__class__ is int:
+        _raise("tvm_qk_rmsnorm_jvp_bwd", r)
+    return r
 
 
 def tvm_attn_check_status(stream=None, raise_on_error=True):

@@ -1,6 +1,8 @@
-"""Builds the CUDA library in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds the CUDA library in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the native half of its
+Python binding with g++ against the installed PyTorch."""
 import os
 import subprocess
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
@@ -8,6 +10,8 @@ CSRC = os.path.join(_HERE, "csrc")
 LIB_DIR = os.path.join(_HERE, "_lib")
 LIB_PATH = os.path.join(LIB_DIR, "libtvm_attn.so")
 SOURCES = ["tvm_attn_api.cu"]
+BINDING_PATH = os.path.join(LIB_DIR, "_tvm_binding.so")
+BINDING_SOURCE = os.path.join(CSRC, "torch_binding.cpp")
 
 
 def _newest_source_mtime():
@@ -25,22 +29,49 @@ def nvcc_command(out_path, extra=()):
             *extra, "-o", out_path, *[os.path.join(CSRC, s) for s in SOURCES]]
 
 
-def build(force=False, verbose=False, out_path=None):
-    """Compiles libtvm_attn.so if it is missing or older than its sources; returns its path.
-    `out_path` writes the library somewhere else."""
-    global_out = out_path or LIB_PATH
-    if not force and os.path.exists(global_out) and os.path.getmtime(global_out) >= _newest_source_mtime():
-        return global_out
-    os.makedirs(os.path.dirname(global_out), exist_ok=True)
-    tmp = global_out + ".tmp.%d" % os.getpid()
-    extra = ("-Xptxas", "-v") if verbose else ()
-    cmd = nvcc_command(tmp, extra)
+def binding_command(out_path):
+    import torch
+    root = os.path.dirname(torch.__file__)
+    libs = [os.path.join(root, "lib"), "/usr/local/cuda/lib64"]
+    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), "-I", os.path.join(_ROOT, "include"),
+            "-isystem", os.path.join(root, "include"), "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+            "-isystem", "/usr/local/cuda/include", "-isystem", sysconfig.get_paths()["include"], BINDING_SOURCE, "-o", out_path,
+            *["-L" + d for d in libs], "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch", "-ltorch_python"]
+
+
+def build_binding(force=False):
+    """Compiles _tvm_binding.so if it is missing or older than its source; returns its path."""
+    header = os.path.join(_ROOT, "include", "tvm_attn.h")
+    if not force and os.path.exists(BINDING_PATH) and os.path.getmtime(BINDING_PATH) >= max(os.path.getmtime(f) for f in (BINDING_SOURCE, header)):
+        return BINDING_PATH
+    _run(binding_command, BINDING_PATH)
+    return BINDING_PATH
+
+
+def _run(command, path, *args):
+    """Runs command(temporary path, ...) and moves what it wrote to `path`; returns its messages."""
+    os.makedirs(os.path.dirname(path), exist_ok=True)
+    tmp = path + ".tmp.%d" % os.getpid()
+    cmd = command(tmp, *args)
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
-        raise RuntimeError("nvcc failed:\n%s\n%s" % (" ".join(cmd), res.stderr[-8000:]))
+        raise RuntimeError("compilation failed:\n%s\n%s" % (" ".join(cmd), res.stderr[-8000:]))
+    os.replace(tmp, path)
+    return res.stderr
+
+
+def build(force=False, verbose=False, out_path=None):
+    """Compiles libtvm_attn.so if it is missing or older than its sources; returns its path.
+    `out_path` writes the library somewhere else.  The binding's native half is built along with the in-tree library."""
+    global_out = out_path or LIB_PATH
+    if out_path is None:
+        build_binding(force)
+    if not force and os.path.exists(global_out) and os.path.getmtime(global_out) >= _newest_source_mtime():
+        return global_out
+    messages = _run(nvcc_command, global_out, ("-Xptxas", "-v") if verbose else ())
     if verbose:
-        print(res.stderr)
-    os.replace(tmp, global_out)
+        print(messages)
     return global_out
 
 

@@ -22,21 +22,69 @@ namespace tvm_attn {
 
 static std::atomic<uint64_t> g_launches{0};
 
-// Number of SMs of the current device (a fact of the hardware: looked up once per device index); <= 0 on error.
-static int device_sm_count() {
-    static std::atomic<int> cached[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return -1;
-    if (dev < 64) {
-        const int v = cached[dev].load(std::memory_order_relaxed);
-        if (v > 0) return v;
-    }
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return -1;
-    if (dev < 64) cached[dev].store(sms, std::memory_order_relaxed);
-    return sms;
-}
 __device__ int g_status_word = 0;  // raised by a tensor-core kernel whose bounded wait ran out
+
+// What a call needs to know about the current device, looked up once per thread and CUDA context (the lookups cost a
+// small call as much as a launch): a context's id is never used again in a process, so a device reset or a switch of
+// devices is a new lookup.
+struct DeviceFacts {
+    unsigned long long ctx = 0;
+    int sms = 0, major = 0;
+    int* status = nullptr;   // device address of g_status_word
+};
+
+// Driver functions, by the runtime's entry-point lookup (the library does not link the driver).
+template <typename F>
+static F driver_function(const char* name) {
+    void* sym = nullptr;
+    cudaDriverEntryPointQueryResult qres;
+    if (cudaGetDriverEntryPoint(name, &sym, cudaEnableDefault, &qres) != cudaSuccess || qres != cudaDriverEntryPointSuccess) return nullptr;
+    return reinterpret_cast<F>(sym);
+}
+
+// Id of the calling thread's CUDA context, initialising the device if it has none yet; 0 on error.
+static unsigned long long context_id() {
+    static const auto get_current = driver_function<CUresult (*)(CUcontext*)>("cuCtxGetCurrent");
+    static const auto get_id = driver_function<CUresult (*)(CUcontext, unsigned long long*)>("cuCtxGetId");
+    if (!get_current || !get_id) return 0;
+    CUcontext ctx = nullptr;
+    if (get_current(&ctx) != CUDA_SUCCESS) return 0;
+    if (!ctx && (cudaFree(nullptr) != cudaSuccess || get_current(&ctx) != CUDA_SUCCESS || !ctx)) return 0;
+    unsigned long long id = 0;
+    return get_id(ctx, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+static const DeviceFacts* device_facts() {
+    thread_local DeviceFacts facts;
+    const unsigned long long ctx = context_id();
+    if (ctx == 0) return nullptr;
+    if (facts.ctx == ctx) return &facts;
+    DeviceFacts f;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&f.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&f.major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess || f.sms <= 0 ||
+        cudaGetSymbolAddress(reinterpret_cast<void**>(&f.status), g_status_word) != cudaSuccess || !f.status)
+        return nullptr;
+    f.ctx = ctx;
+    facts = f;
+    return &facts;
+}
+
+// The facts of a device that runs the tensor-core kernels.
+static int tensor_core_device(const DeviceFacts** f) {
+    *f = device_facts();
+    return !*f ? TVM_ATTN_CUDA_ERROR : (*f)->major == 10 ? TVM_ATTN_OK : TVM_ATTN_UNSUPPORTED;
+}
+
+// Lets `kern` use `bytes` of dynamic shared memory: set once per thread, context and kernel (KERN is its identity).
+template <auto KERN>
+static bool allow_smem(const DeviceFacts& f, int bytes) {
+    thread_local unsigned long long done = 0;
+    if (done == f.ctx) return true;
+    if (cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+    done = f.ctx;
+    return true;
+}
 
 // Optional per-kernel timing: events recorded around each launch of the most recent call.  While it is
 // disabled (the normal state) a call only reads the atomic flag, so concurrent calls from several host
@@ -181,15 +229,7 @@ typedef CUresult (*encode_tiled_fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_
                                     CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 static encode_tiled_fn get_encode_fn() {
-    static encode_tiled_fn fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void* sym = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &qres) == cudaSuccess &&
-            qres == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<encode_tiled_fn>(sym);
-    });
+    static const encode_tiled_fn fn = driver_function<encode_tiled_fn>("cuTensorMapEncodeTiled");
     return fn;
 }
 
@@ -222,22 +262,9 @@ static int make_tmap3(CUtensorMap* m, const void* ptr, const Shape& s, int rows)
     return r == CUDA_SUCCESS ? TVM_ATTN_OK : TVM_ATTN_CUDA_ERROR;
 }
 
-static int device_is_sm100() {
-    int dev = 0, major = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return TVM_ATTN_CUDA_ERROR;
-    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return TVM_ATTN_CUDA_ERROR;
-    return major == 10 ? TVM_ATTN_OK : TVM_ATTN_UNSUPPORTED;
-}
-
-static int* status_word_ptr() {
-    int* ptr = nullptr;
-    if (cudaGetSymbolAddress(reinterpret_cast<void**>(&ptr), g_status_word) != cudaSuccess) return nullptr;
-    return ptr;
-}
-
 template <int MODE, int NA>
 static int launch_tc(const Shape& s, const void* const own[4], const void* const strm[4], const TcParams& prm,
-                     cudaStream_t st) {
+                     const DeviceFacts& dev, cudaStream_t st) {
     using C = TcCfg<MODE, NA>;
     CUtensorMap mo[4], ms[4];
     for (int t = 0; t < 4; ++t) {
@@ -248,8 +275,7 @@ static int launch_tc(const Shape& s, const void* const own[4], const void* const
         if (rc != TVM_ATTN_OK) return rc;
     }
     auto kern = dual_attn_kernel<MODE, NA>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES) != cudaSuccess)
-        return TVM_ATTN_CUDA_ERROR;
+    if (!allow_smem<dual_attn_kernel<MODE, NA>>(dev, C::SMEM_BYTES)) return TVM_ATTN_CUDA_ERROR;
     const long long grid = s.BH * ((s.N + TC_OWN_ROWS - 1) / TC_OWN_ROWS);
     g_prof.before(st);
     kern<<<(unsigned)grid, TC_THREADS, C::SMEM_BYTES, st>>>(mo[0], mo[1], mo[2], mo[3], ms[0], ms[1], ms[2], ms[3], prm);
@@ -260,13 +286,13 @@ static int launch_tc(const Shape& s, const void* const own[4], const void* const
 
 template <int MODE>
 static int launch_tc_na(const Shape& s, const void* const own[4], const void* const strm[4], const TcParams& prm,
-                        cudaStream_t st) {
-    return s.d <= 64 ? launch_tc<MODE, 1>(s, own, strm, prm, st) : launch_tc<MODE, 2>(s, own, strm, prm, st);
+                        const DeviceFacts& dev, cudaStream_t st) {
+    return launch_tc<MODE, 2>(s, own, strm, prm, dev, st);   // head dims above 80
 }
 
 // Forward for padded head dims up to 80: operands Q, tQ live in tensor memory (jvp_fwd_sm100.cuh).
 template <int DP>
-static int launch_fwd(const Shape& s, const void* const strm[4], const FwdParams& prm, cudaStream_t st) {
+static int launch_fwd(const Shape& s, const void* const strm[4], const FwdParams& prm, const DeviceFacts& dev, cudaStream_t st) {
     using C = FwdCfg<DP>;
     CUtensorMap m[4];
     for (int t = 0; t < 4; ++t) {
@@ -274,14 +300,11 @@ static int launch_fwd(const Shape& s, const void* const strm[4], const FwdParams
         if (rc != TVM_ATTN_OK) return rc;
     }
     auto kern = jvp_fwd_kernel<DP>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES) != cudaSuccess)
-        return TVM_ATTN_CUDA_ERROR;
+    if (!allow_smem<jvp_fwd_kernel<DP>>(dev, C::SMEM_BYTES)) return TVM_ATTN_CUDA_ERROR;
     // one CTA per SM (each needs the whole tensor memory and most of the shared memory of one); the work
     // items go round-robin over them
     const long long items = s.BH * ((s.M + FWD_ROWS - 1) / FWD_ROWS);
-    const int sms = device_sm_count();
-    if (sms <= 0) return TVM_ATTN_CUDA_ERROR;
-    const long long grid = items < sms ? items : sms;
+    const long long grid = items < dev.sms ? items : dev.sms;
     g_prof.before(st);
     kern<<<(unsigned)grid, FWD_THREADS, C::SMEM_BYTES, st>>>(m[0], m[1], m[2], m[3], prm);
     g_prof.after(st);
@@ -291,7 +314,8 @@ static int launch_fwd(const Shape& s, const void* const strm[4], const FwdParams
 
 // One backward pass for padded head dims up to 80 (jvp_bwd_sm100.cuh).  own: X0..X3; strm: E ring (0, 1), L ring (2, 3).
 template <int MODE, int DP>
-static int launch_bwd_pass(const Shape& s, const void* const own[4], const void* const strm[4], BwdParams prm, cudaStream_t st) {
+static int launch_bwd_pass(const Shape& s, const void* const own[4], const void* const strm[4], BwdParams prm,
+                           const DeviceFacts& dev, cudaStream_t st) {
     using C = BwdCfg<MODE, DP>;
     CUtensorMap ms[4], mo[2];
     // DV, DK: keys own, queries stream; DQ: queries own, keys stream
@@ -311,15 +335,14 @@ static int launch_bwd_pass(const Shape& s, const void* const own[4], const void*
     // dtO absent: the specialisation that leaves the tangent path out (only instantiated for the padded head dims
     // 64 and 80 of the transformer shapes; other head dims run the general kernel, which skips what it can)
     constexpr bool HAS_HZ = DP == 64 || DP == 80;
-    auto kern = (HAS_HZ && (prm.absent & ABSENT_HC)) ? jvp_bwd_kernel<MODE, DP, HAS_HZ> : jvp_bwd_kernel<MODE, DP, false>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES) != cudaSuccess)
+    const bool hz = HAS_HZ && (prm.absent & ABSENT_HC);
+    auto kern = hz ? jvp_bwd_kernel<MODE, DP, HAS_HZ> : jvp_bwd_kernel<MODE, DP, false>;
+    if (!(hz ? allow_smem<jvp_bwd_kernel<MODE, DP, HAS_HZ>>(dev, C::SMEM_BYTES) : allow_smem<jvp_bwd_kernel<MODE, DP, false>>(dev, C::SMEM_BYTES)))
         return TVM_ATTN_CUDA_ERROR;
     // one CTA per SM (each needs the whole tensor memory and most of the shared memory of one); the work
     // items go round-robin over them
     const long long items = s.BH * ((prm.o.rows + BWD_ROWS - 1) / BWD_ROWS);
-    const int sms = device_sm_count();
-    if (sms <= 0) return TVM_ATTN_CUDA_ERROR;
-    const long long grid = items < sms ? items : sms;
+    const long long grid = items < dev.sms ? items : dev.sms;
     g_prof.before(st);
     {
         // DK and DQ read nothing that the pass before them writes (DV, DK and DQ all depend on the row-sums
@@ -349,13 +372,13 @@ static int launch_bwd_pass(const Shape& s, const void* const own[4], const void*
 
 template <int MODE>
 static int launch_bwd_pass_dp(const Shape& s, const void* const own[4], const void* const strm[4], const BwdParams& prm,
-                              cudaStream_t st) {
+                              const DeviceFacts& dev, cudaStream_t st) {
     switch (s.dp) {
-        case 16: return launch_bwd_pass<MODE, 16>(s, own, strm, prm, st);
-        case 32: return launch_bwd_pass<MODE, 32>(s, own, strm, prm, st);
-        case 48: return launch_bwd_pass<MODE, 48>(s, own, strm, prm, st);
-        case 64: return launch_bwd_pass<MODE, 64>(s, own, strm, prm, st);
-        default: return launch_bwd_pass<MODE, 80>(s, own, strm, prm, st);
+        case 16: return launch_bwd_pass<MODE, 16>(s, own, strm, prm, dev, st);
+        case 32: return launch_bwd_pass<MODE, 32>(s, own, strm, prm, dev, st);
+        case 48: return launch_bwd_pass<MODE, 48>(s, own, strm, prm, dev, st);
+        case 64: return launch_bwd_pass<MODE, 64>(s, own, strm, prm, dev, st);
+        default: return launch_bwd_pass<MODE, 80>(s, own, strm, prm, dev, st);
     }
 }
 
@@ -533,10 +556,10 @@ int tvm_attn_jvp_fwd(const tvm_attn_params* p, const void* Q, const void* K, con
         return s.fp32 ? simt_fwd<float>(s, Q, K, V, tQ, tK, tV, O, tO, lse, mu, st)
                       : simt_fwd<__nv_bfloat16>(s, Q, K, V, tQ, tK, tV, O, tO, lse, mu, st);
     }
-    rc = device_is_sm100();
+    const DeviceFacts* dev;
+    rc = tensor_core_device(&dev);
     if (rc != TVM_ATTN_OK) return rc;
-    int* status = status_word_ptr();
-    if (!status) return TVM_ATTN_CUDA_ERROR;
+    int* status = dev->status;
     const void* strm[4] = {K, tK, V, tV};
     if (s.dp <= 80) {
         FwdParams f;
@@ -548,18 +571,18 @@ int tvm_attn_jvp_fwd(const tvm_attn_params* p, const void* Q, const void* K, con
         f.O = static_cast<__nv_bfloat16*>(O); f.tO = static_cast<__nv_bfloat16*>(tO);
         f.lse = lse; f.mu = mu; f.status = status;
         switch (s.dp) {
-            case 16: return launch_fwd<16>(s, strm, f, st);
-            case 32: return launch_fwd<32>(s, strm, f, st);
-            case 48: return launch_fwd<48>(s, strm, f, st);
-            case 64: return launch_fwd<64>(s, strm, f, st);
-            default: return launch_fwd<80>(s, strm, f, st);
+            case 16: return launch_fwd<16>(s, strm, f, *dev, st);
+            case 32: return launch_fwd<32>(s, strm, f, *dev, st);
+            case 48: return launch_fwd<48>(s, strm, f, *dev, st);
+            case 64: return launch_fwd<64>(s, strm, f, *dev, st);
+            default: return launch_fwd<80>(s, strm, f, *dev, st);
         }
     }
     if (!s.plain) return TVM_ATTN_UNSUPPORTED;  // head dims above 80: self-attention on packed tensors only
     TcParams prm = base_params(s, status);
     prm.out0 = O; prm.out1 = tO; prm.lse_out = lse; prm.mu_out = mu;
     const void* own[4] = {Q, tQ, Q, tQ};
-    return launch_tc_na<MODE_FWD>(s, own, strm, prm, st);
+    return launch_tc_na<MODE_FWD>(s, own, strm, prm, *dev, st);
 }
 
 int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, const void* V, const void* tQ,
@@ -610,10 +633,10 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
         if (rc != TVM_ATTN_OK) return rc;
         return simt_bwd<__nv_bfloat16>(s, Q, K, V, tQ, tK, tV, lse, mu, dO, dtO, sig1, cvec, dQ, dK, dV, dtQ, dtK, dtV, st);
     }
-    rc = device_is_sm100();
+    const DeviceFacts* dev;
+    rc = tensor_core_device(&dev);
     if (rc != TVM_ATTN_OK) return rc;
-    int* status = status_word_ptr();
-    if (!status) return TVM_ATTN_CUDA_ERROR;
+    int* status = dev->status;
     rc = launch_rowsums<__nv_bfloat16>(s, dO, dtO, O, tO, lse, sig1, cvec, lse2, st);
     if (rc != TVM_ATTN_OK) return rc;
     if (s.dp <= 80) {
@@ -627,7 +650,7 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
             q.out0 = dtO ? static_cast<__nv_bfloat16*>(dtV) : nullptr; q.out1 = static_cast<__nv_bfloat16*>(dV);
             const void* own[4] = {K, tK, K, tK};
             const void* strm[4] = {Q, tQ, dtO, dO};
-            rc = launch_bwd_pass_dp<BWD_DV>(s, own, strm, q, st);
+            rc = launch_bwd_pass_dp<BWD_DV>(s, own, strm, q, *dev, st);
             if (rc != TVM_ATTN_OK) return rc;
         }
         {   // dtK = alpha W^T Q, dK = alpha (dA^T Q + W^T tQ) : owner keys (K, tK, V, tV); stream (Hc, G | Q, tQ)
@@ -635,7 +658,7 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
             q.out0 = dtO ? static_cast<__nv_bfloat16*>(dtK) : nullptr; q.out1 = static_cast<__nv_bfloat16*>(dK);
             const void* own[4] = {K, tK, V, tV};
             const void* strm[4] = {dtO, dO, Q, tQ};
-            rc = launch_bwd_pass_dp<BWD_DK>(s, own, strm, q, st);
+            rc = launch_bwd_pass_dp<BWD_DK>(s, own, strm, q, *dev, st);
             if (rc != TVM_ATTN_OK) return rc;
         }
         {   // dtQ = alpha W K, dQ = alpha (dA K + W tK) : owner queries (Q, tQ, Hc, G); stream (V, tV | K, tK)
@@ -643,7 +666,7 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
             q.out0 = dtO ? static_cast<__nv_bfloat16*>(dtQ) : nullptr; q.out1 = static_cast<__nv_bfloat16*>(dQ);
             const void* own[4] = {Q, tQ, dtO, dO};
             const void* strm[4] = {V, tV, K, tK};
-            rc = launch_bwd_pass_dp<BWD_DQ>(s, own, strm, q, st);
+            rc = launch_bwd_pass_dp<BWD_DQ>(s, own, strm, q, *dev, st);
         }
         return rc;
     }
@@ -653,21 +676,21 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
         TcParams q = prm; q.out0 = dtV; q.out1 = dV;
         const void* own[4] = {K, tK, K, tK};
         const void* strm[4] = {Q, tQ, dtO, dO};
-        rc = launch_tc_na<MODE_DV>(s, own, strm, q, st);
+        rc = launch_tc_na<MODE_DV>(s, own, strm, q, *dev, st);
         if (rc != TVM_ATTN_OK) return rc;
     }
     {   // dtK = alpha W^T Q, dK = alpha (dA^T Q + W^T tQ) : owner keys (K, tK, V, tV), stream (Q, tQ, Hc, G)
         TcParams q = prm; q.out0 = dtK; q.out1 = dK; q.out_scale = s.alpha;
         const void* own[4] = {K, tK, V, tV};
         const void* strm[4] = {Q, tQ, dtO, dO};
-        rc = launch_tc_na<MODE_DK>(s, own, strm, q, st);
+        rc = launch_tc_na<MODE_DK>(s, own, strm, q, *dev, st);
         if (rc != TVM_ATTN_OK) return rc;
     }
     {   // dtQ = alpha W K, dQ = alpha (dA K + W tK) : owner queries (Q, tQ, Hc, G), stream (K, tK, V, tV)
         TcParams q = prm; q.out0 = dtQ; q.out1 = dQ; q.out_scale = s.alpha;
         const void* own[4] = {Q, tQ, dtO, dO};
         const void* strm[4] = {K, tK, V, tV};
-        rc = launch_tc_na<MODE_DQ>(s, own, strm, q, st);
+        rc = launch_tc_na<MODE_DQ>(s, own, strm, q, *dev, st);
     }
     return rc;
 }
@@ -739,9 +762,9 @@ int tvm_qk_rmsnorm_jvp_bwd(const tvm_attn_params* p, float eps, const void* Q, c
 
 int tvm_attn_selftest_timeout(uint64_t limit_ns, void* cuda_stream) {
     if (limit_ns == 0 || limit_ns > 100ull * 1000ull * 1000ull) return TVM_ATTN_INVALID_ARG;
-    int* status = status_word_ptr();
-    if (!status) return TVM_ATTN_CUDA_ERROR;
-    selftest_timeout_kernel<<<1, 32, 0, static_cast<cudaStream_t>(cuda_stream)>>>(status, limit_ns);
+    const DeviceFacts* dev = device_facts();
+    if (!dev) return TVM_ATTN_CUDA_ERROR;
+    selftest_timeout_kernel<<<1, 32, 0, static_cast<cudaStream_t>(cuda_stream)>>>(dev->status, limit_ns);
     g_launches += 1;
     return cuda_status(cudaGetLastError());
 }
