@@ -18,6 +18,9 @@ struct Geom {
     }
 };
 
+// Absent cotangents of a backward call (null dtO = Hc, null dO = G), as bits.
+enum : int { ABSENT_HC = 1, ABSENT_G = 2 };
+
 #ifdef __CUDACC__
 // Sum of v over the `gs` consecutive lanes of a warp that share a row (lanes sub * gs .. sub * gs + gs - 1), returned
 // to all of them.  A power-of-two group is a butterfly; any other size (nine 16-byte chunks for d = 72) has its first

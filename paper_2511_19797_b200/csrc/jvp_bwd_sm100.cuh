@@ -78,7 +78,6 @@ struct BwdParams {
     // the MMAs whose result would be exactly zero are not issued.  out0 may be null when Hc is absent.
     int absent;
 };
-enum : int { ABSENT_HC = 1, ABSENT_G = 2 };
 
 template <int MODE, int DP>
 struct BwdCfg {

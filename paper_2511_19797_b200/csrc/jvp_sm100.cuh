@@ -1,0 +1,1241 @@
+// Attention with a Jacobian-vector product on sm_100a (tcgen05 + TMEM + TMA): the forward and the three passes of the
+// backward (App. C Eq. "sdpa", the definitions under "Step 1", and "Multi-step backward pass" with the standard
+// attention backward for dO summed in) on one skeleton.
+//
+// Carrying a tangent next to a primal is dual-number arithmetic, (a + eps b)(c + eps d) = ac + eps (bc + ad), so every
+// product of the method has the same shape:
+//
+//   pass  owner rows  stream rows  score accumulators (128 x 64 fp32)                    bf16 operands A0, A1    acc0, acc1 (128 x d)
+//   FWD   queries     keys         S = Q K^T, Sd = tQ K^T + Q tK^T                        P~, P~ (T - c)          O~, R
+//   DV    keys        queries      S^T, Sd^T                                              P^T, (P Nn)^T           dtV, dV          (step 6)
+//   DK    keys        queries      S^T, Sd^T, D^T = V Hc^T, X^T = tV Hc^T + V G^T        W^T, dA^T               dtK/alpha, dK/alpha   (steps 2, 4)
+//   DQ    queries     keys         S, Sd, D = Hc V^T, X = G V^T + Hc tV^T                 W, dA                   dtQ/alpha, dQ/alpha   (steps 3, 5)
+//
+//   score pair:  S = X0 Y0^T,  Sd = X1 Y0^T + X0 Y1^T        outputs:  acc0 += A0 B0,  acc1 += A1 B0 + A0 B1
+//
+// with P = 2^(c2 S - lse2), T = alpha Sd, Nn = T - mu, W = P (D - Sigma1), dA = P (X - c) + W Nn; in the forward
+// P~ = 2^(c2 S - m) with a lazily updated row reference m, and O = O~/l, tO = R/l - (mu - c) O.
+//
+// A work item is 128 owner rows of one head, against which the other side streams in tiles of 64 rows.  The grid has
+// one CTA per SM (a CTA needs the whole tensor memory of one); the items go round-robin over the CTAs, and the rings,
+// the score buffers and all barrier phases run on through the items.
+//
+// 16 warps in four warpgroups:
+//   warp 0    loads the owner tiles and the E ring (stream tensors that only the score MMAs read)
+//   warp 1    issues the MMAs
+//   warp 2    loads the L ring (stream tensors the output MMAs read)
+//   warps 4-11   element-wise work: two groups of four warps take the tiles in turn; a thread has one owner row and all
+//             64 columns of the tile
+//   warps 12-15  epilogue: normalise, convert and store an item's accumulators while the next item is under way
+//
+// Why this split.  What bounds a tile is not one unit but the chain scores -> element-wise work -> outputs: passing an
+// mbarrier costs a warp 100 to 250 cycles even when the phase has completed, reading tensor memory 180.  A warp pays that
+// for every other tile and for all of its columns, and nothing is exchanged between warps that share a row (the forward's
+// row maximum is the thread's own).
+//
+// Score MMAs: the two tensors of a stage are interleaved so that they form one K-major operand of 128 rows, and
+// [S | X0 Y1^T] = X0 [Y0 | Y1]^T is one N = 128 MMA per k-step, Sd += X1 Y0^T one N = 64 MMA.
+//
+// Measured on B200 at d = 128 (B 2, H 24, N 4096; one CTA per item, 32-key tiles with all four accumulators in two buffers
+// before): forward 1.40 -> 1.08 ms, DV / DK / DQ 1.33 / 2.82 / 2.92 -> 1.06 / 1.48 / 1.42 ms.
+//
+// Every wait on an mbarrier is bounded; when one gives up the block records a time-out status and all roles leave their
+// loops.
+#pragma once
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <math_constants.h>
+#include <stdint.h>
+#include <type_traits>
+
+#include "geometry.cuh"
+#include "sm100_ptx.cuh"
+
+namespace tvm_attn {
+
+enum : int { PASS_FWD = 0, PASS_DV = 1, PASS_DK = 2, PASS_DQ = 3 };
+
+constexpr int JVP_THREADS = 512;
+constexpr int JVP_ROWS = 128;   // owner rows per item
+constexpr int JVP_BC = 64;      // stream rows per tile
+// Forward, how far the row reference m may lag behind the running maximum (log2 units), and for WIDE head dims how far the
+// centre c of the tangent weights may be from T at the arg-max key before it moves.
+constexpr float JVP_LAZY_LOG2 = 3.0f, JVP_LAZY_LOG2_WIDE = 8.0f, JVP_CENTRE_WIDE = 3.0f;
+constexpr uint64_t JVP_WAIT_LIMIT_NS = 200ull * 1000ull * 1000ull;
+// Registers per thread at launch; setmaxnreg moves them between the four warpgroups (JvpCfg::REGS_*) within what the block
+// was launched with: the host refuses to launch a build whose kernels have fewer.
+constexpr int JVP_REGS = 128;
+
+struct JvpParams {
+    int d, BH, H;
+    Geom o, s;    // owner side and stream side of this pass (FWD, DQ: queries own, keys stream; DV, DK: the other way round)
+    float alpha;      // softmax scale
+    float c2;         // alpha * log2(e)
+    float out_scale;  // factor applied to acc0 / acc1 of the backward passes
+    const __nv_bfloat16* own[4];   // owner tensors X0..X3 (X2, X3: DK, DQ)
+    const __nv_bfloat16* strm[4];  // streamed tensors: E ring (0, 1), L ring (2, 3)
+    __nv_bfloat16* out0;           // acc0 destination: O | dtV | dtK | dtQ
+    __nv_bfloat16* out1;           // acc1 destination: tO | dV | dK | dQ
+    float* lse;                    // FWD: statistics written, packed (B, H, M)
+    float* mu_out;
+    // backward: statistics read, packed (B, H, M); the pre-pass writes the negated ones
+    const float* nlse2;  // -lse * log2(e)
+    const float* mu;
+    const float* nsig1;  // -rowsum(dtO * O)
+    const float* ncvec;  // -rowsum(dO * O) - rowsum(dtO * tO)
+    int* status;         // device status word; non-zero makes the kernel a no-op
+    // Absent cotangents (a null dO or dtO means zero; Sec. 5.3 "detach JVP" is dtO absent): bit 0 = Hc (dtO),
+    // bit 1 = G (dO).  An absent tensor is never loaded; where an MMA still reads its tile, the tile is zeroed once,
+    // and the MMAs whose result would be exactly zero are not issued.  out0 may be null when Hc is absent.
+    int absent;
+};
+
+template <int MODE, int DP>
+struct JvpCfg {
+    static_assert(DP % 16 == 0 && DP >= 16 && DP <= 128, "padded head dim must be 16..128");
+    static constexpr int NPAIR = MODE == PASS_DK || MODE == PASS_DQ ? 2 : 1;   // score pairs
+    static constexpr bool TRANSPOSED = MODE == PASS_DV || MODE == PASS_DK;     // owner rows are keys
+    static constexpr int BC = JVP_BC, KS = DP / 16;
+    static constexpr int NA = DP > 64 ? 2 : 1;             // 64-column swizzle atoms per row
+    // How the columns from 64 on arrive.  Up to 16 of them (DP = 80): 16-byte asynchronous copies, because a 64-column
+    // box hanging over the end of a 144-byte row reads the next row from L2 for nothing; tiles that are only read
+    // K-major (owners, E ring) keep them in an unswizzled block [chunk][row][16 bytes] behind the first atom.  More
+    // than 16 (WIDE): a second box and a second swizzle atom everywhere.
+    static constexpr bool WIDE = DP > 80;
+    static constexpr bool TAIL = NA == 2 && !WIDE;
+    // Owner operands.  The pair of the score MMAs on the tile's critical chain (FWD, DV: the only pair; DK, DQ: the second)
+    // lies in tensor memory as bf16 A operands: an MMA with A in shared memory moves 4 KB of A per k-step through the
+    // shared-memory port.  WIDE: tensor memory has no room, everything is in shared memory.
+    static constexpr bool XT = !WIDE;
+    static constexpr int NOWN = 2 * NPAIR - (XT ? 2 : 0);   // owner tensors in shared memory
+    // FOLD (DV, DK): the per-query statistics belong to the columns of the tile, the same for every thread; read from
+    // shared memory they would cost 512 bytes a warp and column.  Instead they are an extra piece of the score MMAs: each
+    // is split into three bf16 parts in columns of its own behind the stream row, against ones behind the owner row, so
+    // that the accumulators arrive as S - lse/alpha, Sd - mu/alpha, D - Sigma1, X - c.  At d = 72 these columns are the
+    // padding up to 80; other head dims take one more k-step of N = 128.
+    static constexpr bool FOLD = TRANSPOSED && !WIDE;
+    static constexpr int OWN_ATOM = JVP_ROWS * 128, ATOM = BC * 128;
+    static constexpr int OWN_BYTES = OWN_ATOM * (WIDE ? 2 : 1) + (TAIL ? JVP_ROWS * 32 : 0);   // one owner tensor
+    static constexpr int EST_BYTES = ATOM * (WIDE ? 2 : 1) + (TAIL ? BC * 32 : 0);             // one E-ring tile
+    static constexpr int LST_BYTES = ATOM * NA;                                                // one L-ring tile
+    static constexpr int SE = WIDE ? (NPAIR == 2 ? 1 : 2) : TAIL ? 3 : 4;
+    static constexpr int SL = WIDE ? 2 : TAIL && NPAIR == 2 ? 3 : 4;
+    static constexpr int TILE_BYTES = NOWN * OWN_BYTES + SE * 2 * EST_BYTES + SL * 2 * LST_BYTES;
+    // FOLD: statistics of a stage, [Y0 rows, Y1 rows][16 bytes], for the rings the score MMAs read; ones and zeros
+    static constexpr int FOLD_BYTES = 2 * BC * 16;
+    static constexpr int FOLD_E = FOLD ? SE : 0, FOLD_L = FOLD && NPAIR == 2 ? SL : 0;
+    static constexpr int ONES_BYTES = FOLD ? JVP_ROWS * 32 : 0;
+    static constexpr int EFULL_COUNT = TAIL ? 33 : 1;                    // TMA issuer (+ each lane's own copies)
+    static constexpr int LFULL_COUNT = TAIL || (TRANSPOSED && !FOLD) ? 33 : 1;
+    // TMEM columns: accumulators, the owner operands in the gaps behind them (and 8 columns of ones behind the first),
+    // score accumulators (FWD, DV: two buffers of S | Sd; DK, DQ: one of S | Sd | D | X).
+    static constexpr int COL_ACC0 = 0, COL_ACC1 = XT ? 128 : DP, COL_SCORE = 2 * COL_ACC1;
+    static constexpr int COL_X0 = DP, COL_X1 = COL_ACC1 + DP, COL_ONES = COL_X0 + DP / 2;
+    static_assert(!XT || DP + DP / 2 + 8 <= 128, "operands do not fit behind their accumulators");
+    static_assert(COL_SCORE + 4 * BC <= 512, "TMEM over-subscribed");
+    // registers per thread: warpgroup 0, element-wise warps, epilogue warps (which hold an owner row, 4 registers a chunk)
+    static constexpr int REGS_LOAD = MODE == PASS_FWD ? 56 : 64, REGS_ELEM = MODE == PASS_FWD ? 184 : MODE == PASS_DV ? 168 : 176,
+                         REGS_EPI = MODE == PASS_FWD ? 88 : MODE == PASS_DV ? 112 : 96;
+    static_assert(REGS_LOAD + 2 * REGS_ELEM + REGS_EPI <= 4 * JVP_REGS, "more registers than the block has");
+    // barriers
+    static constexpr int B_EFULL = 0;
+    static constexpr int B_LFULL = B_EFULL + SE;
+    static constexpr int B_OWN = B_LFULL + SL;                         // owner tiles in shared memory loaded
+    static constexpr int B_OWNFREE = B_OWN + 1;                        // ... free: the score MMAs of the item are complete
+    static constexpr int B_XRDY = B_OWNFREE + 1;                       // owner operands in tensor memory written
+    static constexpr int B_XFREE = B_XRDY + 1;                         // ... free
+    // MMAs of tile g complete: + (g & 3), phase g >> 2.  The element-wise groups meet every other tile only and the
+    // producers run up to four tiles ahead of or behind the others, so that a parity wait on one barrier, or on a pair,
+    // could take another tile's completion for its own.  They also tell the producers that a ring stage is free: a commit
+    // costs the issuing warp 60 cycles, and a barrier of its own per ring would be one more per tile.
+    static constexpr int B_SFULL = B_XFREE + 1;                        // S (and Sd, except in FWD) written
+    static constexpr int B_XFULL = B_SFULL + 4;                        // FWD: Sd written; DK, DQ: D, X written
+    static constexpr int B_OUTDONE = B_XFULL + 4;                      // output MMAs complete
+    static constexpr int B_EDONE = MODE == PASS_DV ? B_SFULL : B_XFULL;   // the E stage of the tile is free
+    static_assert(SE <= 4 && SL <= 4, "a ring deeper than the completion barriers");
+    // operands written: + half of the tile (DK, DQ), + 2 (g & 1) + half (FWD, DV)
+    static constexpr int B_PREADY = B_OUTDONE + 4;
+    static constexpr int B_SREAD = B_PREADY + 4;                       // DK, DQ: S, Sd read
+    static constexpr int B_FINAL = B_SREAD + 1;                        // the item's last output MMAs complete
+    static constexpr int B_ACCFREE = B_FINAL + 1;                      // the epilogue has read the accumulators
+    static constexpr int B_TURN = B_ACCFREE + 1;                       // FWD: + lane quadrant: row state of the tile decided
+    static constexpr int B_ROWSTAT = B_TURN + 4;                       // FWD: the item's row sums written
+    static constexpr int B_DRAIN = B_ROWSTAT + 1;                      // used once, while winding down after a time-out
+    static constexpr int NBARS = B_DRAIN + 1;
+    static_assert(NBARS <= 56, "barrier table too small");
+    static constexpr int NSTAT = 2 * NPAIR;                            // statistics per query: lse2, mu (, Sigma1, c)
+    static constexpr int STATS_FLOATS = TRANSPOSED && !FOLD ? SL * NSTAT * BC : 0;
+    static constexpr int FWD_FLOATS = MODE == PASS_FWD ? 4 * JVP_ROWS + 2 * 4 * JVP_ROWS : 0;   // row state; row sums per group
+    static constexpr int MISC_BYTES = 56 * 8 + 64 + (STATS_FLOATS + FWD_FLOATS) * 4 + (FOLD_E + FOLD_L) * FOLD_BYTES + ONES_BYTES;
+    static constexpr int SMEM_BYTES = TILE_BYTES + MISC_BYTES;         // from a 1024-byte boundary
+    static_assert(SMEM_BYTES <= 227 * 1024, "shared memory over-subscribed");
+};
+
+// What the roles of a block share.
+template <int MODE, int DP>
+struct JvpBlock {
+    using C = JvpCfg<MODE, DP>;
+    uint32_t own, e, l;          // shared-memory addresses of the owner tiles and the rings
+    uint32_t fold_e, fold_l, ones, zeros;   // FOLD: statistics of the E and L stages; ones and zeros, 128 rows of 16 bytes
+    bool fold_step;                  // FOLD: a k-step of their own (else they are the padding columns of the last one)
+    uint32_t bar0;
+    volatile int* abort_flag;
+    float* stats;                // DV, DK, WIDE: [stage][NSTAT][64]
+    float4* row_state;           // FWD: (m, c, running maximum) of each row
+    float4* row_sums;            // FWD: [group][row] (l, sum P~ (T - c), m, c)
+    int items, row_tiles, T;     // work items, items per head, stream tiles per item
+
+    __device__ __forceinline__ uint32_t bar(int i) const { return bar0 + 8u * static_cast<uint32_t>(i); }
+    __device__ __forceinline__ bool wait(int i, int phase) const {
+        return ptx::mbar_wait_warp(bar(i), phase & 1, abort_flag, JVP_WAIT_LIMIT_NS);
+    }
+    __device__ __forceinline__ bool wait2(int i, int pi, int j, int pj) const {
+        return ptx::mbar_wait2_warp(bar(i), pi & 1, bar(j), pj & 1, abort_flag, JVP_WAIT_LIMIT_NS);
+    }
+    // After the waits for a tile: what other warps copied to it (tails) is ordered before the MMAs that read it.
+    __device__ __forceinline__ void tile_fence() const {
+        if (C::TAIL) ptx::fence_proxy_async_smem();
+        ptx::tc_fence_after_sync();
+    }
+    __device__ __forceinline__ bool done(int i, int g) const { return wait(i + (g & 3), g >> 2); }   // i: B_SFULL, B_XFULL, B_OUTDONE
+    __device__ __forceinline__ uint32_t own_tile(int t) const { return own + t * C::OWN_BYTES; }
+    __device__ __forceinline__ uint32_t e_stage(int s) const { return e + s * 2 * C::EST_BYTES; }
+    __device__ __forceinline__ uint32_t l_stage(int s) const { return l + s * 2 * C::LST_BYTES; }
+    // one arrival per warp, after its tensor-memory accesses
+    __device__ __forceinline__ void arrive(int i, int lane) const {
+        ptx::tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(bar(i));
+    }
+};
+
+// ------------------------------------------------------------------------------------------------ producers
+// Owner tiles of an item (by the E ring's warp): two boxes of 64 rows per tensor and atom, like those of the stream tiles,
+// so that one tensor map serves both.
+template <int MODE, int DP>
+__device__ __forceinline__ void jvp_load_owners(const JvpParams& p, const JvpBlock<MODE, DP>& k, const CUtensorMap* const (&maps)[4], int item, int lane) {
+    using C = JvpCfg<MODE, DP>;
+    constexpr int KT = C::TAIL ? (DP - 64) / 8 : 1, H64 = 64 * 128;
+    const int bh = item / k.row_tiles, row0 = (item - bh * k.row_tiles) * JVP_ROWS;
+    const int cb = bh / p.H, ch = bh - cb * p.H;
+    if (lane == 0) {
+        const uint32_t full = k.bar(C::B_OWN);
+        uint32_t tx = 0;
+#pragma unroll
+        for (int t = 0; t < C::NOWN; ++t) tx += p.own[t] ? C::OWN_ATOM * (C::WIDE ? 2 : 1) : 0;   // null: an absent cotangent
+        ptx::mbar_arrive_expect_tx(full, tx);
+#pragma unroll
+        for (int t = 0; t < C::NOWN; ++t) {
+            if (!p.own[t]) continue;   // its tile is zeroed once
+            const uint32_t dst = k.own_tile(t);
+            ptx::tma_load_4d(dst, maps[t], full, 0, row0, ch, cb);
+            ptx::tma_load_4d(dst + H64, maps[t], full, 0, row0 + 64, ch, cb);
+            if (C::WIDE) {
+                ptx::tma_load_4d(dst + C::OWN_ATOM, maps[t], full, 64, row0, ch, cb);
+                ptx::tma_load_4d(dst + C::OWN_ATOM + H64, maps[t], full, 64, row0 + 64, ch, cb);
+            }
+        }
+    }
+    if constexpr (C::TAIL) {
+        const int ntail = (p.d - 64) >> 3, rows_left = p.o.rows - row0;
+        const size_t d32 = 32 * (size_t)p.o.rs, lane_row = p.o.head_off(bh, p.H) + (size_t)(row0 + lane) * (size_t)p.o.rs + 64;
+#pragma unroll
+        for (int t = 0; t < C::NOWN; ++t) {
+            const __nv_bfloat16* x = p.own[t];
+            const uint32_t tile = k.own_tile(t) + C::OWN_ATOM + lane * 16;
+#pragma unroll
+            for (int c = 0; c < KT; ++c) {
+                if (x && c < ntail) {
+#pragma unroll
+                    for (int rp = 0; rp < JVP_ROWS / 32; ++rp) {
+                        const bool v = lane + 32 * rp < rows_left;
+                        ptx::cp_async_16(tile + (c * JVP_ROWS + 32 * rp) * 16, v ? x + lane_row + rp * d32 + 8 * c : x, v ? 16u : 0u);
+                    }
+                }
+            }
+        }
+        ptx::cp_async_arrive(k.bar(C::B_OWN));
+    }
+}
+
+// Three bf16 parts of x whose sum is x to 24 bits, in the first three of eight columns.
+__device__ __forceinline__ uint4 jvp_split3(float x) {
+    const __nv_bfloat16 hi = __float2bfloat16_rn(x);
+    const float r = x - __bfloat162float(hi);
+    const __nv_bfloat16 mid = __float2bfloat16_rn(r);
+    const __nv_bfloat16 lo = __float2bfloat16_rn(r - __bfloat162float(mid));
+    return make_uint4((uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(mid) << 16), __bfloat16_as_ushort(lo), 0u, 0u);
+}
+constexpr uint32_t JVP_ONES0 = 0x3F803F80u, JVP_ONES1 = 0x00003F80u;   // 1, 1, 1, 0 in bf16: what the parts are multiplied by
+
+// One warp per ring; the E ring's loads the owner tiles too.  Lane 0 issues the TMA boxes; with a tail (DP = 80) or
+// statistics copied as they are (WIDE) all lanes copy those, 16 bytes each, and each lane's arrival on the stage's barrier
+// is left to its copies (a warp that waits for them itself loads no more than one tile per memory latency: 1300 cycles a
+// tile).  FOLD: the lanes split the tile's statistics (loaded one tile ahead) and store the parts.
+template <int MODE, int DP, int RING>
+__device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock<MODE, DP>& k, const CUtensorMap* map0, const CUtensorMap* map1,
+                                              const CUtensorMap* const (&own_maps)[4], int lane) {
+    using C = JvpCfg<MODE, DP>;
+    constexpr int BC = C::BC, S = RING == 0 ? C::SE : C::SL, ATOM = C::ATOM;
+    constexpr int b_full = RING == 0 ? C::B_EFULL : C::B_LFULL, b_done = RING == 0 ? C::B_EDONE : C::B_OUTDONE;
+    constexpr uint32_t TB = RING == 0 ? C::EST_BYTES : C::LST_BYTES;
+    constexpr bool STATS = RING == 1 && C::TRANSPOSED && !C::FOLD;   // this ring carries the statistics as they are
+    constexpr bool FOLDED = C::FOLD && (RING == 0 || C::NPAIR == 2);  // ... as columns of the stream rows
+    constexpr bool OWNERS = RING == 0 && C::NOWN > 0;
+    constexpr bool HAS_CP = C::TAIL || STATS;           // the warp has asynchronous copies of its own
+    constexpr int KT = C::TAIL ? (DP - 64) / 8 : 1;     // 16-byte chunks per row behind column 64, at most
+    [[maybe_unused]] const int ntail = C::TAIL ? (p.d - 64) >> 3 : 0;
+    [[maybe_unused]] const size_t d32 = 32 * (size_t)p.s.rs;   // 32 rows further down, in elements
+    [[maybe_unused]] const size_t tile_elems = (size_t)BC * (size_t)p.s.rs;
+    const uint32_t ring_base = RING == 0 ? k.e : k.l;
+    const __nv_bfloat16* base0 = p.strm[2 * RING];
+    const __nv_bfloat16* base1 = p.strm[2 * RING + 1];
+    // the ring that streams the cotangents (Hc, G): L in DV, E in DK; an absent one is not loaded
+    constexpr bool COT = (MODE == PASS_DV && RING == 1) || (MODE == PASS_DK && RING == 0);
+    const bool has0 = !COT || !(p.absent & ABSENT_HC), has1 = !COT || !(p.absent & ABSENT_G);
+    const uint32_t tx_bytes = ((has0 ? 1 : 0) + (has1 ? 1 : 0)) * ATOM * (C::WIDE ? 2 : 1);
+    // Chunk 0 of row `lane` behind the first atoms: compact blocks in the E ring, a second swizzled atom in the L ring.
+    [[maybe_unused]] const uint32_t dst_lane = 2 * ATOM + (RING == 0 ? lane * 16 : lane * 128);
+    [[maybe_unused]] const uint32_t sw = lane & 7;  // rows 32 apart share it
+    // statistics as they are: 16-byte chunks when the rows of the (B, H, M) arrays are 16-byte aligned, else floats
+    [[maybe_unused]] const bool st16 = (p.s.rows & 3) == 0;
+    [[maybe_unused]] const uint32_t st_base = ptx::smem_u32(k.stats);
+    // FOLD: the two statistics of this ring, the factors that bring them to the accumulators' scale, and where the parts of
+    // (tensor t, row lane + 32 rp) go: block + (t, rp steps)
+    constexpr bool COT_STATS = MODE == PASS_DK && RING == 0;
+    [[maybe_unused]] const float* stat0 = COT_STATS ? p.nsig1 : p.nlse2;
+    [[maybe_unused]] const float* stat1 = COT_STATS ? p.ncvec : p.mu;
+    [[maybe_unused]] const float fac0 = COT_STATS ? 1.0f : 1.0f / p.c2, fac1 = COT_STATS ? 1.0f : -1.0f / p.alpha;
+    [[maybe_unused]] const bool own_step = k.fold_step;
+    [[maybe_unused]] const uint32_t fold_base = own_step ? (RING == 0 ? k.fold_e : k.fold_l) + lane * 16
+                                                         : ring_base + (RING == 0 ? 2 * ATOM + 2 * BC * 16 + lane * 16 : 2 * ATOM + lane * 128 + ((1 ^ sw) << 4));
+    [[maybe_unused]] const uint32_t fold_stage = own_step ? C::FOLD_BYTES : 2 * TB;
+    [[maybe_unused]] const uint32_t fold_t = own_step || RING == 0 ? BC * 16 : ATOM, fold_rp = own_step || RING == 0 ? 32 * 16 : 32 * 128;
+    [[maybe_unused]] float nx[4] = {0.f, 0.f, 0.f, 0.f};   // the next tile's statistics of rows lane, lane + 32
+    [[maybe_unused]] auto load_stats = [&](int bh, int j) {
+        const size_t at = (size_t)bh * p.s.rows + (size_t)j * BC + lane;
+        const int left = p.s.rows - j * BC - lane;   // queries beyond M: zero, like their rows of the operands
+        nx[0] = left > 0 ? __ldg(stat0 + at) : 0.f;
+        nx[1] = left > 0 ? __ldg(stat1 + at) : 0.f;
+        nx[2] = left > 32 ? __ldg(stat0 + at + 32) : 0.f;
+        nx[3] = left > 32 ? __ldg(stat1 + at + 32) : 0.f;
+    };
+    bool ok = true;
+    int s = 0, ph = 0;
+    int g = 0, owners = 0;           // tiles, and items whose owner tiles, have been asked for
+    // In an item's tiles the owner tiles have their turn where what they wait for is about to happen: behind as many of the
+    // item's E tiles as the ring holds.
+    [[maybe_unused]] const int owners_at = min(S, k.T) - 1;
+    if (FOLDED && (int)blockIdx.x < k.items) load_stats(blockIdx.x / k.row_tiles, 0);
+    for (int item = blockIdx.x; ok && item < k.items; item += gridDim.x) {
+        const int bh = item / k.row_tiles;
+        const int cb = bh / p.H, ch = bh - cb * p.H;   // batch and head: coordinates of the 4-D tensor maps
+        // element offset of (row `lane`, column 64) in the stream tensors
+        [[maybe_unused]] const size_t lane_row = p.s.head_off(bh, p.H) + (size_t)lane * (size_t)p.s.rs + 64;
+        [[maybe_unused]] const __nv_bfloat16* src0 = base0 + lane_row;  // advance by one tile per iteration
+        [[maybe_unused]] const __nv_bfloat16* src1 = base1 + lane_row;
+        [[maybe_unused]] const size_t srow = (size_t)bh * p.s.rows;
+        [[maybe_unused]] const float* st_src0 = nullptr;
+        [[maybe_unused]] const float* st_src1 = nullptr;
+        if constexpr (STATS) {
+            st_src0 = (lane < 16 ? p.nlse2 : p.mu) + srow + 4 * (lane & 15);
+            if (C::NSTAT == 4) st_src1 = (lane < 16 ? p.nsig1 : p.ncvec) + srow + 4 * (lane & 15);
+        }
+        for (int j = 0; j < k.T; ++j) {
+            if (OWNERS && j == owners_at) {   // once the score MMAs of the item before are complete
+                ok = owners == 0 || k.wait(C::B_OWNFREE, owners - 1);
+                if (!ok) break;
+                jvp_load_owners(p, k, own_maps, item, lane);
+                ++owners;
+            }
+            if (g >= S) ok = k.done(b_done, g - S);   // the MMAs that read the stage's last tile
+            if (!ok) break;
+            ++g;
+            const int rows_left = p.s.rows - j * BC;  // rows of this tile that exist
+            if constexpr (FOLDED) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {   // (row step i >> 1, tensor i & 1)
+                    const uint4 v = jvp_split3(nx[i] * ((i & 1) ? fac1 : fac0));
+                    ptx::st_shared_v4(fold_base + s * fold_stage + (i & 1) * fold_t + (i >> 1) * fold_rp, v.x, v.y, v.z, v.w);
+                }
+                ptx::fence_proxy_async_smem();
+                __syncwarp();   // lane 0's arrival below is the whole warp's
+            }
+            const uint32_t stage = ring_base + s * 2 * TB;
+            if (lane == 0) {
+                const uint32_t full = k.bar(b_full + s);
+                ptx::mbar_arrive_expect_tx(full, tx_bytes);
+                if (has0) {
+                    ptx::tma_load_4d(stage, map0, full, 0, j * BC, ch, cb);
+                    if (C::WIDE) ptx::tma_load_4d(stage + 2 * ATOM, map0, full, 64, j * BC, ch, cb);
+                }
+                if (has1) {
+                    ptx::tma_load_4d(stage + ATOM, map1, full, 0, j * BC, ch, cb);
+                    if (C::WIDE) ptx::tma_load_4d(stage + 3 * ATOM, map1, full, 64, j * BC, ch, cb);
+                }
+            }
+            if constexpr (FOLDED) {
+                const bool more = j + 1 < k.T;
+                if (more || item + (int)gridDim.x < k.items) load_stats(more ? bh : (item + (int)gridDim.x) / k.row_tiles, more ? j + 1 : 0);
+            }
+            if constexpr (STATS) {
+                // queries beyond M read as zero: their rows of the B operands are zero too
+                const uint32_t slot = st_base + s * (C::NSTAT * BC * 4);
+                if (st16) {
+                    const bool v = 4 * (lane & 15) < rows_left;
+                    const uint32_t dst = slot + (lane >> 4) * 256 + (lane & 15) * 16;
+                    ptx::cp_async_16(dst, v ? st_src0 + j * BC : p.nlse2, v ? 16u : 0u);
+                    if (C::NSTAT == 4) ptx::cp_async_16(dst + 512, v ? st_src1 + j * BC : p.nlse2, v ? 16u : 0u);
+                } else {
+                    for (int c = lane; c < C::NSTAT * BC; c += 32) {
+                        const int stat = c >> 6, r = c & 63;
+                        const float* src = (stat == 0 ? p.nlse2 : stat == 1 ? p.mu : stat == 2 ? p.nsig1 : p.ncvec) + srow + j * BC + r;
+                        const bool v = r < rows_left;
+                        ptx::cp_async_4(slot + c * 4, v ? src : p.nlse2, v ? 4u : 0u);
+                    }
+                }
+            }
+            if constexpr (C::TAIL) {
+#pragma unroll
+                for (int c = 0; c < KT; ++c) {
+                    if (c < ntail) {
+#pragma unroll
+                        for (int rp = 0; rp < BC / 32; ++rp) {
+                            const bool v = lane + 32 * rp < rows_left;
+                            const uint32_t dst = stage + dst_lane + (RING == 0 ? c * 2 * BC * 16 + rp * 32 * 16 : rp * 32 * 128 + ((c ^ sw) << 4));
+                            if (has0) ptx::cp_async_16(dst, v ? src0 + rp * d32 + 8 * c : base0, v ? 16u : 0u);
+                            if (has1) ptx::cp_async_16(dst + (RING == 0 ? BC * 16 : ATOM), v ? src1 + rp * d32 + 8 * c : base1, v ? 16u : 0u);
+                        }
+                    }
+                }
+                src0 += tile_elems;
+                src1 += tile_elems;
+            }
+            if (HAS_CP) ptx::cp_async_arrive(k.bar(b_full + s));
+            if (++s == S) { s = 0; ph ^= 1; }
+        }
+    }
+    if (HAS_CP) ptx::cp_async_wait_all();  // nothing of ours stays in flight
+    if (!ok) {
+        // Winding down after a time-out: the TMA loads this warp started write into this block's shared memory and must
+        // have landed before the block exits.  Stages below s carry the phase of this pass over the ring, the others
+        // the one before.
+        for (int i = 0; i < S; ++i) {
+            const bool cur = i < s;
+            if (!cur && g < S) continue;  // never filled
+            ptx::mbar_wait_drain(k.bar(b_full + i), (cur ? ph : ph ^ 1) & 1, ptx::DRAIN_LIMIT_NS);
+        }
+        if (OWNERS && owners > 0) ptx::mbar_wait_drain(k.bar(C::B_OWN), (owners - 1) & 1, ptx::DRAIN_LIMIT_NS);
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ MMA issue
+// The whole warp runs this in converged control flow; one elected lane issues (one election per batch of MMAs,
+// descriptors as 32-bit halves: see mma_ts_p).  Tensor memory starts at column 0, because the block owns all of it.
+template <int MODE, int DP, bool HZ>
+struct JvpIssue {
+    using C = JvpCfg<MODE, DP>;
+    static constexpr int BC = C::BC, KS = C::KS, ATOM = C::ATOM;
+    static constexpr uint32_t HI_SW = ptx::desc_hi_sw128(1024), HI_TAIL = ptx::desc_hi_nosw(128);
+    static constexpr uint32_t I_S = ptx::idesc_bf16_f32(128, BC, 0, 0), I_S2 = ptx::idesc_bf16_f32(128, 2 * BC, 0, 0);
+    static constexpr uint32_t I_O = ptx::idesc_bf16_f32(128, DP, 0, 1);
+    static __device__ __forceinline__ bool is_tail(int kk) { return C::TAIL && kk >= 4; }
+    // low descriptor halves (start address, leading offset) of k-step kk; the high half is HI_SW, or HI_TAIL in a tail
+    static __device__ __forceinline__ uint32_t own_klo(uint32_t tile, int kk) {   // owner tile, K-major
+        if (kk < 4) return ptx::desc_lo(tile, 16) + 2u * kk;
+        return C::WIDE ? ptx::desc_lo(tile + C::OWN_ATOM, 16) + 2u * (kk - 4) : ptx::desc_lo(tile + C::OWN_ATOM, JVP_ROWS * 16);
+    }
+    static __device__ __forceinline__ uint32_t e_klo(uint32_t stage, int kk) {    // E stage, K-major, rows of Y0 (then Y1)
+        if (kk < 4) return ptx::desc_lo(stage, 16) + 2u * kk;
+        return C::WIDE ? ptx::desc_lo(stage + 2 * ATOM, 16) + 2u * (kk - 4) : ptx::desc_lo(stage + 2 * ATOM, 2 * BC * 16);
+    }
+    static __device__ __forceinline__ uint32_t l_klo(uint32_t stage, int kk) {    // L stage, K-major, rows of Y0 (then Y1)
+        return ptx::desc_lo(stage + (kk >> 2) * 2 * ATOM, 16) + 2u * (kk & 3);
+    }
+    // L stage read MN-major by the output MMAs (tensor t): atoms of 64 d-columns are 2 * ATOM bytes apart, 8-row groups
+    // 1024 bytes, a k-step of 16 stream rows 2048
+    static __device__ __forceinline__ uint32_t l_nlo(uint32_t stage, int t) { return ptx::desc_lo(stage + t * ATOM, 2 * ATOM); }
+
+    // One k-step with A in tensor memory (ATM: a = its columns) or in shared memory (a = the tile).
+    template <bool ATM, uint32_t ACC>
+    static __device__ __forceinline__ void step(uint32_t el, uint32_t col, uint32_t a, int kk, uint32_t b, uint32_t bhi, uint32_t idesc) {
+        if (ATM) ptx::mma_ts_p<ACC>(el, col, a + 8 * kk, b, bhi, idesc);
+        else ptx::mma_ss_p<ACC>(el, col, own_klo(a, kk), is_tail(kk) ? HI_TAIL : HI_SW, b, bhi, idesc);
+    }
+    // The statistics' own k-step (FOLD, where the padding columns do not hold them): `fold` is the stage's block, tensor t0 on.
+    template <bool ATM>
+    static __device__ __forceinline__ void fold_step(uint32_t el, uint32_t col, const JvpBlock<MODE, DP>& k, uint32_t fold, int t0, uint32_t idesc) {
+        const uint32_t b = ptx::desc_lo(fold + t0 * BC * 16, k.zeros - fold);
+        if (ATM) ptx::mma_ts_p<1>(el, col, C::COL_ONES, b, HI_TAIL, idesc);
+        else ptx::mma_ss_p<1>(el, col, ptx::desc_lo(k.ones, k.zeros - k.ones), HI_TAIL, b, HI_TAIL, idesc);
+    }
+    // [S | X0 Y1^T] = X0 [Y0 | Y1]^T, Sd += X1 Y0^T at column col; FROM_L: the stage is one of the L ring.
+    template <bool FROM_L, bool ATM>
+    static __device__ __forceinline__ void pair(uint32_t el, uint32_t col, const JvpBlock<MODE, DP>& k, uint32_t a0, uint32_t a1, uint32_t stage, uint32_t fold,
+                                                bool second, uint32_t mid_bar) {
+#pragma unroll
+        for (int kk = 0; kk < KS; ++kk) {
+            const uint32_t b = FROM_L ? l_klo(stage, kk) : e_klo(stage, kk), bhi = !FROM_L && is_tail(kk) ? HI_TAIL : HI_SW;
+            if (kk == 0) step<ATM, 0>(el, col, a0, kk, b, bhi, I_S2);
+            else step<ATM, 1>(el, col, a0, kk, b, bhi, I_S2);
+        }
+        if (C::FOLD && k.fold_step) fold_step<ATM>(el, col, k, fold, 0, I_S2);
+        if (MODE == PASS_FWD) ptx::mma_commit_p(el, mid_bar);   // S is complete before Sd
+        if (second) {
+#pragma unroll
+            for (int kk = 0; kk < KS; ++kk)
+                step<ATM, 1>(el, col + BC, a1, kk, FROM_L ? l_klo(stage, kk) : e_klo(stage, kk), !FROM_L && is_tail(kk) ? HI_TAIL : HI_SW, I_S);
+        }
+    }
+    // One product X Y^T with Y the t-th tensor of the stage.
+    template <bool FROM_L, bool ATM>
+    static __device__ __forceinline__ void single(uint32_t el, uint32_t col, const JvpBlock<MODE, DP>& k, uint32_t a, uint32_t stage, uint32_t fold, int t) {
+#pragma unroll
+        for (int kk = 0; kk < KS; ++kk) {
+            const bool tail = !FROM_L && is_tail(kk);
+            const uint32_t b = (FROM_L ? l_klo(stage, kk) : e_klo(stage, kk)) + ((uint32_t)(tail ? t * BC * 16 : t * ATOM) >> 4);
+            if (kk == 0) step<ATM, 0>(el, col, a, kk, b, tail ? HI_TAIL : HI_SW, I_S);
+            else step<ATM, 1>(el, col, a, kk, b, tail ? HI_TAIL : HI_SW, I_S);
+        }
+        if (C::FOLD && k.fold_step) fold_step<ATM>(el, col, k, fold, t, I_S);
+    }
+    // Half of acc0 += A0 B0, acc1 += A1 B0 + A0 B1 (k-steps U0, U0 + 1 of four; the operand of a k-step lies at the columns of
+    // the scores it replaces); the terms of an absent tensor are left out, one uniform branch around the unrolled loops.
+    // `first`: the accumulators are overwritten.
+    template <int U0>
+    static __device__ __forceinline__ void outputs(uint32_t el, uint32_t a0, uint32_t a1, uint32_t stage, bool first, int absent) {
+        const uint32_t b0 = l_nlo(stage, 0), b1 = l_nlo(stage, 1);
+        constexpr uint32_t c0 = C::COL_ACC0, c1 = C::COL_ACC1;
+        constexpr bool DV = MODE == PASS_DV;
+        if (!HZ && (MODE == PASS_FWD || absent == 0 || (!DV && !(absent & ABSENT_HC)))) {
+#pragma unroll
+            for (int u = U0; u < U0 + 2; ++u) {
+                const uint32_t off = (uint32_t)(u * 2048) >> 4;
+                if (u == 0 && first) { ptx::mma_ts_p<0>(el, c0, a0, b0, HI_SW, I_O); ptx::mma_ts_p<0>(el, c1, a1, b0, HI_SW, I_O); }
+                else { ptx::mma_ts_p<1>(el, c0, a0 + 16 * u, b0 + off, HI_SW, I_O); ptx::mma_ts_p<1>(el, c1, a1 + 16 * u, b0 + off, HI_SW, I_O); }
+                ptx::mma_ts_p<1>(el, c1, a0 + 16 * u, b1 + off, HI_SW, I_O);
+            }
+        } else if (DV && !HZ && (absent & ABSENT_G)) {   // B1 = G absent
+#pragma unroll
+            for (int u = U0; u < U0 + 2; ++u) {
+                const uint32_t off = (uint32_t)(u * 2048) >> 4;
+                if (u == 0 && first) { ptx::mma_ts_p<0>(el, c0, a0, b0, HI_SW, I_O); ptx::mma_ts_p<0>(el, c1, a1, b0, HI_SW, I_O); }
+                else { ptx::mma_ts_p<1>(el, c0, a0 + 16 * u, b0 + off, HI_SW, I_O); ptx::mma_ts_p<1>(el, c1, a1 + 16 * u, b0 + off, HI_SW, I_O); }
+            }
+        } else {   // Hc absent: DV: acc1 += P^T G alone; DK, DQ: W is exactly zero, acc1 += A1 B0 alone
+            const uint32_t a = DV ? a0 : a1, b = DV ? b1 : b0;
+#pragma unroll
+            for (int u = U0; u < U0 + 2; ++u) {
+                const uint32_t off = (uint32_t)(u * 2048) >> 4;
+                if (u == 0 && first) ptx::mma_ts_p<0>(el, c1, a, b, HI_SW, I_O);
+                else ptx::mma_ts_p<1>(el, c1, a + 16 * u, b + off, HI_SW, I_O);
+            }
+        }
+    }
+};
+
+struct JvpRing {   // stage and phase of a ring's next tile
+    int s = 0, ph = 0;
+    template <int S>
+    __device__ __forceinline__ void next() { if (++s == S) { s = 0; ph ^= 1; } }
+};
+
+// FWD, DV: two score buffers taken in turn, operands written over the scores; pipe order S(0), S(1), out(0), S(2), out(1), ...:
+// S(n + 1) overwrites what out(n - 1) reads, and the pipe keeps the order.
+template <int MODE, int DP, bool HZ>
+__device__ __forceinline__ void jvp_issue_one_pair(const JvpParams& p, const JvpBlock<MODE, DP>& k) {
+    using C = JvpCfg<MODE, DP>;
+    using I = JvpIssue<MODE, DP, HZ>;
+    constexpr int RDY = C::XT ? C::B_XRDY : C::B_OWN, FREE = C::XT ? C::B_XFREE : C::B_OWNFREE;
+    const int n_it = (int)blockIdx.x < k.items ? (k.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+    const int T = k.T, G = n_it * T, absent = p.absent;
+    const uint32_t x0 = C::XT ? C::COL_X0 : k.own_tile(0), x1 = C::XT ? C::COL_X1 : k.own_tile(1);
+    JvpRing e, l;
+    int js = 0, is = 0, jo = 0, it = 0;   // place in its item, and item, of the scores' and of the outputs' tile
+    int n = 0;                            // next tile whose scores are issued
+    auto scores = [&]() -> bool {
+        if (js == 0 && !k.wait(RDY, is)) return false;
+        if (!k.wait(C::B_EFULL + e.s, e.ph)) return false;
+        k.tile_fence();
+        const uint32_t el = ptx::elect_one();
+        const uint32_t col = C::COL_SCORE + (n & 1) * 2 * C::BC, stage = k.e_stage(e.s), fold = k.fold_e + e.s * C::FOLD_BYTES;
+        if (HZ) I::template single<false, C::XT>(el, col, k, x0, stage, fold, 0);
+        else I::template pair<false, C::XT>(el, col, k, x0, x1, stage, fold, true, k.bar(C::B_SFULL + (n & 3)));
+        ptx::mma_commit_p(el, k.bar(C::B_EDONE + (n & 3)));
+        e.next<C::SE>();
+        ++n;
+        if (++js == T) {
+            ptx::mma_commit_p(el, k.bar(FREE));
+            js = 0;
+            ++is;
+        }
+        return true;
+    };
+    for (int g = 0; g < G; ++g) {
+        if (n == g && !scores()) return;
+        // The scores of the next tile go in front of this tile's outputs, unless they open an item whose owner operands are
+        // still on their way: then wherever these turn out to be ready.
+        if (n < G && (js > 0 || ptx::mbar_test_warp(k.bar(RDY), is & 1)) && !scores()) return;
+        const int b = g & 1;
+        if (!k.wait2(C::B_PREADY + 2 * b, g >> 1, C::B_LFULL + l.s, l.ph)) return;
+        // the first tile of an item overwrites the accumulators
+        if (jo == 0 && it > 0 && !k.wait(C::B_ACCFREE, it - 1)) return;
+        k.tile_fence();
+        const uint32_t a0 = C::COL_SCORE + b * 2 * C::BC, stage = k.l_stage(l.s);
+        I::template outputs<0>(ptx::elect_one(), a0, a0 + C::BC, stage, jo == 0, absent);
+        if (n == g + 1 && n < G && ptx::mbar_test_warp(k.bar(RDY), is & 1) && !scores()) return;
+        if (!k.wait(C::B_PREADY + 2 * b + 1, g >> 1)) return;
+        ptx::tc_fence_after_sync();
+        const uint32_t el = ptx::elect_one();
+        I::template outputs<2>(el, a0, a0 + C::BC, stage, false, absent);
+        ptx::mma_commit_p(el, k.bar(C::B_OUTDONE + (g & 3)));
+        l.next<C::SL>();
+        if (++jo == T) {
+            ptx::mma_commit_p(el, k.bar(C::B_FINAL));
+            jo = 0;
+            ++it;
+        }
+    }
+}
+
+// DK, DQ: one buffer of (S, Sd | D, X), the operands W, dA over D, X.  Pipe order: (S, Sd)(n) once (S, Sd)(n - 1) has been read |
+// outputs(n - 1), half by half, as W, dA are written | (D, X)(n), which overwrites them.
+template <int MODE, int DP, bool HZ>
+__device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const JvpBlock<MODE, DP>& k) {
+    using C = JvpCfg<MODE, DP>;
+    using I = JvpIssue<MODE, DP, HZ>;
+    const int T = k.T, absent = p.absent;
+    const uint32_t x0 = k.own_tile(0), x1 = k.own_tile(1);
+    const uint32_t x2 = C::XT ? C::COL_X0 : k.own_tile(2), x3 = C::XT ? C::COL_X1 : k.own_tile(3);
+    constexpr uint32_t cS = C::COL_SCORE, cD = C::COL_SCORE + 2 * C::BC, cX = C::COL_SCORE + 3 * C::BC;
+    JvpRing e, l;
+    int ls = 0, n = 0;   // L stage of the outputs' tile; next tile whose scores are issued
+    auto first = [&](int j) -> bool {
+        if (!k.wait2(C::B_SREAD, n - 1, C::B_LFULL + l.s, l.ph)) return false;   // (a fresh barrier passes for n = 0)
+        k.tile_fence();
+        const uint32_t el = ptx::elect_one(), fold = k.fold_l + l.s * C::FOLD_BYTES;
+        if (HZ) I::template single<true, false>(el, cS, k, x0, k.l_stage(l.s), fold, 0);
+        else I::template pair<true, false>(el, cS, k, x0, x1, k.l_stage(l.s), fold, true, 0);
+        ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
+        if (C::XT && j == T - 1) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE));
+        l.next<C::SL>();
+        return true;
+    };
+    auto second = [&](int j) -> bool {
+        if (!k.wait(C::B_EFULL + e.s, e.ph)) return false;
+        k.tile_fence();
+        const uint32_t el = ptx::elect_one(), fold = k.fold_e + e.s * C::FOLD_BYTES;
+        // HZ: X = G V^T alone: DK: X2 Y3^T (V, and G the stage's second tensor); DQ: X3 Y2^T (G, and V its first)
+        if (HZ) I::template single<false, C::XT>(el, cX, k, MODE == PASS_DK ? x2 : x3, k.e_stage(e.s), fold, MODE == PASS_DK ? 1 : 0);
+        // X3 Y2^T is zero when either factor is an absent cotangent: DK has Y2 = Hc, DQ has X3 = G
+        else I::template pair<false, C::XT>(el, cD, k, x2, x3, k.e_stage(e.s), fold, !(absent & (MODE == PASS_DK ? ABSENT_HC : ABSENT_G)), 0);
+        ptx::mma_commit_p(el, k.bar(C::B_XFULL + (n & 3)));
+        if (j == T - 1) ptx::mma_commit_p(el, k.bar(C::XT ? C::B_XFREE : C::B_OWNFREE));
+        e.next<C::SE>();
+        ++n;
+        return true;
+    };
+    int it = 0;
+    for (int item = blockIdx.x; item < k.items; item += gridDim.x, ++it) {
+        if (!k.wait(C::B_OWN, it) || !first(0)) return;
+        if ((C::XT && !k.wait(C::B_XRDY, it)) || !second(0)) return;
+        if (!k.wait(C::B_ACCFREE, it - 1)) return;    // the first tile overwrites the accumulators
+        for (int j = 0; j < T; ++j) {
+            const int g = n - 1;
+            if (j + 1 < T && !first(j + 1)) return;
+            if (!k.wait(C::B_PREADY, g)) return;
+            ptx::tc_fence_after_sync();
+            const uint32_t stage = k.l_stage(ls);
+            I::template outputs<0>(ptx::elect_one(), cD, cX, stage, j == 0, absent);
+            if (!k.wait(C::B_PREADY + 1, g)) return;
+            ptx::tc_fence_after_sync();
+            const uint32_t el = ptx::elect_one();
+            I::template outputs<2>(el, cD, cX, stage, false, absent);
+            ptx::mma_commit_p(el, k.bar(C::B_OUTDONE + (g & 3)));
+            if (++ls == C::SL) ls = 0;
+            if (j + 1 < T) { if (!second(j + 1)) return; }
+            else ptx::mma_commit_p(el, k.bar(C::B_FINAL));
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ element-wise warps
+// Group `grp` takes the tiles g of its parity; a thread has owner row `row` and the 64 columns of the tile.  Reads of
+// tensor memory are issued for many columns at once (a read costs 180 cycles whatever its width) and released with one
+// arrival per warp; the operands are handed over half by half.
+
+// Forward.  The reference m of a row and the centre c of its tangent weights are shared by the two groups: the warp that
+// has a row's tile g decides whether to move them and hands the row state on to the warp that has tile g + 1 (B_TURN), long
+// before that one needs it.  m follows the running maximum only when a tile maximum exceeds it by more than JVP_LAZY_LOG2
+// (rare after the first tile): then m moves to the new maximum, c to T at the new arg-max key (WIDE: c on its own, whenever
+// it is too far off), and the accumulators are rescaled, R += (c_old - c_new) O~ keeping them consistent.  Centring T keeps the bf16 rounding of P~ (T - c) small where
+// P~ is large, so that tO = R/l - (mu - c) O does not cancel badly on rows with a peaked softmax.
+template <int DP>
+__device__ __forceinline__ void jvp_elem_fwd(const JvpParams& p, const JvpBlock<PASS_FWD, DP>& k, int grp, int q, int lane) {
+    using C = JvpCfg<PASS_FWD, DP>;
+    constexpr int BC = C::BC;
+    const int row = q * 32 + lane;
+    const uint32_t lanes = static_cast<uint32_t>(q * 32) << 16;
+    const uint64_t c2c2 = ptx::pack2(p.c2, p.c2), aa = ptx::pack2(p.alpha, p.alpha);
+    bool ok = true;
+    int it = 0;
+    for (int item = blockIdx.x; ok && item < k.items; item += gridDim.x, ++it) {
+        const int g0 = it * k.T;
+        float m_own = -CUDART_INF_F, c_own = 0.f;   // reference and centre of this thread's sums
+        uint64_t l2 = 0ull, mt2 = 0ull;             // two partial sums each of P~ and of P~ (T - c) over this group's tiles
+        for (int j = (grp ^ g0) & 1; j < k.T; j += 2) {
+            const int g = g0 + j, b = g & 1;
+            const uint32_t sb = lanes + C::COL_SCORE + b * 2 * BC;
+            uint32_t s[64], t[64];
+            ok = k.done(C::B_SFULL, g);   // S is complete before Sd
+            if (!ok) break;
+            ptx::tc_fence_after_sync();
+            ptx::tmem_ld32(sb, s);
+            ptx::tmem_ld32(sb + 32, s + 32);
+            ptx::tmem_wait_ld();
+            const int nvalid = p.s.rows - j * BC;  // columns that are real keys
+            if (nvalid < BC) {
+#pragma unroll
+                for (int c = 0; c < BC; ++c)
+                    if (c >= nvalid) s[c] = __float_as_uint(-CUDART_INF_F);
+            }
+            float mx[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                mx[i] = __uint_as_float(s[16 * i]);
+#pragma unroll
+                for (int c = 1; c < 15; c += 2) mx[i] = ptx::max3(mx[i], __uint_as_float(s[16 * i + c]), __uint_as_float(s[16 * i + c + 1]));
+                mx[i] = fmaxf(mx[i], __uint_as_float(s[16 * i + 15]));
+            }
+            const float top = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+            const float mrow = top * p.c2;         // tile maximum of the row, log2 units
+            ok = k.done(C::B_XFULL, g);
+            if (!ok) break;
+            ptx::tc_fence_after_sync();
+            ptx::tmem_ld32(sb + BC, t);
+            ptx::tmem_ld32(sb + BC + 32, t + 32);
+            if (g > 0) ok = k.wait(C::B_TURN + q, g - 1);
+            if (!ok) break;
+            float m_ref = -CUDART_INF_F, cen = 0.f, m_max = -CUDART_INF_F;
+            if (j > 0) { const float4 st = k.row_state[row]; m_ref = st.x; cen = st.y; m_max = st.z; }
+            ptx::tmem_wait_ld();
+            bool scaling = mrow > m_ref + (C::WIDE ? JVP_LAZY_LOG2_WIDE : JVP_LAZY_LOG2), centring = C::WIDE ? mrow > m_max : scaling;
+            if (__any_sync(0xffffffffu, centring)) {
+                float lt = 0.f;                    // Sd at the arg-max key (the first one)
+#pragma unroll
+                for (int c = BC - 1; c >= 0; --c) lt = __uint_as_float(s[c]) == top ? __uint_as_float(t[c]) : lt;
+                const float tw = lt * p.alpha;
+                if (C::WIDE) {
+                    centring = centring && (j == 0 || fabsf(tw - cen) > JVP_CENTRE_WIDE);
+                    m_max = fmaxf(m_max, mrow);
+                }
+                const float scale = scaling ? ptx::ex2(m_ref - mrow) : 1.0f;
+                const float fix = centring ? cen - tw : 0.f;
+                if (scaling) m_ref = mrow;
+                if (centring) cen = tw;
+                if (j > 0 && (!C::WIDE || __any_sync(0xffffffffu, scaling || centring))) {
+                    // accumulators must be at rest: the value MMAs of tile g - 1 have completed
+                    ok = k.done(C::B_OUTDONE, g - 1);
+                    if (!ok) break;
+                    ptx::tc_fence_after_sync();
+#pragma unroll 1
+                    for (int c0 = 0; c0 < DP; c0 += 8) {   // eight columns at a time: this rare path must not set the register peak
+                        uint32_t o[8], r[8];
+                        ptx::tmem_ld8(lanes + C::COL_ACC0 + c0, o);
+                        ptx::tmem_ld8(lanes + C::COL_ACC1 + c0, r);
+                        ptx::tmem_wait_ld();
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) {
+                            const float ov = __uint_as_float(o[c]);
+                            r[c] = __float_as_uint(scale * fmaf(fix, ov, __uint_as_float(r[c])));
+                            o[c] = __float_as_uint(scale * ov);
+                        }
+                        ptx::tmem_st8(lanes + C::COL_ACC0 + c0, o);
+                        ptx::tmem_st8(lanes + C::COL_ACC1 + c0, r);
+                    }
+                    ptx::tmem_wait_st();
+                }
+                k.row_state[row] = make_float4(m_ref, cen, m_max, 0.f);
+            }
+            k.arrive(C::B_TURN + q, lane);
+            if (__any_sync(0xffffffffu, m_ref != m_own || (C::WIDE && cen != c_own))) {   // the reference has moved since this group's last tile
+                const float scale = ptx::ex2(m_own - m_ref), fix = c_own - cen;
+                float l0, l1, t0, t1;
+                ptx::unpack2(l2, l0, l1);
+                ptx::unpack2(mt2, t0, t1);
+                l2 = ptx::pack2(l0 * scale, l1 * scale);
+                mt2 = ptx::pack2(scale * fmaf(fix, l0, t0), scale * fmaf(fix, l1, t1));
+                m_own = m_ref;
+                c_own = cen;
+            }
+            // ---- P~ = 2^(c2 s - m), P~ (T - c): operands of a k-step (16 keys) at the columns of the scores they replace
+            const uint64_t nm = ptx::pack2(-m_ref, -m_ref), nc = ptx::pack2(-cen, -cen);
+#pragma unroll
+            for (int u = 0; u < BC / 16; ++u) {
+                uint32_t pp[8], ppt[8];
+#pragma unroll
+                for (int c = 0; c < 16; c += 2) {
+                    const uint64_t x2 = ptx::fma2(ptx::pack2u(s[16 * u + c], s[16 * u + c + 1]), c2c2, nm);
+                    float x0, x1;
+                    ptx::unpack2(x2, x0, x1);
+                    const float p0 = ptx::ex2(x0), p1 = ptx::ex2(x1);
+                    const uint64_t p2 = ptx::pack2(p0, p1);
+                    const uint64_t pt2 = ptx::mul2(p2, ptx::fma2(ptx::pack2u(t[16 * u + c], t[16 * u + c + 1]), aa, nc));
+                    l2 = ptx::add2(l2, p2);
+                    mt2 = ptx::add2(mt2, pt2);
+                    float q0, q1;
+                    ptx::unpack2(pt2, q0, q1);
+                    pp[c >> 1] = ptx::pack_bf16(p0, p1);
+                    ppt[c >> 1] = ptx::pack_bf16(q0, q1);
+                }
+                ptx::tmem_st8(sb + 16 * u, pp);
+                ptx::tmem_st8(sb + BC + 16 * u, ppt);
+                if (u & 1) {   // half of the output MMAs may go
+                    ptx::tmem_wait_st();
+                    k.arrive(C::B_PREADY + 2 * b + (u >> 1), lane);
+                }
+            }
+        }
+        if (!ok) break;
+        // the item's sums of this group, for the epilogue (which has read those of the item before)
+        if (it > 0) ok = k.wait(C::B_ACCFREE, it - 1);
+        float l0, l1, t0, t1;
+        ptx::unpack2(l2, l0, l1);
+        ptx::unpack2(mt2, t0, t1);
+        k.row_sums[grp * JVP_ROWS + row] = make_float4(l0 + l1, t0 + t1, m_own, c_own);
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(k.bar(C::B_ROWSTAT));
+    }
+}
+
+// DV: P, P Nn from (S, Sd), written over them.  FOLD: the statistics are in the scores already.
+template <int DP, bool HZ>
+__device__ __forceinline__ void jvp_elem_dv(const JvpParams& p, const JvpBlock<PASS_DV, DP>& k, int grp, int q, int lane) {
+    using C = JvpCfg<PASS_DV, DP>;
+    constexpr int BC = C::BC;
+    const uint32_t lanes = static_cast<uint32_t>(q * 32) << 16;
+    const uint64_t c2c2 = ptx::pack2(p.c2, p.c2), aa = ptx::pack2(p.alpha, p.alpha);
+    const int n_it = (int)blockIdx.x < k.items ? (k.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+    for (int g = grp; g < n_it * k.T; g += 2) {
+        const int b = g & 1;
+        const uint32_t sb = lanes + C::COL_SCORE + b * 2 * BC;
+        if (!k.done(C::B_SFULL, g)) return;
+        if (!C::FOLD && !k.wait(C::B_LFULL + g % C::SL, g / C::SL)) return;   // the tile's statistics
+        ptx::tc_fence_after_sync();
+        uint32_t s[64], t[64];
+        ptx::tmem_ld32(sb, s);
+        if (!HZ) ptx::tmem_ld32(sb + BC, t);
+        ptx::tmem_ld32(sb + 32, s + 32);
+        if (!HZ) ptx::tmem_ld32(sb + BC + 32, t + 32);
+        ptx::tmem_wait_ld();
+        const float* st = C::FOLD ? nullptr : k.stats + (g % C::SL) * C::NSTAT * BC;
+#pragma unroll
+        for (int u = 0; u < BC / 16; ++u) {
+            uint32_t pa0[8], pa1[8];
+#pragma unroll
+            for (int c = 0; c < 16; c += 4) {
+                const int cc = 16 * u + c;
+                [[maybe_unused]] ulonglong2 l4, m4;
+                if (!C::FOLD) l4 = *reinterpret_cast<const ulonglong2*>(st + cc);
+                if (!C::FOLD && !HZ) m4 = *reinterpret_cast<const ulonglong2*>(st + BC + cc);
+#pragma unroll
+                for (int e = 0; e < 4; e += 2) {
+                    const uint64_t s2 = ptx::pack2u(s[cc + e], s[cc + e + 1]);
+                    float x0, x1;
+                    ptx::unpack2(C::FOLD ? ptx::mul2(s2, c2c2) : ptx::fma2(s2, c2c2, e ? l4.y : l4.x), x0, x1);
+                    const float p0 = ptx::ex2(x0), p1 = ptx::ex2(x1);
+                    pa0[(c + e) >> 1] = ptx::pack_bf16(p0, p1);
+                    if (!HZ) {
+                        const uint64_t t2 = ptx::pack2u(t[cc + e], t[cc + e + 1]);
+                        const uint64_t n2 = C::FOLD ? ptx::mul2(t2, aa) : ptx::fma2(t2, aa, ptx::neg2(e ? m4.y : m4.x));
+                        float q0, q1;
+                        ptx::unpack2(ptx::mul2(ptx::pack2(p0, p1), n2), q0, q1);
+                        pa1[(c + e) >> 1] = ptx::pack_bf16(q0, q1);
+                    }
+                }
+            }
+            ptx::tmem_st8(sb + 16 * u, pa0);
+            if (!HZ) ptx::tmem_st8(sb + BC + 16 * u, pa1);
+            if (u & 1) {   // half of the output MMAs may go
+                ptx::tmem_wait_st();
+                k.arrive(C::B_PREADY + 2 * b + (u >> 1), lane);
+            }
+        }
+    }
+}
+
+// DK, DQ.  Phase A: P and Nn from (S, Sd), kept in registers; phase B: W = P (D - Sigma1), dA = P (X - c) + W Nn, written over
+// D and X.  The statistics are in the scores already (FOLD), belong to the columns (DK, WIDE) or to this thread's row (DQ).
+template <int MODE, int DP, bool HZ>
+__device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const JvpBlock<MODE, DP>& k, int grp, int q, int lane) {
+    using C = JvpCfg<MODE, DP>;
+    constexpr int BC = C::BC;
+    constexpr bool FOLD = C::FOLD, COL = C::TRANSPOSED && !FOLD, ROW = !C::TRANSPOSED;
+    const int row = q * 32 + lane;
+    const uint32_t sb = (static_cast<uint32_t>(q * 32) << 16) + C::COL_SCORE;
+    const uint64_t c2c2 = ptx::pack2(p.c2, p.c2), aa = ptx::pack2(p.alpha, p.alpha);
+    // DQ: the statistics of this thread's row in the next item, loaded one item ahead
+    [[maybe_unused]] float n_lse2 = -CUDART_INF_F, n_mu = 0.f, n_s1 = 0.f, n_cv = 0.f;
+    [[maybe_unused]] auto load_stats = [&](int item) {
+        const int bh = item / k.row_tiles, r = (item - bh * k.row_tiles) * JVP_ROWS + row;
+        n_lse2 = -CUDART_INF_F; n_mu = n_s1 = n_cv = 0.f;
+        if (item < k.items && r < p.o.rows) {
+            const size_t at = (size_t)bh * p.o.rows + r;
+            n_lse2 = p.nlse2[at]; n_mu = p.mu[at]; n_s1 = p.nsig1[at]; n_cv = p.ncvec[at];
+        }
+    };
+    if (ROW) load_stats(blockIdx.x);
+    int it = 0;
+    for (int item = blockIdx.x; item < k.items; item += gridDim.x, ++it) {
+        const int g0 = it * k.T;
+        [[maybe_unused]] const uint64_t r_l = ptx::pack2(n_lse2, n_lse2), r_nm = ptx::pack2(-n_mu, -n_mu), r_s = ptx::pack2(n_s1, n_s1), r_c = ptx::pack2(n_cv, n_cv);
+        if (ROW) load_stats(item + gridDim.x);
+        for (int j = (grp ^ g0) & 1; j < k.T; j += 2) {
+            const int g = g0 + j;
+            [[maybe_unused]] const float* st = COL ? k.stats + (g % C::SL) * C::NSTAT * BC : nullptr;
+            uint32_t s[64], t[64];
+            uint64_t P2[32], N2[32];
+            // ---- phase A
+            if (!k.done(C::B_SFULL, g)) return;
+            if (COL && !k.wait(C::B_LFULL + g % C::SL, g / C::SL)) return;   // (complete: those MMAs read the tile's L stage)
+            ptx::tc_fence_after_sync();
+            ptx::tmem_ld32(sb, s);
+            if (!HZ) ptx::tmem_ld32(sb + BC, t);
+            ptx::tmem_ld32(sb + 32, s + 32);
+            if (!HZ) ptx::tmem_ld32(sb + BC + 32, t + 32);
+            ptx::tmem_wait_ld();
+            k.arrive(C::B_SREAD, lane);
+            if (ROW && p.s.rows - j * BC < BC) {   // keys beyond N: P = 0
+                const int nvalid = p.s.rows - j * BC;
+#pragma unroll
+                for (int c = 0; c < BC; ++c)
+                    if (c >= nvalid) s[c] = __float_as_uint(-CUDART_INF_F);   // c2 s = -inf (c2 > 0)
+            }
+#pragma unroll
+            for (int c = 0; c < BC; c += 4) {
+                [[maybe_unused]] ulonglong2 l4, m4;
+                if (COL) l4 = *reinterpret_cast<const ulonglong2*>(st + c);
+                if (COL && !HZ) m4 = *reinterpret_cast<const ulonglong2*>(st + BC + c);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int i = c / 2 + e;
+                    const uint64_t s2 = ptx::pack2u(s[2 * i], s[2 * i + 1]);
+                    float x0, x1;
+                    ptx::unpack2(FOLD ? ptx::mul2(s2, c2c2) : ptx::fma2(s2, c2c2, COL ? (e ? l4.y : l4.x) : r_l), x0, x1);
+                    P2[i] = ptx::pack2(ptx::ex2(x0), ptx::ex2(x1));
+                    if (!HZ) {
+                        const uint64_t ts = ptx::pack2u(t[2 * i], t[2 * i + 1]);
+                        N2[i] = FOLD ? ptx::mul2(ts, aa) : ptx::fma2(ts, aa, COL ? ptx::neg2(e ? m4.y : m4.x) : r_nm);
+                    }
+                }
+            }
+            // ---- phase B, 16 columns (one k-step of the output MMAs) at a time
+            if (!k.done(C::B_XFULL, g)) return;
+            ptx::tc_fence_after_sync();
+#pragma unroll
+            for (int u = 0; u < BC / 16; ++u) {
+                uint32_t dd[16], xx[16];
+                if (!HZ) ptx::tmem_ld16(sb + 2 * BC + 16 * u, dd);
+                ptx::tmem_ld16(sb + 3 * BC + 16 * u, xx);
+                ptx::tmem_wait_ld();
+                uint32_t pa0[8], pa1[8];
+#pragma unroll
+                for (int c = 0; c < 16; c += 4) {
+                    [[maybe_unused]] ulonglong2 s4, c4;
+                    if (COL && !HZ) s4 = *reinterpret_cast<const ulonglong2*>(st + 2 * BC + 16 * u + c);
+                    if (COL) c4 = *reinterpret_cast<const ulonglong2*>(st + 3 * BC + 16 * u + c);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int i = c / 2 + e, gi = 8 * u + i;
+                        uint64_t x2 = ptx::pack2u(xx[2 * i], xx[2 * i + 1]);
+                        if (!FOLD) x2 = ptx::add2(x2, COL ? (e ? c4.y : c4.x) : r_c);
+                        const uint64_t t2 = ptx::mul2(P2[gi], x2);
+                        float d0, d1;
+                        if (HZ) {
+                            ptx::unpack2(t2, d0, d1);
+                        } else {
+                            uint64_t y2 = ptx::pack2u(dd[2 * i], dd[2 * i + 1]);
+                            if (!FOLD) y2 = ptx::add2(y2, COL ? (e ? s4.y : s4.x) : r_s);
+                            const uint64_t w2 = ptx::mul2(P2[gi], y2);
+                            float w0, w1;
+                            ptx::unpack2(w2, w0, w1);
+                            ptx::unpack2(ptx::fma2(w2, N2[gi], t2), d0, d1);
+                            pa0[i] = ptx::pack_bf16(w0, w1);
+                        }
+                        pa1[i] = ptx::pack_bf16(d0, d1);
+                    }
+                }
+                if (!HZ) ptx::tmem_st8(sb + 2 * BC + 16 * u, pa0);
+                ptx::tmem_st8(sb + 3 * BC + 16 * u, pa1);
+                if (u & 1) {   // half of the output MMAs may go
+                    ptx::tmem_wait_st();
+                    k.arrive(C::B_PREADY + (u >> 1), lane);
+                }
+            }
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ epilogue warps
+// A thread has one owner row.  Per item: the owner operands of the next item go to tensor memory as soon as the item's last
+// score MMAs are done with the present ones (XT), then the accumulators are normalised, converted and stored; they are free
+// for the next item once all four warps have read them.
+template <int MODE, int DP>
+__device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<MODE, DP>& k, int q, int lane) {
+    using C = JvpCfg<MODE, DP>;
+    constexpr int NCH = DP / 8;                    // 16-byte chunks of a row
+    constexpr int XT0 = C::NPAIR == 2 ? 2 : 0;     // p.own[XT0], p.own[XT0 + 1] -> tensor memory
+    const int row = q * 32 + lane;
+    const uint32_t lanes = static_cast<uint32_t>(q * 32) << 16;
+    // Row of tensor t in an item; what is beyond the head dim or the tensor, and an absent cotangent, reads as zero.  The
+    // columns of ones that the statistics are multiplied by (FOLD): padding of the first tensor.
+    [[maybe_unused]] auto load_x = [&](int item, int t, uint4 (&v)[NCH]) {
+        const int bh = item / k.row_tiles, row0 = (item - bh * k.row_tiles) * JVP_ROWS;
+        const __nv_bfloat16* x = p.own[XT0 + t];
+        const bool valid = x && row0 + row < p.o.rows;
+        const __nv_bfloat16* src = x + (p.o.head_off(bh, p.H) + (size_t)(row0 + row) * (size_t)p.o.rs);
+#pragma unroll
+        for (int c = 0; c < NCH; ++c) {
+            v[c] = make_uint4(0, 0, 0, 0);
+            if (valid && 8 * c < p.d) v[c] = __ldg(reinterpret_cast<const uint4*>(src + 8 * c));
+        }
+        if (C::FOLD && t == 0 && !k.fold_step) { v[NCH - 1].x = JVP_ONES0; v[NCH - 1].y = JVP_ONES1; }
+    };
+    [[maybe_unused]] auto store_x = [&](int t, const uint4 (&v)[NCH]) {
+#pragma unroll
+        for (int c = 0; c < NCH; c += 2) {
+            const uint32_t r[8] = {v[c].x, v[c].y, v[c].z, v[c].w, v[c + 1].x, v[c + 1].y, v[c + 1].z, v[c + 1].w};
+            ptx::tmem_st8(lanes + (t ? C::COL_X1 : C::COL_X0) + 4 * c, r);
+        }
+    };
+    [[maybe_unused]] uint4 v0[NCH], v1[NCH];
+    if (C::XT && (int)blockIdx.x < k.items) {
+        if (C::FOLD) {
+            const uint32_t r[8] = {JVP_ONES0, JVP_ONES1, 0u, 0u, 0u, 0u, 0u, 0u};
+            ptx::tmem_st8(lanes + C::COL_ONES, r);
+        }
+        load_x(blockIdx.x, 0, v0);
+        store_x(0, v0);
+        load_x(blockIdx.x, 1, v0);
+        store_x(1, v0);
+        ptx::tmem_wait_st();
+        k.arrive(C::B_XRDY, lane);
+    }
+    int it = 0;
+    for (int item = blockIdx.x; item < k.items; item += gridDim.x, ++it) {
+        if (C::XT && item + (int)gridDim.x < k.items) {
+            load_x(item + gridDim.x, 0, v0);                       // in flight during the wait
+            if (MODE == PASS_DV) load_x(item + gridDim.x, 1, v1);   // (the other passes have no registers for the second)
+            if (!k.wait(C::B_XFREE, it)) return;
+            ptx::tc_fence_after_sync();
+            store_x(0, v0);
+            if (MODE != PASS_DV) load_x(item + gridDim.x, 1, v0);
+            store_x(1, MODE == PASS_DV ? v1 : v0);
+            ptx::tmem_wait_st();
+            k.arrive(C::B_XRDY, lane);
+        }
+        const int bh = item / k.row_tiles, row0 = (item - bh * k.row_tiles) * JVP_ROWS;
+        const size_t off = p.o.head_off(bh, p.H) + (size_t)(row0 + row) * (size_t)p.o.rs;
+        // lane pairs write the two rows of the pair one after the other, each as complete 32-byte sectors
+        const bool ok_even = row0 + (row & ~1) < p.o.rows, ok_odd = row0 + (row | 1) < p.o.rows;
+        float f0 = p.out_scale, mun = 0.f;
+        if constexpr (MODE == PASS_FWD) {   // O = O~/l, tO = R/l - (mu - c) O
+            if (!k.wait(C::B_ROWSTAT, it)) return;
+            const int last = (it * k.T + k.T - 1) & 1;   // the group whose reference is the accumulators'
+            const float4 f = k.row_sums[last * JVP_ROWS + row], o = k.row_sums[(last ^ 1) * JVP_ROWS + row];
+            const float scale = ptx::ex2(o.z - f.z);     // (a group without a tile: m = -inf, factor 0)
+            const float l = fmaf(o.x, scale, f.x), mt = f.y + scale * fmaf(o.w - f.w, o.x, o.y);
+            f0 = 1.0f / l;
+            mun = mt * f0;
+            if (row0 + row < p.o.rows) {
+                const size_t at = (size_t)bh * p.o.rows + row0 + row;
+                p.lse[at] = (f.z + log2f(l)) * 0.6931471805599453f;
+                p.mu_out[at] = f.w + mun;
+            }
+        }
+        if (!k.wait(C::B_FINAL, it)) return;
+        ptx::tc_fence_after_sync();
+#pragma unroll 1
+        for (int ch = 0; ch < C::KS; ++ch) {
+            uint32_t x0[16], x1[16], q0[8], q1[8];
+            ptx::tmem_ld16(lanes + C::COL_ACC0 + 16 * ch, x0);
+            ptx::tmem_ld16(lanes + C::COL_ACC1 + 16 * ch, x1);
+            ptx::tmem_wait_ld();
+            if (ch == C::KS - 1) k.arrive(C::B_ACCFREE, lane);
+#pragma unroll
+            for (int c = 0; c < 16; c += 2) {
+                float a0 = __uint_as_float(x0[c]) * f0, a1 = __uint_as_float(x0[c + 1]) * f0;
+                float b0 = __uint_as_float(x1[c]) * f0, b1 = __uint_as_float(x1[c + 1]) * f0;
+                if (MODE == PASS_FWD) { b0 = fmaf(-mun, a0, b0); b1 = fmaf(-mun, a1, b1); }
+                q0[c >> 1] = ptx::pack_bf16(a0, a1);
+                q1[c >> 1] = ptx::pack_bf16(b0, b1);
+            }
+            if (16 * ch >= p.d) continue;
+            const bool has_hi = 16 * ch + 8 < p.d;
+            store_row_pairs(p.out1 + off + 16 * ch, p.o.rs, lane, ok_even, ok_odd, has_hi, make_uint4(q1[0], q1[1], q1[2], q1[3]), make_uint4(q1[4], q1[5], q1[6], q1[7]));
+            if (p.out0)   // null with Hc absent: acc0 was never written, its gradient is zero
+                store_row_pairs(p.out0 + off + 16 * ch, p.o.rs, lane, ok_even, ok_odd, has_hi, make_uint4(q0[0], q0[1], q0[2], q0[3]), make_uint4(q0[4], q0[5], q0[6], q0[7]));
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ the kernel
+// HZ: the cotangent Hc = dtO is absent (the "detach JVP" setting), known at compile time: everything that only feeds the
+// tangent path is left out -- Sd, Nn, D, W and their MMAs -- and what remains is the standard attention backward: P from
+// S, dA = P (G V^T - rowsum(G O)), dV = P^T G, dK = alpha dA^T Q, dQ = alpha dA K.
+template <int MODE, int DP, bool HZ>
+__global__ void __launch_bounds__(JVP_THREADS, 1)
+jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUtensorMap s1, const __grid_constant__ CUtensorMap s2,
+           const __grid_constant__ CUtensorMap s3, const __grid_constant__ CUtensorMap o0, const __grid_constant__ CUtensorMap o1,
+           const __grid_constant__ CUtensorMap o2, const __grid_constant__ CUtensorMap o3, const __grid_constant__ JvpParams p) {
+    using C = JvpCfg<MODE, DP>;
+    constexpr int BC = C::BC;
+    constexpr bool DEPENDENT = MODE == PASS_DK || MODE == PASS_DQ;   // launched as a programmatic dependent of the pass before
+    // the next backward pass in the stream, if launched as a programmatic dependent, may start as SMs free up
+    if (MODE != PASS_FWD) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (*reinterpret_cast<volatile int*>(p.status) != 0) {  // an earlier kernel timed out
+        if (DEPENDENT && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+        return;
+    }
+    extern __shared__ __align__(1024) uint8_t jvp_smem[];
+    uint8_t* misc = jvp_smem + C::TILE_BYTES;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 56 * 8);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 56 * 8 + 16);
+
+    JvpBlock<MODE, DP> k;
+    k.own = ptx::smem_u32(jvp_smem);
+    k.e = k.own + C::NOWN * C::OWN_BYTES;
+    k.l = k.e + C::SE * 2 * C::EST_BYTES;
+    k.bar0 = ptx::smem_u32(misc);
+    k.abort_flag = abort_flag;
+    k.stats = reinterpret_cast<float*>(misc + 56 * 8 + 64);
+    k.row_state = reinterpret_cast<float4*>(k.stats + C::STATS_FLOATS);
+    k.row_sums = reinterpret_cast<float4*>(k.row_state + JVP_ROWS);
+    uint8_t* fold = reinterpret_cast<uint8_t*>(k.stats + C::STATS_FLOATS + C::FWD_FLOATS);
+    k.fold_e = ptx::smem_u32(fold);
+    k.fold_l = k.fold_e + C::FOLD_E * C::FOLD_BYTES;
+    k.ones = k.fold_l + C::FOLD_L * C::FOLD_BYTES;
+    k.zeros = k.ones + JVP_ROWS * 16;
+    k.fold_step = C::FOLD && (C::NA == 1 || p.d == DP);
+    k.row_tiles = (p.o.rows + JVP_ROWS - 1) / JVP_ROWS;
+    k.items = p.BH * k.row_tiles;
+    k.T = (p.s.rows + BC - 1) / BC;
+
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        *abort_flag = 0;
+        auto init = [&](int b, int n, int count) { for (int i = 0; i < n; ++i) ptx::mbar_init(k.bar(b + i), count); };
+        init(C::B_EFULL, C::SE, C::EFULL_COUNT);
+        init(C::B_LFULL, C::SL, C::LFULL_COUNT);
+        init(C::B_OWN, 1, C::TAIL ? 33 : 1);
+        init(C::B_OWNFREE, 1, 1);
+        init(C::B_XRDY, 1, 4);
+        init(C::B_XFREE, 1, 1);
+        init(C::B_SFULL, 12, 1);       // SFULL, XFULL, OUTDONE
+        init(C::B_PREADY, 5, 4);       // PREADY, SREAD: the four warps of a group
+        init(C::B_FINAL, 1, 1);
+        init(C::B_ACCFREE, 1, 4);
+        init(C::B_TURN, 4, 1);
+        init(C::B_ROWSTAT, 1, 8);
+        init(C::B_DRAIN, 1, 1);
+        ptx::fence_mbar_init();
+    }
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    if (C::TAIL && ((p.d - 64) >> 3) < 2) {
+        // The 16-byte chunk behind the copied columns (d = 72) pads the head dim to a multiple of 16: zeroed once, never
+        // written again.  Owners and E ring: the second chunk block; L ring: chunk 1 of the second atom, which lies at
+        // physical chunk 1 ^ (r & 7) of row r.  Where the columns hold statistics (FOLD), the first owner tensor has the
+        // ones there.
+        for (int i = threadIdx.x; i < C::NOWN * JVP_ROWS; i += JVP_THREADS)
+            *reinterpret_cast<uint4*>(jvp_smem + (i / JVP_ROWS) * C::OWN_BYTES + C::OWN_ATOM + (JVP_ROWS + i % JVP_ROWS) * 16) =
+                C::FOLD && i < JVP_ROWS ? make_uint4(JVP_ONES0, JVP_ONES1, 0, 0) : zero;
+        uint8_t* e = jvp_smem + C::NOWN * C::OWN_BYTES;
+        for (int i = threadIdx.x; i < C::SE * 2 * BC; i += JVP_THREADS)
+            *reinterpret_cast<uint4*>(e + (i / (2 * BC)) * 2 * C::EST_BYTES + 2 * C::ATOM + (2 * BC + i % (2 * BC)) * 16) = zero;
+        uint8_t* l = e + C::SE * 2 * C::EST_BYTES;
+        for (int i = threadIdx.x; i < C::SL * 2 * BC; i += JVP_THREADS) {
+            const int t = i / BC, r = i - t * BC;
+            *reinterpret_cast<uint4*>(l + (t >> 1) * 2 * C::LST_BYTES + (2 + (t & 1)) * C::ATOM + r * 128 + ((1 ^ (r & 7)) << 4)) = zero;
+        }
+    }
+    if (!HZ && MODE == PASS_DK && p.absent) {
+        // both cotangent tiles of an E stage are read by one N = 128 MMA: the never-loaded one must read as zero
+        const int t = (p.absent & ABSENT_HC) ? 0 : 1;
+        uint8_t* e = jvp_smem + C::NOWN * C::OWN_BYTES;
+        for (int st = 0; st < C::SE; ++st) {
+            uint8_t* stage = e + st * 2 * C::EST_BYTES;
+            for (int i = threadIdx.x; i < BC * 8; i += JVP_THREADS) {
+                *reinterpret_cast<uint4*>(stage + t * C::ATOM + i * 16) = zero;
+                if (C::WIDE) *reinterpret_cast<uint4*>(stage + (2 + t) * C::ATOM + i * 16) = zero;
+            }
+            if (C::TAIL)
+                for (int i = threadIdx.x; i < 2 * BC; i += JVP_THREADS)
+                    *reinterpret_cast<uint4*>(stage + 2 * C::ATOM + ((i / BC) * 2 * BC + t * BC + i % BC) * 16) = zero;
+        }
+    }
+    if (C::FOLD)
+        for (int i = threadIdx.x; i < 2 * JVP_ROWS; i += JVP_THREADS)
+            *reinterpret_cast<uint4*>(fold + (C::FOLD_E + C::FOLD_L) * C::FOLD_BYTES + i * 16) = i < JVP_ROWS ? make_uint4(JVP_ONES0, JVP_ONES1, 0, 0) : zero;
+    if (!HZ && MODE == PASS_DQ && !C::XT && p.absent)   // an absent cotangent is an owner tile of zeros
+        for (int t = 2; t < 4; ++t)
+            if (!p.own[t])
+                for (int i = threadIdx.x; i < C::OWN_BYTES / 16; i += JVP_THREADS) *reinterpret_cast<uint4*>(jvp_smem + t * C::OWN_BYTES + i * 16) = zero;
+    ptx::fence_proxy_async_smem();
+    if (warp == 1) {
+        ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
+        ptx::tmem_relinquish();
+    }
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    ptx::tc_fence_after_sync();
+    // The whole tensor memory starts at 0 and the shared memory of a kernel without static arrays at a 1024-byte boundary:
+    // the roles take both for granted.
+    const bool placed = *tmem_slot == 0 && (k.own & 1023) == 0;
+    if (!placed && threadIdx.x == 0) *abort_flag = 1;
+
+    // warpgroup 0: loads and MMA issue; 1, 2: element-wise; 3: epilogue
+    if (warp < 4) {
+        ptx::setmaxnreg_dec<C::REGS_LOAD>();
+        if (placed) {
+            const CUtensorMap* const maps[4] = {&o0, &o1, &o2, &o3};
+            if (warp == 0) jvp_load_ring<MODE, DP, 0>(p, k, &s0, &s1, maps, lane);
+            else if (warp == 2) jvp_load_ring<MODE, DP, 1>(p, k, &s2, &s3, maps, lane);
+            else if (warp == 1) {
+                if constexpr (C::NPAIR == 1) jvp_issue_one_pair<MODE, DP, HZ>(p, k);
+                else jvp_issue_two_pairs<MODE, DP, HZ>(p, k);
+            }
+        }
+        if (warp == 1 && *abort_flag && placed) {
+            // after a time-out: the queued MMAs must be done before the tensor memory is given back
+            ptx::mma_commit_elect(k.bar(C::B_DRAIN));
+            ptx::mbar_wait_drain(k.bar(C::B_DRAIN), 0, ptx::DRAIN_LIMIT_NS);
+        }
+    } else if (warp < 12) {
+        ptx::setmaxnreg_inc<C::REGS_ELEM>();
+        if (placed) {
+            const int grp = (warp - 4) >> 2, q = warp & 3;
+            if constexpr (MODE == PASS_FWD) jvp_elem_fwd<DP>(p, k, grp, q, lane);
+            else if constexpr (MODE == PASS_DV) jvp_elem_dv<DP, HZ>(p, k, grp, q, lane);
+            else jvp_elem_two_pairs<MODE, DP, HZ>(p, k, grp, q, lane);
+        }
+    } else {
+        ptx::setmaxnreg_dec<C::REGS_EPI>();
+        if (placed) jvp_epilogue(p, k, warp & 3, lane);
+    }
+
+    // ---------------------------------------------------------------------- teardown
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    if (warp == 1) {
+        ptx::tc_fence_after_sync();
+        ptx::tmem_dealloc(*tmem_slot, 512);
+    }
+    if (threadIdx.x == 0 && *abort_flag) atomicExch(p.status, 1);
+    // DK and DQ start while the pass before them still runs and read nothing it writes; they must still not complete
+    // before it, or completion of the last pass would not imply that the gradients of the earlier ones are written.
+    // (No effect on a launch without the attribute.)
+    if (DEPENDENT && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+}  // namespace tvm_attn

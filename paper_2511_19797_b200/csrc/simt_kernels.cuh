@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(ROWSUM_THREADS)
 bwd_rowsums_kernel(const T* __restrict__ G, const T* __restrict__ Hc, const T* __restrict__ O,
                    const T* __restrict__ tO, const float* __restrict__ lse, float* __restrict__ sig1,
                    float* __restrict__ cvec, float* __restrict__ lse2, long long rows, Geom qg, int H, int d, int cpr,
-                   int gs) {
+                   int gs, float sign) {
     constexpr int VEC = 16 / (int)sizeof(T);
     const int lane = threadIdx.x & 31;
     const int rpw = 32 / gs;                  // rows per warp and step
@@ -233,7 +233,7 @@ bwd_rowsums_kernel(const T* __restrict__ G, const T* __restrict__ Hc, const T* _
         }
         s1 = lane_group_sum(s1, gs, lane);
         cc = lane_group_sum(cc, gs, lane);
-        if (c == 0 && sub < rpw && row < rows) { sig1[row] = s1; cvec[row] = cc; lse2[row] = lse[row] * 1.4426950408889634f; }
+        if (c == 0 && sub < rpw && row < rows) { sig1[row] = sign * s1; cvec[row] = sign * cc; lse2[row] = sign * (lse[row] * 1.4426950408889634f); }
     }
 }
 

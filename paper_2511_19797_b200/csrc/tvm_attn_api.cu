@@ -12,9 +12,9 @@
 #include <mutex>
 #include <utility>
 
-#include "dual_attn_sm100.cuh"
 #include "jvp_bwd_sm100.cuh"
 #include "jvp_fwd_sm100.cuh"
+#include "jvp_sm100.cuh"
 #include "qk_rmsnorm.cuh"
 #include "simt_kernels.cuh"
 
@@ -82,6 +82,19 @@ static bool allow_smem(const DeviceFacts& f, int bytes) {
     thread_local unsigned long long done = 0;
     if (done == f.ctx) return true;
     if (cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+    done = f.ctx;
+    return true;
+}
+
+// The same for the kernels whose warpgroups redistribute registers, with a check that they were compiled to the number
+// that is redistributed (fewer would make them wait for registers that do not exist).
+template <auto KERN>
+static bool prepare_kernel(const DeviceFacts& f, int smem_bytes) {
+    thread_local unsigned long long done = 0;
+    if (done == f.ctx) return true;
+    cudaFuncAttributes attr;
+    if (cudaFuncGetAttributes(&attr, KERN) != cudaSuccess || attr.numRegs != JVP_REGS || attr.sharedSizeBytes != 0) return false;
+    if (cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes) != cudaSuccess) return false;
     done = f.ctx;
     return true;
 }
@@ -183,7 +196,7 @@ static bool q_packed(const Shape& s) {
 
 template <typename T>
 static int launch_rowsums(const Shape& s, const void* G, const void* Hc, const void* O, const void* tO, const float* lse,
-                          float* sig1, float* cvec, float* lse2, cudaStream_t st) {
+                          float* sig1, float* cvec, float* lse2, float sign, cudaStream_t st) {
     const long long rows = s.BH * s.M;
     const int cpr = s.d * (int)sizeof(T) / 16;  // 16-byte chunks per row (d % 8 == 0)
     const int gs = cpr;                          // lanes per row
@@ -192,7 +205,7 @@ static int launch_rowsums(const Shape& s, const void* G, const void* Hc, const v
     const unsigned grid = (unsigned)((rows + rows_per_block - 1) / rows_per_block);
     g_prof.before(st);
     bwd_rowsums_kernel<T><<<grid, ROWSUM_THREADS, 0, st>>>((const T*)G, (const T*)Hc, (const T*)O, (const T*)tO, lse, sig1,
-                                                           cvec, lse2, rows, s.q, q_packed(s) ? 0 : s.H, s.d, cpr, gs);
+                                                           cvec, lse2, rows, s.q, q_packed(s) ? 0 : s.H, s.d, cpr, gs, sign);
     g_prof.after(st);
     g_launches += 1;
     return cuda_status(cudaGetLastError());
@@ -248,46 +261,81 @@ static int make_tmap(CUtensorMap* m, const void* ptr, const Shape& s, const Geom
     return r == CUDA_SUCCESS ? TVM_ATTN_OK : TVM_ATTN_CUDA_ERROR;
 }
 
-// Packed (B,H,N,d) bf16 viewed as a 3-D tensor (d, N, B*H): the kernels for head dims above 80.
-static int make_tmap3(CUtensorMap* m, const void* ptr, const Shape& s, int rows) {
-    encode_tiled_fn fn = get_encode_fn();
-    if (!fn) return TVM_ATTN_CUDA_ERROR;
-    cuuint64_t dims[3] = {(cuuint64_t)s.d, (cuuint64_t)s.N, (cuuint64_t)s.BH};
-    cuuint64_t strides[2] = {(cuuint64_t)s.d * 2, (cuuint64_t)s.N * s.d * 2};
-    cuuint32_t box[3] = {64, (cuuint32_t)rows, 1};
-    cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? TVM_ATTN_OK : TVM_ATTN_CUDA_ERROR;
-}
+// A tensor of a call and its map (boxes of 64 columns x 64 rows: one map serves a tensor in every role it has in the passes
+// of a call).  An absent cotangent is never loaded: its map is that of a present tensor and unused.
+struct Operand {
+    const __nv_bfloat16* ptr;
+    const CUtensorMap* map;
+};
 
-template <int MODE, int NA>
-static int launch_tc(const Shape& s, const void* const own[4], const void* const strm[4], const TcParams& prm,
-                     const DeviceFacts& dev, cudaStream_t st) {
-    using C = TcCfg<MODE, NA>;
-    CUtensorMap mo[4], ms[4];
+template <int MODE, int DP, bool HZ>
+static int launch_pass(const Shape& s, const Operand (&own)[4], const Operand (&strm)[4], JvpParams prm, const DeviceFacts& dev, cudaStream_t st) {
+    using C = JvpCfg<MODE, DP>;
+    constexpr auto kern = jvp_kernel<MODE, DP, HZ>;
+    if (!prepare_kernel<kern>(dev, C::SMEM_BYTES)) return TVM_ATTN_CUDA_ERROR;
+    // DV, DK: keys own, queries stream; FWD, DQ: queries own, keys stream
+    prm.o = C::TRANSPOSED ? s.k : s.q;
+    prm.s = C::TRANSPOSED ? s.q : s.k;
     for (int t = 0; t < 4; ++t) {
-        const void* po = own[t < C::NOWN ? t : 0];
-        int rc = make_tmap3(&mo[t], po, s, TC_OWN_ROWS);
-        if (rc != TVM_ATTN_OK) return rc;
-        rc = make_tmap3(&ms[t], strm[t], s, C::BC);
-        if (rc != TVM_ATTN_OK) return rc;
+        prm.own[t] = own[t].ptr;
+        prm.strm[t] = strm[t].ptr;
     }
-    auto kern = dual_attn_kernel<MODE, NA>;
-    if (!allow_smem<dual_attn_kernel<MODE, NA>>(dev, C::SMEM_BYTES)) return TVM_ATTN_CUDA_ERROR;
-    const long long grid = s.BH * ((s.N + TC_OWN_ROWS - 1) / TC_OWN_ROWS);
+    // one CTA per SM (each needs the whole tensor memory and most of the shared memory of one); the work
+    // items go round-robin over them
+    const long long items = s.BH * ((prm.o.rows + JVP_ROWS - 1) / JVP_ROWS);
     g_prof.before(st);
-    kern<<<(unsigned)grid, TC_THREADS, C::SMEM_BYTES, st>>>(mo[0], mo[1], mo[2], mo[3], ms[0], ms[1], ms[2], ms[3], prm);
+    // DK and DQ read nothing that the pass before them writes (DV, DK and DQ all depend on the row-sums pre-pass only,
+    // which has completed before DV starts), so their CTAs may fill the SMs that the last, partial wave of the pass
+    // before leaves idle: programmatic dependent launch, with every CTA of these kernels releasing its dependents at
+    // once.  None waits for its primary before it works; each waits for it once at the very end (griddepcontrol.wait in
+    // the teardown), so that DQ cannot complete before DK, nor DK before DV: work enqueued behind the call still sees all
+    // six gradients.  Not while per-kernel events are being recorded: they would time overlapping kernels.
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(items < dev.sms ? items : dev.sms));
+    cfg.blockDim = dim3(JVP_THREADS);
+    cfg.dynamicSmemBytes = C::SMEM_BYTES;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = ((MODE == PASS_DK || MODE == PASS_DQ) && !g_prof.enabled.load(std::memory_order_relaxed)) ? 1 : 0;
+    if (cudaLaunchKernelEx(&cfg, kern, *strm[0].map, *strm[1].map, *strm[2].map, *strm[3].map, *own[0].map, *own[1].map, *own[2].map,
+                           *own[3].map, prm) != cudaSuccess)
+        return cuda_status(cudaGetLastError());
     g_prof.after(st);
     g_launches += 1;
     return cuda_status(cudaGetLastError());
 }
 
+// Padded head dims up to this one run the kernels of jvp_fwd_sm100.cuh and jvp_bwd_sm100.cuh.
+#ifndef JVP_MIN
+#define JVP_MIN 80
+#endif
+template <int MODE, int DP>
+static int launch_pass_hz(const Shape& s, const Operand (&own)[4], const Operand (&strm)[4], const JvpParams& prm, const DeviceFacts& dev, cudaStream_t st) {
+    if constexpr (DP <= JVP_MIN) return TVM_ATTN_UNSUPPORTED;
+    else {
+        // dtO absent: the specialisation that leaves the tangent path out (only instantiated for the padded head dims
+        // 64 and 80 of the transformer shapes; other head dims run the general kernel, which skips what it can)
+        if constexpr (MODE != PASS_FWD && (DP == 64 || DP == 80))
+            if (prm.absent & ABSENT_HC) return launch_pass<MODE, DP, true>(s, own, strm, prm, dev, st);
+        return launch_pass<MODE, DP, false>(s, own, strm, prm, dev, st);
+    }
+}
+
 template <int MODE>
-static int launch_tc_na(const Shape& s, const void* const own[4], const void* const strm[4], const TcParams& prm,
-                        const DeviceFacts& dev, cudaStream_t st) {
-    return launch_tc<MODE, 2>(s, own, strm, prm, dev, st);   // head dims above 80
+static int launch_pass_dp(const Shape& s, const Operand (&own)[4], const Operand (&strm)[4], const JvpParams& prm, const DeviceFacts& dev, cudaStream_t st) {
+    switch (s.dp) {
+        case 16: return launch_pass_hz<MODE, 16>(s, own, strm, prm, dev, st);
+        case 32: return launch_pass_hz<MODE, 32>(s, own, strm, prm, dev, st);
+        case 48: return launch_pass_hz<MODE, 48>(s, own, strm, prm, dev, st);
+        case 64: return launch_pass_hz<MODE, 64>(s, own, strm, prm, dev, st);
+        case 80: return launch_pass_hz<MODE, 80>(s, own, strm, prm, dev, st);
+        case 96: return launch_pass_hz<MODE, 96>(s, own, strm, prm, dev, st);
+        case 112: return launch_pass_hz<MODE, 112>(s, own, strm, prm, dev, st);
+        default: return launch_pass_hz<MODE, 128>(s, own, strm, prm, dev, st);
+    }
 }
 
 // Forward for padded head dims up to 80: operands Q, tQ live in tensor memory (jvp_fwd_sm100.cuh).
@@ -380,17 +428,6 @@ static int launch_bwd_pass_dp(const Shape& s, const void* const own[4], const vo
         case 64: return launch_bwd_pass<MODE, 64>(s, own, strm, prm, dev, st);
         default: return launch_bwd_pass<MODE, 80>(s, own, strm, prm, dev, st);
     }
-}
-
-static TcParams base_params(const Shape& s, int* status) {
-    TcParams prm;
-    std::memset(&prm, 0, sizeof prm);
-    prm.N = s.N; prm.d = s.d; prm.dp = s.dp; prm.BH = (int)s.BH;
-    prm.alpha = s.alpha;
-    prm.c2 = s.alpha * 1.4426950408889634f;
-    prm.out_scale = 1.0f;
-    prm.status = status;
-    return prm;
 }
 
 // Scratch of tvm_attn_jvp_bwd_noalloc: three floats per row, for callers that cannot allocate.  In host code
@@ -561,7 +598,7 @@ int tvm_attn_jvp_fwd(const tvm_attn_params* p, const void* Q, const void* K, con
     if (rc != TVM_ATTN_OK) return rc;
     int* status = dev->status;
     const void* strm[4] = {K, tK, V, tV};
-    if (s.dp <= 80) {
+    if (s.dp <= JVP_MIN) {
         FwdParams f;
         f.d = s.d; f.BH = (int)s.BH; f.H = s.H; f.q = s.q; f.k = s.k;
         f.alpha = s.alpha; f.c2 = s.alpha * 1.4426950408889634f;
@@ -578,11 +615,22 @@ int tvm_attn_jvp_fwd(const tvm_attn_params* p, const void* Q, const void* K, con
             default: return launch_fwd<80>(s, strm, f, *dev, st);
         }
     }
-    if (!s.plain) return TVM_ATTN_UNSUPPORTED;  // head dims above 80: self-attention on packed tensors only
-    TcParams prm = base_params(s, status);
-    prm.out0 = O; prm.out1 = tO; prm.lse_out = lse; prm.mu_out = mu;
-    const void* own[4] = {Q, tQ, Q, tQ};
-    return launch_tc_na<MODE_FWD>(s, own, strm, prm, *dev, st);
+    if (s.dp > 80 && !s.plain) return TVM_ATTN_UNSUPPORTED;  // head dims above 80: self-attention on packed tensors only
+    CUtensorMap maps[6];
+    const void* in[6] = {Q, tQ, K, tK, V, tV};
+    Operand x[6];
+    for (int t = 0; t < 6; ++t) {
+        rc = make_tmap(&maps[t], in[t], s, t < 2 ? s.q : s.k, JVP_BC);
+        if (rc != TVM_ATTN_OK) return rc;
+        x[t] = {static_cast<const __nv_bfloat16*>(in[t]), &maps[t]};
+    }
+    JvpParams f;
+    std::memset(&f, 0, sizeof f);
+    f.d = s.d; f.BH = (int)s.BH; f.H = s.H;
+    f.alpha = s.alpha; f.c2 = s.alpha * 1.4426950408889634f;
+    f.out0 = static_cast<__nv_bfloat16*>(O); f.out1 = static_cast<__nv_bfloat16*>(tO);
+    f.lse = lse; f.mu_out = mu; f.status = status;
+    return launch_pass_dp<PASS_FWD>(s, {x[0], x[1], x[0], x[1]}, {x[2], x[3], x[4], x[5]}, f, *dev, st);
 }
 
 int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, const void* V, const void* tQ,
@@ -625,11 +673,11 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
     }
     if (s.simt) {
         if (s.fp32) {
-            rc = launch_rowsums<float>(s, dO, dtO, O, tO, lse, sig1, cvec, lse2, st);
+            rc = launch_rowsums<float>(s, dO, dtO, O, tO, lse, sig1, cvec, lse2, 1.0f, st);
             if (rc != TVM_ATTN_OK) return rc;
             return simt_bwd<float>(s, Q, K, V, tQ, tK, tV, lse, mu, dO, dtO, sig1, cvec, dQ, dK, dV, dtQ, dtK, dtV, st);
         }
-        rc = launch_rowsums<__nv_bfloat16>(s, dO, dtO, O, tO, lse, sig1, cvec, lse2, st);
+        rc = launch_rowsums<__nv_bfloat16>(s, dO, dtO, O, tO, lse, sig1, cvec, lse2, 1.0f, st);
         if (rc != TVM_ATTN_OK) return rc;
         return simt_bwd<__nv_bfloat16>(s, Q, K, V, tQ, tK, tV, lse, mu, dO, dtO, sig1, cvec, dQ, dK, dV, dtQ, dtK, dtV, st);
     }
@@ -637,9 +685,9 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
     rc = tensor_core_device(&dev);
     if (rc != TVM_ATTN_OK) return rc;
     int* status = dev->status;
-    rc = launch_rowsums<__nv_bfloat16>(s, dO, dtO, O, tO, lse, sig1, cvec, lse2, st);
+    rc = launch_rowsums<__nv_bfloat16>(s, dO, dtO, O, tO, lse, sig1, cvec, lse2, s.dp <= JVP_MIN ? 1.0f : -1.0f, st);
     if (rc != TVM_ATTN_OK) return rc;
-    if (s.dp <= 80) {
+    if (s.dp <= JVP_MIN) {
         BwdParams b;
         std::memset(&b, 0, sizeof b);
         b.d = s.d; b.BH = (int)s.BH; b.H = s.H;
@@ -670,29 +718,36 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
         }
         return rc;
     }
-    TcParams prm = base_params(s, status);
-    prm.lse = lse; prm.mu = mu; prm.sig1 = sig1; prm.cvec = cvec;
-    {   // dtV = P^T Hc, dV = P^T G + (P*Nn)^T Hc : owner keys (K, tK), stream queries (Q, tQ | Hc, G)
-        TcParams q = prm; q.out0 = dtV; q.out1 = dV;
-        const void* own[4] = {K, tK, K, tK};
-        const void* strm[4] = {Q, tQ, dtO, dO};
-        rc = launch_tc_na<MODE_DV>(s, own, strm, q, *dev, st);
+    CUtensorMap maps[8];
+    const void* in[8] = {Q, tQ, dtO, dO, K, tK, V, tV};
+    Operand x[8];
+    for (int t = 0; t < 8; ++t) {
+        x[t] = {static_cast<const __nv_bfloat16*>(in[t]), in[t] ? &maps[t] : &maps[0]};
+        rc = in[t] ? make_tmap(&maps[t], in[t], s, t < 4 ? s.q : s.k, JVP_BC) : TVM_ATTN_OK;
         if (rc != TVM_ATTN_OK) return rc;
     }
-    {   // dtK = alpha W^T Q, dK = alpha (dA^T Q + W^T tQ) : owner keys (K, tK, V, tV), stream (Q, tQ, Hc, G)
-        TcParams q = prm; q.out0 = dtK; q.out1 = dK; q.out_scale = s.alpha;
-        const void* own[4] = {K, tK, V, tV};
-        const void* strm[4] = {Q, tQ, dtO, dO};
-        rc = launch_tc_na<MODE_DK>(s, own, strm, q, *dev, st);
-        if (rc != TVM_ATTN_OK) return rc;
-    }
-    {   // dtQ = alpha W K, dQ = alpha (dA K + W tK) : owner queries (Q, tQ, Hc, G), stream (K, tK, V, tV)
-        TcParams q = prm; q.out0 = dtQ; q.out1 = dQ; q.out_scale = s.alpha;
-        const void* own[4] = {Q, tQ, dtO, dO};
-        const void* strm[4] = {K, tK, V, tV};
-        rc = launch_tc_na<MODE_DQ>(s, own, strm, q, *dev, st);
-    }
-    return rc;
+    const Operand &xQ = x[0], &xtQ = x[1], &xH = x[2], &xG = x[3], &xK = x[4], &xtK = x[5], &xV = x[6], &xtV = x[7];
+    JvpParams b;
+    std::memset(&b, 0, sizeof b);
+    b.d = s.d; b.BH = (int)s.BH; b.H = s.H;
+    b.alpha = s.alpha; b.c2 = s.alpha * 1.4426950408889634f;
+    b.nlse2 = lse2; b.mu = mu; b.nsig1 = sig1; b.ncvec = cvec; b.status = status; b.absent = absent;
+    auto outputs = [&](void* tangent, void* primal, float scale) {
+        b.out0 = dtO ? static_cast<__nv_bfloat16*>(tangent) : nullptr;
+        b.out1 = static_cast<__nv_bfloat16*>(primal);
+        b.out_scale = scale;
+    };
+    // dtV = P^T Hc, dV = P^T G + (P*Nn)^T Hc : owner keys (K, tK); stream queries (Q, tQ | Hc, G)
+    outputs(dtV, dV, 1.0f);
+    rc = launch_pass_dp<PASS_DV>(s, {xK, xtK, xK, xtK}, {xQ, xtQ, xH, xG}, b, *dev, st);
+    if (rc != TVM_ATTN_OK) return rc;
+    // dtK = alpha W^T Q, dK = alpha (dA^T Q + W^T tQ) : owner keys (K, tK, V, tV); stream (Hc, G | Q, tQ)
+    outputs(dtK, dK, s.alpha);
+    rc = launch_pass_dp<PASS_DK>(s, {xK, xtK, xV, xtV}, {xH, xG, xQ, xtQ}, b, *dev, st);
+    if (rc != TVM_ATTN_OK) return rc;
+    // dtQ = alpha W K, dQ = alpha (dA K + W tK) : owner queries (Q, tQ, Hc, G); stream (V, tV | K, tK)
+    outputs(dtQ, dQ, s.alpha);
+    return launch_pass_dp<PASS_DQ>(s, {xQ, xtQ, xH, xG}, {xV, xtV, xK, xtK}, b, *dev, st);
 }
 
 int tvm_attn_jvp_bwd_noalloc(const tvm_attn_params* p, const void* Q, const void* K, const void* V, const void* tQ,

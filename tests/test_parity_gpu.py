@@ -64,6 +64,13 @@ def test_ragged_and_degenerate_shapes(B, H, N, d, mode):
         assert_within(errs, BF16_FWD, BF16_BWD, BF16_STATS)
 
 
+# head dims above 80: several items per CTA, an odd number of tiles, ragged rows, both 16-column tails
+@pytest.mark.parametrize("B,H,N,d,peaky", [(3, 50, 192, 96, 0.0), (2, 40, 300, 128, 0.0), (1, 90, 130, 112, 0.1), (1, 2, 1, 88, 0.0), (4, 80, 65, 120, 0.0)])
+def test_wide_head_dims_with_several_items_per_block(B, H, N, d, peaky):
+    errs, _, _ = run_case(inputs.custom(B, H, N, d, seed=60 + d, peaky_frac=peaky), oracle_heads=[0, B * H // 2, B * H - 1])
+    assert_within(errs, BF16_FWD, BF16_BWD, BF16_STATS)
+
+
 @pytest.mark.parametrize("B,H,N,d", [(3, 50, 192, 72), (3, 50, 320, 64), (5, 61, 65, 72), (2, 80, 200, 40),
                                      (4, 50, 64, 72), (4, 50, 33, 40)])
 def test_several_work_items_per_cta(B, H, N, d):
