@@ -24,20 +24,22 @@
 //   warp 0    loads the owner tiles and the E ring (stream tensors that only the score MMAs read)
 //   warp 1    issues the MMAs
 //   warp 2    loads the L ring (stream tensors the output MMAs read)
-//   warps 4-11   element-wise work: two groups of four warps take the tiles in turn; a thread has one owner row and all
-//             64 columns of the tile
+//   warp 3    DV, DK: puts the per-query statistics into the tiles (FOLD below)
+//   warps 4-11   element-wise work, two groups of four warps
 //   warps 12-15  epilogue: normalise, convert and store an item's accumulators while the next item is under way
 //
 // Why this split.  What bounds a tile is not one unit but the chain scores -> element-wise work -> outputs: passing an
-// mbarrier costs a warp 100 to 250 cycles even when the phase has completed, reading tensor memory 180.  A warp pays that
-// for every other tile and for all of its columns, and nothing is exchanged between warps that share a row (the forward's
-// row maximum is the thread's own).
+// mbarrier costs a warp 100 to 250 cycles even when the phase has completed, reading tensor memory 180, whether it has 16
+// columns to work on or 64, and the warps of a scheduler take issue slots from the one that issues the MMAs: eight
+// element-wise warps with many columns each, the accumulators' way out on warps of its own.
 //
 // Score MMAs: the two tensors of a stage are interleaved so that they form one K-major operand of 128 rows, and
 // [S | X0 Y1^T] = X0 [Y0 | Y1]^T is one N = 128 MMA per k-step, Sd += X1 Y0^T one N = 64 MMA.
 //
 // Measured on B200 at d = 128 (B 2, H 24, N 4096; one CTA per item, 32-key tiles with all four accumulators in two buffers
-// before): forward 1.40 -> 1.08 ms, DV / DK / DQ 1.33 / 2.82 / 2.92 -> 1.06 / 1.48 / 1.42 ms.
+// before): forward 1.40 -> 1.08 ms, DV / DK / DQ 1.33 / 2.82 / 2.92 -> 1.06 / 1.48 / 1.42 ms.  At d <= 80 (two
+// element-wise groups on alternate tiles, which also wrote the outputs, before): d = 64 (8, 16, 4096) forward 1.94 -> 1.75 ms, backward 7.37 -> 6.12 ms;
+// d = 72 (16, 16, 1024) forward 321 -> 306 us, backward 1.22 -> 1.08 ms.
 //
 // Every wait on an mbarrier is bounded; when one gives up the block records a time-out status and all roles leave their
 // loops.
@@ -68,7 +70,8 @@ constexpr uint64_t JVP_WAIT_LIMIT_NS = 200ull * 1000ull * 1000ull;
 constexpr int JVP_REGS = 128;
 
 struct JvpParams {
-    int d, BH, H;
+    int d, H;
+    int items, row_tiles, T;   // work items (128 owner rows of a head), items per head, stream tiles per item
     Geom o, s;    // owner side and stream side of this pass (FWD, DQ: queries own, keys stream; DV, DK: the other way round)
     float alpha;      // softmax scale
     float c2;         // alpha * log2(e)
@@ -126,8 +129,8 @@ struct JvpCfg {
     static constexpr int FOLD_BYTES = 2 * BC * 16;
     static constexpr int FOLD_E = FOLD ? SE : 0, FOLD_L = FOLD && NPAIR == 2 ? SL : 0;
     static constexpr int ONES_BYTES = FOLD ? JVP_ROWS * 32 : 0;
-    static constexpr int EFULL_COUNT = TAIL ? 33 : 1;                    // TMA issuer (+ each lane's own copies)
-    static constexpr int LFULL_COUNT = TAIL || (TRANSPOSED && !FOLD) ? 33 : 1;
+    static constexpr int EFULL_COUNT = 1 + (TAIL ? 32 : 0) + (FOLD_E ? 1 : 0);   // TMA issuer, each lane's own copies, warp 3
+    static constexpr int LFULL_COUNT = 1 + (TAIL || (TRANSPOSED && !FOLD) ? 32 : 0) + (FOLD_L ? 1 : 0);
     // TMEM columns: accumulators, the owner operands in the gaps behind them (and 8 columns of ones behind the first),
     // score accumulators (FWD, DV: two buffers of S | Sd; DK, DQ: one of S | Sd | D | X).
     static constexpr int COL_ACC0 = 0, COL_ACC1 = XT ? 128 : DP, COL_SCORE = 2 * COL_ACC1;
@@ -135,8 +138,7 @@ struct JvpCfg {
     static_assert(!XT || DP + DP / 2 + 8 <= 128, "operands do not fit behind their accumulators");
     static_assert(COL_SCORE + 4 * BC <= 512, "TMEM over-subscribed");
     // registers per thread: warpgroup 0, element-wise warps, epilogue warps (which hold an owner row, 4 registers a chunk)
-    static constexpr int REGS_LOAD = MODE == PASS_FWD ? 56 : 64, REGS_ELEM = MODE == PASS_FWD ? 184 : MODE == PASS_DV ? 168 : 176,
-                         REGS_EPI = MODE == PASS_FWD ? 88 : MODE == PASS_DV ? 112 : 96;
+    static constexpr int REGS_LOAD = MODE == PASS_FWD ? 56 : 96, REGS_ELEM = MODE == PASS_FWD ? 184 : 152, REGS_EPI = MODE == PASS_FWD ? 88 : 112;
     static_assert(REGS_LOAD + 2 * REGS_ELEM + REGS_EPI <= 4 * JVP_REGS, "more registers than the block has");
     // barriers
     static constexpr int B_EFULL = 0;
@@ -172,26 +174,43 @@ struct JvpCfg {
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory over-subscribed");
 };
 
-// What the roles of a block share.
+// A value that is to stay in a register (kernel parameters are otherwise read from constant memory wherever they are used,
+// which costs a dependent instruction 30 cycles more).
+__device__ __forceinline__ int jvp_pin(int v) {
+    asm volatile("" : "+r"(v));
+    return v;
+}
+
+// What the roles of a block share: addresses, all of them the base of its shared memory plus constants (the element-wise
+// warps have no registers to spare for more), and waits.
 template <int MODE, int DP>
 struct JvpBlock {
     using C = JvpCfg<MODE, DP>;
-    uint32_t own, e, l;          // shared-memory addresses of the owner tiles and the rings
-    uint32_t fold_e, fold_l, ones, zeros;   // FOLD: statistics of the E and L stages; ones and zeros, 128 rows of 16 bytes
-    bool fold_step;                  // FOLD: a k-step of their own (else they are the padding columns of the last one)
-    uint32_t bar0;
-    volatile int* abort_flag;
-    float* stats;                // DV, DK, WIDE: [stage][NSTAT][64]
-    float4* row_state;           // FWD: (m, c, running maximum) of each row
-    float4* row_sums;            // FWD: [group][row] (l, sum P~ (T - c), m, c)
-    int items, row_tiles, T;     // work items, items per head, stream tiles per item
+    uint32_t base;
+    const JvpParams& p;
+    static constexpr uint32_t E = C::NOWN * C::OWN_BYTES, L = E + C::SE * 2 * C::EST_BYTES, MISC = C::TILE_BYTES, SLOT = MISC + 56 * 8, ABORT = SLOT + 16;
+    static constexpr uint32_t STATS = SLOT + 64;                              // DV, DK, WIDE: [stage][NSTAT][64] floats
+    static constexpr uint32_t ROW_STATE = STATS + C::STATS_FLOATS * 4;        // FWD: float4 (m, c, running maximum) of each row
+    static constexpr uint32_t ROW_SUMS = ROW_STATE + 16 * JVP_ROWS;           // FWD: [group][row] float4 (l, sum P~ (T - c), m, c)
+    static constexpr uint32_t FOLD_E = ROW_STATE + C::FWD_FLOATS * 4;         // FOLD: statistics of the E and the L stages,
+    static constexpr uint32_t FOLD_L = FOLD_E + C::FOLD_E * C::FOLD_BYTES;    // ones and zeros, 128 rows of 16 bytes
+    static constexpr uint32_t ONES = FOLD_L + C::FOLD_L * C::FOLD_BYTES, ZEROS = ONES + JVP_ROWS * 16;
 
-    __device__ __forceinline__ uint32_t bar(int i) const { return bar0 + 8u * static_cast<uint32_t>(i); }
+    // A copy for a role with registers to spare: the base stays in one.
+    __device__ __forceinline__ JvpBlock pinned() const {
+        JvpBlock r = *this;
+        asm volatile("" : "+r"(r.base));
+        return r;
+    }
+    // FOLD: the statistics have a k-step of their own (else they are the padding columns of the last one)
+    __device__ __forceinline__ bool fold_step() const { return C::FOLD && (C::NA == 1 || p.d == DP); }
+    __device__ __forceinline__ uint32_t bar(int i) const { return base + MISC + 8u * static_cast<uint32_t>(i); }
     __device__ __forceinline__ bool wait(int i, int phase) const {
-        return ptx::mbar_wait_warp(bar(i), phase & 1, abort_flag, JVP_WAIT_LIMIT_NS);
+        return ptx::mbar_wait_warp_s(bar(i), phase & 1, base + ABORT, JVP_WAIT_LIMIT_NS);
     }
     __device__ __forceinline__ bool wait2(int i, int pi, int j, int pj) const {
-        return ptx::mbar_wait2_warp(bar(i), pi & 1, bar(j), pj & 1, abort_flag, JVP_WAIT_LIMIT_NS);
+        if (ptx::mbar_test2_warp(bar(i), pi & 1, bar(j), pj & 1)) return true;
+        return wait(i, pi) && wait(j, pj);
     }
     // After the waits for a tile: what other warps copied to it (tails) is ordered before the MMAs that read it.
     __device__ __forceinline__ void tile_fence() const {
@@ -199,9 +218,10 @@ struct JvpBlock {
         ptx::tc_fence_after_sync();
     }
     __device__ __forceinline__ bool done(int i, int g) const { return wait(i + (g & 3), g >> 2); }   // i: B_SFULL, B_XFULL, B_OUTDONE
-    __device__ __forceinline__ uint32_t own_tile(int t) const { return own + t * C::OWN_BYTES; }
-    __device__ __forceinline__ uint32_t e_stage(int s) const { return e + s * 2 * C::EST_BYTES; }
-    __device__ __forceinline__ uint32_t l_stage(int s) const { return l + s * 2 * C::LST_BYTES; }
+    __device__ __forceinline__ uint32_t own_tile(int t) const { return base + t * C::OWN_BYTES; }
+    __device__ __forceinline__ const float* stats(int s) const { return static_cast<const float*>(__cvta_shared_to_generic(base + STATS + s * C::NSTAT * C::BC * 4)); }
+    __device__ __forceinline__ float4& row_state(int r) const { return *static_cast<float4*>(__cvta_shared_to_generic(base + ROW_STATE + 16 * r)); }
+    __device__ __forceinline__ float4& row_sums(int r) const { return *static_cast<float4*>(__cvta_shared_to_generic(base + ROW_SUMS + 16 * r)); }
     // one arrival per warp, after its tensor-memory accesses
     __device__ __forceinline__ void arrive(int i, int lane) const {
         ptx::tc_fence_before_sync();
@@ -217,7 +237,7 @@ template <int MODE, int DP>
 __device__ __forceinline__ void jvp_load_owners(const JvpParams& p, const JvpBlock<MODE, DP>& k, const CUtensorMap* const (&maps)[4], int item, int lane) {
     using C = JvpCfg<MODE, DP>;
     constexpr int KT = C::TAIL ? (DP - 64) / 8 : 1, H64 = 64 * 128;
-    const int bh = item / k.row_tiles, row0 = (item - bh * k.row_tiles) * JVP_ROWS;
+    const int bh = item / p.row_tiles, row0 = (item - bh * p.row_tiles) * JVP_ROWS;
     const int cb = bh / p.H, ch = bh - cb * p.H;
     if (lane == 0) {
         const uint32_t full = k.bar(C::B_OWN);
@@ -259,36 +279,28 @@ __device__ __forceinline__ void jvp_load_owners(const JvpParams& p, const JvpBlo
     }
 }
 
-// Three bf16 parts of x whose sum is x to 24 bits, in the first three of eight columns.
-__device__ __forceinline__ uint4 jvp_split3(float x) {
-    const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-    const float r = x - __bfloat162float(hi);
-    const __nv_bfloat16 mid = __float2bfloat16_rn(r);
-    const __nv_bfloat16 lo = __float2bfloat16_rn(r - __bfloat162float(mid));
-    return make_uint4((uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(mid) << 16), __bfloat16_as_ushort(lo), 0u, 0u);
-}
-constexpr uint32_t JVP_ONES0 = 0x3F803F80u, JVP_ONES1 = 0x00003F80u;   // 1, 1, 1, 0 in bf16: what the parts are multiplied by
-
-// One warp per ring; the E ring's loads the owner tiles too.  Lane 0 issues the TMA boxes; with a tail (DP = 80) or
+// One warp per ring; the E ring's loads the owner tiles too.  One lane issues the TMA boxes; with a tail (DP = 80) or
 // statistics copied as they are (WIDE) all lanes copy those, 16 bytes each, and each lane's arrival on the stage's barrier
-// is left to its copies (a warp that waits for them itself loads no more than one tile per memory latency: 1300 cycles a
-// tile).  FOLD: the lanes split the tile's statistics (loaded one tile ahead) and store the parts.
+// is left to its copies (a warp that waits for them itself loads no more than one tile per memory latency).  These loops
+// run next to element-wise warps that leave them few issue slots, and a ring is refilled no faster than they run: what does
+// not depend on the tile is set up before them, and tiles whose rows all exist take a path without predicates.
 template <int MODE, int DP, int RING>
-__device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock<MODE, DP>& k, const CUtensorMap* map0, const CUtensorMap* map1,
+__device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock<MODE, DP>& shared, const CUtensorMap* map0, const CUtensorMap* map1,
                                               const CUtensorMap* const (&own_maps)[4], int lane) {
     using C = JvpCfg<MODE, DP>;
+    const JvpBlock<MODE, DP> k = shared.pinned();
+    const int T = jvp_pin(p.T), rows = jvp_pin(p.s.rows);
     constexpr int BC = C::BC, S = RING == 0 ? C::SE : C::SL, ATOM = C::ATOM;
     constexpr int b_full = RING == 0 ? C::B_EFULL : C::B_LFULL, b_done = RING == 0 ? C::B_EDONE : C::B_OUTDONE;
     constexpr uint32_t TB = RING == 0 ? C::EST_BYTES : C::LST_BYTES;
     constexpr bool STATS = RING == 1 && C::TRANSPOSED && !C::FOLD;   // this ring carries the statistics as they are
-    constexpr bool FOLDED = C::FOLD && (RING == 0 || C::NPAIR == 2);  // ... as columns of the stream rows
     constexpr bool OWNERS = RING == 0 && C::NOWN > 0;
     constexpr bool HAS_CP = C::TAIL || STATS;           // the warp has asynchronous copies of its own
     constexpr int KT = C::TAIL ? (DP - 64) / 8 : 1;     // 16-byte chunks per row behind column 64, at most
     [[maybe_unused]] const int ntail = C::TAIL ? (p.d - 64) >> 3 : 0;
     [[maybe_unused]] const size_t d32 = 32 * (size_t)p.s.rs;   // 32 rows further down, in elements
     [[maybe_unused]] const size_t tile_elems = (size_t)BC * (size_t)p.s.rs;
-    const uint32_t ring_base = RING == 0 ? k.e : k.l;
+    const uint32_t ring_base = k.base + (RING == 0 ? k.E : k.L);
     const __nv_bfloat16* base0 = p.strm[2 * RING];
     const __nv_bfloat16* base1 = p.strm[2 * RING + 1];
     // the ring that streams the cotangents (Hc, G): L in DV, E in DK; an absent one is not loaded
@@ -296,40 +308,20 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
     const bool has0 = !COT || !(p.absent & ABSENT_HC), has1 = !COT || !(p.absent & ABSENT_G);
     const uint32_t tx_bytes = ((has0 ? 1 : 0) + (has1 ? 1 : 0)) * ATOM * (C::WIDE ? 2 : 1);
     // Chunk 0 of row `lane` behind the first atoms: compact blocks in the E ring, a second swizzled atom in the L ring.
-    [[maybe_unused]] const uint32_t dst_lane = 2 * ATOM + (RING == 0 ? lane * 16 : lane * 128);
     [[maybe_unused]] const uint32_t sw = lane & 7;  // rows 32 apart share it
+    [[maybe_unused]] const uint32_t dst_lane = 2 * ATOM + (RING == 0 ? lane * 16 : lane * 128);
     // statistics as they are: 16-byte chunks when the rows of the (B, H, M) arrays are 16-byte aligned, else floats
     [[maybe_unused]] const bool st16 = (p.s.rows & 3) == 0;
-    [[maybe_unused]] const uint32_t st_base = ptx::smem_u32(k.stats);
-    // FOLD: the two statistics of this ring, the factors that bring them to the accumulators' scale, and where the parts of
-    // (tensor t, row lane + 32 rp) go: block + (t, rp steps)
-    constexpr bool COT_STATS = MODE == PASS_DK && RING == 0;
-    [[maybe_unused]] const float* stat0 = COT_STATS ? p.nsig1 : p.nlse2;
-    [[maybe_unused]] const float* stat1 = COT_STATS ? p.ncvec : p.mu;
-    [[maybe_unused]] const float fac0 = COT_STATS ? 1.0f : 1.0f / p.c2, fac1 = COT_STATS ? 1.0f : -1.0f / p.alpha;
-    [[maybe_unused]] const bool own_step = k.fold_step;
-    [[maybe_unused]] const uint32_t fold_base = own_step ? (RING == 0 ? k.fold_e : k.fold_l) + lane * 16
-                                                         : ring_base + (RING == 0 ? 2 * ATOM + 2 * BC * 16 + lane * 16 : 2 * ATOM + lane * 128 + ((1 ^ sw) << 4));
-    [[maybe_unused]] const uint32_t fold_stage = own_step ? C::FOLD_BYTES : 2 * TB;
-    [[maybe_unused]] const uint32_t fold_t = own_step || RING == 0 ? BC * 16 : ATOM, fold_rp = own_step || RING == 0 ? 32 * 16 : 32 * 128;
-    [[maybe_unused]] float nx[4] = {0.f, 0.f, 0.f, 0.f};   // the next tile's statistics of rows lane, lane + 32
-    [[maybe_unused]] auto load_stats = [&](int bh, int j) {
-        const size_t at = (size_t)bh * p.s.rows + (size_t)j * BC + lane;
-        const int left = p.s.rows - j * BC - lane;   // queries beyond M: zero, like their rows of the operands
-        nx[0] = left > 0 ? __ldg(stat0 + at) : 0.f;
-        nx[1] = left > 0 ? __ldg(stat1 + at) : 0.f;
-        nx[2] = left > 32 ? __ldg(stat0 + at + 32) : 0.f;
-        nx[3] = left > 32 ? __ldg(stat1 + at + 32) : 0.f;
-    };
+    [[maybe_unused]] const uint32_t st_base = k.base + k.STATS;
     bool ok = true;
     int s = 0, ph = 0;
     int g = 0, owners = 0;           // tiles, and items whose owner tiles, have been asked for
+    uint32_t stage = ring_base, full = k.bar(b_full);
     // In an item's tiles the owner tiles have their turn where what they wait for is about to happen: behind as many of the
     // item's E tiles as the ring holds.
-    [[maybe_unused]] const int owners_at = min(S, k.T) - 1;
-    if (FOLDED && (int)blockIdx.x < k.items) load_stats(blockIdx.x / k.row_tiles, 0);
-    for (int item = blockIdx.x; ok && item < k.items; item += gridDim.x) {
-        const int bh = item / k.row_tiles;
+    [[maybe_unused]] const int owners_at = min(S, T) - 1;
+    for (int item = blockIdx.x; ok && item < p.items; item += gridDim.x) {
+        const int bh = item / p.row_tiles;
         const int cb = bh / p.H, ch = bh - cb * p.H;   // batch and head: coordinates of the 4-D tensor maps
         // element offset of (row `lane`, column 64) in the stream tensors
         [[maybe_unused]] const size_t lane_row = p.s.head_off(bh, p.H) + (size_t)lane * (size_t)p.s.rs + 64;
@@ -342,7 +334,7 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
             st_src0 = (lane < 16 ? p.nlse2 : p.mu) + srow + 4 * (lane & 15);
             if (C::NSTAT == 4) st_src1 = (lane < 16 ? p.nsig1 : p.ncvec) + srow + 4 * (lane & 15);
         }
-        for (int j = 0; j < k.T; ++j) {
+        for (int j = 0; j < T; ++j) {
             if (OWNERS && j == owners_at) {   // once the score MMAs of the item before are complete
                 ok = owners == 0 || k.wait(C::B_OWNFREE, owners - 1);
                 if (!ok) break;
@@ -352,19 +344,8 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
             if (g >= S) ok = k.done(b_done, g - S);   // the MMAs that read the stage's last tile
             if (!ok) break;
             ++g;
-            const int rows_left = p.s.rows - j * BC;  // rows of this tile that exist
-            if constexpr (FOLDED) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {   // (row step i >> 1, tensor i & 1)
-                    const uint4 v = jvp_split3(nx[i] * ((i & 1) ? fac1 : fac0));
-                    ptx::st_shared_v4(fold_base + s * fold_stage + (i & 1) * fold_t + (i >> 1) * fold_rp, v.x, v.y, v.z, v.w);
-                }
-                ptx::fence_proxy_async_smem();
-                __syncwarp();   // lane 0's arrival below is the whole warp's
-            }
-            const uint32_t stage = ring_base + s * 2 * TB;
-            if (lane == 0) {
-                const uint32_t full = k.bar(b_full + s);
+            [[maybe_unused]] const int rows_left = rows - j * BC;  // rows of this tile that exist
+            if (ptx::elect_one()) {
                 ptx::mbar_arrive_expect_tx(full, tx_bytes);
                 if (has0) {
                     ptx::tma_load_4d(stage, map0, full, 0, j * BC, ch, cb);
@@ -375,10 +356,7 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
                     if (C::WIDE) ptx::tma_load_4d(stage + 3 * ATOM, map1, full, 64, j * BC, ch, cb);
                 }
             }
-            if constexpr (FOLDED) {
-                const bool more = j + 1 < k.T;
-                if (more || item + (int)gridDim.x < k.items) load_stats(more ? bh : (item + (int)gridDim.x) / k.row_tiles, more ? j + 1 : 0);
-            }
+            __syncwarp();
             if constexpr (STATS) {
                 // queries beyond M read as zero: their rows of the B operands are zero too
                 const uint32_t slot = st_base + s * (C::NSTAT * BC * 4);
@@ -397,23 +375,32 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
                 }
             }
             if constexpr (C::TAIL) {
+                const uint32_t d0 = stage + dst_lane;
+                constexpr uint32_t T1 = RING == 0 ? BC * 16 : ATOM, R1 = RING == 0 ? 32 * 16 : 32 * 128;   // second tensor, second 32 rows
 #pragma unroll
                 for (int c = 0; c < KT; ++c) {
                     if (c < ntail) {
+                        const uint32_t dst = d0 + (RING == 0 ? c * 2 * BC * 16 : (c ^ sw) << 4);
+                        if (__builtin_expect(rows_left >= BC, 1)) {
+                            if (has0) { ptx::cp_async_16(dst, src0 + 8 * c); ptx::cp_async_16(dst + R1, src0 + d32 + 8 * c); }
+                            if (has1) { ptx::cp_async_16(dst + T1, src1 + 8 * c); ptx::cp_async_16(dst + T1 + R1, src1 + d32 + 8 * c); }
+                        } else {
 #pragma unroll
-                        for (int rp = 0; rp < BC / 32; ++rp) {
-                            const bool v = lane + 32 * rp < rows_left;
-                            const uint32_t dst = stage + dst_lane + (RING == 0 ? c * 2 * BC * 16 + rp * 32 * 16 : rp * 32 * 128 + ((c ^ sw) << 4));
-                            if (has0) ptx::cp_async_16(dst, v ? src0 + rp * d32 + 8 * c : base0, v ? 16u : 0u);
-                            if (has1) ptx::cp_async_16(dst + (RING == 0 ? BC * 16 : ATOM), v ? src1 + rp * d32 + 8 * c : base1, v ? 16u : 0u);
+                            for (int rp = 0; rp < 2; ++rp) {
+                                const bool v = lane + 32 * rp < rows_left;
+                                if (has0) ptx::cp_async_16(dst + rp * R1, v ? src0 + rp * d32 + 8 * c : base0, v ? 16u : 0u);
+                                if (has1) ptx::cp_async_16(dst + rp * R1 + T1, v ? src1 + rp * d32 + 8 * c : base1, v ? 16u : 0u);
+                            }
                         }
                     }
                 }
                 src0 += tile_elems;
                 src1 += tile_elems;
             }
-            if (HAS_CP) ptx::cp_async_arrive(k.bar(b_full + s));
-            if (++s == S) { s = 0; ph ^= 1; }
+            if (HAS_CP) ptx::cp_async_arrive(full);
+            stage += 2 * TB;
+            full += 8;
+            if (++s == S) { s = 0; ph ^= 1; stage = ring_base; full = k.bar(b_full); }
         }
     }
     if (HAS_CP) ptx::cp_async_wait_all();  // nothing of ours stays in flight
@@ -430,240 +417,331 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
     }
 }
 
+// FOLD.  Each statistic is stored as three bf16 parts whose sum is its 24 bits, in the first three of eight columns, against
+// ones in the owner operand.
+constexpr uint32_t JVP_ONES0 = 0x3F803F80u, JVP_ONES1 = 0x00003F80u;   // 1, 1, 1, 0 in bf16
+__device__ __forceinline__ void jvp_split3(float a, float b, uint2& pa, uint2& pb) {   // two values at once
+    const uint32_t h = ptx::pack_bf16(a, b);
+    a -= __uint_as_float(h << 16); b -= __uint_as_float(h & 0xffff0000u);
+    const uint32_t m = ptx::pack_bf16(a, b);
+    a -= __uint_as_float(m << 16); b -= __uint_as_float(m & 0xffff0000u);
+    const uint32_t l = ptx::pack_bf16(a, b);
+    pa = make_uint2(__byte_perm(h, m, 0x5410), l & 0xffffu);
+    pb = make_uint2(__byte_perm(h, m, 0x7632), l >> 16);
+}
+
+// Warp 3: the statistics of the stream rows lane and lane + 32 of a tile, for the E ring (DV: lse, mu; DK: Sigma1, c) and the
+// L ring (DK: lse, mu), loaded one tile ahead.
+template <int MODE, int DP>
+__device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE, DP>& shared, int lane) {
+    using C = JvpCfg<MODE, DP>;
+    const JvpBlock<MODE, DP> k = shared.pinned();
+    const int T = jvp_pin(p.T);
+    constexpr int BC = C::BC;
+    // where the parts of (tensor t, row lane + 32 r) of a stage go: base + stage * step + t * t_step + r * r_step
+    struct Dst { uint32_t base, step, t_step, r_step; };
+    const uint32_t sw = lane & 7;
+    const bool own = k.fold_step();
+    const Dst de = own ? Dst{k.base + k.FOLD_E + lane * 16, (uint32_t)C::FOLD_BYTES, BC * 16, 32 * 16}
+                       : Dst{k.base + k.E + 2 * C::ATOM + 2 * BC * 16 + lane * 16, 2u * C::EST_BYTES, BC * 16, 32 * 16};
+    [[maybe_unused]] const Dst dl = own ? Dst{k.base + k.FOLD_L + lane * 16, (uint32_t)C::FOLD_BYTES, BC * 16, 32 * 16}
+                                        : Dst{k.base + k.L + 2 * C::ATOM + lane * 128 + ((1 ^ sw) << 4), 2u * C::LST_BYTES, C::ATOM, 32 * 128};
+    const float f_lse = 1.0f / p.c2, f_mu = -1.0f / p.alpha;   // to the scale of S and Sd
+    float a[4], b[4];   // (statistic of tensor 0, of tensor 1) of the two rows: lse, mu | Sigma1, c
+    auto load = [&](int bh, int j) {
+        const int left = p.s.rows - j * BC - lane;   // queries beyond M: zero, like their rows of the operands
+        const size_t at = (size_t)bh * p.s.rows + (size_t)j * BC + lane;
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const bool v = left > 32 * r;
+            a[2 * r] = v ? __ldg(p.nlse2 + at + 32 * r) : 0.f;
+            a[2 * r + 1] = v ? __ldg(p.mu + at + 32 * r) : 0.f;
+            if (C::NPAIR == 2) {
+                b[2 * r] = v ? __ldg(p.nsig1 + at + 32 * r) : 0.f;
+                b[2 * r + 1] = v ? __ldg(p.ncvec + at + 32 * r) : 0.f;
+            }
+        }
+    };
+    auto put = [&](const Dst& d, int stage, int full, float x0, float x1, float y0, float y1) {
+        const uint32_t at = d.base + stage * d.step;
+        uint2 u, v;
+        jvp_split3(x0, x1, u, v);
+        ptx::st_shared_v4(at, u.x, u.y, 0u, 0u);
+        ptx::st_shared_v4(at + d.t_step, v.x, v.y, 0u, 0u);
+        jvp_split3(y0, y1, u, v);
+        ptx::st_shared_v4(at + d.r_step, u.x, u.y, 0u, 0u);
+        ptx::st_shared_v4(at + d.t_step + d.r_step, v.x, v.y, 0u, 0u);
+        ptx::fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(k.bar(full + stage));
+    };
+    if ((int)blockIdx.x < p.items) load(blockIdx.x / p.row_tiles, 0);
+    int g = 0, se = 0, sl = 0;
+    for (int item = blockIdx.x; item < p.items; item += gridDim.x) {
+        const int bh = item / p.row_tiles, next = item + (int)gridDim.x;
+        for (int j = 0; j < T; ++j, ++g) {
+            if (C::NPAIR == 2) {
+                if (g >= C::SL && !k.done(C::B_OUTDONE, g - C::SL)) return;
+                put(dl, sl, C::B_LFULL, a[0] * f_lse, a[1] * f_mu, a[2] * f_lse, a[3] * f_mu);
+                if (++sl == C::SL) sl = 0;
+            }
+            if (g >= C::SE && !k.done(C::B_EDONE, g - C::SE)) return;
+            if (C::NPAIR == 2) put(de, se, C::B_EFULL, b[0], b[1], b[2], b[3]);
+            else put(de, se, C::B_EFULL, a[0] * f_lse, a[1] * f_mu, a[2] * f_lse, a[3] * f_mu);
+            if (++se == C::SE) se = 0;
+            const bool more = j + 1 < T;
+            if (more || next < p.items) load(more ? bh : next / p.row_tiles, more ? j + 1 : 0);
+        }
+    }
+}
+
 // ------------------------------------------------------------------------------------------------ MMA issue
 // The whole warp runs this in converged control flow; one elected lane issues (one election per batch of MMAs,
 // descriptors as 32-bit halves: see mma_ts_p).  Tensor memory starts at column 0, because the block owns all of it.
-template <int MODE, int DP, bool HZ>
+//
+// The tensor pipe takes about four MMAs ahead, 130 to 250 cycles of work; whatever the issuing warp does between two
+// batches beyond that leaves the pipe idle.  A wait for a barrier that has completed costs it 85 cycles, a commit 60, a
+// dependent scalar instruction ten.  So: ring positions are carried along as descriptors (every descriptor of a batch is
+// the carried one plus a constant), barriers of the rings are tested ahead, in front of the batch before, what depends on
+// the item stays out of the tile's path, and which cotangent is absent (ABS) is a template parameter.
+struct JvpSlot {   // a ring's next tile: stage, phase, low descriptor halves of the stage and of its statistics
+    uint32_t lo, fold, lo0, fold0;
+    int s = 0, ph = 0;
+    __device__ __forceinline__ JvpSlot(uint32_t lo_, uint32_t fold_) : lo(lo_), fold(fold_), lo0(lo_), fold0(fold_) {}
+    template <int S, uint32_t STEP, uint32_t FSTEP>
+    __device__ __forceinline__ void next() {
+        lo += STEP;
+        fold += FSTEP;
+        if (++s == S) { s = 0; ph ^= 1; lo = lo0; fold = fold0; }
+    }
+};
+
+template <int MODE, int DP, bool HZ, int ABS>
 struct JvpIssue {
     using C = JvpCfg<MODE, DP>;
+    using Block = JvpBlock<MODE, DP>;
     static constexpr int BC = C::BC, KS = C::KS, ATOM = C::ATOM;
     static constexpr uint32_t HI_SW = ptx::desc_hi_sw128(1024), HI_TAIL = ptx::desc_hi_nosw(128);
     static constexpr uint32_t I_S = ptx::idesc_bf16_f32(128, BC, 0, 0), I_S2 = ptx::idesc_bf16_f32(128, 2 * BC, 0, 0);
     static constexpr uint32_t I_O = ptx::idesc_bf16_f32(128, DP, 0, 1);
-    static __device__ __forceinline__ bool is_tail(int kk) { return C::TAIL && kk >= 4; }
-    // low descriptor halves (start address, leading offset) of k-step kk; the high half is HI_SW, or HI_TAIL in a tail
-    static __device__ __forceinline__ uint32_t own_klo(uint32_t tile, int kk) {   // owner tile, K-major
-        if (kk < 4) return ptx::desc_lo(tile, 16) + 2u * kk;
-        return C::WIDE ? ptx::desc_lo(tile + C::OWN_ATOM, 16) + 2u * (kk - 4) : ptx::desc_lo(tile + C::OWN_ATOM, JVP_ROWS * 16);
+    // Low descriptor half of an address with leading offset 16 (K-major, swizzled); other operands are that plus constants.
+    static constexpr uint32_t LBO16 = 1u << 16;
+    static __host__ __device__ constexpr uint32_t lbo(uint32_t bytes) { return ((bytes >> 4) << 16) - LBO16; }
+    static constexpr uint32_t E_STEP = (2 * C::EST_BYTES) >> 4, L_STEP = (2 * C::LST_BYTES) >> 4;
+    static constexpr uint32_t F_STEP = (C::FOLD_BYTES >> 4) - ((C::FOLD_BYTES >> 4) << 16);   // the zeros behind come nearer
+    static __device__ __forceinline__ JvpSlot e_slot(const Block& k) { return JvpSlot(ptx::desc_lo(k.base + k.E, 16), ptx::desc_lo(k.base + k.FOLD_E, k.ZEROS - k.FOLD_E)); }
+    static __device__ __forceinline__ JvpSlot l_slot(const Block& k) { return JvpSlot(ptx::desc_lo(k.base + k.L, 16), ptx::desc_lo(k.base + k.FOLD_L, k.ZEROS - k.FOLD_L)); }
+
+    static __host__ __device__ constexpr bool is_tail(int kk) { return C::TAIL && kk >= 4; }
+    // k-step kk of a K-major operand, relative to its tile or stage: owner tile | E stage (rows of Y0, then Y1) | L stage
+    static __host__ __device__ constexpr uint32_t own_k(int kk) {
+        return kk < 4 ? 2u * kk : C::WIDE ? ((uint32_t)C::OWN_ATOM >> 4) + 2u * (kk - 4) : ((uint32_t)C::OWN_ATOM >> 4) + lbo(JVP_ROWS * 16);
     }
-    static __device__ __forceinline__ uint32_t e_klo(uint32_t stage, int kk) {    // E stage, K-major, rows of Y0 (then Y1)
-        if (kk < 4) return ptx::desc_lo(stage, 16) + 2u * kk;
-        return C::WIDE ? ptx::desc_lo(stage + 2 * ATOM, 16) + 2u * (kk - 4) : ptx::desc_lo(stage + 2 * ATOM, 2 * BC * 16);
+    static __host__ __device__ constexpr uint32_t e_k(int kk) {
+        return kk < 4 ? 2u * kk : C::WIDE ? (2u * ATOM >> 4) + 2u * (kk - 4) : (2u * ATOM >> 4) + lbo(2 * BC * 16);
     }
-    static __device__ __forceinline__ uint32_t l_klo(uint32_t stage, int kk) {    // L stage, K-major, rows of Y0 (then Y1)
-        return ptx::desc_lo(stage + (kk >> 2) * 2 * ATOM, 16) + 2u * (kk & 3);
-    }
+    static __host__ __device__ constexpr uint32_t l_k(int kk) { return (uint32_t)((kk >> 2) * 2 * ATOM >> 4) + 2u * (kk & 3); }
     // L stage read MN-major by the output MMAs (tensor t): atoms of 64 d-columns are 2 * ATOM bytes apart, 8-row groups
     // 1024 bytes, a k-step of 16 stream rows 2048
-    static __device__ __forceinline__ uint32_t l_nlo(uint32_t stage, int t) { return ptx::desc_lo(stage + t * ATOM, 2 * ATOM); }
+    static __host__ __device__ constexpr uint32_t l_n(int t, int u) { return (uint32_t)(t * ATOM + u * 2048) / 16 + lbo(2 * ATOM); }
 
-    // One k-step with A in tensor memory (ATM: a = its columns) or in shared memory (a = the tile).
+    // One k-step with A in tensor memory (ATM: a = its columns) or in shared memory (a = the tile's descriptor).
     template <bool ATM, uint32_t ACC>
     static __device__ __forceinline__ void step(uint32_t el, uint32_t col, uint32_t a, int kk, uint32_t b, uint32_t bhi, uint32_t idesc) {
         if (ATM) ptx::mma_ts_p<ACC>(el, col, a + 8 * kk, b, bhi, idesc);
-        else ptx::mma_ss_p<ACC>(el, col, own_klo(a, kk), is_tail(kk) ? HI_TAIL : HI_SW, b, bhi, idesc);
+        else ptx::mma_ss_p<ACC>(el, col, a + own_k(kk), is_tail(kk) ? HI_TAIL : HI_SW, b, bhi, idesc);
     }
-    // The statistics' own k-step (FOLD, where the padding columns do not hold them): `fold` is the stage's block, tensor t0 on.
+    // The statistics' own k-step (FOLD, where the padding columns do not hold them), tensor t0 on.
     template <bool ATM>
-    static __device__ __forceinline__ void fold_step(uint32_t el, uint32_t col, const JvpBlock<MODE, DP>& k, uint32_t fold, int t0, uint32_t idesc) {
-        const uint32_t b = ptx::desc_lo(fold + t0 * BC * 16, k.zeros - fold);
+    static __device__ __forceinline__ void fold_step(uint32_t el, uint32_t col, const Block& k, uint32_t fold, int t0, uint32_t idesc) {
+        const uint32_t b = fold + (uint32_t)(t0 * BC * 16 >> 4) - ((uint32_t)(t0 * BC * 16 >> 4) << 16);
         if (ATM) ptx::mma_ts_p<1>(el, col, C::COL_ONES, b, HI_TAIL, idesc);
-        else ptx::mma_ss_p<1>(el, col, ptx::desc_lo(k.ones, k.zeros - k.ones), HI_TAIL, b, HI_TAIL, idesc);
+        else ptx::mma_ss_p<1>(el, col, ptx::desc_lo(k.base + k.ONES, JVP_ROWS * 16), HI_TAIL, b, HI_TAIL, idesc);
     }
     // [S | X0 Y1^T] = X0 [Y0 | Y1]^T, Sd += X1 Y0^T at column col; FROM_L: the stage is one of the L ring.
-    template <bool FROM_L, bool ATM>
-    static __device__ __forceinline__ void pair(uint32_t el, uint32_t col, const JvpBlock<MODE, DP>& k, uint32_t a0, uint32_t a1, uint32_t stage, uint32_t fold,
-                                                bool second, uint32_t mid_bar) {
+    template <bool FROM_L, bool ATM, bool SECOND>
+    static __device__ __forceinline__ void pair(uint32_t el, uint32_t col, const Block& k, uint32_t a0, uint32_t a1, uint32_t lo, uint32_t fold, uint32_t mid_bar) {
 #pragma unroll
         for (int kk = 0; kk < KS; ++kk) {
-            const uint32_t b = FROM_L ? l_klo(stage, kk) : e_klo(stage, kk), bhi = !FROM_L && is_tail(kk) ? HI_TAIL : HI_SW;
+            const uint32_t b = lo + (FROM_L ? l_k(kk) : e_k(kk)), bhi = !FROM_L && is_tail(kk) ? HI_TAIL : HI_SW;
             if (kk == 0) step<ATM, 0>(el, col, a0, kk, b, bhi, I_S2);
             else step<ATM, 1>(el, col, a0, kk, b, bhi, I_S2);
         }
-        if (C::FOLD && k.fold_step) fold_step<ATM>(el, col, k, fold, 0, I_S2);
+        if (k.fold_step()) fold_step<ATM>(el, col, k, fold, 0, I_S2);
         if (MODE == PASS_FWD) ptx::mma_commit_p(el, mid_bar);   // S is complete before Sd
-        if (second) {
+        if (SECOND) {
 #pragma unroll
             for (int kk = 0; kk < KS; ++kk)
-                step<ATM, 1>(el, col + BC, a1, kk, FROM_L ? l_klo(stage, kk) : e_klo(stage, kk), !FROM_L && is_tail(kk) ? HI_TAIL : HI_SW, I_S);
+                step<ATM, 1>(el, col + BC, a1, kk, lo + (FROM_L ? l_k(kk) : e_k(kk)), !FROM_L && is_tail(kk) ? HI_TAIL : HI_SW, I_S);
         }
     }
-    // One product X Y^T with Y the t-th tensor of the stage.
-    template <bool FROM_L, bool ATM>
-    static __device__ __forceinline__ void single(uint32_t el, uint32_t col, const JvpBlock<MODE, DP>& k, uint32_t a, uint32_t stage, uint32_t fold, int t) {
+    // One product X Y^T with Y the T-th tensor of the stage.
+    template <bool FROM_L, bool ATM, int T>
+    static __device__ __forceinline__ void single(uint32_t el, uint32_t col, const Block& k, uint32_t a, uint32_t lo, uint32_t fold) {
 #pragma unroll
         for (int kk = 0; kk < KS; ++kk) {
             const bool tail = !FROM_L && is_tail(kk);
-            const uint32_t b = (FROM_L ? l_klo(stage, kk) : e_klo(stage, kk)) + ((uint32_t)(tail ? t * BC * 16 : t * ATOM) >> 4);
+            const uint32_t b = lo + (FROM_L ? l_k(kk) : e_k(kk)) + ((uint32_t)(tail ? T * BC * 16 : T * ATOM) >> 4);
             if (kk == 0) step<ATM, 0>(el, col, a, kk, b, tail ? HI_TAIL : HI_SW, I_S);
             else step<ATM, 1>(el, col, a, kk, b, tail ? HI_TAIL : HI_SW, I_S);
         }
-        if (C::FOLD && k.fold_step) fold_step<ATM>(el, col, k, fold, t, I_S);
+        if (k.fold_step()) fold_step<ATM>(el, col, k, fold, T, I_S);
     }
     // Half of acc0 += A0 B0, acc1 += A1 B0 + A0 B1 (k-steps U0, U0 + 1 of four; the operand of a k-step lies at the columns of
-    // the scores it replaces); the terms of an absent tensor are left out, one uniform branch around the unrolled loops.
-    // `first`: the accumulators are overwritten.
+    // the scores it replaces); the terms of an absent tensor are left out.  acc = 0: the accumulators are overwritten.
     template <int U0>
-    static __device__ __forceinline__ void outputs(uint32_t el, uint32_t a0, uint32_t a1, uint32_t stage, bool first, int absent) {
-        const uint32_t b0 = l_nlo(stage, 0), b1 = l_nlo(stage, 1);
+    static __device__ __forceinline__ void outputs(uint32_t el, uint32_t a0, uint32_t a1, uint32_t lo, uint32_t acc) {
         constexpr uint32_t c0 = C::COL_ACC0, c1 = C::COL_ACC1;
-        constexpr bool DV = MODE == PASS_DV;
-        if (!HZ && (MODE == PASS_FWD || absent == 0 || (!DV && !(absent & ABSENT_HC)))) {
+        constexpr bool DV = MODE == PASS_DV, B0 = !HZ && !(DV && (ABS & ABSENT_HC)), A0 = !HZ && !(!DV && (ABS & ABSENT_HC)), B1 = !(DV && (ABS & ABSENT_G));
+        // (DV: Hc is B0, G is B1; DK, DQ with Hc absent: A0 = W is exactly zero)
+        constexpr bool T0 = A0 && B0, T1 = !DV ? true : B0, T2 = DV ? B1 : A0;   // A0 B0, A1 B0, A0 B1
 #pragma unroll
-            for (int u = U0; u < U0 + 2; ++u) {
-                const uint32_t off = (uint32_t)(u * 2048) >> 4;
-                if (u == 0 && first) { ptx::mma_ts_p<0>(el, c0, a0, b0, HI_SW, I_O); ptx::mma_ts_p<0>(el, c1, a1, b0, HI_SW, I_O); }
-                else { ptx::mma_ts_p<1>(el, c0, a0 + 16 * u, b0 + off, HI_SW, I_O); ptx::mma_ts_p<1>(el, c1, a1 + 16 * u, b0 + off, HI_SW, I_O); }
-                ptx::mma_ts_p<1>(el, c1, a0 + 16 * u, b1 + off, HI_SW, I_O);
-            }
-        } else if (DV && !HZ && (absent & ABSENT_G)) {   // B1 = G absent
-#pragma unroll
-            for (int u = U0; u < U0 + 2; ++u) {
-                const uint32_t off = (uint32_t)(u * 2048) >> 4;
-                if (u == 0 && first) { ptx::mma_ts_p<0>(el, c0, a0, b0, HI_SW, I_O); ptx::mma_ts_p<0>(el, c1, a1, b0, HI_SW, I_O); }
-                else { ptx::mma_ts_p<1>(el, c0, a0 + 16 * u, b0 + off, HI_SW, I_O); ptx::mma_ts_p<1>(el, c1, a1 + 16 * u, b0 + off, HI_SW, I_O); }
-            }
-        } else {   // Hc absent: DV: acc1 += P^T G alone; DK, DQ: W is exactly zero, acc1 += A1 B0 alone
-            const uint32_t a = DV ? a0 : a1, b = DV ? b1 : b0;
-#pragma unroll
-            for (int u = U0; u < U0 + 2; ++u) {
-                const uint32_t off = (uint32_t)(u * 2048) >> 4;
-                if (u == 0 && first) ptx::mma_ts_p<0>(el, c1, a, b, HI_SW, I_O);
-                else ptx::mma_ts_p<1>(el, c1, a + 16 * u, b + off, HI_SW, I_O);
-            }
+        for (int u = U0; u < U0 + 2; ++u) {
+            const uint32_t b0 = lo + l_n(0, u), b1 = lo + l_n(1, u);
+            if (T0) { if (u == 0) ptx::mma_ts_acc(el, c0, a0, b0, HI_SW, I_O, acc); else ptx::mma_ts_p<1>(el, c0, a0 + 16 * u, b0, HI_SW, I_O); }
+            if (T1) { if (u == 0) ptx::mma_ts_acc(el, c1, a1, b0, HI_SW, I_O, acc); else ptx::mma_ts_p<1>(el, c1, a1 + 16 * u, b0, HI_SW, I_O); }
+            if (T2) { if (u == 0 && !T1) ptx::mma_ts_acc(el, c1, a0, b1, HI_SW, I_O, acc); else ptx::mma_ts_p<1>(el, c1, a0 + 16 * u, b1, HI_SW, I_O); }
         }
     }
-};
-
-struct JvpRing {   // stage and phase of a ring's next tile
-    int s = 0, ph = 0;
-    template <int S>
-    __device__ __forceinline__ void next() { if (++s == S) { s = 0; ph ^= 1; } }
 };
 
 // FWD, DV: two score buffers taken in turn, operands written over the scores; pipe order S(0), S(1), out(0), S(2), out(1), ...:
 // S(n + 1) overwrites what out(n - 1) reads, and the pipe keeps the order.
-template <int MODE, int DP, bool HZ>
-__device__ __forceinline__ void jvp_issue_one_pair(const JvpParams& p, const JvpBlock<MODE, DP>& k) {
+template <int MODE, int DP, bool HZ, int ABS>
+__device__ __forceinline__ void jvp_issue_one_pair(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
     using C = JvpCfg<MODE, DP>;
-    using I = JvpIssue<MODE, DP, HZ>;
+    using I = JvpIssue<MODE, DP, HZ, ABS>;
     constexpr int RDY = C::XT ? C::B_XRDY : C::B_OWN, FREE = C::XT ? C::B_XFREE : C::B_OWNFREE;
-    const int n_it = (int)blockIdx.x < k.items ? (k.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-    const int T = k.T, G = n_it * T, absent = p.absent;
-    const uint32_t x0 = C::XT ? C::COL_X0 : k.own_tile(0), x1 = C::XT ? C::COL_X1 : k.own_tile(1);
-    JvpRing e, l;
-    int js = 0, is = 0, jo = 0, it = 0;   // place in its item, and item, of the scores' and of the outputs' tile
-    int n = 0;                            // next tile whose scores are issued
-    auto scores = [&]() -> bool {
-        if (js == 0 && !k.wait(RDY, is)) return false;
-        if (!k.wait(C::B_EFULL + e.s, e.ph)) return false;
-        k.tile_fence();
-        const uint32_t el = ptx::elect_one();
-        const uint32_t col = C::COL_SCORE + (n & 1) * 2 * C::BC, stage = k.e_stage(e.s), fold = k.fold_e + e.s * C::FOLD_BYTES;
-        if (HZ) I::template single<false, C::XT>(el, col, k, x0, stage, fold, 0);
-        else I::template pair<false, C::XT>(el, col, k, x0, x1, stage, fold, true, k.bar(C::B_SFULL + (n & 3)));
-        ptx::mma_commit_p(el, k.bar(C::B_EDONE + (n & 3)));
-        e.next<C::SE>();
-        ++n;
-        if (++js == T) {
-            ptx::mma_commit_p(el, k.bar(FREE));
-            js = 0;
-            ++is;
-        }
-        return true;
-    };
-    for (int g = 0; g < G; ++g) {
-        if (n == g && !scores()) return;
-        // The scores of the next tile go in front of this tile's outputs, unless they open an item whose owner operands are
-        // still on their way: then wherever these turn out to be ready.
-        if (n < G && (js > 0 || ptx::mbar_test_warp(k.bar(RDY), is & 1)) && !scores()) return;
-        const int b = g & 1;
-        if (!k.wait2(C::B_PREADY + 2 * b, g >> 1, C::B_LFULL + l.s, l.ph)) return;
-        // the first tile of an item overwrites the accumulators
-        if (jo == 0 && it > 0 && !k.wait(C::B_ACCFREE, it - 1)) return;
-        k.tile_fence();
-        const uint32_t a0 = C::COL_SCORE + b * 2 * C::BC, stage = k.l_stage(l.s);
-        I::template outputs<0>(ptx::elect_one(), a0, a0 + C::BC, stage, jo == 0, absent);
-        if (n == g + 1 && n < G && ptx::mbar_test_warp(k.bar(RDY), is & 1) && !scores()) return;
-        if (!k.wait(C::B_PREADY + 2 * b + 1, g >> 1)) return;
-        ptx::tc_fence_after_sync();
-        const uint32_t el = ptx::elect_one();
-        I::template outputs<2>(el, a0, a0 + C::BC, stage, false, absent);
-        ptx::mma_commit_p(el, k.bar(C::B_OUTDONE + (g & 3)));
-        l.next<C::SL>();
-        if (++jo == T) {
-            ptx::mma_commit_p(el, k.bar(C::B_FINAL));
-            jo = 0;
-            ++it;
+    const JvpBlock<MODE, DP> k = shared.pinned();
+    const int T = jvp_pin(p.T), items = jvp_pin(p.items);
+    const uint32_t x0 = C::XT ? C::COL_X0 : ptx::desc_lo(k.own_tile(0), 16), x1 = C::XT ? C::COL_X1 : ptx::desc_lo(k.own_tile(1), 16);
+    JvpSlot e = I::e_slot(k), l = I::l_slot(k);
+    int n = 0;                 // next tile whose scores are issued
+    bool e_ready = false;      // its E stage was seen full
+    int g = 0, it = 0;
+    bool opened = false;       // the first scores of the item have been issued
+    for (int item = blockIdx.x; item < items; item += gridDim.x, ++it) {
+        const bool more = item + (int)gridDim.x < items;
+        if (!opened && !k.wait(RDY, it)) return;
+        if (it > 0 && !k.wait(C::B_ACCFREE, it - 1)) return;   // the first tile overwrites the accumulators
+        for (int j = opened ? 0 : -1; j < T; ++j) {
+            // The scores of the next tile go in front of this tile's outputs.  Where they open an item they do if its owner
+            // operands are there already, else they follow when the loop gets there.
+            bool go = j + 1 < T;
+            if (!go) go = opened = more && ptx::mbar_test_warp(k.bar(RDY), (it + 1) & 1);
+            if (go) {
+                if (!e_ready && !k.wait(C::B_EFULL + e.s, e.ph)) return;
+                k.tile_fence();
+                const uint32_t el = ptx::elect_one();
+                const uint32_t col = C::COL_SCORE + (n & 1) * 2 * C::BC;
+                if (HZ) I::template single<false, C::XT, 0>(el, col, k, x0, e.lo, e.fold);
+                else I::template pair<false, C::XT, true>(el, col, k, x0, x1, e.lo, e.fold, k.bar(C::B_SFULL + (n & 3)));
+                ptx::mma_commit_p(el, k.bar(C::B_EDONE + (n & 3)));
+                if (j + 2 == T || (T == 1 && j == 0)) ptx::mma_commit_p(el, k.bar(FREE));   // the item's last scores
+                e.template next<C::SE, I::E_STEP, I::F_STEP>();
+                ++n;
+            }
+            e_ready = ptx::mbar_test_warp(k.bar(C::B_EFULL + e.s), e.ph);
+            if (j < 0) continue;
+            const int b = g & 1;
+            if (!k.wait2(C::B_PREADY + 2 * b, g >> 1, C::B_LFULL + l.s, l.ph)) return;
+            k.tile_fence();
+            const uint32_t a0 = C::COL_SCORE + b * 2 * C::BC;
+            I::template outputs<0>(ptx::elect_one(), a0, a0 + C::BC, l.lo, j > 0 ? 1u : 0u);
+            if (!k.wait(C::B_PREADY + 2 * b + 1, g >> 1)) return;
+            ptx::tc_fence_after_sync();
+            const uint32_t el = ptx::elect_one();
+            I::template outputs<2>(el, a0, a0 + C::BC, l.lo, 1u);
+            ptx::mma_commit_p(el, k.bar(C::B_OUTDONE + (g & 3)));
+            if (j == T - 1) ptx::mma_commit_p(el, k.bar(C::B_FINAL));
+            l.template next<C::SL, I::L_STEP, 0>();
+            ++g;
         }
     }
 }
 
 // DK, DQ: one buffer of (S, Sd | D, X), the operands W, dA over D, X.  Pipe order: (S, Sd)(n) once (S, Sd)(n - 1) has been read |
 // outputs(n - 1), half by half, as W, dA are written | (D, X)(n), which overwrites them.
-template <int MODE, int DP, bool HZ>
-__device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const JvpBlock<MODE, DP>& k) {
+template <int MODE, int DP, bool HZ, int ABS>
+__device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
     using C = JvpCfg<MODE, DP>;
-    using I = JvpIssue<MODE, DP, HZ>;
-    const int T = k.T, absent = p.absent;
-    const uint32_t x0 = k.own_tile(0), x1 = k.own_tile(1);
-    const uint32_t x2 = C::XT ? C::COL_X0 : k.own_tile(2), x3 = C::XT ? C::COL_X1 : k.own_tile(3);
+    using I = JvpIssue<MODE, DP, HZ, ABS>;
+    const JvpBlock<MODE, DP> k = shared.pinned();
+    const int T = jvp_pin(p.T), items = jvp_pin(p.items);
+    const uint32_t x0 = ptx::desc_lo(k.own_tile(0), 16), x1 = ptx::desc_lo(k.own_tile(1), 16);
+    const uint32_t x2 = C::XT ? C::COL_X0 : ptx::desc_lo(k.own_tile(2), 16), x3 = C::XT ? C::COL_X1 : ptx::desc_lo(k.own_tile(3), 16);
     constexpr uint32_t cS = C::COL_SCORE, cD = C::COL_SCORE + 2 * C::BC, cX = C::COL_SCORE + 3 * C::BC;
-    JvpRing e, l;
-    int ls = 0, n = 0;   // L stage of the outputs' tile; next tile whose scores are issued
-    auto first = [&](int j) -> bool {
-        if (!k.wait2(C::B_SREAD, n - 1, C::B_LFULL + l.s, l.ph)) return false;   // (a fresh barrier passes for n = 0)
-        k.tile_fence();
-        const uint32_t el = ptx::elect_one(), fold = k.fold_l + l.s * C::FOLD_BYTES;
-        if (HZ) I::template single<true, false>(el, cS, k, x0, k.l_stage(l.s), fold, 0);
-        else I::template pair<true, false>(el, cS, k, x0, x1, k.l_stage(l.s), fold, true, 0);
-        ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
-        if (C::XT && j == T - 1) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE));
-        l.next<C::SL>();
-        return true;
-    };
-    auto second = [&](int j) -> bool {
-        if (!k.wait(C::B_EFULL + e.s, e.ph)) return false;
-        k.tile_fence();
-        const uint32_t el = ptx::elect_one(), fold = k.fold_e + e.s * C::FOLD_BYTES;
-        // HZ: X = G V^T alone: DK: X2 Y3^T (V, and G the stage's second tensor); DQ: X3 Y2^T (G, and V its first)
-        if (HZ) I::template single<false, C::XT>(el, cX, k, MODE == PASS_DK ? x2 : x3, k.e_stage(e.s), fold, MODE == PASS_DK ? 1 : 0);
-        // X3 Y2^T is zero when either factor is an absent cotangent: DK has Y2 = Hc, DQ has X3 = G
-        else I::template pair<false, C::XT>(el, cD, k, x2, x3, k.e_stage(e.s), fold, !(absent & (MODE == PASS_DK ? ABSENT_HC : ABSENT_G)), 0);
-        ptx::mma_commit_p(el, k.bar(C::B_XFULL + (n & 3)));
-        if (j == T - 1) ptx::mma_commit_p(el, k.bar(C::XT ? C::B_XFREE : C::B_OWNFREE));
-        e.next<C::SE>();
-        ++n;
-        return true;
-    };
+    // X3 Y2^T is zero when either factor is an absent cotangent: DK has Y2 = Hc, DQ has X3 = G
+    constexpr bool X3 = !(ABS & (MODE == PASS_DK ? ABSENT_HC : ABSENT_G));
+    JvpSlot e = I::e_slot(k), l = I::l_slot(k);
+    uint32_t lo = l.lo;        // L stage of the outputs' tile
+    int n = 0;                 // next tile whose scores are issued
+    bool e_ready = false;
     int it = 0;
-    for (int item = blockIdx.x; item < k.items; item += gridDim.x, ++it) {
-        if (!k.wait(C::B_OWN, it) || !first(0)) return;
-        if ((C::XT && !k.wait(C::B_XRDY, it)) || !second(0)) return;
-        if (!k.wait(C::B_ACCFREE, it - 1)) return;    // the first tile overwrites the accumulators
-        for (int j = 0; j < T; ++j) {
-            const int g = n - 1;
-            if (j + 1 < T && !first(j + 1)) return;
-            if (!k.wait(C::B_PREADY, g)) return;
-            ptx::tc_fence_after_sync();
-            const uint32_t stage = k.l_stage(ls);
-            I::template outputs<0>(ptx::elect_one(), cD, cX, stage, j == 0, absent);
-            if (!k.wait(C::B_PREADY + 1, g)) return;
-            ptx::tc_fence_after_sync();
-            const uint32_t el = ptx::elect_one();
-            I::template outputs<2>(el, cD, cX, stage, false, absent);
-            ptx::mma_commit_p(el, k.bar(C::B_OUTDONE + (g & 3)));
-            if (++ls == C::SL) ls = 0;
-            if (j + 1 < T) { if (!second(j + 1)) return; }
-            else ptx::mma_commit_p(el, k.bar(C::B_FINAL));
+    for (int item = blockIdx.x; item < items; item += gridDim.x, ++it) {
+        if (!k.wait(C::B_OWN, it)) return;
+        for (int j = -1; j < T; ++j) {
+            if (j + 1 < T) {   // (S, Sd) of the next tile
+                if (!k.wait2(C::B_SREAD, n - 1, C::B_LFULL + l.s, l.ph)) return;   // (a fresh barrier passes for n = 0)
+                k.tile_fence();
+                const uint32_t el = ptx::elect_one();
+                if (HZ) I::template single<true, false, 0>(el, cS, k, x0, l.lo, l.fold);
+                else I::template pair<true, false, true>(el, cS, k, x0, x1, l.lo, l.fold, 0);
+                ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
+                if (C::XT && j + 2 == T) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE));
+                l.template next<C::SL, I::L_STEP, I::F_STEP>();
+            }
+            e_ready = ptx::mbar_test_warp(k.bar(C::B_EFULL + e.s), e.ph);
+            if (j >= 0) {      // outputs
+                if (!k.wait(C::B_PREADY, n - 1)) return;
+                if (j == 0 && !k.wait(C::B_ACCFREE, it - 1)) return;    // the first tile overwrites the accumulators
+                ptx::tc_fence_after_sync();
+                I::template outputs<0>(ptx::elect_one(), cD, cX, lo, j > 0 ? 1u : 0u);
+                if (!k.wait(C::B_PREADY + 1, n - 1)) return;
+                ptx::tc_fence_after_sync();
+                const uint32_t el = ptx::elect_one();
+                I::template outputs<2>(el, cD, cX, lo, 1u);
+                ptx::mma_commit_p(el, k.bar(C::B_OUTDONE + ((n - 1) & 3)));
+                if (j == T - 1) ptx::mma_commit_p(el, k.bar(C::B_FINAL));
+                lo = lo + I::L_STEP == l.lo0 + C::SL * I::L_STEP ? l.lo0 : lo + I::L_STEP;
+            } else if (C::XT && !k.wait(C::B_XRDY, it)) {
+                return;
+            }
+            if (j + 1 < T) {   // (D, X) of the next tile
+                if (!e_ready && !k.wait(C::B_EFULL + e.s, e.ph)) return;
+                k.tile_fence();
+                const uint32_t el = ptx::elect_one();
+                // HZ: X = G V^T alone: DK: X2 Y3^T (V, and G the stage's second tensor); DQ: X3 Y2^T (G, and V its first)
+                if (HZ) I::template single<false, C::XT, MODE == PASS_DK ? 1 : 0>(el, cX, k, MODE == PASS_DK ? x2 : x3, e.lo, e.fold);
+                else I::template pair<false, C::XT, X3>(el, cD, k, x2, x3, e.lo, e.fold, 0);
+                ptx::mma_commit_p(el, k.bar(C::B_XFULL + (n & 3)));
+                if (j + 2 == T) ptx::mma_commit_p(el, k.bar(C::XT ? C::B_XFREE : C::B_OWNFREE));
+                e.template next<C::SE, I::E_STEP, I::F_STEP>();
+                ++n;
+            }
         }
     }
 }
 
+// Which cotangent is absent is decided here, once.
+template <int MODE, int DP, bool HZ, int ABS>
+__device__ __forceinline__ void jvp_issue_abs(const JvpParams& p, const JvpBlock<MODE, DP>& k) {
+    if constexpr (JvpCfg<MODE, DP>::NPAIR == 1) jvp_issue_one_pair<MODE, DP, HZ, ABS>(p, k);
+    else jvp_issue_two_pairs<MODE, DP, HZ, ABS>(p, k);
+}
+template <int MODE, int DP, bool HZ>
+__device__ __forceinline__ void jvp_issue(const JvpParams& p, const JvpBlock<MODE, DP>& k) {
+    if (MODE == PASS_FWD || HZ || p.absent == 0) jvp_issue_abs<MODE, DP, HZ, 0>(p, k);
+    else if (p.absent == ABSENT_HC) jvp_issue_abs<MODE, DP, HZ, ABSENT_HC>(p, k);
+    else jvp_issue_abs<MODE, DP, HZ, ABSENT_G>(p, k);
+}
+
 // ------------------------------------------------------------------------------------------------ element-wise warps
-// Group `grp` takes the tiles g of its parity; a thread has owner row `row` and the 64 columns of the tile.  Reads of
-// tensor memory are issued for many columns at once (a read costs 180 cycles whatever its width) and released with one
-// arrival per warp; the operands are handed over half by half.
+// Forward: the two groups take the tiles in turn; a thread has owner row `row` and the 64 columns of the tile.  Backward: all
+// eight warps work on every tile; a thread has the 32 columns of its group's half.  (With one score buffer, or in the
+// backward's shorter DV tile, the tensor pipe waits for how long a tile takes; the forward measured 8 % slower that way,
+// with the row maxima to exchange.)  Reads of tensor memory are issued for many columns at once (a read costs 180 cycles
+// whatever its width) and released with one arrival per warp; the operands are handed over half by half.
 
 // Forward.  The reference m of a row and the centre c of its tangent weights are shared by the two groups: the warp that
 // has a row's tile g decides whether to move them and hands the row state on to the warp that has tile g + 1 (B_TURN), long
@@ -680,11 +758,11 @@ __device__ __forceinline__ void jvp_elem_fwd(const JvpParams& p, const JvpBlock<
     const uint64_t c2c2 = ptx::pack2(p.c2, p.c2), aa = ptx::pack2(p.alpha, p.alpha);
     bool ok = true;
     int it = 0;
-    for (int item = blockIdx.x; ok && item < k.items; item += gridDim.x, ++it) {
-        const int g0 = it * k.T;
+    for (int item = blockIdx.x; ok && item < p.items; item += gridDim.x, ++it) {
+        const int g0 = it * p.T;
         float m_own = -CUDART_INF_F, c_own = 0.f;   // reference and centre of this thread's sums
         uint64_t l2 = 0ull, mt2 = 0ull;             // two partial sums each of P~ and of P~ (T - c) over this group's tiles
-        for (int j = (grp ^ g0) & 1; j < k.T; j += 2) {
+        for (int j = (grp ^ g0) & 1; j < p.T; j += 2) {
             const int g = g0 + j, b = g & 1;
             const uint32_t sb = lanes + C::COL_SCORE + b * 2 * BC;
             uint32_t s[64], t[64];
@@ -695,7 +773,7 @@ __device__ __forceinline__ void jvp_elem_fwd(const JvpParams& p, const JvpBlock<
             ptx::tmem_ld32(sb + 32, s + 32);
             ptx::tmem_wait_ld();
             const int nvalid = p.s.rows - j * BC;  // columns that are real keys
-            if (nvalid < BC) {
+            if (__builtin_expect(nvalid < BC, 0)) {
 #pragma unroll
                 for (int c = 0; c < BC; ++c)
                     if (c >= nvalid) s[c] = __float_as_uint(-CUDART_INF_F);
@@ -713,15 +791,15 @@ __device__ __forceinline__ void jvp_elem_fwd(const JvpParams& p, const JvpBlock<
             ok = k.done(C::B_XFULL, g);
             if (!ok) break;
             ptx::tc_fence_after_sync();
-            ptx::tmem_ld32(sb + BC, t);
-            ptx::tmem_ld32(sb + BC + 32, t + 32);
             if (g > 0) ok = k.wait(C::B_TURN + q, g - 1);
             if (!ok) break;
             float m_ref = -CUDART_INF_F, cen = 0.f, m_max = -CUDART_INF_F;
-            if (j > 0) { const float4 st = k.row_state[row]; m_ref = st.x; cen = st.y; m_max = st.z; }
-            ptx::tmem_wait_ld();
+            if (j > 0) { const float4 st = k.row_state(row); m_ref = st.x; cen = st.y; m_max = st.z; }
             bool scaling = mrow > m_ref + (C::WIDE ? JVP_LAZY_LOG2_WIDE : JVP_LAZY_LOG2), centring = C::WIDE ? mrow > m_max : scaling;
-            if (__any_sync(0xffffffffu, centring)) {
+            if (__builtin_expect(__any_sync(0xffffffffu, centring), 0)) {
+                ptx::tmem_ld32(sb + BC, t);
+                ptx::tmem_ld32(sb + BC + 32, t + 32);
+                ptx::tmem_wait_ld();
                 float lt = 0.f;                    // Sd at the arg-max key (the first one)
 #pragma unroll
                 for (int c = BC - 1; c >= 0; --c) lt = __uint_as_float(s[c]) == top ? __uint_as_float(t[c]) : lt;
@@ -756,10 +834,10 @@ __device__ __forceinline__ void jvp_elem_fwd(const JvpParams& p, const JvpBlock<
                     }
                     ptx::tmem_wait_st();
                 }
-                k.row_state[row] = make_float4(m_ref, cen, m_max, 0.f);
+                k.row_state(row) = make_float4(m_ref, cen, m_max, 0.f);
             }
             k.arrive(C::B_TURN + q, lane);
-            if (__any_sync(0xffffffffu, m_ref != m_own || (C::WIDE && cen != c_own))) {   // the reference has moved since this group's last tile
+            if (__builtin_expect(__any_sync(0xffffffffu, m_ref != m_own || (C::WIDE && cen != c_own)), 0)) {   // the reference has moved since this group's last tile
                 const float scale = ptx::ex2(m_own - m_ref), fix = c_own - cen;
                 float l0, l1, t0, t1;
                 ptx::unpack2(l2, l0, l1);
@@ -771,30 +849,39 @@ __device__ __forceinline__ void jvp_elem_fwd(const JvpParams& p, const JvpBlock<
             }
             // ---- P~ = 2^(c2 s - m), P~ (T - c): operands of a k-step (16 keys) at the columns of the scores they replace
             const uint64_t nm = ptx::pack2(-m_ref, -m_ref), nc = ptx::pack2(-cen, -cen);
+#pragma unroll 1
+            for (int h = 0; h < BC; h += 32) {   // rolled: half the code (the roles of a scheduler share its instruction cache)
+                ptx::tmem_ld32(sb + h, s);
+                ptx::tmem_ld32(sb + BC + h, t);
+                ptx::tmem_wait_ld();
+                if (__builtin_expect(nvalid < BC, 0)) {
 #pragma unroll
-            for (int u = 0; u < BC / 16; ++u) {
-                uint32_t pp[8], ppt[8];
+                    for (int c = 0; c < 32; ++c)
+                        if (h + c >= nvalid) s[c] = __float_as_uint(-CUDART_INF_F);
+                }
 #pragma unroll
-                for (int c = 0; c < 16; c += 2) {
-                    const uint64_t x2 = ptx::fma2(ptx::pack2u(s[16 * u + c], s[16 * u + c + 1]), c2c2, nm);
-                    float x0, x1;
-                    ptx::unpack2(x2, x0, x1);
-                    const float p0 = ptx::ex2(x0), p1 = ptx::ex2(x1);
-                    const uint64_t p2 = ptx::pack2(p0, p1);
-                    const uint64_t pt2 = ptx::mul2(p2, ptx::fma2(ptx::pack2u(t[16 * u + c], t[16 * u + c + 1]), aa, nc));
-                    l2 = ptx::add2(l2, p2);
-                    mt2 = ptx::add2(mt2, pt2);
-                    float q0, q1;
-                    ptx::unpack2(pt2, q0, q1);
-                    pp[c >> 1] = ptx::pack_bf16(p0, p1);
-                    ppt[c >> 1] = ptx::pack_bf16(q0, q1);
+                for (int u = 0; u < 2; ++u) {
+                    uint32_t pp[8], ppt[8];
+#pragma unroll
+                    for (int c = 0; c < 16; c += 2) {
+                        const uint64_t x2 = ptx::fma2(ptx::pack2u(s[16 * u + c], s[16 * u + c + 1]), c2c2, nm);
+                        float x0, x1;
+                        ptx::unpack2(x2, x0, x1);
+                        const float p0 = ptx::ex2(x0), p1 = ptx::ex2(x1);
+                        const uint64_t p2 = ptx::pack2(p0, p1);
+                        const uint64_t pt2 = ptx::mul2(p2, ptx::fma2(ptx::pack2u(t[16 * u + c], t[16 * u + c + 1]), aa, nc));
+                        l2 = ptx::add2(l2, p2);
+                        mt2 = ptx::add2(mt2, pt2);
+                        float q0, q1;
+                        ptx::unpack2(pt2, q0, q1);
+                        pp[c >> 1] = ptx::pack_bf16(p0, p1);
+                        ppt[c >> 1] = ptx::pack_bf16(q0, q1);
+                    }
+                    ptx::tmem_st8(sb + h + 16 * u, pp);
+                    ptx::tmem_st8(sb + BC + h + 16 * u, ppt);
                 }
-                ptx::tmem_st8(sb + 16 * u, pp);
-                ptx::tmem_st8(sb + BC + 16 * u, ppt);
-                if (u & 1) {   // half of the output MMAs may go
-                    ptx::tmem_wait_st();
-                    k.arrive(C::B_PREADY + 2 * b + (u >> 1), lane);
-                }
+                ptx::tmem_wait_st();
+                k.arrive(C::B_PREADY + 2 * b + (h >> 5), lane);   // half of the output MMAs may go
             }
         }
         if (!ok) break;
@@ -803,7 +890,7 @@ __device__ __forceinline__ void jvp_elem_fwd(const JvpParams& p, const JvpBlock<
         float l0, l1, t0, t1;
         ptx::unpack2(l2, l0, l1);
         ptx::unpack2(mt2, t0, t1);
-        k.row_sums[grp * JVP_ROWS + row] = make_float4(l0 + l1, t0 + t1, m_own, c_own);
+        k.row_sums(grp * JVP_ROWS + row) = make_float4(l0 + l1, t0 + t1, m_own, c_own);
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(k.bar(C::B_ROWSTAT));
     }
@@ -813,25 +900,23 @@ __device__ __forceinline__ void jvp_elem_fwd(const JvpParams& p, const JvpBlock<
 template <int DP, bool HZ>
 __device__ __forceinline__ void jvp_elem_dv(const JvpParams& p, const JvpBlock<PASS_DV, DP>& k, int grp, int q, int lane) {
     using C = JvpCfg<PASS_DV, DP>;
-    constexpr int BC = C::BC;
-    const uint32_t lanes = static_cast<uint32_t>(q * 32) << 16;
+    constexpr int BC = C::BC, HC = BC / 2;
+    const uint32_t sb0 = (static_cast<uint32_t>(q * 32) << 16) + C::COL_SCORE + grp * HC;
     const uint64_t c2c2 = ptx::pack2(p.c2, p.c2), aa = ptx::pack2(p.alpha, p.alpha);
-    const int n_it = (int)blockIdx.x < k.items ? (k.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-    for (int g = grp; g < n_it * k.T; g += 2) {
+    const int n_it = (int)blockIdx.x < p.items ? (p.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+    for (int g = 0; g < n_it * p.T; ++g) {
         const int b = g & 1;
-        const uint32_t sb = lanes + C::COL_SCORE + b * 2 * BC;
+        const uint32_t sb = sb0 + b * 2 * BC;
         if (!k.done(C::B_SFULL, g)) return;
         if (!C::FOLD && !k.wait(C::B_LFULL + g % C::SL, g / C::SL)) return;   // the tile's statistics
         ptx::tc_fence_after_sync();
-        uint32_t s[64], t[64];
+        uint32_t s[HC], t[HC];
         ptx::tmem_ld32(sb, s);
         if (!HZ) ptx::tmem_ld32(sb + BC, t);
-        ptx::tmem_ld32(sb + 32, s + 32);
-        if (!HZ) ptx::tmem_ld32(sb + BC + 32, t + 32);
         ptx::tmem_wait_ld();
-        const float* st = C::FOLD ? nullptr : k.stats + (g % C::SL) * C::NSTAT * BC;
+        const float* st = C::FOLD ? nullptr : k.stats(g % C::SL) + grp * HC;
 #pragma unroll
-        for (int u = 0; u < BC / 16; ++u) {
+        for (int u = 0; u < HC / 16; ++u) {
             uint32_t pa0[8], pa1[8];
 #pragma unroll
             for (int c = 0; c < 16; c += 4) {
@@ -857,11 +942,9 @@ __device__ __forceinline__ void jvp_elem_dv(const JvpParams& p, const JvpBlock<P
             }
             ptx::tmem_st8(sb + 16 * u, pa0);
             if (!HZ) ptx::tmem_st8(sb + BC + 16 * u, pa1);
-            if (u & 1) {   // half of the output MMAs may go
-                ptx::tmem_wait_st();
-                k.arrive(C::B_PREADY + 2 * b + (u >> 1), lane);
-            }
         }
+        ptx::tmem_wait_st();
+        k.arrive(C::B_PREADY + 2 * b + grp, lane);
     }
 }
 
@@ -870,75 +953,73 @@ __device__ __forceinline__ void jvp_elem_dv(const JvpParams& p, const JvpBlock<P
 template <int MODE, int DP, bool HZ>
 __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const JvpBlock<MODE, DP>& k, int grp, int q, int lane) {
     using C = JvpCfg<MODE, DP>;
-    constexpr int BC = C::BC;
+    constexpr int BC = C::BC, HC = BC / 2;
     constexpr bool FOLD = C::FOLD, COL = C::TRANSPOSED && !FOLD, ROW = !C::TRANSPOSED;
     const int row = q * 32 + lane;
-    const uint32_t sb = (static_cast<uint32_t>(q * 32) << 16) + C::COL_SCORE;
+    const uint32_t sb = (static_cast<uint32_t>(q * 32) << 16) + C::COL_SCORE + grp * HC;
     const uint64_t c2c2 = ptx::pack2(p.c2, p.c2), aa = ptx::pack2(p.alpha, p.alpha);
     // DQ: the statistics of this thread's row in the next item, loaded one item ahead
     [[maybe_unused]] float n_lse2 = -CUDART_INF_F, n_mu = 0.f, n_s1 = 0.f, n_cv = 0.f;
     [[maybe_unused]] auto load_stats = [&](int item) {
-        const int bh = item / k.row_tiles, r = (item - bh * k.row_tiles) * JVP_ROWS + row;
+        const int bh = item / p.row_tiles, r = (item - bh * p.row_tiles) * JVP_ROWS + row;
         n_lse2 = -CUDART_INF_F; n_mu = n_s1 = n_cv = 0.f;
-        if (item < k.items && r < p.o.rows) {
+        if (item < p.items && r < p.o.rows) {
             const size_t at = (size_t)bh * p.o.rows + r;
             n_lse2 = p.nlse2[at]; n_mu = p.mu[at]; n_s1 = p.nsig1[at]; n_cv = p.ncvec[at];
         }
     };
     if (ROW) load_stats(blockIdx.x);
-    int it = 0;
-    for (int item = blockIdx.x; item < k.items; item += gridDim.x, ++it) {
-        const int g0 = it * k.T;
+    int g = 0;
+    for (int item = blockIdx.x; item < p.items; item += gridDim.x) {
         [[maybe_unused]] const uint64_t r_l = ptx::pack2(n_lse2, n_lse2), r_nm = ptx::pack2(-n_mu, -n_mu), r_s = ptx::pack2(n_s1, n_s1), r_c = ptx::pack2(n_cv, n_cv);
         if (ROW) load_stats(item + gridDim.x);
-        for (int j = (grp ^ g0) & 1; j < k.T; j += 2) {
-            const int g = g0 + j;
-            [[maybe_unused]] const float* st = COL ? k.stats + (g % C::SL) * C::NSTAT * BC : nullptr;
-            uint32_t s[64], t[64];
-            uint64_t P2[32], N2[32];
+        for (int j = 0; j < p.T; ++j, ++g) {
+            [[maybe_unused]] const float* st = COL ? k.stats(g % C::SL) + grp * HC : nullptr;
+            uint64_t P2[HC / 2], N2[HC / 2];
             // ---- phase A
             if (!k.done(C::B_SFULL, g)) return;
             if (COL && !k.wait(C::B_LFULL + g % C::SL, g / C::SL)) return;   // (complete: those MMAs read the tile's L stage)
             ptx::tc_fence_after_sync();
-            ptx::tmem_ld32(sb, s);
-            if (!HZ) ptx::tmem_ld32(sb + BC, t);
-            ptx::tmem_ld32(sb + 32, s + 32);
-            if (!HZ) ptx::tmem_ld32(sb + BC + 32, t + 32);
-            ptx::tmem_wait_ld();
-            k.arrive(C::B_SREAD, lane);
-            if (ROW && p.s.rows - j * BC < BC) {   // keys beyond N: P = 0
-                const int nvalid = p.s.rows - j * BC;
+            {
+                uint32_t s[HC], t[HC];
+                ptx::tmem_ld32(sb, s);
+                if (!HZ) ptx::tmem_ld32(sb + BC, t);
+                ptx::tmem_wait_ld();
+                k.arrive(C::B_SREAD, lane);
+                const int nvalid = p.s.rows - j * BC - grp * HC;
+                if (ROW && __builtin_expect(nvalid < HC, 0)) {   // keys beyond N: P = 0
 #pragma unroll
-                for (int c = 0; c < BC; ++c)
-                    if (c >= nvalid) s[c] = __float_as_uint(-CUDART_INF_F);   // c2 s = -inf (c2 > 0)
-            }
+                    for (int c = 0; c < HC; ++c)
+                        if (c >= nvalid) s[c] = __float_as_uint(-CUDART_INF_F);   // c2 s = -inf (c2 > 0)
+                }
 #pragma unroll
-            for (int c = 0; c < BC; c += 4) {
-                [[maybe_unused]] ulonglong2 l4, m4;
-                if (COL) l4 = *reinterpret_cast<const ulonglong2*>(st + c);
-                if (COL && !HZ) m4 = *reinterpret_cast<const ulonglong2*>(st + BC + c);
+                for (int c = 0; c < HC; c += 4) {
+                    [[maybe_unused]] ulonglong2 l4, m4;
+                    if (COL) l4 = *reinterpret_cast<const ulonglong2*>(st + c);
+                    if (COL && !HZ) m4 = *reinterpret_cast<const ulonglong2*>(st + BC + c);
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int i = c / 2 + e;
-                    const uint64_t s2 = ptx::pack2u(s[2 * i], s[2 * i + 1]);
-                    float x0, x1;
-                    ptx::unpack2(FOLD ? ptx::mul2(s2, c2c2) : ptx::fma2(s2, c2c2, COL ? (e ? l4.y : l4.x) : r_l), x0, x1);
-                    P2[i] = ptx::pack2(ptx::ex2(x0), ptx::ex2(x1));
-                    if (!HZ) {
-                        const uint64_t ts = ptx::pack2u(t[2 * i], t[2 * i + 1]);
-                        N2[i] = FOLD ? ptx::mul2(ts, aa) : ptx::fma2(ts, aa, COL ? ptx::neg2(e ? m4.y : m4.x) : r_nm);
+                    for (int e = 0; e < 2; ++e) {
+                        const int i = c / 2 + e;
+                        const uint64_t s2 = ptx::pack2u(s[2 * i], s[2 * i + 1]);
+                        float x0, x1;
+                        ptx::unpack2(FOLD ? ptx::mul2(s2, c2c2) : ptx::fma2(s2, c2c2, COL ? (e ? l4.y : l4.x) : r_l), x0, x1);
+                        P2[i] = ptx::pack2(ptx::ex2(x0), ptx::ex2(x1));
+                        if (!HZ) {
+                            const uint64_t ts = ptx::pack2u(t[2 * i], t[2 * i + 1]);
+                            N2[i] = FOLD ? ptx::mul2(ts, aa) : ptx::fma2(ts, aa, COL ? ptx::neg2(e ? m4.y : m4.x) : r_nm);
+                        }
                     }
                 }
             }
-            // ---- phase B, 16 columns (one k-step of the output MMAs) at a time
+            // ---- phase B
             if (!k.done(C::B_XFULL, g)) return;
             ptx::tc_fence_after_sync();
+            uint32_t dd[HC], xx[HC];
+            if (!HZ) ptx::tmem_ld32(sb + 2 * BC, dd);
+            ptx::tmem_ld32(sb + 3 * BC, xx);
+            ptx::tmem_wait_ld();
 #pragma unroll
-            for (int u = 0; u < BC / 16; ++u) {
-                uint32_t dd[16], xx[16];
-                if (!HZ) ptx::tmem_ld16(sb + 2 * BC + 16 * u, dd);
-                ptx::tmem_ld16(sb + 3 * BC + 16 * u, xx);
-                ptx::tmem_wait_ld();
+            for (int u = 0; u < HC / 16; ++u) {
                 uint32_t pa0[8], pa1[8];
 #pragma unroll
                 for (int c = 0; c < 16; c += 4) {
@@ -948,14 +1029,14 @@ __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const Jvp
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         const int i = c / 2 + e, gi = 8 * u + i;
-                        uint64_t x2 = ptx::pack2u(xx[2 * i], xx[2 * i + 1]);
+                        uint64_t x2 = ptx::pack2u(xx[2 * gi], xx[2 * gi + 1]);
                         if (!FOLD) x2 = ptx::add2(x2, COL ? (e ? c4.y : c4.x) : r_c);
                         const uint64_t t2 = ptx::mul2(P2[gi], x2);
                         float d0, d1;
                         if (HZ) {
                             ptx::unpack2(t2, d0, d1);
                         } else {
-                            uint64_t y2 = ptx::pack2u(dd[2 * i], dd[2 * i + 1]);
+                            uint64_t y2 = ptx::pack2u(dd[2 * gi], dd[2 * gi + 1]);
                             if (!FOLD) y2 = ptx::add2(y2, COL ? (e ? s4.y : s4.x) : r_s);
                             const uint64_t w2 = ptx::mul2(P2[gi], y2);
                             float w0, w1;
@@ -968,11 +1049,9 @@ __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const Jvp
                 }
                 if (!HZ) ptx::tmem_st8(sb + 2 * BC + 16 * u, pa0);
                 ptx::tmem_st8(sb + 3 * BC + 16 * u, pa1);
-                if (u & 1) {   // half of the output MMAs may go
-                    ptx::tmem_wait_st();
-                    k.arrive(C::B_PREADY + (u >> 1), lane);
-                }
             }
+            ptx::tmem_wait_st();
+            k.arrive(C::B_PREADY + grp, lane);
         }
     }
 }
@@ -991,7 +1070,7 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
     // Row of tensor t in an item; what is beyond the head dim or the tensor, and an absent cotangent, reads as zero.  The
     // columns of ones that the statistics are multiplied by (FOLD): padding of the first tensor.
     [[maybe_unused]] auto load_x = [&](int item, int t, uint4 (&v)[NCH]) {
-        const int bh = item / k.row_tiles, row0 = (item - bh * k.row_tiles) * JVP_ROWS;
+        const int bh = item / p.row_tiles, row0 = (item - bh * p.row_tiles) * JVP_ROWS;
         const __nv_bfloat16* x = p.own[XT0 + t];
         const bool valid = x && row0 + row < p.o.rows;
         const __nv_bfloat16* src = x + (p.o.head_off(bh, p.H) + (size_t)(row0 + row) * (size_t)p.o.rs);
@@ -1000,7 +1079,7 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
             v[c] = make_uint4(0, 0, 0, 0);
             if (valid && 8 * c < p.d) v[c] = __ldg(reinterpret_cast<const uint4*>(src + 8 * c));
         }
-        if (C::FOLD && t == 0 && !k.fold_step) { v[NCH - 1].x = JVP_ONES0; v[NCH - 1].y = JVP_ONES1; }
+        if (C::FOLD && t == 0 && !k.fold_step()) { v[NCH - 1].x = JVP_ONES0; v[NCH - 1].y = JVP_ONES1; }
     };
     [[maybe_unused]] auto store_x = [&](int t, const uint4 (&v)[NCH]) {
 #pragma unroll
@@ -1010,7 +1089,7 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
         }
     };
     [[maybe_unused]] uint4 v0[NCH], v1[NCH];
-    if (C::XT && (int)blockIdx.x < k.items) {
+    if (C::XT && (int)blockIdx.x < p.items) {
         if (C::FOLD) {
             const uint32_t r[8] = {JVP_ONES0, JVP_ONES1, 0u, 0u, 0u, 0u, 0u, 0u};
             ptx::tmem_st8(lanes + C::COL_ONES, r);
@@ -1023,27 +1102,27 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
         k.arrive(C::B_XRDY, lane);
     }
     int it = 0;
-    for (int item = blockIdx.x; item < k.items; item += gridDim.x, ++it) {
-        if (C::XT && item + (int)gridDim.x < k.items) {
+    for (int item = blockIdx.x; item < p.items; item += gridDim.x, ++it) {
+        if (C::XT && item + (int)gridDim.x < p.items) {
             load_x(item + gridDim.x, 0, v0);                       // in flight during the wait
-            if (MODE == PASS_DV) load_x(item + gridDim.x, 1, v1);   // (the other passes have no registers for the second)
+            if (MODE != PASS_FWD) load_x(item + gridDim.x, 1, v1);   // (the forward has no registers for the second)
             if (!k.wait(C::B_XFREE, it)) return;
             ptx::tc_fence_after_sync();
             store_x(0, v0);
-            if (MODE != PASS_DV) load_x(item + gridDim.x, 1, v0);
-            store_x(1, MODE == PASS_DV ? v1 : v0);
+            if (MODE == PASS_FWD) load_x(item + gridDim.x, 1, v0);
+            store_x(1, MODE != PASS_FWD ? v1 : v0);
             ptx::tmem_wait_st();
             k.arrive(C::B_XRDY, lane);
         }
-        const int bh = item / k.row_tiles, row0 = (item - bh * k.row_tiles) * JVP_ROWS;
+        const int bh = item / p.row_tiles, row0 = (item - bh * p.row_tiles) * JVP_ROWS;
         const size_t off = p.o.head_off(bh, p.H) + (size_t)(row0 + row) * (size_t)p.o.rs;
         // lane pairs write the two rows of the pair one after the other, each as complete 32-byte sectors
         const bool ok_even = row0 + (row & ~1) < p.o.rows, ok_odd = row0 + (row | 1) < p.o.rows;
         float f0 = p.out_scale, mun = 0.f;
         if constexpr (MODE == PASS_FWD) {   // O = O~/l, tO = R/l - (mu - c) O
             if (!k.wait(C::B_ROWSTAT, it)) return;
-            const int last = (it * k.T + k.T - 1) & 1;   // the group whose reference is the accumulators'
-            const float4 f = k.row_sums[last * JVP_ROWS + row], o = k.row_sums[(last ^ 1) * JVP_ROWS + row];
+            const int last = (it * p.T + p.T - 1) & 1;   // the group whose reference is the accumulators'
+            const float4 f = k.row_sums(last * JVP_ROWS + row), o = k.row_sums((last ^ 1) * JVP_ROWS + row);
             const float scale = ptx::ex2(o.z - f.z);     // (a group without a tile: m = -inf, factor 0)
             const float l = fmaf(o.x, scale, f.x), mt = f.y + scale * fmaf(o.w - f.w, o.x, o.y);
             f0 = 1.0f / l;
@@ -1099,28 +1178,9 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
         return;
     }
     extern __shared__ __align__(1024) uint8_t jvp_smem[];
-    uint8_t* misc = jvp_smem + C::TILE_BYTES;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 56 * 8);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 56 * 8 + 16);
-
-    JvpBlock<MODE, DP> k;
-    k.own = ptx::smem_u32(jvp_smem);
-    k.e = k.own + C::NOWN * C::OWN_BYTES;
-    k.l = k.e + C::SE * 2 * C::EST_BYTES;
-    k.bar0 = ptx::smem_u32(misc);
-    k.abort_flag = abort_flag;
-    k.stats = reinterpret_cast<float*>(misc + 56 * 8 + 64);
-    k.row_state = reinterpret_cast<float4*>(k.stats + C::STATS_FLOATS);
-    k.row_sums = reinterpret_cast<float4*>(k.row_state + JVP_ROWS);
-    uint8_t* fold = reinterpret_cast<uint8_t*>(k.stats + C::STATS_FLOATS + C::FWD_FLOATS);
-    k.fold_e = ptx::smem_u32(fold);
-    k.fold_l = k.fold_e + C::FOLD_E * C::FOLD_BYTES;
-    k.ones = k.fold_l + C::FOLD_L * C::FOLD_BYTES;
-    k.zeros = k.ones + JVP_ROWS * 16;
-    k.fold_step = C::FOLD && (C::NA == 1 || p.d == DP);
-    k.row_tiles = (p.o.rows + JVP_ROWS - 1) / JVP_ROWS;
-    k.items = p.BH * k.row_tiles;
-    k.T = (p.s.rows + BC - 1) / BC;
+    const JvpBlock<MODE, DP> k{ptx::smem_u32(jvp_smem), p};
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(jvp_smem + k.SLOT);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(jvp_smem + k.ABORT);
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -1133,7 +1193,8 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
         init(C::B_XRDY, 1, 4);
         init(C::B_XFREE, 1, 1);
         init(C::B_SFULL, 12, 1);       // SFULL, XFULL, OUTDONE
-        init(C::B_PREADY, 5, 4);       // PREADY, SREAD: the four warps of a group
+        init(C::B_PREADY, 4, 4);       // the four warps of a group
+        init(C::B_SREAD, 1, 8);
         init(C::B_FINAL, 1, 1);
         init(C::B_ACCFREE, 1, 4);
         init(C::B_TURN, 4, 1);
@@ -1176,7 +1237,7 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
     }
     if (C::FOLD)
         for (int i = threadIdx.x; i < 2 * JVP_ROWS; i += JVP_THREADS)
-            *reinterpret_cast<uint4*>(fold + (C::FOLD_E + C::FOLD_L) * C::FOLD_BYTES + i * 16) = i < JVP_ROWS ? make_uint4(JVP_ONES0, JVP_ONES1, 0, 0) : zero;
+            *reinterpret_cast<uint4*>(jvp_smem + k.ONES + i * 16) = i < JVP_ROWS ? make_uint4(JVP_ONES0, JVP_ONES1, 0, 0) : zero;
     if (!HZ && MODE == PASS_DQ && !C::XT && p.absent)   // an absent cotangent is an owner tile of zeros
         for (int t = 2; t < 4; ++t)
             if (!p.own[t])
@@ -1191,7 +1252,7 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
     ptx::tc_fence_after_sync();
     // The whole tensor memory starts at 0 and the shared memory of a kernel without static arrays at a 1024-byte boundary:
     // the roles take both for granted.
-    const bool placed = *tmem_slot == 0 && (k.own & 1023) == 0;
+    const bool placed = *tmem_slot == 0 && (k.base & 1023) == 0;
     if (!placed && threadIdx.x == 0) *abort_flag = 1;
 
     // warpgroup 0: loads and MMA issue; 1, 2: element-wise; 3: epilogue
@@ -1201,10 +1262,8 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
             const CUtensorMap* const maps[4] = {&o0, &o1, &o2, &o3};
             if (warp == 0) jvp_load_ring<MODE, DP, 0>(p, k, &s0, &s1, maps, lane);
             else if (warp == 2) jvp_load_ring<MODE, DP, 1>(p, k, &s2, &s3, maps, lane);
-            else if (warp == 1) {
-                if constexpr (C::NPAIR == 1) jvp_issue_one_pair<MODE, DP, HZ>(p, k);
-                else jvp_issue_two_pairs<MODE, DP, HZ>(p, k);
-            }
+            else if (warp == 1) jvp_issue<MODE, DP, HZ>(p, k);
+            else if constexpr (C::FOLD) jvp_fold<MODE, DP>(p, k, lane);
         }
         if (warp == 1 && *abort_flag && placed) {
             // after a time-out: the queued MMAs must be done before the tensor memory is given back

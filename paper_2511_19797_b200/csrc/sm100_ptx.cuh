@@ -85,22 +85,11 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
-// ---------------------------------------------------------------- TMA (tiled, 3-D, no multicast)
-__device__ __forceinline__ void prefetch_tmap(const void* tmap) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");
-}
-// Loads one box of a 3-D tensor map into shared memory; completion is signalled on `bar` as
-// transaction bytes.  c0 is the innermost (element) coordinate and must be a multiple of 8 for
-// 16-bit elements.
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
-        : "memory");
-}
+// ---------------------------------------------------------------- TMA (tiled, no multicast)
 
-// The same for a 4-D tensor map (element, row, head, batch): tensors whose heads and batches have strides of
-// their own, e.g. a (B, rows, H, d) slice of a fused projection read in place.
+// Loads one box of a 4-D tensor map (element, row, head, batch: a (B, rows, H, d) slice of a fused projection is read in
+// place) into shared memory; completion is signalled on `bar` as transaction bytes.  c0 is the innermost (element)
+// coordinate and must be a multiple of 8 for 16-bit elements.
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2, int c3) {
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
@@ -138,13 +127,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
         : "r"(taddr)
         : "memory");
 }
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
-        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-          "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-        : "memory");
-}
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
@@ -157,6 +139,9 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
 __device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src, uint32_t src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
+__device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
 // The same for 4 bytes (sources that are only 4-byte aligned).
 __device__ __forceinline__ void cp_async_4(uint32_t dst, const void* src, uint32_t src_bytes) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
@@ -166,22 +151,12 @@ __device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int PENDING>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
-}
 
 // 32 lanes x 8 consecutive 32-bit columns.
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "r"(taddr)
-                 : "memory");
-}
-__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t* r) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};"
-                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3])
                  : "memory");
 }
 // 32 lanes x 32 consecutive 32-bit columns.
@@ -198,79 +173,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
 }
 
 // ---------------------------------------------------------------- tcgen05.mma (kind::f16, 1 CTA)
-// 64-bit shared-memory matrix descriptor: start address, leading/stride byte offsets (all >> 4),
-// descriptor version 1 (bits 46-47) and the swizzle mode in bits 61-63 (2 = 128-byte swizzle).
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-    uint64_t d = 0;
-    d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
-    d |= static_cast<uint64_t>((lbo_bytes >> 4) & 0x3FFFu) << 16;
-    d |= static_cast<uint64_t>((sbo_bytes >> 4) & 0x3FFFu) << 32;
-    d |= static_cast<uint64_t>(1) << 46;
-    d |= static_cast<uint64_t>(2) << 61;
-    return d;
-}
-// Same descriptor without swizzle: core matrices of 8 rows x 16 bytes, each contiguous (128 bytes).
-// For a K-major operand lbo_bytes is the distance between the core matrices of the two 16-byte
-// halves of a k-step, sbo_bytes the distance between 8-row groups.
-__device__ __forceinline__ uint64_t smem_desc_nosw(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-    uint64_t d = 0;
-    d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
-    d |= static_cast<uint64_t>((lbo_bytes >> 4) & 0x3FFFu) << 16;
-    d |= static_cast<uint64_t>((sbo_bytes >> 4) & 0x3FFFu) << 32;
-    d |= static_cast<uint64_t>(1) << 46;
-    return d;
-}
 // 32-bit instruction descriptor: fp32 accumulate (bits 4-5 = 1), bf16 A and B (bits 7-9, 10-12 = 1),
 // A/B major-ness (bits 15, 16; 0 = K-major, 1 = MN-major), N >> 3 in bits 17-22, M >> 4 in bits 24-28.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(uint32_t M, uint32_t N, uint32_t a_mn_major, uint32_t b_mn_major) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn_major << 15) | (b_mn_major << 16) | ((N >> 3) << 17) |
            ((M >> 4) << 24);
 }
-// D[tmem] (+)= A[smem] * B[smem]
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// D[tmem] (+)= A[tmem] * B[smem]   (A: 128 lanes x K/2 packed bf16 columns)
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// Arrives once on `bar` when every tcgen05 operation this thread issued before has completed.
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
 
-// Warp-collective forms: the whole warp executes the call in converged control flow and one elected
-// lane issues the instruction.  Keeping the surrounding loop warp-uniform lets the compiler hold the
-// descriptors in uniform registers; issued from a divergent `lane == 0` branch the same MMA costs
-// about 45 cycles of issue time, more than a 128 x 64 x 16 MMA takes to execute.
-__device__ __forceinline__ void mma_ss_elect(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .pred e;\n\t"
-        "elect.sync _|e, 0xffffffff;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void mma_ts_elect(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .pred e;\n\t"
-        "elect.sync _|e, 0xffffffff;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
 __device__ __forceinline__ void mma_commit_elect(uint32_t bar) {
     asm volatile(
         "{\n\t.reg .pred e;\n\t"
@@ -303,6 +212,16 @@ __device__ __forceinline__ void mma_ts_p(uint32_t el, uint32_t d_tmem, uint32_t 
         ::"r"(el), "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "n"(ACC)
         : "memory");
 }
+__device__ __forceinline__ void mma_ts_acc(uint32_t el, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .pred e;\n\t.reg .b64 b;\n\t"
+        "setp.ne.b32 e, %0, 0;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "mov.b64 b, {%3, %4};\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%1], [%2], b, %5, p;\n\t}"
+        ::"r"(el), "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
 template <uint32_t ACC>
 __device__ __forceinline__ void mma_ss_p(uint32_t el, uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc) {
     asm volatile(
@@ -330,33 +249,28 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
     return __all_sync(0xffffffffu, ok);
 }
 
-// A turn counter in shared memory orders steps of two warps: `turn_post` publishes a count, `turn_wait_warp`
-// waits (bounded like mbar_wait; warp-uniform result) until it has reached `want`.
-__device__ __forceinline__ void turn_post(uint32_t addr, uint32_t value) {
-    asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(addr), "r"(value) : "memory");
-}
-__device__ __forceinline__ uint32_t turn_read(uint32_t addr) {
-    uint32_t v;
-    asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ bool turn_wait_warp(uint32_t addr, uint32_t want, volatile int* abort_flag, uint64_t limit_ns) {
-    bool ok = true;
-    if (turn_read(addr) < want) {
-        const uint64_t t0 = globaltimer_ns();
-        for (uint32_t it = 1;; ++it) {
-            if (turn_read(addr) >= want) break;
-            if ((it & 255u) == 0u) {
-                if (*abort_flag) { ok = false; break; }
-                if (globaltimer_ns() - t0 > limit_ns) {
-                    *abort_flag = 1;
-                    ok = false;
-                    break;
-                }
-            }
-        }
-    }
+// The same with the abort flag given by its shared-memory address (one register instead of two where a role has none to
+// spare).
+__device__ __forceinline__ bool mbar_wait_warp_s(uint32_t bar, uint32_t parity, uint32_t abort_addr, uint64_t limit_ns) {
+    bool ok = mbar_try_wait(bar, parity);
+    for (int it = 0; it < 256 && !ok; ++it) ok = mbar_try_wait(bar, parity);
+    if (__builtin_expect(__all_sync(0xffffffffu, ok), 1)) return true;
+    if (!ok) ok = mbar_wait(bar, parity, static_cast<volatile int*>(__cvta_shared_to_generic(abort_addr)), limit_ns);
     return __all_sync(0xffffffffu, ok);
+}
+// Non-blocking test of two mbarrier phases at once; warp-uniform result.
+__device__ __forceinline__ bool mbar_test2_warp(uint32_t b0, uint32_t p0, uint32_t b1, uint32_t p1) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred a;\n\t.reg .pred b;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 a, [%1], %2;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 b, [%3], %4;\n\t"
+        "and.pred a, a, b;\n\t"
+        "selp.u32 %0, 1, 0, a;\n\t}"
+        : "=r"(ok)
+        : "r"(b0), "r"(p0), "r"(b1), "r"(p1)
+        : "memory");
+    return __all_sync(0xffffffffu, ok != 0);
 }
 
 // Non-blocking test of one mbarrier phase; warp-uniform result.
@@ -368,44 +282,6 @@ __device__ __forceinline__ bool mbar_test_warp(uint32_t bar, uint32_t parity) {
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
         : "r"(bar), "r"(parity)
-        : "memory");
-    return __all_sync(0xffffffffu, ok != 0);
-}
-
-// Bounded wait for two mbarrier phases, executed by a whole warp; warp-uniform result.  Both are polled back
-// to back first, so that when both have completed (the steady state of a pipeline) one shared-memory round
-// trip replaces two serial ones.
-__device__ __forceinline__ bool mbar_wait2_warp(uint32_t b0, uint32_t p0, uint32_t b1, uint32_t p1, volatile int* abort_flag,
-                                                uint64_t limit_ns) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred a;\n\t.reg .pred b;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 a, [%1], %2;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 b, [%3], %4;\n\t"
-        "and.pred a, a, b;\n\t"
-        "selp.u32 %0, 1, 0, a;\n\t}"
-        : "=r"(ok)
-        : "r"(b0), "r"(p0), "r"(b1), "r"(p1)
-        : "memory");
-    if (__all_sync(0xffffffffu, ok != 0)) return true;
-    if (!mbar_wait_warp(b0, p0, abort_flag, limit_ns)) return false;
-    return mbar_wait_warp(b1, p1, abort_flag, limit_ns);
-}
-
-// Non-blocking test of three mbarrier phases at once; the three polls are issued back to back so
-// that their shared-memory round trips overlap.  Warp-uniform result.  In the steady state of a
-// pipeline all three have completed and one round trip replaces three serial waits.
-__device__ __forceinline__ bool mbar_test3_warp(uint32_t b0, uint32_t p0, uint32_t b1, uint32_t p1, uint32_t b2, uint32_t p2) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred a;\n\t.reg .pred b;\n\t.reg .pred c;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 a, [%1], %2;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 b, [%3], %4;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 c, [%5], %6;\n\t"
-        "and.pred a, a, b;\n\tand.pred a, a, c;\n\t"
-        "selp.u32 %0, 1, 0, a;\n\t}"
-        : "=r"(ok)
-        : "r"(b0), "r"(p0), "r"(b1), "r"(p1), "r"(b2), "r"(p2)
         : "memory");
     return __all_sync(0xffffffffu, ok != 0);
 }
@@ -463,9 +339,6 @@ template <int REGS>
 __device__ __forceinline__ void setmaxnreg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS)); }
 template <int REGS>
 __device__ __forceinline__ void setmaxnreg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS)); }
-__device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t nthreads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
 
 }  // namespace ptx
 }  // namespace tvm_attn

@@ -12,8 +12,6 @@
 #include <mutex>
 #include <utility>
 
-#include "jvp_bwd_sm100.cuh"
-#include "jvp_fwd_sm100.cuh"
 #include "jvp_sm100.cuh"
 #include "qk_rmsnorm.cuh"
 #include "simt_kernels.cuh"
@@ -76,18 +74,9 @@ static int tensor_core_device(const DeviceFacts** f) {
     return !*f ? TVM_ATTN_CUDA_ERROR : (*f)->major == 10 ? TVM_ATTN_OK : TVM_ATTN_UNSUPPORTED;
 }
 
-// Lets `kern` use `bytes` of dynamic shared memory: set once per thread, context and kernel (KERN is its identity).
-template <auto KERN>
-static bool allow_smem(const DeviceFacts& f, int bytes) {
-    thread_local unsigned long long done = 0;
-    if (done == f.ctx) return true;
-    if (cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
-    done = f.ctx;
-    return true;
-}
-
-// The same for the kernels whose warpgroups redistribute registers, with a check that they were compiled to the number
-// that is redistributed (fewer would make them wait for registers that do not exist).
+// Prepares a tensor-core kernel for launches, once per thread and context (KERN is its identity): its dynamic shared
+// memory, and a check that it was compiled to the registers its warpgroups redistribute (fewer would make them wait for
+// registers that do not exist).
 template <auto KERN>
 static bool prepare_kernel(const DeviceFacts& f, int smem_bytes) {
     thread_local unsigned long long done = 0;
@@ -247,13 +236,13 @@ static encode_tiled_fn get_encode_fn() {
 }
 
 // A bf16 tensor of one side viewed as a 4-D tensor (d, rows, H, B) with that side's strides; a box is 64 columns x
-// `rows` rows of one head with the 128-byte swizzle; columns or rows beyond the tensor read as zero.
-static int make_tmap(CUtensorMap* m, const void* ptr, const Shape& s, const Geom& g, int rows) {
+// 64 rows of one head with the 128-byte swizzle; columns or rows beyond the tensor read as zero.
+static int make_tmap(CUtensorMap* m, const void* ptr, const Shape& s, const Geom& g) {
     encode_tiled_fn fn = get_encode_fn();
     if (!fn) return TVM_ATTN_CUDA_ERROR;
     cuuint64_t dims[4] = {(cuuint64_t)s.d, (cuuint64_t)g.rows, (cuuint64_t)s.H, (cuuint64_t)s.B};
     cuuint64_t strides[3] = {(cuuint64_t)g.rs * 2, (cuuint64_t)g.hs * 2, (cuuint64_t)g.bs * 2};
-    cuuint32_t box[4] = {64, (cuuint32_t)rows, 1, 1};
+    cuuint32_t box[4] = {64, JVP_BC, 1, 1};
     cuuint32_t estr[4] = {1, 1, 1, 1};
     CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -282,7 +271,9 @@ static int launch_pass(const Shape& s, const Operand (&own)[4], const Operand (&
     }
     // one CTA per SM (each needs the whole tensor memory and most of the shared memory of one); the work
     // items go round-robin over them
-    const long long items = s.BH * ((prm.o.rows + JVP_ROWS - 1) / JVP_ROWS);
+    prm.row_tiles = (prm.o.rows + JVP_ROWS - 1) / JVP_ROWS;
+    prm.items = (int)(s.BH * prm.row_tiles);
+    prm.T = (prm.s.rows + JVP_BC - 1) / JVP_BC;
     g_prof.before(st);
     // DK and DQ read nothing that the pass before them writes (DV, DK and DQ all depend on the row-sums pre-pass only,
     // which has completed before DV starts), so their CTAs may fill the SMs that the last, partial wave of the pass
@@ -291,7 +282,7 @@ static int launch_pass(const Shape& s, const Operand (&own)[4], const Operand (&
     // the teardown), so that DQ cannot complete before DK, nor DK before DV: work enqueued behind the call still sees all
     // six gradients.  Not while per-kernel events are being recorded: they would time overlapping kernels.
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(items < dev.sms ? items : dev.sms));
+    cfg.gridDim = dim3((unsigned)(prm.items < dev.sms ? prm.items : dev.sms));
     cfg.blockDim = dim3(JVP_THREADS);
     cfg.dynamicSmemBytes = C::SMEM_BYTES;
     cfg.stream = st;
@@ -308,20 +299,13 @@ static int launch_pass(const Shape& s, const Operand (&own)[4], const Operand (&
     return cuda_status(cudaGetLastError());
 }
 
-// Padded head dims up to this one run the kernels of jvp_fwd_sm100.cuh and jvp_bwd_sm100.cuh.
-#ifndef JVP_MIN
-#define JVP_MIN 80
-#endif
 template <int MODE, int DP>
 static int launch_pass_hz(const Shape& s, const Operand (&own)[4], const Operand (&strm)[4], const JvpParams& prm, const DeviceFacts& dev, cudaStream_t st) {
-    if constexpr (DP <= JVP_MIN) return TVM_ATTN_UNSUPPORTED;
-    else {
-        // dtO absent: the specialisation that leaves the tangent path out (only instantiated for the padded head dims
-        // 64 and 80 of the transformer shapes; other head dims run the general kernel, which skips what it can)
-        if constexpr (MODE != PASS_FWD && (DP == 64 || DP == 80))
-            if (prm.absent & ABSENT_HC) return launch_pass<MODE, DP, true>(s, own, strm, prm, dev, st);
-        return launch_pass<MODE, DP, false>(s, own, strm, prm, dev, st);
-    }
+    // dtO absent: the specialisation that leaves the tangent path out (only instantiated for the padded head dims
+    // 64 and 80 of the transformer shapes; other head dims run the general kernel, which skips what it can)
+    if constexpr (MODE != PASS_FWD && (DP == 64 || DP == 80))
+        if (prm.absent & ABSENT_HC) return launch_pass<MODE, DP, true>(s, own, strm, prm, dev, st);
+    return launch_pass<MODE, DP, false>(s, own, strm, prm, dev, st);
 }
 
 template <int MODE>
@@ -335,98 +319,6 @@ static int launch_pass_dp(const Shape& s, const Operand (&own)[4], const Operand
         case 96: return launch_pass_hz<MODE, 96>(s, own, strm, prm, dev, st);
         case 112: return launch_pass_hz<MODE, 112>(s, own, strm, prm, dev, st);
         default: return launch_pass_hz<MODE, 128>(s, own, strm, prm, dev, st);
-    }
-}
-
-// Forward for padded head dims up to 80: operands Q, tQ live in tensor memory (jvp_fwd_sm100.cuh).
-template <int DP>
-static int launch_fwd(const Shape& s, const void* const strm[4], const FwdParams& prm, const DeviceFacts& dev, cudaStream_t st) {
-    using C = FwdCfg<DP>;
-    CUtensorMap m[4];
-    for (int t = 0; t < 4; ++t) {
-        const int rc = make_tmap(&m[t], strm[t], s, s.k, FWD_BC);
-        if (rc != TVM_ATTN_OK) return rc;
-    }
-    auto kern = jvp_fwd_kernel<DP>;
-    if (!allow_smem<jvp_fwd_kernel<DP>>(dev, C::SMEM_BYTES)) return TVM_ATTN_CUDA_ERROR;
-    // one CTA per SM (each needs the whole tensor memory and most of the shared memory of one); the work
-    // items go round-robin over them
-    const long long items = s.BH * ((s.M + FWD_ROWS - 1) / FWD_ROWS);
-    const long long grid = items < dev.sms ? items : dev.sms;
-    g_prof.before(st);
-    kern<<<(unsigned)grid, FWD_THREADS, C::SMEM_BYTES, st>>>(m[0], m[1], m[2], m[3], prm);
-    g_prof.after(st);
-    g_launches += 1;
-    return cuda_status(cudaGetLastError());
-}
-
-// One backward pass for padded head dims up to 80 (jvp_bwd_sm100.cuh).  own: X0..X3; strm: E ring (0, 1), L ring (2, 3).
-template <int MODE, int DP>
-static int launch_bwd_pass(const Shape& s, const void* const own[4], const void* const strm[4], BwdParams prm,
-                           const DeviceFacts& dev, cudaStream_t st) {
-    using C = BwdCfg<MODE, DP>;
-    CUtensorMap ms[4], mo[2];
-    // DV, DK: keys own, queries stream; DQ: queries own, keys stream
-    prm.o = MODE == BWD_DQ ? s.q : s.k;
-    prm.s = MODE == BWD_DQ ? s.k : s.q;
-    for (int t = 0; t < 4; ++t) {
-        // an absent cotangent (null) is never loaded: its map is built on a present tensor and stays unused
-        const int rc = make_tmap(&ms[t], strm[t] ? strm[t] : strm[t ^ 1], s, prm.s, C::BC);
-        if (rc != TVM_ATTN_OK) return rc;
-        prm.strm[t] = static_cast<const __nv_bfloat16*>(strm[t]);
-        prm.own[t] = static_cast<const __nv_bfloat16*>(own[t]);
-    }
-    for (int t = 0; t < 2; ++t) {
-        const int rc = make_tmap(&mo[t], own[C::NPAIR == 2 ? C::XS0 + t : t], s, prm.o, BWD_ROWS);  // never a cotangent
-        if (rc != TVM_ATTN_OK) return rc;
-    }
-    // dtO absent: the specialisation that leaves the tangent path out (only instantiated for the padded head dims
-    // 64 and 80 of the transformer shapes; other head dims run the general kernel, which skips what it can)
-    constexpr bool HAS_HZ = DP == 64 || DP == 80;
-    const bool hz = HAS_HZ && (prm.absent & ABSENT_HC);
-    auto kern = hz ? jvp_bwd_kernel<MODE, DP, HAS_HZ> : jvp_bwd_kernel<MODE, DP, false>;
-    if (!(hz ? allow_smem<jvp_bwd_kernel<MODE, DP, HAS_HZ>>(dev, C::SMEM_BYTES) : allow_smem<jvp_bwd_kernel<MODE, DP, false>>(dev, C::SMEM_BYTES)))
-        return TVM_ATTN_CUDA_ERROR;
-    // one CTA per SM (each needs the whole tensor memory and most of the shared memory of one); the work
-    // items go round-robin over them
-    const long long items = s.BH * ((prm.o.rows + BWD_ROWS - 1) / BWD_ROWS);
-    const long long grid = items < dev.sms ? items : dev.sms;
-    g_prof.before(st);
-    {
-        // DK and DQ read nothing that the pass before them writes (DV, DK and DQ all depend on the row-sums
-        // pre-pass only, which has completed before DV starts), so their CTAs may fill the SMs that the last,
-        // partial wave of the pass before leaves idle: programmatic dependent launch, with every CTA of these
-        // kernels releasing its dependents at once.  None waits for its primary before it works; each waits for
-        // it once at the very end (griddepcontrol.wait in the teardown), so that DQ cannot complete before DK, nor
-        // DK before DV: work enqueued behind the call still sees all six gradients.  Not while per-kernel events
-        // are being recorded: they would time overlapping kernels.
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)grid);
-        cfg.blockDim = dim3(BWD_THREADS);
-        cfg.dynamicSmemBytes = C::SMEM_BYTES;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = (MODE != BWD_DV && !g_prof.enabled.load(std::memory_order_relaxed)) ? 1 : 0;
-        if (cudaLaunchKernelEx(&cfg, kern, ms[0], ms[1], ms[2], ms[3], mo[0], mo[1], prm) != cudaSuccess)
-            return cuda_status(cudaGetLastError());
-    }
-    g_prof.after(st);
-    g_launches += 1;
-    return cuda_status(cudaGetLastError());
-}
-
-template <int MODE>
-static int launch_bwd_pass_dp(const Shape& s, const void* const own[4], const void* const strm[4], const BwdParams& prm,
-                              const DeviceFacts& dev, cudaStream_t st) {
-    switch (s.dp) {
-        case 16: return launch_bwd_pass<MODE, 16>(s, own, strm, prm, dev, st);
-        case 32: return launch_bwd_pass<MODE, 32>(s, own, strm, prm, dev, st);
-        case 48: return launch_bwd_pass<MODE, 48>(s, own, strm, prm, dev, st);
-        case 64: return launch_bwd_pass<MODE, 64>(s, own, strm, prm, dev, st);
-        default: return launch_bwd_pass<MODE, 80>(s, own, strm, prm, dev, st);
     }
 }
 
@@ -596,40 +488,21 @@ int tvm_attn_jvp_fwd(const tvm_attn_params* p, const void* Q, const void* K, con
     const DeviceFacts* dev;
     rc = tensor_core_device(&dev);
     if (rc != TVM_ATTN_OK) return rc;
-    int* status = dev->status;
-    const void* strm[4] = {K, tK, V, tV};
-    if (s.dp <= JVP_MIN) {
-        FwdParams f;
-        f.d = s.d; f.BH = (int)s.BH; f.H = s.H; f.q = s.q; f.k = s.k;
-        f.alpha = s.alpha; f.c2 = s.alpha * 1.4426950408889634f;
-        f.Q = static_cast<const __nv_bfloat16*>(Q); f.tQ = static_cast<const __nv_bfloat16*>(tQ);
-        f.K = static_cast<const __nv_bfloat16*>(K); f.tK = static_cast<const __nv_bfloat16*>(tK);
-        f.V = static_cast<const __nv_bfloat16*>(V); f.tV = static_cast<const __nv_bfloat16*>(tV);
-        f.O = static_cast<__nv_bfloat16*>(O); f.tO = static_cast<__nv_bfloat16*>(tO);
-        f.lse = lse; f.mu = mu; f.status = status;
-        switch (s.dp) {
-            case 16: return launch_fwd<16>(s, strm, f, *dev, st);
-            case 32: return launch_fwd<32>(s, strm, f, *dev, st);
-            case 48: return launch_fwd<48>(s, strm, f, *dev, st);
-            case 64: return launch_fwd<64>(s, strm, f, *dev, st);
-            default: return launch_fwd<80>(s, strm, f, *dev, st);
-        }
-    }
     if (s.dp > 80 && !s.plain) return TVM_ATTN_UNSUPPORTED;  // head dims above 80: self-attention on packed tensors only
     CUtensorMap maps[6];
     const void* in[6] = {Q, tQ, K, tK, V, tV};
     Operand x[6];
     for (int t = 0; t < 6; ++t) {
-        rc = make_tmap(&maps[t], in[t], s, t < 2 ? s.q : s.k, JVP_BC);
+        rc = make_tmap(&maps[t], in[t], s, t < 2 ? s.q : s.k);
         if (rc != TVM_ATTN_OK) return rc;
         x[t] = {static_cast<const __nv_bfloat16*>(in[t]), &maps[t]};
     }
     JvpParams f;
     std::memset(&f, 0, sizeof f);
-    f.d = s.d; f.BH = (int)s.BH; f.H = s.H;
+    f.d = s.d; f.H = s.H;
     f.alpha = s.alpha; f.c2 = s.alpha * 1.4426950408889634f;
     f.out0 = static_cast<__nv_bfloat16*>(O); f.out1 = static_cast<__nv_bfloat16*>(tO);
-    f.lse = lse; f.mu_out = mu; f.status = status;
+    f.lse = lse; f.mu_out = mu; f.status = dev->status;
     return launch_pass_dp<PASS_FWD>(s, {x[0], x[1], x[0], x[1]}, {x[2], x[3], x[4], x[5]}, f, *dev, st);
 }
 
@@ -684,54 +557,22 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
     const DeviceFacts* dev;
     rc = tensor_core_device(&dev);
     if (rc != TVM_ATTN_OK) return rc;
-    int* status = dev->status;
-    rc = launch_rowsums<__nv_bfloat16>(s, dO, dtO, O, tO, lse, sig1, cvec, lse2, s.dp <= JVP_MIN ? 1.0f : -1.0f, st);
+    rc = launch_rowsums<__nv_bfloat16>(s, dO, dtO, O, tO, lse, sig1, cvec, lse2, -1.0f, st);
     if (rc != TVM_ATTN_OK) return rc;
-    if (s.dp <= JVP_MIN) {
-        BwdParams b;
-        std::memset(&b, 0, sizeof b);
-        b.d = s.d; b.BH = (int)s.BH; b.H = s.H;
-        b.alpha = s.alpha; b.c2 = s.alpha * 1.4426950408889634f;
-        b.lse2 = lse2; b.mu = mu; b.sig1 = sig1; b.cvec = cvec; b.status = status; b.absent = absent;
-        {   // dtV = P^T Hc, dV = P^T G + (P*Nn)^T Hc : owner keys (K, tK); stream queries (Q, tQ | Hc, G)
-            BwdParams q = b; q.out_scale = 1.0f;
-            q.out0 = dtO ? static_cast<__nv_bfloat16*>(dtV) : nullptr; q.out1 = static_cast<__nv_bfloat16*>(dV);
-            const void* own[4] = {K, tK, K, tK};
-            const void* strm[4] = {Q, tQ, dtO, dO};
-            rc = launch_bwd_pass_dp<BWD_DV>(s, own, strm, q, *dev, st);
-            if (rc != TVM_ATTN_OK) return rc;
-        }
-        {   // dtK = alpha W^T Q, dK = alpha (dA^T Q + W^T tQ) : owner keys (K, tK, V, tV); stream (Hc, G | Q, tQ)
-            BwdParams q = b; q.out_scale = s.alpha;
-            q.out0 = dtO ? static_cast<__nv_bfloat16*>(dtK) : nullptr; q.out1 = static_cast<__nv_bfloat16*>(dK);
-            const void* own[4] = {K, tK, V, tV};
-            const void* strm[4] = {dtO, dO, Q, tQ};
-            rc = launch_bwd_pass_dp<BWD_DK>(s, own, strm, q, *dev, st);
-            if (rc != TVM_ATTN_OK) return rc;
-        }
-        {   // dtQ = alpha W K, dQ = alpha (dA K + W tK) : owner queries (Q, tQ, Hc, G); stream (V, tV | K, tK)
-            BwdParams q = b; q.out_scale = s.alpha;
-            q.out0 = dtO ? static_cast<__nv_bfloat16*>(dtQ) : nullptr; q.out1 = static_cast<__nv_bfloat16*>(dQ);
-            const void* own[4] = {Q, tQ, dtO, dO};
-            const void* strm[4] = {V, tV, K, tK};
-            rc = launch_bwd_pass_dp<BWD_DQ>(s, own, strm, q, *dev, st);
-        }
-        return rc;
-    }
     CUtensorMap maps[8];
     const void* in[8] = {Q, tQ, dtO, dO, K, tK, V, tV};
     Operand x[8];
     for (int t = 0; t < 8; ++t) {
         x[t] = {static_cast<const __nv_bfloat16*>(in[t]), in[t] ? &maps[t] : &maps[0]};
-        rc = in[t] ? make_tmap(&maps[t], in[t], s, t < 4 ? s.q : s.k, JVP_BC) : TVM_ATTN_OK;
+        rc = in[t] ? make_tmap(&maps[t], in[t], s, t < 4 ? s.q : s.k) : TVM_ATTN_OK;
         if (rc != TVM_ATTN_OK) return rc;
     }
     const Operand &xQ = x[0], &xtQ = x[1], &xH = x[2], &xG = x[3], &xK = x[4], &xtK = x[5], &xV = x[6], &xtV = x[7];
     JvpParams b;
     std::memset(&b, 0, sizeof b);
-    b.d = s.d; b.BH = (int)s.BH; b.H = s.H;
+    b.d = s.d; b.H = s.H;
     b.alpha = s.alpha; b.c2 = s.alpha * 1.4426950408889634f;
-    b.nlse2 = lse2; b.mu = mu; b.nsig1 = sig1; b.ncvec = cvec; b.status = status; b.absent = absent;
+    b.nlse2 = lse2; b.mu = mu; b.nsig1 = sig1; b.ncvec = cvec; b.status = dev->status; b.absent = absent;
     auto outputs = [&](void* tangent, void* primal, float scale) {
         b.out0 = dtO ? static_cast<__nv_bfloat16*>(tangent) : nullptr;
         b.out1 = static_cast<__nv_bfloat16*>(primal);
