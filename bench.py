@@ -28,17 +28,17 @@ METRIC = "attn_jvp_fwd_bwd_tflops"
 UNIT = "TFLOP/s"
 NOMINAL_BF16_TFLOPS = 2250.0
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
-# GEMM units (2*B*H*N^2*d FLOP each, true d) each kernel EXECUTES by design.  The backward passes recompute
-# scores: together they execute 24 units for the 15 the method counts (3 recompute + 3 cotangent-score + 9 output).
-KERNEL_GEMMS = {"fwd": 6, "bwd_rowsums": 0, "bwd_dv": 6, "bwd_dk": 9, "bwd_dq": 9}
+# GEMM units (2*B*H*N^2*d FLOP each, true d) each kernel EXECUTES by design, and the (B,H,N,d) tensors it reads + writes once
+# (its algorithmic HBM bytes, in units of one tensor).  The method counts 15 units for the backward (3 recompute +
+# 3 cotangent-score + 9 output).  Up to head dim 80 one kernel makes dK and dV and one dQ, each with scores of its own:
+# 21 units; above that dV and dK have a kernel each: 24.  Without dtO what is left is S, G V^T and one or two outputs.
+FWD_KERNEL = {"fwd": (6, 8)}
+BWD_KERNELS = {"narrow": {"bwd_rowsums": (0, 4), "bwd_dkv": (12, 12), "bwd_dq": (9, 10)},
+               "wide": {"bwd_rowsums": (0, 4), "bwd_dv": (6, 8), "bwd_dk": (9, 10), "bwd_dq": (9, 10)},
+               "detach": {"bwd_rowsums": (0, 2), "bwd_dkv": (4, 6), "bwd_dq": (3, 5)}}
 BWD_CREDITED_GEMMS = 15
-BWD_TC = ("bwd_dv", "bwd_dk", "bwd_dq")
-# (B,H,N,d) tensors each kernel reads + writes once (its algorithmic HBM bytes, in units of one tensor)
-KERNEL_TENSORS = {"fwd": 8, "bwd_rowsums": 4, "bwd_dv": 8, "bwd_dk": 10, "bwd_dq": 10}
-# dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu capture summarised in
-# profiles/jvp_fwd_bwd_kernels_dit512.md (that workload only; None for anything else, and None once a kernel
-# has changed since the capture)
-NCU_TRAFFIC_BYTES = {"dit512": {"fwd": 280.0e6, "bwd_dv": 281.5e6, "bwd_dk": 366.3e6, "bwd_dq": 363.7e6}}
+# dram__bytes_read.sum + dram__bytes_write.sum per launch from an ncu capture of the present kernels (None where there is none)
+NCU_TRAFFIC_BYTES = {}
 
 
 def load_peaks():
@@ -221,8 +221,10 @@ def main():
     detach = args.variant == "detach"
     if detach:  # standard attention backward: S recompute, dP, dV, dK, dQ = 5 GEMM units
         f_bwd = f_bwd * 5.0 / 15.0
-        KERNEL_GEMMS.update({"bwd_dv": 4, "bwd_dk": 6, "bwd_dq": 7})   # what the three passes still execute
-        KERNEL_TENSORS.update({"bwd_rowsums": 2, "bwd_dv": 6, "bwd_dk": 8, "bwd_dq": 8})
+    bwd_kernels = BWD_KERNELS["wide" if wl.d > 80 else "detach" if detach else "narrow"]
+    kernels = dict(FWD_KERNEL, **bwd_kernels)
+    kernel_gemms, kernel_tensors = {k: v[0] for k, v in kernels.items()}, {k: v[1] for k, v in kernels.items()}
+    bwd_tc = tuple(k for k in bwd_kernels if kernel_gemms[k])
     host = {k: v.to(torch.bfloat16).pin_memory() for k, v in inputs.make_inputs(wl).items()}
     x = {k: v.to(dev) for k, v in host.items()}
     shape = x["Q"].shape
@@ -294,13 +296,13 @@ def main():
 
     # per-kernel durations (CUDA events recorded by the library around each launch)
     binding.tvm_attn_set_profiling(True)
-    per_kernel = {k: [] for k in KERNEL_GEMMS}
+    per_kernel = {k: [] for k in kernel_gemms}
     for _ in range(min(args.steps, 20)):
         fwd()
         per_kernel["fwd"].append(binding.tvm_attn_get_profile()[0])
         bwd()
         prof = binding.tvm_attn_get_profile()
-        for k, v in zip(("bwd_rowsums", "bwd_dv", "bwd_dk", "bwd_dq"), prof):
+        for k, v in zip(bwd_kernels, prof):
             per_kernel[k].append(v)
     binding.tvm_attn_set_profiling(False)
     kernel_ms = {k: statistics.mean(v) for k, v in per_kernel.items() if v}
@@ -411,19 +413,19 @@ def main():
         return {"frac_of_burst_peak": tf / peaks["bf16_tflops"], "frac_of_sustained_peak": tf / peaks["bf16_tflops_sustained"],
                 "frac_of_nominal": tf / NOMINAL_BF16_TFLOPS}
 
-    # the dominant kernels: the three tensor-core passes of the backward, taken together
-    tc_ms = sum(kernel_ms[k] for k in BWD_TC)
+    # the dominant kernels: the tensor-core passes of the backward, taken together
+    tc_ms = sum(kernel_ms[k] for k in bwd_tc)
     credited_units = 5 if detach else BWD_CREDITED_GEMMS
     credited = credited_units * unit_flops / (tc_ms * 1e-3) / 1e12
-    executed = sum(KERNEL_GEMMS[k] for k in BWD_TC) * unit_flops / (tc_ms * 1e-3) / 1e12
-    tc_bytes = sum(KERNEL_TENSORS[k] for k in BWD_TC) * tensor_bytes
+    executed = sum(kernel_gemms[k] for k in bwd_tc) * unit_flops / (tc_ms * 1e-3) / 1e12
+    tc_bytes = sum(kernel_tensors[k] for k in bwd_tc) * tensor_bytes
     tc_gbs = tc_bytes / (tc_ms * 1e-3) / 1e9
     # whole-step bounds: analytic FLOP against the tensor peak, compulsory bytes (every kernel's own tensors once)
     # against the HBM peak; the larger fraction names the binding bound
-    step_bytes = sum(KERNEL_TENSORS[k] for k in kernel_ms) * tensor_bytes
+    step_bytes = sum(kernel_tensors[k] for k in kernel_ms) * tensor_bytes
     step_tensor_frac = (f_fwd + f_bwd) / (ms_step * 1e-3) / 1e12 / peak
     step_hbm_frac = step_bytes / (ms_step * 1e-3) / 1e9 / peaks["hbm_gbs"]
-    fwd_hbm_frac = KERNEL_TENSORS["fwd"] * tensor_bytes / (ms_fwd / args.steps * 1e-3) / 1e9 / peaks["hbm_gbs"]
+    fwd_hbm_frac = kernel_tensors["fwd"] * tensor_bytes / (ms_fwd / args.steps * 1e-3) / 1e9 / peaks["hbm_gbs"]
     traffic = NCU_TRAFFIC_BYTES.get(args.workload)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
@@ -444,17 +446,17 @@ def main():
         "kernels_ms": kernel_ms,
         "kernels_cycles": {k: cycles(v) for k, v in kernel_ms.items()},
         "kernels_share": {k: v / total_k for k, v in kernel_ms.items()},
-        "kernels_executed_tflops": {k: KERNEL_GEMMS[k] * unit_flops / (v * 1e-3) / 1e12 for k, v in kernel_ms.items() if KERNEL_GEMMS[k]},
+        "kernels_executed_tflops": {k: kernel_gemms[k] * unit_flops / (v * 1e-3) / 1e12 for k, v in kernel_ms.items() if kernel_gemms[k]},
         "roofline": {"bound": "tensor" if step_tensor_frac >= step_hbm_frac else "hbm",
-                     "kernel": "+".join(BWD_TC), "achieved": credited, "peak": peak, "unit": "TFLOP/s",
+                     "kernel": "+".join(bwd_tc), "achieved": credited, "peak": peak, "unit": "TFLOP/s",
                      "frac": credited / peak, "peak_source": peak_note,
                      "achieved_executed": executed, "frac_executed": executed / peak,
-                     "note": "achieved = the method's own %d GEMM units of the backward / summed duration of the three "
+                     "note": "achieved = the method's own %d GEMM units of the backward / summed duration of the "
                              "tensor-core passes; achieved_executed counts the %d units they execute (scores recomputed per pass)"
-                             % (credited_units, sum(KERNEL_GEMMS[k] for k in BWD_TC)),
+                             % (credited_units, sum(kernel_gemms[k] for k in bwd_tc)),
                      "flops_per_launch": credited_units * unit_flops,
-                     "flops_executed_per_launch": sum(KERNEL_GEMMS[k] for k in BWD_TC) * unit_flops,
-                     "traffic": None if not traffic else sum(traffic[k] for k in BWD_TC),
+                     "flops_executed_per_launch": sum(kernel_gemms[k] for k in bwd_tc) * unit_flops,
+                     "traffic": None if not traffic else sum(traffic[k] for k in bwd_tc),
                      "hbm": {"achieved": tc_gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": tc_gbs / peaks["hbm_gbs"],
                              "bytes_per_launch": tc_bytes},
                      "step": {"tensor_frac": step_tensor_frac, "hbm_frac": step_hbm_frac, "bytes": step_bytes}},

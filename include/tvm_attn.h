@@ -211,9 +211,10 @@ int tvm_attn_selftest_timeout(uint64_t limit_ns, void* cuda_stream);
  * Per-kernel timing aid (no counterpart in the paper).  While enabled, tvm_attn_jvp_fwd/bwd record
  * CUDA events on the caller's stream around every kernel they launch.  tvm_attn_get_profile waits
  * for the most recent profiled call and writes the duration in milliseconds of each of its kernels
- * to ms[0..], in launch order (forward: 1 kernel; backward: row sums, dV/dtV, dK/dtK, dQ/dtQ), and
- * returns how many it wrote (at most `capacity`), or a negative status.  Process-wide state: use
- * from one host thread at a time.  Creates CUDA events, no device memory.
+ * to ms[0..], in launch order (forward: 1 kernel; backward: row sums, dK/dtK/dV/dtV, dQ/dtQ up to
+ * head dim 80, row sums, dV/dtV, dK/dtK, dQ/dtQ above), and returns how many it wrote (at most
+ * `capacity`), or a negative status.  Process-wide state: use from one host thread at a time.
+ * Creates CUDA events, no device memory.
  */
 int tvm_attn_set_profiling(int enable);
 int tvm_attn_get_profile(float* ms, int capacity);

@@ -9,6 +9,7 @@
 //   FWD   queries     keys         S = Q K^T, Sd = tQ K^T + Q tK^T                        P~, P~ (T - c)          O~, R
 //   DV    keys        queries      S^T, Sd^T                                              P^T, (P Nn)^T           dtV, dV          (step 6)
 //   DK    keys        queries      S^T, Sd^T, D^T = V Hc^T, X^T = tV Hc^T + V G^T        W^T, dA^T               dtK/alpha, dK/alpha   (steps 2, 4)
+//   DKV   keys        queries      as DK                                                  as DV; as DK            as DV; as DK (acc2, acc3)
 //   DQ    queries     keys         S, Sd, D = Hc V^T, X = G V^T + Hc tV^T                 W, dA                   dtQ/alpha, dQ/alpha   (steps 3, 5)
 //
 //   score pair:  S = X0 Y0^T,  Sd = X1 Y0^T + X0 Y1^T        outputs:  acc0 += A0 B0,  acc1 += A1 B0 + A0 B1
@@ -16,7 +17,10 @@
 // with P = 2^(c2 S - lse2), T = alpha Sd, Nn = T - mu, W = P (D - Sigma1), dA = P (X - c) + W Nn; in the forward
 // P~ = 2^(c2 S - m) with a lazily updated row reference m, and O = O~/l, tO = R/l - (mu - c) O.
 //
-// A work item is 128 owner rows of one head, against which the other side streams in tiles of 64 rows.  The grid has
+// DKV does DV's and DK's work with one computation of the scores, and one exponential, instead of two.  Its four accumulators
+// leave tensor memory for four score blocks of 64 columns at d <= 64 and of 48 at d <= 80; above that DV and DK run on their own.
+//
+// A work item is 128 owner rows of one head, against which the other side streams in tiles of 64 rows (48).  The grid has
 // one CTA per SM (a CTA needs the whole tensor memory of one); the items go round-robin over the CTAs, and the rings,
 // the score buffers and all barrier phases run on through the items.
 //
@@ -24,7 +28,7 @@
 //   warp 0    loads the owner tiles and the E ring (stream tensors that only the score MMAs read)
 //   warp 1    issues the MMAs
 //   warp 2    loads the L ring (stream tensors the output MMAs read)
-//   warp 3    DV, DK: puts the per-query statistics into the tiles (FOLD below)
+//   warp 3    DKV: puts the per-query statistics into the tiles (FOLD below)
 //   warps 4-11   element-wise work, two groups of four warps
 //   warps 12-15  epilogue: normalise, convert and store an item's accumulators while the next item is under way
 //
@@ -38,8 +42,9 @@
 //
 // Measured on B200 at d = 128 (B 2, H 24, N 4096; one CTA per item, 32-key tiles with all four accumulators in two buffers
 // before): forward 1.40 -> 1.08 ms, DV / DK / DQ 1.33 / 2.82 / 2.92 -> 1.06 / 1.48 / 1.42 ms.  At d <= 80 (two
-// element-wise groups on alternate tiles, which also wrote the outputs, before): d = 64 (8, 16, 4096) forward 1.94 -> 1.75 ms, backward 7.37 -> 6.12 ms;
-// d = 72 (16, 16, 1024) forward 321 -> 306 us, backward 1.22 -> 1.08 ms.
+// element-wise groups on alternate tiles, which also wrote the outputs, before): d = 64 (8, 16, 4096) forward 1.94 -> 1.75 ms,
+// backward 7.37 -> 6.12 ms, with DV and DK in one pass 5.45 ms; d = 72 (16, 16, 1024) forward 321 -> 306 us, backward
+// 1.22 -> 1.08 -> 1.01 ms.
 //
 // Every wait on an mbarrier is bounded; when one gives up the block records a time-out status and all roles leave their
 // loops.
@@ -56,11 +61,11 @@
 
 namespace tvm_attn {
 
-enum : int { PASS_FWD = 0, PASS_DV = 1, PASS_DK = 2, PASS_DQ = 3 };
+enum : int { PASS_FWD = 0, PASS_DV = 1, PASS_DK = 2, PASS_DQ = 3, PASS_DKV = 4 };
 
 constexpr int JVP_THREADS = 512;
 constexpr int JVP_ROWS = 128;   // owner rows per item
-constexpr int JVP_BC = 64;      // stream rows per tile
+constexpr int JVP_BC = 64;      // stream rows per tile (DKV at padded head dim 80: 48)
 // Forward, how far the row reference m may lag behind the running maximum (log2 units), and for WIDE head dims how far the
 // centre c of the tangent weights may be from T at the arg-max key before it moves.
 constexpr float JVP_LAZY_LOG2 = 3.0f, JVP_LAZY_LOG2_WIDE = 8.0f, JVP_CENTRE_WIDE = 3.0f;
@@ -72,14 +77,16 @@ constexpr int JVP_REGS = 128;
 struct JvpParams {
     int d, H;
     int items, row_tiles, T;   // work items (128 owner rows of a head), items per head, stream tiles per item
-    Geom o, s;    // owner side and stream side of this pass (FWD, DQ: queries own, keys stream; DV, DK: the other way round)
+    Geom o, s;    // owner side and stream side of this pass (FWD, DQ: queries own, keys stream; DV, DK, DKV: the other way round)
     float alpha;      // softmax scale
     float c2;         // alpha * log2(e)
     float out_scale;  // factor applied to acc0 / acc1 of the backward passes
-    const __nv_bfloat16* own[4];   // owner tensors X0..X3 (X2, X3: DK, DQ)
+    const __nv_bfloat16* own[4];   // owner tensors X0..X3 (X2, X3: DK, DKV, DQ)
     const __nv_bfloat16* strm[4];  // streamed tensors: E ring (0, 1), L ring (2, 3)
     __nv_bfloat16* out0;           // acc0 destination: O | dtV | dtK | dtQ
     __nv_bfloat16* out1;           // acc1 destination: tO | dV | dK | dQ
+    __nv_bfloat16* out2;           // DKV: dtK
+    __nv_bfloat16* out3;           //      dK
     float* lse;                    // FWD: statistics written, packed (B, H, M)
     float* mu_out;
     // backward: statistics read, packed (B, H, M); the pre-pass writes the negated ones
@@ -97,9 +104,11 @@ struct JvpParams {
 template <int MODE, int DP>
 struct JvpCfg {
     static_assert(DP % 16 == 0 && DP >= 16 && DP <= 128, "padded head dim must be 16..128");
-    static constexpr int NPAIR = MODE == PASS_DK || MODE == PASS_DQ ? 2 : 1;   // score pairs
-    static constexpr bool TRANSPOSED = MODE == PASS_DV || MODE == PASS_DK;     // owner rows are keys
-    static constexpr int BC = JVP_BC, KS = DP / 16;
+    static constexpr bool DKV = MODE == PASS_DKV;
+    static constexpr int NPAIR = MODE == PASS_FWD || MODE == PASS_DV ? 1 : 2;  // score pairs
+    static constexpr bool TRANSPOSED = MODE != PASS_FWD && MODE != PASS_DQ;    // owner rows are keys
+    // Stream rows per tile.  Four accumulators of DP columns and four of BC have to fit into 512.
+    static constexpr int BC = DKV && DP > 64 ? 48 : JVP_BC, KS = DP / 16;
     static constexpr int NA = DP > 64 ? 2 : 1;             // 64-column swizzle atoms per row
     // How the columns from 64 on arrive.  Up to 16 of them (DP = 80): 16-byte asynchronous copies, because a 64-column
     // box hanging over the end of a 144-byte row reads the next row from L2 for nothing; tiles that are only read
@@ -107,23 +116,26 @@ struct JvpCfg {
     // than 16 (WIDE): a second box and a second swizzle atom everywhere.
     static constexpr bool WIDE = DP > 80;
     static constexpr bool TAIL = NA == 2 && !WIDE;
+    static_assert(WIDE || (MODE != PASS_DV && MODE != PASS_DK), "DV and DK on their own: only where DKV does not fit");
+    static_assert(!WIDE || !DKV, "DKV: four accumulators do not fit");
+    static constexpr bool E_MN = DKV;                      // the E ring is read MN-major too: swizzled atoms like the L ring's
     // Owner operands.  The pair of the score MMAs on the tile's critical chain (FWD, DV: the only pair; DK, DQ: the second)
     // lies in tensor memory as bf16 A operands: an MMA with A in shared memory moves 4 KB of A per k-step through the
-    // shared-memory port.  WIDE: tensor memory has no room, everything is in shared memory.
-    static constexpr bool XT = !WIDE;
+    // shared-memory port.  WIDE, DKV: tensor memory has no room, everything is in shared memory.
+    static constexpr bool XT = !WIDE && !DKV;
     static constexpr int NOWN = 2 * NPAIR - (XT ? 2 : 0);   // owner tensors in shared memory
-    // FOLD (DV, DK): the per-query statistics belong to the columns of the tile, the same for every thread; read from
+    // FOLD (DKV): the per-query statistics belong to the columns of the tile, the same for every thread; read from
     // shared memory they would cost 512 bytes a warp and column.  Instead they are an extra piece of the score MMAs: each
     // is split into three bf16 parts in columns of its own behind the stream row, against ones behind the owner row, so
     // that the accumulators arrive as S - lse/alpha, Sd - mu/alpha, D - Sigma1, X - c.  At d = 72 these columns are the
     // padding up to 80; other head dims take one more k-step of N = 128.
-    static constexpr bool FOLD = TRANSPOSED && !WIDE;
+    static constexpr bool FOLD = DKV;
     static constexpr int OWN_ATOM = JVP_ROWS * 128, ATOM = BC * 128;
     static constexpr int OWN_BYTES = OWN_ATOM * (WIDE ? 2 : 1) + (TAIL ? JVP_ROWS * 32 : 0);   // one owner tensor
-    static constexpr int EST_BYTES = ATOM * (WIDE ? 2 : 1) + (TAIL ? BC * 32 : 0);             // one E-ring tile
+    static constexpr int EST_BYTES = E_MN ? ATOM * NA : ATOM * (WIDE ? 2 : 1) + (TAIL ? BC * 32 : 0);   // one E-ring tile
     static constexpr int LST_BYTES = ATOM * NA;                                                // one L-ring tile
-    static constexpr int SE = WIDE ? (NPAIR == 2 ? 1 : 2) : TAIL ? 3 : 4;
-    static constexpr int SL = WIDE ? 2 : TAIL && NPAIR == 2 ? 3 : 4;
+    static constexpr int SE = WIDE ? (NPAIR == 2 ? 1 : 2) : DKV ? (TAIL ? 2 : 3) : TAIL ? 3 : 4;
+    static constexpr int SL = WIDE ? 2 : DKV ? (TAIL ? 3 : 4) : TAIL && NPAIR == 2 ? 3 : 4;
     static constexpr int TILE_BYTES = NOWN * OWN_BYTES + SE * 2 * EST_BYTES + SL * 2 * LST_BYTES;
     // FOLD: statistics of a stage, [Y0 rows, Y1 rows][16 bytes], for the rings the score MMAs read; ones and zeros
     static constexpr int FOLD_BYTES = 2 * BC * 16;
@@ -131,11 +143,13 @@ struct JvpCfg {
     static constexpr int ONES_BYTES = FOLD ? JVP_ROWS * 32 : 0;
     static constexpr int EFULL_COUNT = 1 + (TAIL ? 32 : 0) + (FOLD_E ? 1 : 0);   // TMA issuer, each lane's own copies, warp 3
     static constexpr int LFULL_COUNT = 1 + (TAIL || (TRANSPOSED && !FOLD) ? 32 : 0) + (FOLD_L ? 1 : 0);
-    // TMEM columns: accumulators, the owner operands in the gaps behind them (and 8 columns of ones behind the first),
+    // TMEM columns: accumulators, the owner operands in the gaps behind them,
     // score accumulators (FWD, DV: two buffers of S | Sd; DK, DQ: one of S | Sd | D | X).
-    static constexpr int COL_ACC0 = 0, COL_ACC1 = XT ? 128 : DP, COL_SCORE = 2 * COL_ACC1;
-    static constexpr int COL_X0 = DP, COL_X1 = COL_ACC1 + DP, COL_ONES = COL_X0 + DP / 2;
-    static_assert(!XT || DP + DP / 2 + 8 <= 128, "operands do not fit behind their accumulators");
+    static constexpr int NACC = DKV ? 4 : 2;
+    static constexpr int KLO = BC / 32;                    // k-steps of an output in its first part
+    static constexpr int COL_ACC0 = 0, COL_ACC1 = XT ? 128 : DP, COL_SCORE = NACC * COL_ACC1;
+    static constexpr int COL_X0 = DP, COL_X1 = COL_ACC1 + DP;
+    static_assert(!XT || DP + DP / 2 <= 128, "operands do not fit behind their accumulators");
     static_assert(COL_SCORE + 4 * BC <= 512, "TMEM over-subscribed");
     // registers per thread: warpgroup 0, element-wise warps, epilogue warps (which hold an owner row, 4 registers a chunk)
     static constexpr int REGS_LOAD = MODE == PASS_FWD ? 56 : 96, REGS_ELEM = MODE == PASS_FWD ? 184 : 152, REGS_EPI = MODE == PASS_FWD ? 88 : 112;
@@ -154,10 +168,11 @@ struct JvpCfg {
     static constexpr int B_SFULL = B_XFREE + 1;                        // S (and Sd, except in FWD) written
     static constexpr int B_XFULL = B_SFULL + 4;                        // FWD: Sd written; DK, DQ: D, X written
     static constexpr int B_OUTDONE = B_XFULL + 4;                      // output MMAs complete
-    static constexpr int B_EDONE = MODE == PASS_DV ? B_SFULL : B_XFULL;   // the E stage of the tile is free
+    static constexpr int B_O1DONE = B_OUTDONE + 4;                     // DKV: ... of the first pair (OUTDONE: of the second)
+    static constexpr int B_EDONE = DKV ? B_O1DONE : MODE == PASS_DV ? B_SFULL : B_XFULL;   // the E stage of the tile is free
     static_assert(SE <= 4 && SL <= 4, "a ring deeper than the completion barriers");
-    // operands written: + half of the tile (DK, DQ), + 2 (g & 1) + half (FWD, DV)
-    static constexpr int B_PREADY = B_OUTDONE + 4;
+    // operands written: + half of the tile (DK, DQ), + 2 (g & 1) + half (FWD, DV), + 2 pair + part (DKV)
+    static constexpr int B_PREADY = B_O1DONE + 4;
     static constexpr int B_SREAD = B_PREADY + 4;                       // DK, DQ: S, Sd read
     static constexpr int B_FINAL = B_SREAD + 1;                        // the item's last output MMAs complete
     static constexpr int B_ACCFREE = B_FINAL + 1;                      // the epilogue has read the accumulators
@@ -303,13 +318,14 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
     const uint32_t ring_base = k.base + (RING == 0 ? k.E : k.L);
     const __nv_bfloat16* base0 = p.strm[2 * RING];
     const __nv_bfloat16* base1 = p.strm[2 * RING + 1];
-    // the ring that streams the cotangents (Hc, G): L in DV, E in DK; an absent one is not loaded
-    constexpr bool COT = (MODE == PASS_DV && RING == 1) || (MODE == PASS_DK && RING == 0);
+    // the ring that streams the cotangents (Hc, G): L in DV, E in DK and DKV; an absent one is not loaded
+    constexpr bool COT = (MODE == PASS_DV && RING == 1) || ((MODE == PASS_DK || C::DKV) && RING == 0);
     const bool has0 = !COT || !(p.absent & ABSENT_HC), has1 = !COT || !(p.absent & ABSENT_G);
     const uint32_t tx_bytes = ((has0 ? 1 : 0) + (has1 ? 1 : 0)) * ATOM * (C::WIDE ? 2 : 1);
     // Chunk 0 of row `lane` behind the first atoms: compact blocks in the E ring, a second swizzled atom in the L ring.
     [[maybe_unused]] const uint32_t sw = lane & 7;  // rows 32 apart share it
-    [[maybe_unused]] const uint32_t dst_lane = 2 * ATOM + (RING == 0 ? lane * 16 : lane * 128);
+    constexpr bool FLAT = RING == 0 && !C::E_MN;
+    [[maybe_unused]] const uint32_t dst_lane = 2 * ATOM + (FLAT ? lane * 16 : lane * 128);
     // statistics as they are: 16-byte chunks when the rows of the (B, H, M) arrays are 16-byte aligned, else floats
     [[maybe_unused]] const bool st16 = (p.s.rows & 3) == 0;
     [[maybe_unused]] const uint32_t st_base = k.base + k.STATS;
@@ -376,18 +392,20 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
             }
             if constexpr (C::TAIL) {
                 const uint32_t d0 = stage + dst_lane;
-                constexpr uint32_t T1 = RING == 0 ? BC * 16 : ATOM, R1 = RING == 0 ? 32 * 16 : 32 * 128;   // second tensor, second 32 rows
+                constexpr uint32_t T1 = FLAT ? BC * 16 : ATOM, R1 = FLAT ? 32 * 16 : 32 * 128;   // second tensor, second 32 rows
+                const bool hi = BC == 64 || lane < BC - 32;   // the lane has a second row
 #pragma unroll
                 for (int c = 0; c < KT; ++c) {
                     if (c < ntail) {
-                        const uint32_t dst = d0 + (RING == 0 ? c * 2 * BC * 16 : (c ^ sw) << 4);
+                        const uint32_t dst = d0 + (FLAT ? c * 2 * BC * 16 : (c ^ sw) << 4);
                         if (__builtin_expect(rows_left >= BC, 1)) {
-                            if (has0) { ptx::cp_async_16(dst, src0 + 8 * c); ptx::cp_async_16(dst + R1, src0 + d32 + 8 * c); }
-                            if (has1) { ptx::cp_async_16(dst + T1, src1 + 8 * c); ptx::cp_async_16(dst + T1 + R1, src1 + d32 + 8 * c); }
+                            if (has0) { ptx::cp_async_16(dst, src0 + 8 * c); if (hi) ptx::cp_async_16(dst + R1, src0 + d32 + 8 * c); }
+                            if (has1) { ptx::cp_async_16(dst + T1, src1 + 8 * c); if (hi) ptx::cp_async_16(dst + T1 + R1, src1 + d32 + 8 * c); }
                         } else {
 #pragma unroll
                             for (int rp = 0; rp < 2; ++rp) {
                                 const bool v = lane + 32 * rp < rows_left;
+                                if (rp == 1 && !hi) continue;
                                 if (has0) ptx::cp_async_16(dst + rp * R1, v ? src0 + rp * d32 + 8 * c : base0, v ? 16u : 0u);
                                 if (has1) ptx::cp_async_16(dst + rp * R1 + T1, v ? src1 + rp * d32 + 8 * c : base1, v ? 16u : 0u);
                             }
@@ -430,8 +448,8 @@ __device__ __forceinline__ void jvp_split3(float a, float b, uint2& pa, uint2& p
     pb = make_uint2(__byte_perm(h, m, 0x7632), l >> 16);
 }
 
-// Warp 3: the statistics of the stream rows lane and lane + 32 of a tile, for the E ring (DV: lse, mu; DK: Sigma1, c) and the
-// L ring (DK: lse, mu), loaded one tile ahead.
+// Warp 3: the statistics of the stream rows lane and lane + 32 of a tile, for the L ring (lse, mu) and the E ring (Sigma1, c),
+// loaded one tile ahead.
 template <int MODE, int DP>
 __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE, DP>& shared, int lane) {
     using C = JvpCfg<MODE, DP>;
@@ -443,8 +461,8 @@ __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE
     const uint32_t sw = lane & 7;
     const bool own = k.fold_step();
     const Dst de = own ? Dst{k.base + k.FOLD_E + lane * 16, (uint32_t)C::FOLD_BYTES, BC * 16, 32 * 16}
-                       : Dst{k.base + k.E + 2 * C::ATOM + 2 * BC * 16 + lane * 16, 2u * C::EST_BYTES, BC * 16, 32 * 16};
-    [[maybe_unused]] const Dst dl = own ? Dst{k.base + k.FOLD_L + lane * 16, (uint32_t)C::FOLD_BYTES, BC * 16, 32 * 16}
+                       : Dst{k.base + k.E + 2 * C::ATOM + lane * 128 + ((1 ^ sw) << 4), 2u * C::EST_BYTES, C::ATOM, 32 * 128};
+    const Dst dl = own ? Dst{k.base + k.FOLD_L + lane * 16, (uint32_t)C::FOLD_BYTES, BC * 16, 32 * 16}
                                         : Dst{k.base + k.L + 2 * C::ATOM + lane * 128 + ((1 ^ sw) << 4), 2u * C::LST_BYTES, C::ATOM, 32 * 128};
     const float f_lse = 1.0f / p.c2, f_mu = -1.0f / p.alpha;   // to the scale of S and Sd
     float a[4], b[4];   // (statistic of tensor 0, of tensor 1) of the two rows: lse, mu | Sigma1, c
@@ -456,10 +474,8 @@ __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE
             const bool v = left > 32 * r;
             a[2 * r] = v ? __ldg(p.nlse2 + at + 32 * r) : 0.f;
             a[2 * r + 1] = v ? __ldg(p.mu + at + 32 * r) : 0.f;
-            if (C::NPAIR == 2) {
-                b[2 * r] = v ? __ldg(p.nsig1 + at + 32 * r) : 0.f;
-                b[2 * r + 1] = v ? __ldg(p.ncvec + at + 32 * r) : 0.f;
-            }
+            b[2 * r] = v ? __ldg(p.nsig1 + at + 32 * r) : 0.f;
+            b[2 * r + 1] = v ? __ldg(p.ncvec + at + 32 * r) : 0.f;
         }
     };
     auto put = [&](const Dst& d, int stage, int full, float x0, float x1, float y0, float y1) {
@@ -468,9 +484,11 @@ __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE
         jvp_split3(x0, x1, u, v);
         ptx::st_shared_v4(at, u.x, u.y, 0u, 0u);
         ptx::st_shared_v4(at + d.t_step, v.x, v.y, 0u, 0u);
-        jvp_split3(y0, y1, u, v);
-        ptx::st_shared_v4(at + d.r_step, u.x, u.y, 0u, 0u);
-        ptx::st_shared_v4(at + d.t_step + d.r_step, v.x, v.y, 0u, 0u);
+        if (BC == 64 || lane < BC - 32) {   // the lane has a second row
+            jvp_split3(y0, y1, u, v);
+            ptx::st_shared_v4(at + d.r_step, u.x, u.y, 0u, 0u);
+            ptx::st_shared_v4(at + d.t_step + d.r_step, v.x, v.y, 0u, 0u);
+        }
         ptx::fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(k.bar(full + stage));
@@ -480,14 +498,11 @@ __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE
     for (int item = blockIdx.x; item < p.items; item += gridDim.x) {
         const int bh = item / p.row_tiles, next = item + (int)gridDim.x;
         for (int j = 0; j < T; ++j, ++g) {
-            if (C::NPAIR == 2) {
-                if (g >= C::SL && !k.done(C::B_OUTDONE, g - C::SL)) return;
-                put(dl, sl, C::B_LFULL, a[0] * f_lse, a[1] * f_mu, a[2] * f_lse, a[3] * f_mu);
-                if (++sl == C::SL) sl = 0;
-            }
+            if (g >= C::SL && !k.done(C::B_OUTDONE, g - C::SL)) return;
+            put(dl, sl, C::B_LFULL, a[0] * f_lse, a[1] * f_mu, a[2] * f_lse, a[3] * f_mu);
+            if (++sl == C::SL) sl = 0;
             if (g >= C::SE && !k.done(C::B_EDONE, g - C::SE)) return;
-            if (C::NPAIR == 2) put(de, se, C::B_EFULL, b[0], b[1], b[2], b[3]);
-            else put(de, se, C::B_EFULL, a[0] * f_lse, a[1] * f_mu, a[2] * f_lse, a[3] * f_mu);
+            put(de, se, C::B_EFULL, b[0], b[1], b[2], b[3]);
             if (++se == C::SE) se = 0;
             const bool more = j + 1 < T;
             if (more || next < p.items) load(more ? bh : next / p.row_tiles, more ? j + 1 : 0);
@@ -533,12 +548,13 @@ struct JvpIssue {
     static __device__ __forceinline__ JvpSlot l_slot(const Block& k) { return JvpSlot(ptx::desc_lo(k.base + k.L, 16), ptx::desc_lo(k.base + k.FOLD_L, k.ZEROS - k.FOLD_L)); }
 
     static __host__ __device__ constexpr bool is_tail(int kk) { return C::TAIL && kk >= 4; }
+    static __host__ __device__ constexpr bool flat(bool from_l, int kk) { return is_tail(kk) && !from_l && !C::E_MN; }   // an unswizzled tail
     // k-step kk of a K-major operand, relative to its tile or stage: owner tile | E stage (rows of Y0, then Y1) | L stage
     static __host__ __device__ constexpr uint32_t own_k(int kk) {
         return kk < 4 ? 2u * kk : C::WIDE ? ((uint32_t)C::OWN_ATOM >> 4) + 2u * (kk - 4) : ((uint32_t)C::OWN_ATOM >> 4) + lbo(JVP_ROWS * 16);
     }
     static __host__ __device__ constexpr uint32_t e_k(int kk) {
-        return kk < 4 ? 2u * kk : C::WIDE ? (2u * ATOM >> 4) + 2u * (kk - 4) : (2u * ATOM >> 4) + lbo(2 * BC * 16);
+        return C::E_MN ? l_k(kk) : kk < 4 ? 2u * kk : C::WIDE ? (2u * ATOM >> 4) + 2u * (kk - 4) : (2u * ATOM >> 4) + lbo(2 * BC * 16);
     }
     static __host__ __device__ constexpr uint32_t l_k(int kk) { return (uint32_t)((kk >> 2) * 2 * ATOM >> 4) + 2u * (kk & 3); }
     // L stage read MN-major by the output MMAs (tensor t): atoms of 64 d-columns are 2 * ATOM bytes apart, 8-row groups
@@ -552,27 +568,25 @@ struct JvpIssue {
         else ptx::mma_ss_p<ACC>(el, col, a + own_k(kk), is_tail(kk) ? HI_TAIL : HI_SW, b, bhi, idesc);
     }
     // The statistics' own k-step (FOLD, where the padding columns do not hold them), tensor t0 on.
-    template <bool ATM>
     static __device__ __forceinline__ void fold_step(uint32_t el, uint32_t col, const Block& k, uint32_t fold, int t0, uint32_t idesc) {
         const uint32_t b = fold + (uint32_t)(t0 * BC * 16 >> 4) - ((uint32_t)(t0 * BC * 16 >> 4) << 16);
-        if (ATM) ptx::mma_ts_p<1>(el, col, C::COL_ONES, b, HI_TAIL, idesc);
-        else ptx::mma_ss_p<1>(el, col, ptx::desc_lo(k.base + k.ONES, JVP_ROWS * 16), HI_TAIL, b, HI_TAIL, idesc);
+        ptx::mma_ss_p<1>(el, col, ptx::desc_lo(k.base + k.ONES, JVP_ROWS * 16), HI_TAIL, b, HI_TAIL, idesc);
     }
     // [S | X0 Y1^T] = X0 [Y0 | Y1]^T, Sd += X1 Y0^T at column col; FROM_L: the stage is one of the L ring.
     template <bool FROM_L, bool ATM, bool SECOND>
     static __device__ __forceinline__ void pair(uint32_t el, uint32_t col, const Block& k, uint32_t a0, uint32_t a1, uint32_t lo, uint32_t fold, uint32_t mid_bar) {
 #pragma unroll
         for (int kk = 0; kk < KS; ++kk) {
-            const uint32_t b = lo + (FROM_L ? l_k(kk) : e_k(kk)), bhi = !FROM_L && is_tail(kk) ? HI_TAIL : HI_SW;
+            const uint32_t b = lo + (FROM_L ? l_k(kk) : e_k(kk)), bhi = flat(FROM_L, kk) ? HI_TAIL : HI_SW;
             if (kk == 0) step<ATM, 0>(el, col, a0, kk, b, bhi, I_S2);
             else step<ATM, 1>(el, col, a0, kk, b, bhi, I_S2);
         }
-        if (k.fold_step()) fold_step<ATM>(el, col, k, fold, 0, I_S2);
+        if (k.fold_step()) fold_step(el, col, k, fold, 0, I_S2);
         if (MODE == PASS_FWD) ptx::mma_commit_p(el, mid_bar);   // S is complete before Sd
         if (SECOND) {
 #pragma unroll
             for (int kk = 0; kk < KS; ++kk)
-                step<ATM, 1>(el, col + BC, a1, kk, lo + (FROM_L ? l_k(kk) : e_k(kk)), !FROM_L && is_tail(kk) ? HI_TAIL : HI_SW, I_S);
+                step<ATM, 1>(el, col + BC, a1, kk, lo + (FROM_L ? l_k(kk) : e_k(kk)), flat(FROM_L, kk) ? HI_TAIL : HI_SW, I_S);
         }
     }
     // One product X Y^T with Y the T-th tensor of the stage.
@@ -580,12 +594,12 @@ struct JvpIssue {
     static __device__ __forceinline__ void single(uint32_t el, uint32_t col, const Block& k, uint32_t a, uint32_t lo, uint32_t fold) {
 #pragma unroll
         for (int kk = 0; kk < KS; ++kk) {
-            const bool tail = !FROM_L && is_tail(kk);
+            const bool tail = flat(FROM_L, kk);
             const uint32_t b = lo + (FROM_L ? l_k(kk) : e_k(kk)) + ((uint32_t)(tail ? T * BC * 16 : T * ATOM) >> 4);
             if (kk == 0) step<ATM, 0>(el, col, a, kk, b, tail ? HI_TAIL : HI_SW, I_S);
             else step<ATM, 1>(el, col, a, kk, b, tail ? HI_TAIL : HI_SW, I_S);
         }
-        if (k.fold_step()) fold_step<ATM>(el, col, k, fold, T, I_S);
+        if (k.fold_step()) fold_step(el, col, k, fold, T, I_S);
     }
     // Half of acc0 += A0 B0, acc1 += A1 B0 + A0 B1 (k-steps U0, U0 + 1 of four; the operand of a k-step lies at the columns of
     // the scores it replaces); the terms of an absent tensor are left out.  acc = 0: the accumulators are overwritten.
@@ -603,7 +617,93 @@ struct JvpIssue {
             if (T2) { if (u == 0 && !T1) ptx::mma_ts_acc(el, c1, a0, b1, HI_SW, I_O, acc); else ptx::mma_ts_p<1>(el, c1, a0 + 16 * u, b1, HI_SW, I_O); }
         }
     }
+    // DKV: k-steps U0 .. U1 - 1 of acc[C] += A0 B0, acc[C + 1] += A1 B0 + A0 B1 (T0, T1, T2: which of the three there are).
+    template <int U0, int U1, bool T0, bool T1, bool T2, int ACC>
+    static __device__ __forceinline__ void dkv_outputs(uint32_t el, uint32_t a0, uint32_t a1, uint32_t lo, uint32_t acc) {
+        constexpr uint32_t c0 = ACC * DP, c1 = c0 + DP;
+#pragma unroll
+        for (int u = U0; u < U1; ++u) {
+            const uint32_t b0 = lo + l_n(0, u), b1 = lo + l_n(1, u), o = 16u * u;
+            if (T0) { if (u == 0) ptx::mma_ts_acc(el, c0, a0, b0, HI_SW, I_O, acc); else ptx::mma_ts_p<1>(el, c0, a0 + o, b0, HI_SW, I_O); }
+            if (T1) { if (u == 0) ptx::mma_ts_acc(el, c1, a1, b0, HI_SW, I_O, acc); else ptx::mma_ts_p<1>(el, c1, a1 + o, b0, HI_SW, I_O); }
+            if (T2) { if (u == 0 && !T1) ptx::mma_ts_acc(el, c1, a0, b1, HI_SW, I_O, acc); else ptx::mma_ts_p<1>(el, c1, a0 + o, b1, HI_SW, I_O); }
+        }
+    }
 };
+
+// DKV: one buffer of (S, Sd | D, X), operands written over the scores.  Pipe order: outputs of the first pair (P, P Nn)(n - 1) |
+// (S, Sd)(n) | outputs of the second pair (W, dA)(n - 1) | (D, X)(n): what the element-wise warps do to one pair runs under
+// the MMAs of the other, so that no unit waits for the whole chain of a tile.  (d = 64, per 64 queries: MMAs of 1860 cycles
+// instead of 2250 in two passes, half the exponentials and loads.)
+template <int MODE, int DP, bool HZ, int ABS>
+__device__ __forceinline__ void jvp_issue_dkv(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
+    using C = JvpCfg<MODE, DP>;
+    using I = JvpIssue<MODE, DP, HZ, ABS>;
+    constexpr int NU = C::BC / 16, LO = C::KLO, BC = C::BC;   // k-steps of an output; those of its first part
+    const JvpBlock<MODE, DP> k = shared.pinned();
+    const int T = jvp_pin(p.T), items = jvp_pin(p.items);
+    const uint32_t x0 = ptx::desc_lo(k.own_tile(0), 16), x1 = ptx::desc_lo(k.own_tile(1), 16);
+    const uint32_t x2 = ptx::desc_lo(k.own_tile(2), 16), x3 = ptx::desc_lo(k.own_tile(3), 16);
+    constexpr uint32_t cS = C::COL_SCORE, cT = cS + BC, cD = cS + 2 * BC, cX = cS + 3 * BC;
+    constexpr bool H = !HZ && !(ABS & ABSENT_HC), G = !(ABS & ABSENT_G);
+    JvpSlot e = I::e_slot(k), l = I::l_slot(k);   // next tile of the scores
+    uint32_t elo = e.lo, llo = l.lo;              // stages of the outputs' tile
+    int n = 0, it = 0;                            // next tile whose scores are issued
+    bool ready = false;
+    for (int item = blockIdx.x; item < items; item += gridDim.x, ++it) {
+        if (!k.wait(C::B_OWN, it)) return;
+        for (int j = -1; j < T; ++j) {
+            const uint32_t acc = j > 0 ? 1u : 0u;
+            if (j >= 0) {   // dtV += P^T Hc, dV += (P Nn)^T Hc + P^T G
+                if (!k.wait(C::B_PREADY, n - 1)) return;
+                if (j == 0 && !k.wait(C::B_ACCFREE, it - 1)) return;    // the first tile overwrites the accumulators
+                ptx::tc_fence_after_sync();
+                uint32_t el = ptx::elect_one();
+                I::template dkv_outputs<0, LO, H, H, G, 0>(el, cS, cT, elo, acc);
+                if (!k.wait(C::B_PREADY + 1, n - 1)) return;
+                ptx::tc_fence_after_sync();
+                el = ptx::elect_one();
+                I::template dkv_outputs<LO, NU, H, H, G, 0>(el, cS, cT, elo, acc);
+                ptx::mma_commit_p(el, k.bar(C::B_O1DONE + ((n - 1) & 3)));
+                elo = elo + I::E_STEP == e.lo0 + C::SE * I::E_STEP ? e.lo0 : elo + I::E_STEP;
+            }
+            if (j + 1 < T) {   // (S, Sd) of the next tile
+                if (!k.wait(C::B_LFULL + l.s, l.ph)) return;
+                k.tile_fence();
+                const uint32_t el = ptx::elect_one();
+                if (HZ) I::template single<true, false, 0>(el, cS, k, x0, l.lo, l.fold);
+                else I::template pair<true, false, true>(el, cS, k, x0, x1, l.lo, l.fold, 0);
+                ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
+                l.template next<C::SL, I::L_STEP, I::F_STEP>();
+                ready = ptx::mbar_test_warp(k.bar(C::B_EFULL + e.s), e.ph);
+            }
+            if (j >= 0) {   // dtK += W^T Q, dK += dA^T Q + W^T tQ
+                if (!k.wait(C::B_PREADY + 2, n - 1)) return;
+                ptx::tc_fence_after_sync();
+                uint32_t el = ptx::elect_one();
+                I::template dkv_outputs<0, LO, H, true, H, 2>(el, cD, cX, llo, acc);
+                if (!k.wait(C::B_PREADY + 3, n - 1)) return;
+                ptx::tc_fence_after_sync();
+                el = ptx::elect_one();
+                I::template dkv_outputs<LO, NU, H, true, H, 2>(el, cD, cX, llo, acc);
+                ptx::mma_commit_p(el, k.bar(C::B_OUTDONE + ((n - 1) & 3)));
+                if (j == T - 1) ptx::mma_commit_p(el, k.bar(C::B_FINAL));
+                llo = llo + I::L_STEP == l.lo0 + C::SL * I::L_STEP ? l.lo0 : llo + I::L_STEP;
+            }
+            if (j + 1 < T) {   // (D, X) of the next tile
+                if (!ready && !k.wait(C::B_EFULL + e.s, e.ph)) return;
+                k.tile_fence();
+                const uint32_t el = ptx::elect_one();
+                if (HZ) I::template single<false, false, 1>(el, cX, k, x2, e.lo, e.fold);   // X = V G^T alone
+                else I::template pair<false, false, H>(el, cD, k, x2, x3, e.lo, e.fold, 0);  // (tV Hc^T is zero with Hc absent)
+                ptx::mma_commit_p(el, k.bar(C::B_XFULL + (n & 3)));
+                if (j + 2 == T) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE));
+                e.template next<C::SE, I::E_STEP, I::F_STEP>();
+                ++n;
+            }
+        }
+    }
+}
 
 // FWD, DV: two score buffers taken in turn, operands written over the scores; pipe order S(0), S(1), out(0), S(2), out(1), ...:
 // S(n + 1) overwrites what out(n - 1) reads, and the pipe keeps the order.
@@ -726,7 +826,8 @@ __device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const Jv
 // Which cotangent is absent is decided here, once.
 template <int MODE, int DP, bool HZ, int ABS>
 __device__ __forceinline__ void jvp_issue_abs(const JvpParams& p, const JvpBlock<MODE, DP>& k) {
-    if constexpr (JvpCfg<MODE, DP>::NPAIR == 1) jvp_issue_one_pair<MODE, DP, HZ, ABS>(p, k);
+    if constexpr (MODE == PASS_DKV) jvp_issue_dkv<MODE, DP, HZ, ABS>(p, k);
+    else if constexpr (JvpCfg<MODE, DP>::NPAIR == 1) jvp_issue_one_pair<MODE, DP, HZ, ABS>(p, k);
     else jvp_issue_two_pairs<MODE, DP, HZ, ABS>(p, k);
 }
 template <int MODE, int DP, bool HZ>
@@ -896,7 +997,7 @@ __device__ __forceinline__ void jvp_elem_fwd(const JvpParams& p, const JvpBlock<
     }
 }
 
-// DV: P, P Nn from (S, Sd), written over them.  FOLD: the statistics are in the scores already.
+// DV: P, P Nn from (S, Sd), written over them.
 template <int DP, bool HZ>
 __device__ __forceinline__ void jvp_elem_dv(const JvpParams& p, const JvpBlock<PASS_DV, DP>& k, int grp, int q, int lane) {
     using C = JvpCfg<PASS_DV, DP>;
@@ -908,32 +1009,33 @@ __device__ __forceinline__ void jvp_elem_dv(const JvpParams& p, const JvpBlock<P
         const int b = g & 1;
         const uint32_t sb = sb0 + b * 2 * BC;
         if (!k.done(C::B_SFULL, g)) return;
-        if (!C::FOLD && !k.wait(C::B_LFULL + g % C::SL, g / C::SL)) return;   // the tile's statistics
+        if (!k.wait(C::B_LFULL + g % C::SL, g / C::SL)) return;   // the tile's statistics
         ptx::tc_fence_after_sync();
         uint32_t s[HC], t[HC];
         ptx::tmem_ld32(sb, s);
         if (!HZ) ptx::tmem_ld32(sb + BC, t);
         ptx::tmem_wait_ld();
-        const float* st = C::FOLD ? nullptr : k.stats(g % C::SL) + grp * HC;
+        const float* st = k.stats(g % C::SL) + grp * HC;
 #pragma unroll
         for (int u = 0; u < HC / 16; ++u) {
             uint32_t pa0[8], pa1[8];
 #pragma unroll
             for (int c = 0; c < 16; c += 4) {
                 const int cc = 16 * u + c;
-                [[maybe_unused]] ulonglong2 l4, m4;
-                if (!C::FOLD) l4 = *reinterpret_cast<const ulonglong2*>(st + cc);
-                if (!C::FOLD && !HZ) m4 = *reinterpret_cast<const ulonglong2*>(st + BC + cc);
+                ulonglong2 l4;
+                [[maybe_unused]] ulonglong2 m4;
+                l4 = *reinterpret_cast<const ulonglong2*>(st + cc);
+                if (!HZ) m4 = *reinterpret_cast<const ulonglong2*>(st + BC + cc);
 #pragma unroll
                 for (int e = 0; e < 4; e += 2) {
                     const uint64_t s2 = ptx::pack2u(s[cc + e], s[cc + e + 1]);
                     float x0, x1;
-                    ptx::unpack2(C::FOLD ? ptx::mul2(s2, c2c2) : ptx::fma2(s2, c2c2, e ? l4.y : l4.x), x0, x1);
+                    ptx::unpack2(ptx::fma2(s2, c2c2, e ? l4.y : l4.x), x0, x1);
                     const float p0 = ptx::ex2(x0), p1 = ptx::ex2(x1);
                     pa0[(c + e) >> 1] = ptx::pack_bf16(p0, p1);
                     if (!HZ) {
                         const uint64_t t2 = ptx::pack2u(t[cc + e], t[cc + e + 1]);
-                        const uint64_t n2 = C::FOLD ? ptx::mul2(t2, aa) : ptx::fma2(t2, aa, ptx::neg2(e ? m4.y : m4.x));
+                        const uint64_t n2 = ptx::fma2(t2, aa, ptx::neg2(e ? m4.y : m4.x));
                         float q0, q1;
                         ptx::unpack2(ptx::mul2(ptx::pack2(p0, p1), n2), q0, q1);
                         pa1[(c + e) >> 1] = ptx::pack_bf16(q0, q1);
@@ -949,12 +1051,12 @@ __device__ __forceinline__ void jvp_elem_dv(const JvpParams& p, const JvpBlock<P
 }
 
 // DK, DQ.  Phase A: P and Nn from (S, Sd), kept in registers; phase B: W = P (D - Sigma1), dA = P (X - c) + W Nn, written over
-// D and X.  The statistics are in the scores already (FOLD), belong to the columns (DK, WIDE) or to this thread's row (DQ).
+// D and X.  The statistics belong to the columns (DK) or to this thread's row (DQ).
 template <int MODE, int DP, bool HZ>
 __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const JvpBlock<MODE, DP>& k, int grp, int q, int lane) {
     using C = JvpCfg<MODE, DP>;
     constexpr int BC = C::BC, HC = BC / 2;
-    constexpr bool FOLD = C::FOLD, COL = C::TRANSPOSED && !FOLD, ROW = !C::TRANSPOSED;
+    constexpr bool COL = C::TRANSPOSED, ROW = !COL;
     const int row = q * 32 + lane;
     const uint32_t sb = (static_cast<uint32_t>(q * 32) << 16) + C::COL_SCORE + grp * HC;
     const uint64_t c2c2 = ptx::pack2(p.c2, p.c2), aa = ptx::pack2(p.alpha, p.alpha);
@@ -1002,11 +1104,11 @@ __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const Jvp
                         const int i = c / 2 + e;
                         const uint64_t s2 = ptx::pack2u(s[2 * i], s[2 * i + 1]);
                         float x0, x1;
-                        ptx::unpack2(FOLD ? ptx::mul2(s2, c2c2) : ptx::fma2(s2, c2c2, COL ? (e ? l4.y : l4.x) : r_l), x0, x1);
+                        ptx::unpack2(ptx::fma2(s2, c2c2, COL ? (e ? l4.y : l4.x) : r_l), x0, x1);
                         P2[i] = ptx::pack2(ptx::ex2(x0), ptx::ex2(x1));
                         if (!HZ) {
                             const uint64_t ts = ptx::pack2u(t[2 * i], t[2 * i + 1]);
-                            N2[i] = FOLD ? ptx::mul2(ts, aa) : ptx::fma2(ts, aa, COL ? ptx::neg2(e ? m4.y : m4.x) : r_nm);
+                            N2[i] = ptx::fma2(ts, aa, COL ? ptx::neg2(e ? m4.y : m4.x) : r_nm);
                         }
                     }
                 }
@@ -1030,14 +1132,14 @@ __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const Jvp
                     for (int e = 0; e < 2; ++e) {
                         const int i = c / 2 + e, gi = 8 * u + i;
                         uint64_t x2 = ptx::pack2u(xx[2 * gi], xx[2 * gi + 1]);
-                        if (!FOLD) x2 = ptx::add2(x2, COL ? (e ? c4.y : c4.x) : r_c);
+                        x2 = ptx::add2(x2, COL ? (e ? c4.y : c4.x) : r_c);
                         const uint64_t t2 = ptx::mul2(P2[gi], x2);
                         float d0, d1;
                         if (HZ) {
                             ptx::unpack2(t2, d0, d1);
                         } else {
                             uint64_t y2 = ptx::pack2u(dd[2 * gi], dd[2 * gi + 1]);
-                            if (!FOLD) y2 = ptx::add2(y2, COL ? (e ? s4.y : s4.x) : r_s);
+                            y2 = ptx::add2(y2, COL ? (e ? s4.y : s4.x) : r_s);
                             const uint64_t w2 = ptx::mul2(P2[gi], y2);
                             float w0, w1;
                             ptx::unpack2(w2, w0, w1);
@@ -1056,6 +1158,88 @@ __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const Jvp
     }
 }
 
+// DKV.  Both halves of a tile's work in place: P, P Nn over S, Sd, then W, dA over D, X.  A warp has 16 rows of its lane
+// quadrant (the two groups share the 32) and all columns, so that the operand of a k-step, which replaces 16 columns, is never
+// put together by two warps, whatever the width of the tile.  The statistics are in the scores already, so it does not
+// matter which element of a row a thread holds: 16 lanes x 256 bits are read, and two neighbouring values packed make
+// 16 lanes x 128 bits.
+template <int DP, bool HZ>
+__device__ __forceinline__ void jvp_elem_dkv(const JvpParams& p, const JvpBlock<PASS_DKV, DP>& k, int grp, int q, int lane) {
+    using C = JvpCfg<PASS_DKV, DP>;
+    constexpr int BC = C::BC, NU = BC / 16, LO = C::KLO;
+    const uint32_t sb = (static_cast<uint32_t>(q * 32 + grp * 16) << 16) + C::COL_SCORE;
+    const uint64_t c2c2 = ptx::pack2(p.c2, p.c2), aa = ptx::pack2(p.alpha, p.alpha);
+    const int n_it = (int)blockIdx.x < p.items ? (p.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+    for (int g = 0; g < n_it * p.T; ++g) {
+        uint64_t P2[4 * NU], N2[4 * NU];
+        uint32_t y[8 * NU], x[8 * NU];   // S, Sd, then D, X
+        if (!k.done(C::B_SFULL, g)) return;
+        ptx::tc_fence_after_sync();
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            ptx::tmem_ld16_256x2(sb + 16 * u, y + 8 * u);
+            if (!HZ) ptx::tmem_ld16_256x2(sb + BC + 16 * u, x + 8 * u);
+        }
+        ptx::tmem_wait_ld();
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            uint32_t a0[4], a1[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int c = 4 * u + i;
+                float x0, x1;
+                ptx::unpack2(ptx::mul2(ptx::pack2u(y[2 * c], y[2 * c + 1]), c2c2), x0, x1);
+                x0 = ptx::ex2(x0); x1 = ptx::ex2(x1);
+                P2[c] = ptx::pack2(x0, x1);
+                a0[i] = ptx::pack_bf16(x0, x1);
+                if (!HZ) {
+                    N2[c] = ptx::mul2(ptx::pack2u(x[2 * c], x[2 * c + 1]), aa);
+                    ptx::unpack2(ptx::mul2(P2[c], N2[c]), x0, x1);
+                    a1[i] = ptx::pack_bf16(x0, x1);
+                }
+            }
+            ptx::tmem_st16_128x2(sb + 16 * u, a0);
+            if (!HZ) ptx::tmem_st16_128x2(sb + BC + 16 * u, a1);
+            if (u == LO - 1 || u == NU - 1) {
+                ptx::tmem_wait_st();
+                k.arrive(C::B_PREADY + (u == NU - 1), lane);
+            }
+        }
+        if (!k.done(C::B_XFULL, g)) return;
+        ptx::tc_fence_after_sync();
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            if (!HZ) ptx::tmem_ld16_256x2(sb + 2 * BC + 16 * u, y + 8 * u);
+            ptx::tmem_ld16_256x2(sb + 3 * BC + 16 * u, x + 8 * u);
+        }
+        ptx::tmem_wait_ld();
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            uint32_t a0[4], a1[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int c = 4 * u + i;
+                uint64_t t2 = ptx::mul2(P2[c], ptx::pack2u(x[2 * c], x[2 * c + 1]));
+                float x0, x1;
+                if (!HZ) {
+                    const uint64_t w2 = ptx::mul2(P2[c], ptx::pack2u(y[2 * c], y[2 * c + 1]));
+                    ptx::unpack2(w2, x0, x1);
+                    a0[i] = ptx::pack_bf16(x0, x1);
+                    t2 = ptx::fma2(w2, N2[c], t2);
+                }
+                ptx::unpack2(t2, x0, x1);
+                a1[i] = ptx::pack_bf16(x0, x1);
+            }
+            if (!HZ) ptx::tmem_st16_128x2(sb + 2 * BC + 16 * u, a0);
+            ptx::tmem_st16_128x2(sb + 3 * BC + 16 * u, a1);
+            if (u == LO - 1 || u == NU - 1) {
+                ptx::tmem_wait_st();
+                k.arrive(C::B_PREADY + 2 + (u == NU - 1), lane);
+            }
+        }
+    }
+}
+
 // ------------------------------------------------------------------------------------------------ epilogue warps
 // A thread has one owner row.  Per item: the owner operands of the next item go to tensor memory as soon as the item's last
 // score MMAs are done with the present ones (XT), then the accumulators are normalised, converted and stored; they are free
@@ -1067,8 +1251,7 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
     constexpr int XT0 = C::NPAIR == 2 ? 2 : 0;     // p.own[XT0], p.own[XT0 + 1] -> tensor memory
     const int row = q * 32 + lane;
     const uint32_t lanes = static_cast<uint32_t>(q * 32) << 16;
-    // Row of tensor t in an item; what is beyond the head dim or the tensor, and an absent cotangent, reads as zero.  The
-    // columns of ones that the statistics are multiplied by (FOLD): padding of the first tensor.
+    // Row of tensor t in an item; what is beyond the head dim or the tensor, and an absent cotangent, reads as zero.
     [[maybe_unused]] auto load_x = [&](int item, int t, uint4 (&v)[NCH]) {
         const int bh = item / p.row_tiles, row0 = (item - bh * p.row_tiles) * JVP_ROWS;
         const __nv_bfloat16* x = p.own[XT0 + t];
@@ -1079,7 +1262,6 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
             v[c] = make_uint4(0, 0, 0, 0);
             if (valid && 8 * c < p.d) v[c] = __ldg(reinterpret_cast<const uint4*>(src + 8 * c));
         }
-        if (C::FOLD && t == 0 && !k.fold_step()) { v[NCH - 1].x = JVP_ONES0; v[NCH - 1].y = JVP_ONES1; }
     };
     [[maybe_unused]] auto store_x = [&](int t, const uint4 (&v)[NCH]) {
 #pragma unroll
@@ -1090,10 +1272,6 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
     };
     [[maybe_unused]] uint4 v0[NCH], v1[NCH];
     if (C::XT && (int)blockIdx.x < p.items) {
-        if (C::FOLD) {
-            const uint32_t r[8] = {JVP_ONES0, JVP_ONES1, 0u, 0u, 0u, 0u, 0u, 0u};
-            ptx::tmem_st8(lanes + C::COL_ONES, r);
-        }
         load_x(blockIdx.x, 0, v0);
         store_x(0, v0);
         load_x(blockIdx.x, 1, v0);
@@ -1136,12 +1314,18 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
         if (!k.wait(C::B_FINAL, it)) return;
         ptx::tc_fence_after_sync();
 #pragma unroll 1
-        for (int ch = 0; ch < C::KS; ++ch) {
+        for (int i = 0; i < C::KS * (C::NACC / 2); ++i) {
+            const bool second = C::DKV && i >= C::KS;      // the second pair of accumulators
+            const int ch = second ? i - C::KS : i;
+            const uint32_t at = lanes + 16 * ch + (second ? 2 * C::COL_ACC1 : 0);
+            __nv_bfloat16* const out0 = second ? p.out2 : p.out0;
+            __nv_bfloat16* const out1 = second ? p.out3 : p.out1;
+            if (C::DKV) f0 = second ? p.out_scale : 1.0f;
             uint32_t x0[16], x1[16], q0[8], q1[8];
-            ptx::tmem_ld16(lanes + C::COL_ACC0 + 16 * ch, x0);
-            ptx::tmem_ld16(lanes + C::COL_ACC1 + 16 * ch, x1);
+            ptx::tmem_ld16(at + C::COL_ACC0, x0);
+            ptx::tmem_ld16(at + C::COL_ACC1, x1);
             ptx::tmem_wait_ld();
-            if (ch == C::KS - 1) k.arrive(C::B_ACCFREE, lane);
+            if (i == C::KS * (C::NACC / 2) - 1) k.arrive(C::B_ACCFREE, lane);
 #pragma unroll
             for (int c = 0; c < 16; c += 2) {
                 float a0 = __uint_as_float(x0[c]) * f0, a1 = __uint_as_float(x0[c + 1]) * f0;
@@ -1152,9 +1336,9 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
             }
             if (16 * ch >= p.d) continue;
             const bool has_hi = 16 * ch + 8 < p.d;
-            store_row_pairs(p.out1 + off + 16 * ch, p.o.rs, lane, ok_even, ok_odd, has_hi, make_uint4(q1[0], q1[1], q1[2], q1[3]), make_uint4(q1[4], q1[5], q1[6], q1[7]));
-            if (p.out0)   // null with Hc absent: acc0 was never written, its gradient is zero
-                store_row_pairs(p.out0 + off + 16 * ch, p.o.rs, lane, ok_even, ok_odd, has_hi, make_uint4(q0[0], q0[1], q0[2], q0[3]), make_uint4(q0[4], q0[5], q0[6], q0[7]));
+            store_row_pairs(out1 + off + 16 * ch, p.o.rs, lane, ok_even, ok_odd, has_hi, make_uint4(q1[0], q1[1], q1[2], q1[3]), make_uint4(q1[4], q1[5], q1[6], q1[7]));
+            if (out0)   // null with Hc absent: acc0 was never written, its gradient is zero
+                store_row_pairs(out0 + off + 16 * ch, p.o.rs, lane, ok_even, ok_odd, has_hi, make_uint4(q0[0], q0[1], q0[2], q0[3]), make_uint4(q0[4], q0[5], q0[6], q0[7]));
         }
     }
 }
@@ -1192,8 +1376,8 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
         init(C::B_OWNFREE, 1, 1);
         init(C::B_XRDY, 1, 4);
         init(C::B_XFREE, 1, 1);
-        init(C::B_SFULL, 12, 1);       // SFULL, XFULL, OUTDONE
-        init(C::B_PREADY, 4, 4);       // the four warps of a group
+        init(C::B_SFULL, 16, 1);       // SFULL, XFULL, OUTDONE, O1DONE
+        init(C::B_PREADY, 4, C::DKV ? 8 : 4);   // (of four: the warps of a group)
         init(C::B_SREAD, 1, 8);
         init(C::B_FINAL, 1, 1);
         init(C::B_ACCFREE, 1, 4);
@@ -1206,33 +1390,32 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
     if (C::TAIL && ((p.d - 64) >> 3) < 2) {
         // The 16-byte chunk behind the copied columns (d = 72) pads the head dim to a multiple of 16: zeroed once, never
         // written again.  Owners and E ring: the second chunk block; L ring: chunk 1 of the second atom, which lies at
-        // physical chunk 1 ^ (r & 7) of row r.  Where the columns hold statistics (FOLD), the first owner tensor has the
-        // ones there.
+        // physical chunk 1 ^ (r & 7) of row r.  FOLD: the stages have the statistics there, the first owner tensor of a pair
+        // the ones.
         for (int i = threadIdx.x; i < C::NOWN * JVP_ROWS; i += JVP_THREADS)
             *reinterpret_cast<uint4*>(jvp_smem + (i / JVP_ROWS) * C::OWN_BYTES + C::OWN_ATOM + (JVP_ROWS + i % JVP_ROWS) * 16) =
-                C::FOLD && i < JVP_ROWS ? make_uint4(JVP_ONES0, JVP_ONES1, 0, 0) : zero;
-        uint8_t* e = jvp_smem + C::NOWN * C::OWN_BYTES;
-        for (int i = threadIdx.x; i < C::SE * 2 * BC; i += JVP_THREADS)
-            *reinterpret_cast<uint4*>(e + (i / (2 * BC)) * 2 * C::EST_BYTES + 2 * C::ATOM + (2 * BC + i % (2 * BC)) * 16) = zero;
-        uint8_t* l = e + C::SE * 2 * C::EST_BYTES;
-        for (int i = threadIdx.x; i < C::SL * 2 * BC; i += JVP_THREADS) {
-            const int t = i / BC, r = i - t * BC;
-            *reinterpret_cast<uint4*>(l + (t >> 1) * 2 * C::LST_BYTES + (2 + (t & 1)) * C::ATOM + r * 128 + ((1 ^ (r & 7)) << 4)) = zero;
+                C::FOLD && !(i / JVP_ROWS & 1) ? make_uint4(JVP_ONES0, JVP_ONES1, 0, 0) : zero;
+        if (!C::FOLD) {
+            uint8_t* e = jvp_smem + C::NOWN * C::OWN_BYTES;
+            for (int i = threadIdx.x; i < C::SE * 2 * BC; i += JVP_THREADS)
+                *reinterpret_cast<uint4*>(e + (i / (2 * BC)) * 2 * C::EST_BYTES + 2 * C::ATOM + (2 * BC + i % (2 * BC)) * 16) = zero;
+            uint8_t* l = e + C::SE * 2 * C::EST_BYTES;
+            for (int i = threadIdx.x; i < C::SL * 2 * BC; i += JVP_THREADS) {
+                const int t = i / BC, r = i - t * BC;
+                *reinterpret_cast<uint4*>(l + (t >> 1) * 2 * C::LST_BYTES + (2 + (t & 1)) * C::ATOM + r * 128 + ((1 ^ (r & 7)) << 4)) = zero;
+            }
         }
     }
-    if (!HZ && MODE == PASS_DK && p.absent) {
-        // both cotangent tiles of an E stage are read by one N = 128 MMA: the never-loaded one must read as zero
+    if (!HZ && (MODE == PASS_DK || C::DKV) && p.absent) {
+        // both cotangent tiles of an E stage are read by one MMA: the never-loaded one must read as zero
         const int t = (p.absent & ABSENT_HC) ? 0 : 1;
         uint8_t* e = jvp_smem + C::NOWN * C::OWN_BYTES;
         for (int st = 0; st < C::SE; ++st) {
             uint8_t* stage = e + st * 2 * C::EST_BYTES;
             for (int i = threadIdx.x; i < BC * 8; i += JVP_THREADS) {
                 *reinterpret_cast<uint4*>(stage + t * C::ATOM + i * 16) = zero;
-                if (C::WIDE) *reinterpret_cast<uint4*>(stage + (2 + t) * C::ATOM + i * 16) = zero;
+                if (C::NA == 2) *reinterpret_cast<uint4*>(stage + (2 + t) * C::ATOM + i * 16) = zero;
             }
-            if (C::TAIL)
-                for (int i = threadIdx.x; i < 2 * BC; i += JVP_THREADS)
-                    *reinterpret_cast<uint4*>(stage + 2 * C::ATOM + ((i / BC) * 2 * BC + t * BC + i % BC) * 16) = zero;
         }
     }
     if (C::FOLD)
@@ -1275,6 +1458,7 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
         if (placed) {
             const int grp = (warp - 4) >> 2, q = warp & 3;
             if constexpr (MODE == PASS_FWD) jvp_elem_fwd<DP>(p, k, grp, q, lane);
+            else if constexpr (MODE == PASS_DKV) jvp_elem_dkv<DP, HZ>(p, k, grp, q, lane);
             else if constexpr (MODE == PASS_DV) jvp_elem_dv<DP, HZ>(p, k, grp, q, lane);
             else jvp_elem_two_pairs<MODE, DP, HZ>(p, k, grp, q, lane);
         }

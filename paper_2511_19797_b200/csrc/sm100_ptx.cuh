@@ -159,6 +159,19 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
                  : "r"(taddr)
                  : "memory");
 }
+// 16 lanes (from a multiple of 16) x 16 columns: thread t has r[0, 1] = columns 2 (t % 4), 2 (t % 4) + 1 of lane t / 4, r[2, 3] the
+// same of lane 8 + t / 4, r[4..7] the same 8 columns further on.
+__device__ __forceinline__ void tmem_ld16_256x2(uint32_t taddr, uint32_t* r) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+}
+// 16 lanes x 8 columns: thread t has r[0] = column t % 4 of lane t / 4, r[1] the same of lane 8 + t / 4, r[2, 3] the same 4 columns
+// further on: where the values of tmem_ld16_256x2 belong once two neighbours have been packed into one column.
+__device__ __forceinline__ void tmem_st16_128x2(uint32_t taddr, const uint32_t* r) {
+    asm volatile("tcgen05.st.sync.aligned.16x128b.x2.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
 // 32 lanes x 32 consecutive 32-bit columns.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
     asm volatile(

@@ -236,13 +236,13 @@ static encode_tiled_fn get_encode_fn() {
 }
 
 // A bf16 tensor of one side viewed as a 4-D tensor (d, rows, H, B) with that side's strides; a box is 64 columns x
-// 64 rows of one head with the 128-byte swizzle; columns or rows beyond the tensor read as zero.
-static int make_tmap(CUtensorMap* m, const void* ptr, const Shape& s, const Geom& g) {
+// `box_rows` rows of one head with the 128-byte swizzle; columns or rows beyond the tensor read as zero.
+static int make_tmap(CUtensorMap* m, const void* ptr, const Shape& s, const Geom& g, int box_rows = JVP_BC) {
     encode_tiled_fn fn = get_encode_fn();
     if (!fn) return TVM_ATTN_CUDA_ERROR;
     cuuint64_t dims[4] = {(cuuint64_t)s.d, (cuuint64_t)g.rows, (cuuint64_t)s.H, (cuuint64_t)s.B};
     cuuint64_t strides[3] = {(cuuint64_t)g.rs * 2, (cuuint64_t)g.hs * 2, (cuuint64_t)g.bs * 2};
-    cuuint32_t box[4] = {64, JVP_BC, 1, 1};
+    cuuint32_t box[4] = {64, (cuuint32_t)box_rows, 1, 1};
     cuuint32_t estr[4] = {1, 1, 1, 1};
     CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -250,8 +250,8 @@ static int make_tmap(CUtensorMap* m, const void* ptr, const Shape& s, const Geom
     return r == CUDA_SUCCESS ? TVM_ATTN_OK : TVM_ATTN_CUDA_ERROR;
 }
 
-// A tensor of a call and its map (boxes of 64 columns x 64 rows: one map serves a tensor in every role it has in the passes
-// of a call).  An absent cotangent is never loaded: its map is that of a present tensor and unused.
+// A tensor of a call and its map (with boxes of 64 rows one map serves a tensor in every role it has in the passes of a
+// call, except as a stream of shorter tiles).  An absent cotangent is never loaded: its map is that of a present tensor and unused.
 struct Operand {
     const __nv_bfloat16* ptr;
     const CUtensorMap* map;
@@ -273,13 +273,13 @@ static int launch_pass(const Shape& s, const Operand (&own)[4], const Operand (&
     // items go round-robin over them
     prm.row_tiles = (prm.o.rows + JVP_ROWS - 1) / JVP_ROWS;
     prm.items = (int)(s.BH * prm.row_tiles);
-    prm.T = (prm.s.rows + JVP_BC - 1) / JVP_BC;
+    prm.T = (prm.s.rows + C::BC - 1) / C::BC;
     g_prof.before(st);
-    // DK and DQ read nothing that the pass before them writes (DV, DK and DQ all depend on the row-sums pre-pass only,
-    // which has completed before DV starts), so their CTAs may fill the SMs that the last, partial wave of the pass
+    // DK and DQ read nothing that the pass before them writes (all passes depend on the row-sums pre-pass only, which has
+    // completed before the first of them starts), so their CTAs may fill the SMs that the last, partial wave of the pass
     // before leaves idle: programmatic dependent launch, with every CTA of these kernels releasing its dependents at
     // once.  None waits for its primary before it works; each waits for it once at the very end (griddepcontrol.wait in
-    // the teardown), so that DQ cannot complete before DK, nor DK before DV: work enqueued behind the call still sees all
+    // the teardown), so that no pass can complete before the one in front of it: work enqueued behind the call still sees all
     // six gradients.  Not while per-kernel events are being recorded: they would time overlapping kernels.
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(prm.items < dev.sms ? prm.items : dev.sms));
@@ -308,17 +308,18 @@ static int launch_pass_hz(const Shape& s, const Operand (&own)[4], const Operand
     return launch_pass<MODE, DP, false>(s, own, strm, prm, dev, st);
 }
 
-template <int MODE>
+// The passes there are: FWD and DQ for every head dim; DKV where its four accumulators fit into tensor memory next to the
+// scores, DV and DK where they do not.
+static constexpr bool pass_exists(int mode, int dp) { return mode == PASS_DKV ? dp <= 80 : mode == PASS_DV || mode == PASS_DK ? dp > 80 : true; }
+
+template <int MODE, int DP = 16>
 static int launch_pass_dp(const Shape& s, const Operand (&own)[4], const Operand (&strm)[4], const JvpParams& prm, const DeviceFacts& dev, cudaStream_t st) {
-    switch (s.dp) {
-        case 16: return launch_pass_hz<MODE, 16>(s, own, strm, prm, dev, st);
-        case 32: return launch_pass_hz<MODE, 32>(s, own, strm, prm, dev, st);
-        case 48: return launch_pass_hz<MODE, 48>(s, own, strm, prm, dev, st);
-        case 64: return launch_pass_hz<MODE, 64>(s, own, strm, prm, dev, st);
-        case 80: return launch_pass_hz<MODE, 80>(s, own, strm, prm, dev, st);
-        case 96: return launch_pass_hz<MODE, 96>(s, own, strm, prm, dev, st);
-        case 112: return launch_pass_hz<MODE, 112>(s, own, strm, prm, dev, st);
-        default: return launch_pass_hz<MODE, 128>(s, own, strm, prm, dev, st);
+    if constexpr (DP > 128) {
+        return TVM_ATTN_UNSUPPORTED;
+    } else {
+        if constexpr (pass_exists(MODE, DP))
+            if (s.dp == DP) return launch_pass_hz<MODE, DP>(s, own, strm, prm, dev, st);
+        return launch_pass_dp<MODE, DP + 16>(s, own, strm, prm, dev, st);
     }
 }
 
@@ -559,12 +560,21 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
     if (rc != TVM_ATTN_OK) return rc;
     rc = launch_rowsums<__nv_bfloat16>(s, dO, dtO, O, tO, lse, sig1, cvec, lse2, -1.0f, st);
     if (rc != TVM_ATTN_OK) return rc;
-    CUtensorMap maps[8];
+    CUtensorMap maps[12];
     const void* in[8] = {Q, tQ, dtO, dO, K, tK, V, tV};
-    Operand x[8];
+    Operand x[12];
     for (int t = 0; t < 8; ++t) {
         x[t] = {static_cast<const __nv_bfloat16*>(in[t]), in[t] ? &maps[t] : &maps[0]};
         rc = in[t] ? make_tmap(&maps[t], in[t], s, t < 4 ? s.q : s.k) : TVM_ATTN_OK;
+        if (rc != TVM_ATTN_OK) return rc;
+    }
+    // the query side as DKV streams it
+    const int short_rows = s.dp == 80 ? JvpCfg<PASS_DKV, 80>::BC : JVP_BC;
+    for (int t = 0; t < 4; ++t) {
+        x[8 + t] = x[t];
+        if (short_rows == JVP_BC || !in[t]) continue;
+        x[8 + t].map = &maps[8 + t];
+        rc = make_tmap(&maps[8 + t], in[t], s, s.q, short_rows);
         if (rc != TVM_ATTN_OK) return rc;
     }
     const Operand &xQ = x[0], &xtQ = x[1], &xH = x[2], &xG = x[3], &xK = x[4], &xtK = x[5], &xV = x[6], &xtV = x[7];
@@ -573,18 +583,25 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
     b.d = s.d; b.H = s.H;
     b.alpha = s.alpha; b.c2 = s.alpha * 1.4426950408889634f;
     b.nlse2 = lse2; b.mu = mu; b.nsig1 = sig1; b.ncvec = cvec; b.status = dev->status; b.absent = absent;
+    auto bf16 = [](void* ptr) { return static_cast<__nv_bfloat16*>(ptr); };
     auto outputs = [&](void* tangent, void* primal, float scale) {
-        b.out0 = dtO ? static_cast<__nv_bfloat16*>(tangent) : nullptr;
-        b.out1 = static_cast<__nv_bfloat16*>(primal);
+        b.out0 = dtO ? bf16(tangent) : nullptr;
+        b.out1 = bf16(primal);
         b.out_scale = scale;
     };
-    // dtV = P^T Hc, dV = P^T G + (P*Nn)^T Hc : owner keys (K, tK); stream queries (Q, tQ | Hc, G)
-    outputs(dtV, dV, 1.0f);
-    rc = launch_pass_dp<PASS_DV>(s, {xK, xtK, xK, xtK}, {xQ, xtQ, xH, xG}, b, *dev, st);
-    if (rc != TVM_ATTN_OK) return rc;
-    // dtK = alpha W^T Q, dK = alpha (dA^T Q + W^T tQ) : owner keys (K, tK, V, tV); stream (Hc, G | Q, tQ)
-    outputs(dtK, dK, s.alpha);
-    rc = launch_pass_dp<PASS_DK>(s, {xK, xtK, xV, xtV}, {xH, xG, xQ, xtQ}, b, *dev, st);
+    // dtV = P^T Hc, dV = P^T G + (P*Nn)^T Hc; dtK = alpha W^T Q, dK = alpha (dA^T Q + W^T tQ) : owner keys, stream queries
+    if (pass_exists(PASS_DKV, s.dp)) {
+        outputs(dtV, dV, s.alpha);
+        b.out2 = dtO ? bf16(dtK) : nullptr;
+        b.out3 = bf16(dK);
+        rc = launch_pass_dp<PASS_DKV>(s, {xK, xtK, xV, xtV}, {x[10], x[11], x[8], x[9]}, b, *dev, st);
+    } else {
+        outputs(dtV, dV, 1.0f);
+        rc = launch_pass_dp<PASS_DV>(s, {xK, xtK, xK, xtK}, {xQ, xtQ, xH, xG}, b, *dev, st);
+        if (rc != TVM_ATTN_OK) return rc;
+        outputs(dtK, dK, s.alpha);
+        rc = launch_pass_dp<PASS_DK>(s, {xK, xtK, xV, xtV}, {xH, xG, xQ, xtQ}, b, *dev, st);
+    }
     if (rc != TVM_ATTN_OK) return rc;
     // dtQ = alpha W K, dQ = alpha (dA K + W tK) : owner queries (Q, tQ, Hc, G); stream (V, tV | K, tK)
     outputs(dtQ, dQ, s.alpha);

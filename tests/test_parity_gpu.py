@@ -71,6 +71,14 @@ def test_wide_head_dims_with_several_items_per_block(B, H, N, d, peaky):
     assert_within(errs, BF16_FWD, BF16_BWD, BF16_STATS)
 
 
+# key and value gradients of one pass: edges of its query tiles (48 rows at d = 72 and 80, else 64) and of the 128 keys of an item
+@pytest.mark.parametrize("absent", [None, "dtO", "dO"])
+@pytest.mark.parametrize("N,d", [(1, 72), (47, 72), (48, 80), (49, 72), (97, 80), (145, 72), (33, 64), (64, 64), (127, 48), (193, 16)])
+def test_key_gradients_at_tile_edges(N, d, absent):
+    errs, _, _ = run_case(inputs.custom(2, 3, N, d, seed=80 + N + d), absent=absent)
+    assert_within(errs, BF16_FWD, BF16_BWD, BF16_STATS)
+
+
 @pytest.mark.parametrize("B,H,N,d", [(3, 50, 192, 72), (3, 50, 320, 64), (5, 61, 65, 72), (2, 80, 200, 40),
                                      (4, 50, 64, 72), (4, 50, 33, 40)])
 def test_several_work_items_per_cta(B, H, N, d):
