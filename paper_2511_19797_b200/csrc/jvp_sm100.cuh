@@ -146,7 +146,6 @@ struct JvpCfg {
     // TMEM columns: accumulators, the owner operands in the gaps behind them,
     // score accumulators (FWD, DV: two buffers of S | Sd; DK, DQ: one of S | Sd | D | X).
     static constexpr int NACC = DKV ? 4 : 2;
-    static constexpr int KLO = BC / 32;                    // k-steps of an output in its first part
     static constexpr int COL_ACC0 = 0, COL_ACC1 = XT ? 128 : DP, COL_SCORE = NACC * COL_ACC1;
     static constexpr int COL_X0 = DP, COL_X1 = COL_ACC1 + DP;
     static_assert(!XT || DP + DP / 2 <= 128, "operands do not fit behind their accumulators");
@@ -157,9 +156,10 @@ struct JvpCfg {
     // barriers
     static constexpr int B_EFULL = 0;
     static constexpr int B_LFULL = B_EFULL + SE;
+    static constexpr int OWN_SETS = DKV ? 2 : 1;                       // owner tiles with barriers of their own (DKV: K, tK | V, tV)
     static constexpr int B_OWN = B_LFULL + SL;                         // owner tiles in shared memory loaded
-    static constexpr int B_OWNFREE = B_OWN + 1;                        // ... free: the score MMAs of the item are complete
-    static constexpr int B_XRDY = B_OWNFREE + 1;                       // owner operands in tensor memory written
+    static constexpr int B_OWNFREE = B_OWN + OWN_SETS;                 // ... free: the score MMAs of the item are complete
+    static constexpr int B_XRDY = B_OWNFREE + OWN_SETS;                       // owner operands in tensor memory written
     static constexpr int B_XFREE = B_XRDY + 1;                         // ... free
     // MMAs of tile g complete: + (g & 3), phase g >> 2.  The element-wise groups meet every other tile only and the
     // producers run up to four tiles ahead of or behind the others, so that a parity wait on one barrier, or on a pair,
@@ -168,11 +168,12 @@ struct JvpCfg {
     static constexpr int B_SFULL = B_XFREE + 1;                        // S (and Sd, except in FWD) written
     static constexpr int B_XFULL = B_SFULL + 4;                        // FWD: Sd written; DK, DQ: D, X written
     static constexpr int B_OUTDONE = B_XFULL + 4;                      // output MMAs complete
-    static constexpr int B_O1DONE = B_OUTDONE + 4;                     // DKV: ... of the first pair (OUTDONE: of the second)
-    static constexpr int B_EDONE = DKV ? B_O1DONE : MODE == PASS_DV ? B_SFULL : B_XFULL;   // the E stage of the tile is free
+    // The stage of a tile is free.  DKV: its output MMAs are in front of the next tile's scores, whose completion implies theirs.
+    static constexpr int B_EDONE = DKV || MODE == PASS_DV ? B_SFULL : B_XFULL, EDONE_NEXT = DKV ? 1 : 0;
+    static constexpr int B_LDONE = DKV ? B_XFULL : B_OUTDONE, LDONE_NEXT = EDONE_NEXT;
     static_assert(SE <= 4 && SL <= 4, "a ring deeper than the completion barriers");
-    // operands written: + half of the tile (DK, DQ), + 2 (g & 1) + half (FWD, DV), + 2 pair + part (DKV)
-    static constexpr int B_PREADY = B_O1DONE + 4;
+    // operands written: + half of the tile (DK, DQ), + 2 (g & 1) + half (FWD, DV), + pair (DKV)
+    static constexpr int B_PREADY = B_OUTDONE + 4;
     static constexpr int B_SREAD = B_PREADY + 4;                       // DK, DQ: S, Sd read
     static constexpr int B_FINAL = B_SREAD + 1;                        // the item's last output MMAs complete
     static constexpr int B_ACCFREE = B_FINAL + 1;                      // the epilogue has read the accumulators
@@ -246,23 +247,24 @@ struct JvpBlock {
 };
 
 // ------------------------------------------------------------------------------------------------ producers
-// Owner tiles of an item (by the E ring's warp): two boxes of 64 rows per tensor and atom, like those of the stream tiles,
+// A set of owner tiles of an item (by the E ring's warp): two boxes of 64 rows per tensor and atom, like those of the stream tiles,
 // so that one tensor map serves both.
-template <int MODE, int DP>
+template <int MODE, int DP, int SET>
 __device__ __forceinline__ void jvp_load_owners(const JvpParams& p, const JvpBlock<MODE, DP>& k, const CUtensorMap* const (&maps)[4], int item, int lane) {
     using C = JvpCfg<MODE, DP>;
+    constexpr int T0 = SET * (C::NOWN / C::OWN_SETS), T1 = T0 + C::NOWN / C::OWN_SETS;
     constexpr int KT = C::TAIL ? (DP - 64) / 8 : 1, H64 = 64 * 128;
     const int bh = item / p.row_tiles, row0 = (item - bh * p.row_tiles) * JVP_ROWS;
     const int cb = bh / p.H, ch = bh - cb * p.H;
     if (lane == 0) {
-        const uint32_t full = k.bar(C::B_OWN);
+        const uint32_t full = k.bar(C::B_OWN + SET);
         uint32_t tx = 0;
 #pragma unroll
-        for (int t = 0; t < C::NOWN; ++t) tx += p.own[t] ? C::OWN_ATOM * (C::WIDE ? 2 : 1) : 0;   // null: an absent cotangent
+        for (int t = T0; t < T1; ++t) tx += p.own[t] ? C::OWN_ATOM * (C::WIDE ? 2 : 1) : 0;   // null: absent, or not read
         ptx::mbar_arrive_expect_tx(full, tx);
 #pragma unroll
-        for (int t = 0; t < C::NOWN; ++t) {
-            if (!p.own[t]) continue;   // its tile is zeroed once
+        for (int t = T0; t < T1; ++t) {
+            if (!p.own[t]) continue;   // (its tile is zeroed once)
             const uint32_t dst = k.own_tile(t);
             ptx::tma_load_4d(dst, maps[t], full, 0, row0, ch, cb);
             ptx::tma_load_4d(dst + H64, maps[t], full, 0, row0 + 64, ch, cb);
@@ -276,7 +278,7 @@ __device__ __forceinline__ void jvp_load_owners(const JvpParams& p, const JvpBlo
         const int ntail = (p.d - 64) >> 3, rows_left = p.o.rows - row0;
         const size_t d32 = 32 * (size_t)p.o.rs, lane_row = p.o.head_off(bh, p.H) + (size_t)(row0 + lane) * (size_t)p.o.rs + 64;
 #pragma unroll
-        for (int t = 0; t < C::NOWN; ++t) {
+        for (int t = T0; t < T1; ++t) {
             const __nv_bfloat16* x = p.own[t];
             const uint32_t tile = k.own_tile(t) + C::OWN_ATOM + lane * 16;
 #pragma unroll
@@ -290,7 +292,7 @@ __device__ __forceinline__ void jvp_load_owners(const JvpParams& p, const JvpBlo
                 }
             }
         }
-        ptx::cp_async_arrive(k.bar(C::B_OWN));
+        ptx::cp_async_arrive(k.bar(C::B_OWN + SET));
     }
 }
 
@@ -299,14 +301,14 @@ __device__ __forceinline__ void jvp_load_owners(const JvpParams& p, const JvpBlo
 // is left to its copies (a warp that waits for them itself loads no more than one tile per memory latency).  These loops
 // run next to element-wise warps that leave them few issue slots, and a ring is refilled no faster than they run: what does
 // not depend on the tile is set up before them, and tiles whose rows all exist take a path without predicates.
-template <int MODE, int DP, int RING>
+template <int MODE, int DP, bool HZ, int RING>
 __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock<MODE, DP>& shared, const CUtensorMap* map0, const CUtensorMap* map1,
                                               const CUtensorMap* const (&own_maps)[4], int lane) {
     using C = JvpCfg<MODE, DP>;
     const JvpBlock<MODE, DP> k = shared.pinned();
     const int T = jvp_pin(p.T), rows = jvp_pin(p.s.rows);
     constexpr int BC = C::BC, S = RING == 0 ? C::SE : C::SL, ATOM = C::ATOM;
-    constexpr int b_full = RING == 0 ? C::B_EFULL : C::B_LFULL, b_done = RING == 0 ? C::B_EDONE : C::B_OUTDONE;
+    constexpr int b_full = RING == 0 ? C::B_EFULL : C::B_LFULL, b_done = RING == 0 ? C::B_EDONE : C::B_LDONE, next = RING == 0 ? C::EDONE_NEXT : C::LDONE_NEXT;
     constexpr uint32_t TB = RING == 0 ? C::EST_BYTES : C::LST_BYTES;
     constexpr bool STATS = RING == 1 && C::TRANSPOSED && !C::FOLD;   // this ring carries the statistics as they are
     constexpr bool OWNERS = RING == 0 && C::NOWN > 0;
@@ -318,9 +320,10 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
     const uint32_t ring_base = k.base + (RING == 0 ? k.E : k.L);
     const __nv_bfloat16* base0 = p.strm[2 * RING];
     const __nv_bfloat16* base1 = p.strm[2 * RING + 1];
-    // the ring that streams the cotangents (Hc, G): L in DV, E in DK and DKV; an absent one is not loaded
+    // The ring that streams the cotangents (Hc, G): L in DV, E in DK and DKV; an absent one (null) is not loaded, nor, with HZ,
+    // are the tangents.
     constexpr bool COT = (MODE == PASS_DV && RING == 1) || ((MODE == PASS_DK || C::DKV) && RING == 0);
-    const bool has0 = !COT || !(p.absent & ABSENT_HC), has1 = !COT || !(p.absent & ABSENT_G);
+    const bool has0 = COT ? !HZ && base0 : true, has1 = COT ? HZ || base1 : !HZ;
     const uint32_t tx_bytes = ((has0 ? 1 : 0) + (has1 ? 1 : 0)) * ATOM * (C::WIDE ? 2 : 1);
     // Chunk 0 of row `lane` behind the first atoms: compact blocks in the E ring, a second swizzled atom in the L ring.
     [[maybe_unused]] const uint32_t sw = lane & 7;  // rows 32 apart share it
@@ -332,6 +335,7 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
     bool ok = true;
     int s = 0, ph = 0;
     int g = 0, owners = 0;           // tiles, and items whose owner tiles, have been asked for
+    [[maybe_unused]] int owners0 = 0;   // one more item's first set has
     uint32_t stage = ring_base, full = k.bar(b_full);
     // In an item's tiles the owner tiles have their turn where what they wait for is about to happen: behind as many of the
     // item's E tiles as the ring holds.
@@ -354,10 +358,15 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
             if (OWNERS && j == owners_at) {   // once the score MMAs of the item before are complete
                 ok = owners == 0 || k.wait(C::B_OWNFREE, owners - 1);
                 if (!ok) break;
-                jvp_load_owners(p, k, own_maps, item, lane);
+                jvp_load_owners<MODE, DP, 0>(p, k, own_maps, item, lane);
+                if constexpr (C::OWN_SETS == 2) {
+                    ok = owners == 0 || k.wait(C::B_OWNFREE + 1, owners - 1);
+                    if (!ok) { owners0 = 1; break; }
+                    jvp_load_owners<MODE, DP, 1>(p, k, own_maps, item, lane);
+                }
                 ++owners;
             }
-            if (g >= S) ok = k.done(b_done, g - S);   // the MMAs that read the stage's last tile
+            if (g >= S) ok = k.done(b_done, g - S + next);   // the MMAs that read the stage's last tile
             if (!ok) break;
             ++g;
             [[maybe_unused]] const int rows_left = rows - j * BC;  // rows of this tile that exist
@@ -431,7 +440,8 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
             if (!cur && g < S) continue;  // never filled
             ptx::mbar_wait_drain(k.bar(b_full + i), (cur ? ph : ph ^ 1) & 1, ptx::DRAIN_LIMIT_NS);
         }
-        if (OWNERS && owners > 0) ptx::mbar_wait_drain(k.bar(C::B_OWN), (owners - 1) & 1, ptx::DRAIN_LIMIT_NS);
+        if (OWNERS && owners + owners0 > 0) ptx::mbar_wait_drain(k.bar(C::B_OWN), (owners + owners0 - 1) & 1, ptx::DRAIN_LIMIT_NS);
+        if (OWNERS && C::OWN_SETS == 2 && owners > 0) ptx::mbar_wait_drain(k.bar(C::B_OWN + 1), (owners - 1) & 1, ptx::DRAIN_LIMIT_NS);
     }
 }
 
@@ -498,10 +508,10 @@ __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE
     for (int item = blockIdx.x; item < p.items; item += gridDim.x) {
         const int bh = item / p.row_tiles, next = item + (int)gridDim.x;
         for (int j = 0; j < T; ++j, ++g) {
-            if (g >= C::SL && !k.done(C::B_OUTDONE, g - C::SL)) return;
+            if (g >= C::SL && !k.done(C::B_LDONE, g - C::SL + C::LDONE_NEXT)) return;
             put(dl, sl, C::B_LFULL, a[0] * f_lse, a[1] * f_mu, a[2] * f_lse, a[3] * f_mu);
             if (++sl == C::SL) sl = 0;
-            if (g >= C::SE && !k.done(C::B_EDONE, g - C::SE)) return;
+            if (g >= C::SE && !k.done(C::B_EDONE, g - C::SE + C::EDONE_NEXT)) return;
             put(de, se, C::B_EFULL, b[0], b[1], b[2], b[3]);
             if (++se == C::SE) se = 0;
             const bool more = j + 1 < T;
@@ -512,7 +522,7 @@ __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE
 
 // ------------------------------------------------------------------------------------------------ MMA issue
 // The whole warp runs this in converged control flow; one elected lane issues (one election per batch of MMAs,
-// descriptors as 32-bit halves: see mma_ts_p).  Tensor memory starts at column 0, because the block owns all of it.
+// descriptors as 32-bit halves: see mma_ts_acc).  Tensor memory starts at column 0, because the block owns all of it.
 //
 // The tensor pipe takes about four MMAs ahead, 130 to 250 cycles of work; whatever the issuing warp does between two
 // batches beyond that leaves the pipe idle.  A wait for a barrier that has completed costs it 85 cycles, a commit 60, a
@@ -561,11 +571,27 @@ struct JvpIssue {
     // 1024 bytes, a k-step of 16 stream rows 2048
     static __host__ __device__ constexpr uint32_t l_n(int t, int u) { return (uint32_t)(t * ATOM + u * 2048) / 16 + lbo(2 * ATOM); }
 
+    // Long batches are loops: their code, run once a tile by one warp, else pushes the element-wise loops out of the instruction
+    // cache (head dims above 64: 4 to 8 % of a pass; DKV 3 %).  Short ones (d <= 64, without dtO) pay more for the loops.
+    static constexpr int UNROLL = !HZ && (DP > 64 || C::DKV) ? 1 : 8;
     // One k-step with A in tensor memory (ATM: a = its columns) or in shared memory (a = the tile's descriptor).
-    template <bool ATM, uint32_t ACC>
-    static __device__ __forceinline__ void step(uint32_t el, uint32_t col, uint32_t a, int kk, uint32_t b, uint32_t bhi, uint32_t idesc) {
-        if (ATM) ptx::mma_ts_p<ACC>(el, col, a + 8 * kk, b, bhi, idesc);
-        else ptx::mma_ss_p<ACC>(el, col, a + own_k(kk), is_tail(kk) ? HI_TAIL : HI_SW, b, bhi, idesc);
+    template <bool ATM>
+    static __device__ __forceinline__ void step(uint32_t el, uint32_t col, uint32_t a, uint32_t ahi, uint32_t b, uint32_t bhi, uint32_t idesc, uint32_t acc) {
+        if (ATM) ptx::mma_ts_acc(el, col, a, b, bhi, idesc, acc);
+        else ptx::mma_ss_acc(el, col, a, ahi, b, bhi, idesc, acc);
+    }
+    // The k-steps of a K-major product: f(a offset, a hi, b offset, b hi, first ? 0 : 1).
+    template <bool FROM_L, bool ATM, class F>
+    static __device__ __forceinline__ void ksteps(F f) {
+        constexpr int K0 = KS < 4 ? KS : 4;
+#pragma unroll UNROLL
+        for (int kk = 0; kk < K0; ++kk) f(ATM ? 8u * kk : 2u * kk, HI_SW, 2u * kk, HI_SW, kk ? 1u : 0u);
+        if constexpr (KS > 4) {
+            constexpr uint32_t b4 = FROM_L ? l_k(4) : e_k(4);
+#pragma unroll UNROLL
+            for (int kk = 0; kk < KS - 4; ++kk)
+                f(ATM ? 32u + 8u * kk : own_k(4) + 2u * kk, is_tail(4) ? HI_TAIL : HI_SW, b4 + 2u * kk, flat(FROM_L, 4) ? HI_TAIL : HI_SW, 1u);
+        }
     }
     // The statistics' own k-step (FOLD, where the padding columns do not hold them), tensor t0 on.
     static __device__ __forceinline__ void fold_step(uint32_t el, uint32_t col, const Block& k, uint32_t fold, int t0, uint32_t idesc) {
@@ -575,30 +601,24 @@ struct JvpIssue {
     // [S | X0 Y1^T] = X0 [Y0 | Y1]^T, Sd += X1 Y0^T at column col; FROM_L: the stage is one of the L ring.
     template <bool FROM_L, bool ATM, bool SECOND>
     static __device__ __forceinline__ void pair(uint32_t el, uint32_t col, const Block& k, uint32_t a0, uint32_t a1, uint32_t lo, uint32_t fold, uint32_t mid_bar) {
-#pragma unroll
-        for (int kk = 0; kk < KS; ++kk) {
-            const uint32_t b = lo + (FROM_L ? l_k(kk) : e_k(kk)), bhi = flat(FROM_L, kk) ? HI_TAIL : HI_SW;
-            if (kk == 0) step<ATM, 0>(el, col, a0, kk, b, bhi, I_S2);
-            else step<ATM, 1>(el, col, a0, kk, b, bhi, I_S2);
-        }
+        ksteps<FROM_L, ATM>([&](uint32_t ao, uint32_t ahi, uint32_t bo, uint32_t bhi, uint32_t acc) {
+            step<ATM>(el, col, a0 + ao, ahi, lo + bo, bhi, I_S2, acc);
+            if (SECOND && MODE != PASS_FWD) step<ATM>(el, col + BC, a1 + ao, ahi, lo + bo, bhi, I_S, 1u);
+        });
         if (k.fold_step()) fold_step(el, col, k, fold, 0, I_S2);
-        if (MODE == PASS_FWD) ptx::mma_commit_p(el, mid_bar);   // S is complete before Sd
-        if (SECOND) {
-#pragma unroll
-            for (int kk = 0; kk < KS; ++kk)
-                step<ATM, 1>(el, col + BC, a1, kk, lo + (FROM_L ? l_k(kk) : e_k(kk)), flat(FROM_L, kk) ? HI_TAIL : HI_SW, I_S);
+        if (MODE == PASS_FWD) {
+            ptx::mma_commit_p(el, mid_bar);   // S is complete before Sd
+            ksteps<FROM_L, ATM>([&](uint32_t ao, uint32_t ahi, uint32_t bo, uint32_t bhi, uint32_t) {
+                step<ATM>(el, col + BC, a1 + ao, ahi, lo + bo, bhi, I_S, 1u);
+            });
         }
     }
     // One product X Y^T with Y the T-th tensor of the stage.
     template <bool FROM_L, bool ATM, int T>
     static __device__ __forceinline__ void single(uint32_t el, uint32_t col, const Block& k, uint32_t a, uint32_t lo, uint32_t fold) {
-#pragma unroll
-        for (int kk = 0; kk < KS; ++kk) {
-            const bool tail = flat(FROM_L, kk);
-            const uint32_t b = lo + (FROM_L ? l_k(kk) : e_k(kk)) + ((uint32_t)(tail ? T * BC * 16 : T * ATOM) >> 4);
-            if (kk == 0) step<ATM, 0>(el, col, a, kk, b, tail ? HI_TAIL : HI_SW, I_S);
-            else step<ATM, 1>(el, col, a, kk, b, tail ? HI_TAIL : HI_SW, I_S);
-        }
+        ksteps<FROM_L, ATM>([&](uint32_t ao, uint32_t ahi, uint32_t bo, uint32_t bhi, uint32_t acc) {
+            step<ATM>(el, col, a + ao, ahi, lo + bo + ((uint32_t)(bhi == HI_TAIL ? T * BC * 16 : T * ATOM) >> 4), bhi, I_S, acc);
+        });
         if (k.fold_step()) fold_step(el, col, k, fold, T, I_S);
     }
     // Half of acc0 += A0 B0, acc1 += A1 B0 + A0 B1 (k-steps U0, U0 + 1 of four; the operand of a k-step lies at the columns of
@@ -609,24 +629,24 @@ struct JvpIssue {
         constexpr bool DV = MODE == PASS_DV, B0 = !HZ && !(DV && (ABS & ABSENT_HC)), A0 = !HZ && !(!DV && (ABS & ABSENT_HC)), B1 = !(DV && (ABS & ABSENT_G));
         // (DV: Hc is B0, G is B1; DK, DQ with Hc absent: A0 = W is exactly zero)
         constexpr bool T0 = A0 && B0, T1 = !DV ? true : B0, T2 = DV ? B1 : A0;   // A0 B0, A1 B0, A0 B1
-#pragma unroll
+#pragma unroll UNROLL
         for (int u = U0; u < U0 + 2; ++u) {
-            const uint32_t b0 = lo + l_n(0, u), b1 = lo + l_n(1, u);
-            if (T0) { if (u == 0) ptx::mma_ts_acc(el, c0, a0, b0, HI_SW, I_O, acc); else ptx::mma_ts_p<1>(el, c0, a0 + 16 * u, b0, HI_SW, I_O); }
-            if (T1) { if (u == 0) ptx::mma_ts_acc(el, c1, a1, b0, HI_SW, I_O, acc); else ptx::mma_ts_p<1>(el, c1, a1 + 16 * u, b0, HI_SW, I_O); }
-            if (T2) { if (u == 0 && !T1) ptx::mma_ts_acc(el, c1, a0, b1, HI_SW, I_O, acc); else ptx::mma_ts_p<1>(el, c1, a0 + 16 * u, b1, HI_SW, I_O); }
+            const uint32_t b0 = lo + l_n(0, 0) + 128u * u, b1 = lo + l_n(1, 0) + 128u * u, o = 16u * u, first = U0 > 0 || u > 0 ? 1u : acc;
+            if (T0) ptx::mma_ts_acc(el, c0, a0 + o, b0, HI_SW, I_O, first);
+            if (T1) ptx::mma_ts_acc(el, c1, a1 + o, b0, HI_SW, I_O, first);
+            if (T2) ptx::mma_ts_acc(el, c1, a0 + o, b1, HI_SW, I_O, T1 ? 1u : first);
         }
     }
-    // DKV: k-steps U0 .. U1 - 1 of acc[C] += A0 B0, acc[C + 1] += A1 B0 + A0 B1 (T0, T1, T2: which of the three there are).
-    template <int U0, int U1, bool T0, bool T1, bool T2, int ACC>
+    // DKV: acc[C] += A0 B0, acc[C + 1] += A1 B0 + A0 B1 (T0, T1, T2: which of the three there are).
+    template <bool T0, bool T1, bool T2, int ACC>
     static __device__ __forceinline__ void dkv_outputs(uint32_t el, uint32_t a0, uint32_t a1, uint32_t lo, uint32_t acc) {
         constexpr uint32_t c0 = ACC * DP, c1 = c0 + DP;
-#pragma unroll
-        for (int u = U0; u < U1; ++u) {
-            const uint32_t b0 = lo + l_n(0, u), b1 = lo + l_n(1, u), o = 16u * u;
-            if (T0) { if (u == 0) ptx::mma_ts_acc(el, c0, a0, b0, HI_SW, I_O, acc); else ptx::mma_ts_p<1>(el, c0, a0 + o, b0, HI_SW, I_O); }
-            if (T1) { if (u == 0) ptx::mma_ts_acc(el, c1, a1, b0, HI_SW, I_O, acc); else ptx::mma_ts_p<1>(el, c1, a1 + o, b0, HI_SW, I_O); }
-            if (T2) { if (u == 0 && !T1) ptx::mma_ts_acc(el, c1, a0, b1, HI_SW, I_O, acc); else ptx::mma_ts_p<1>(el, c1, a0 + o, b1, HI_SW, I_O); }
+#pragma unroll UNROLL
+        for (int u = 0; u < BC / 16; ++u) {
+            const uint32_t b0 = lo + l_n(0, 0) + 128u * u, b1 = lo + l_n(1, 0) + 128u * u, o = 16u * u, first = u > 0 ? 1u : acc;
+            if (T0) ptx::mma_ts_acc(el, c0, a0 + o, b0, HI_SW, I_O, first);
+            if (T1) ptx::mma_ts_acc(el, c1, a1 + o, b0, HI_SW, I_O, first);
+            if (T2) ptx::mma_ts_acc(el, c1, a0 + o, b1, HI_SW, I_O, T1 ? 1u : first);
         }
     }
 };
@@ -634,12 +654,16 @@ struct JvpIssue {
 // DKV: one buffer of (S, Sd | D, X), operands written over the scores.  Pipe order: outputs of the first pair (P, P Nn)(n - 1) |
 // (S, Sd)(n) | outputs of the second pair (W, dA)(n - 1) | (D, X)(n): what the element-wise warps do to one pair runs under
 // the MMAs of the other, so that no unit waits for the whole chain of a tile.  (d = 64, per 64 queries: MMAs of 1860 cycles
-// instead of 2250 in two passes, half the exponentials and loads.)
+// instead of 2250 in two passes, half the exponentials and loads.)  The element-wise warps are done 400 to 800 cycles before
+// their operands' turn, so this warp waits and commits twice per tile and no more: for the operands as a whole, together with
+// the next stage of the ring, and one completion for outputs and scores.  (Operands handed over in halves, a wait per barrier
+// and four commits: d = 72 (16, 16, 1024) 1034 -> 994 us for the backward, without dtO 656 -> 544.)  What bounds a tile now
+// is the pipe with two operands in shared memory, whose port the loads share: 2950 cycles, 2490 with nothing to load or compute.
 template <int MODE, int DP, bool HZ, int ABS>
 __device__ __forceinline__ void jvp_issue_dkv(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
     using C = JvpCfg<MODE, DP>;
     using I = JvpIssue<MODE, DP, HZ, ABS>;
-    constexpr int NU = C::BC / 16, LO = C::KLO, BC = C::BC;   // k-steps of an output; those of its first part
+    constexpr int BC = C::BC;
     const JvpBlock<MODE, DP> k = shared.pinned();
     const int T = jvp_pin(p.T), items = jvp_pin(p.items);
     const uint32_t x0 = ptx::desc_lo(k.own_tile(0), 16), x1 = ptx::desc_lo(k.own_tile(1), 16);
@@ -649,57 +673,49 @@ __device__ __forceinline__ void jvp_issue_dkv(const JvpParams& p, const JvpBlock
     JvpSlot e = I::e_slot(k), l = I::l_slot(k);   // next tile of the scores
     uint32_t elo = e.lo, llo = l.lo;              // stages of the outputs' tile
     int n = 0, it = 0;                            // next tile whose scores are issued
-    bool ready = false;
     for (int item = blockIdx.x; item < items; item += gridDim.x, ++it) {
         if (!k.wait(C::B_OWN, it)) return;
+        bool ready = false;                       // what the next batch waits for was seen complete
         for (int j = -1; j < T; ++j) {
+            const bool out = j >= 0, score = j + 1 < T;
             const uint32_t acc = j > 0 ? 1u : 0u;
-            if (j >= 0) {   // dtV += P^T Hc, dV += (P Nn)^T Hc + P^T G
-                if (!k.wait(C::B_PREADY, n - 1)) return;
-                if (j == 0 && !k.wait(C::B_ACCFREE, it - 1)) return;    // the first tile overwrites the accumulators
-                ptx::tc_fence_after_sync();
-                uint32_t el = ptx::elect_one();
-                I::template dkv_outputs<0, LO, H, H, G, 0>(el, cS, cT, elo, acc);
-                if (!k.wait(C::B_PREADY + 1, n - 1)) return;
-                ptx::tc_fence_after_sync();
-                el = ptx::elect_one();
-                I::template dkv_outputs<LO, NU, H, H, G, 0>(el, cS, cT, elo, acc);
-                ptx::mma_commit_p(el, k.bar(C::B_O1DONE + ((n - 1) & 3)));
-                elo = elo + I::E_STEP == e.lo0 + C::SE * I::E_STEP ? e.lo0 : elo + I::E_STEP;
-            }
-            if (j + 1 < T) {   // (S, Sd) of the next tile
-                if (!k.wait(C::B_LFULL + l.s, l.ph)) return;
-                k.tile_fence();
-                const uint32_t el = ptx::elect_one();
+            // dtV += P^T Hc, dV += (P Nn)^T Hc + P^T G | (S, Sd) of the next tile
+            if (!ready && !(score ? k.wait2(C::B_PREADY, n - 1, C::B_LFULL + l.s, l.ph) : k.wait(C::B_PREADY, n - 1))) return;
+            if (j == 0 && it > 0 && !k.wait(C::B_ACCFREE, it - 1)) return;    // the first tile overwrites the accumulators
+            k.tile_fence();
+            uint32_t el = ptx::elect_one();
+            if (out) I::template dkv_outputs<H, H, G, 0>(el, cS, cT, elo, acc);
+            if (score) {
+                ready = ptx::mbar_test2_warp(k.bar(C::B_PREADY + 1), (n - 1) & 1, k.bar(C::B_EFULL + e.s), e.ph);
                 if (HZ) I::template single<true, false, 0>(el, cS, k, x0, l.lo, l.fold);
                 else I::template pair<true, false, true>(el, cS, k, x0, x1, l.lo, l.fold, 0);
                 ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
+                if (j + 2 == T) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE));
                 l.template next<C::SL, I::L_STEP, I::F_STEP>();
-                ready = ptx::mbar_test_warp(k.bar(C::B_EFULL + e.s), e.ph);
+            } else {
+                ready = false;
             }
-            if (j >= 0) {   // dtK += W^T Q, dK += dA^T Q + W^T tQ
-                if (!k.wait(C::B_PREADY + 2, n - 1)) return;
-                ptx::tc_fence_after_sync();
-                uint32_t el = ptx::elect_one();
-                I::template dkv_outputs<0, LO, H, true, H, 2>(el, cD, cX, llo, acc);
-                if (!k.wait(C::B_PREADY + 3, n - 1)) return;
-                ptx::tc_fence_after_sync();
-                el = ptx::elect_one();
-                I::template dkv_outputs<LO, NU, H, true, H, 2>(el, cD, cX, llo, acc);
-                ptx::mma_commit_p(el, k.bar(C::B_OUTDONE + ((n - 1) & 3)));
-                if (j == T - 1) ptx::mma_commit_p(el, k.bar(C::B_FINAL));
+            // dtK += W^T Q, dK += dA^T Q + W^T tQ | (D, X) of the next tile
+            if (!ready && !(score ? k.wait2(C::B_PREADY + 1, n - 1, C::B_EFULL + e.s, e.ph) : k.wait(C::B_PREADY + 1, n - 1))) return;
+            if (!out && !k.wait(C::B_OWN + 1, it)) return;
+            k.tile_fence();
+            el = ptx::elect_one();
+            if (out) {
+                I::template dkv_outputs<H, true, H, 2>(el, cD, cX, llo, acc);
+                elo = elo + I::E_STEP == e.lo0 + C::SE * I::E_STEP ? e.lo0 : elo + I::E_STEP;
                 llo = llo + I::L_STEP == l.lo0 + C::SL * I::L_STEP ? l.lo0 : llo + I::L_STEP;
             }
-            if (j + 1 < T) {   // (D, X) of the next tile
-                if (!ready && !k.wait(C::B_EFULL + e.s, e.ph)) return;
-                k.tile_fence();
-                const uint32_t el = ptx::elect_one();
+            if (score) {
+                // (the stage of the tile after the next one, where there is one)
+                ready = j + 2 < T && ptx::mbar_test2_warp(k.bar(C::B_PREADY), n & 1, k.bar(C::B_LFULL + l.s), l.ph);
                 if (HZ) I::template single<false, false, 1>(el, cX, k, x2, e.lo, e.fold);   // X = V G^T alone
                 else I::template pair<false, false, H>(el, cD, k, x2, x3, e.lo, e.fold, 0);  // (tV Hc^T is zero with Hc absent)
                 ptx::mma_commit_p(el, k.bar(C::B_XFULL + (n & 3)));
-                if (j + 2 == T) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE));
+                if (j + 2 == T) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE + 1));
                 e.template next<C::SE, I::E_STEP, I::F_STEP>();
                 ++n;
+            } else {
+                ptx::mma_commit_p(el, k.bar(C::B_FINAL));
             }
         }
     }
@@ -1166,7 +1182,7 @@ __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const Jvp
 template <int DP, bool HZ>
 __device__ __forceinline__ void jvp_elem_dkv(const JvpParams& p, const JvpBlock<PASS_DKV, DP>& k, int grp, int q, int lane) {
     using C = JvpCfg<PASS_DKV, DP>;
-    constexpr int BC = C::BC, NU = BC / 16, LO = C::KLO;
+    constexpr int BC = C::BC, NU = BC / 16;
     const uint32_t sb = (static_cast<uint32_t>(q * 32 + grp * 16) << 16) + C::COL_SCORE;
     const uint64_t c2c2 = ptx::pack2(p.c2, p.c2), aa = ptx::pack2(p.alpha, p.alpha);
     const int n_it = (int)blockIdx.x < p.items ? (p.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
@@ -1200,11 +1216,9 @@ __device__ __forceinline__ void jvp_elem_dkv(const JvpParams& p, const JvpBlock<
             }
             ptx::tmem_st16_128x2(sb + 16 * u, a0);
             if (!HZ) ptx::tmem_st16_128x2(sb + BC + 16 * u, a1);
-            if (u == LO - 1 || u == NU - 1) {
-                ptx::tmem_wait_st();
-                k.arrive(C::B_PREADY + (u == NU - 1), lane);
-            }
         }
+        ptx::tmem_wait_st();
+        k.arrive(C::B_PREADY, lane);
         if (!k.done(C::B_XFULL, g)) return;
         ptx::tc_fence_after_sync();
 #pragma unroll
@@ -1232,11 +1246,9 @@ __device__ __forceinline__ void jvp_elem_dkv(const JvpParams& p, const JvpBlock<
             }
             if (!HZ) ptx::tmem_st16_128x2(sb + 2 * BC + 16 * u, a0);
             ptx::tmem_st16_128x2(sb + 3 * BC + 16 * u, a1);
-            if (u == LO - 1 || u == NU - 1) {
-                ptx::tmem_wait_st();
-                k.arrive(C::B_PREADY + 2 + (u == NU - 1), lane);
-            }
         }
+        ptx::tmem_wait_st();
+        k.arrive(C::B_PREADY + 1, lane);
     }
 }
 
@@ -1372,11 +1384,11 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
         auto init = [&](int b, int n, int count) { for (int i = 0; i < n; ++i) ptx::mbar_init(k.bar(b + i), count); };
         init(C::B_EFULL, C::SE, C::EFULL_COUNT);
         init(C::B_LFULL, C::SL, C::LFULL_COUNT);
-        init(C::B_OWN, 1, C::TAIL ? 33 : 1);
-        init(C::B_OWNFREE, 1, 1);
+        init(C::B_OWN, C::OWN_SETS, C::TAIL ? 33 : 1);
+        init(C::B_OWNFREE, C::OWN_SETS, 1);
         init(C::B_XRDY, 1, 4);
         init(C::B_XFREE, 1, 1);
-        init(C::B_SFULL, 16, 1);       // SFULL, XFULL, OUTDONE, O1DONE
+        init(C::B_SFULL, 12, 1);       // SFULL, XFULL, OUTDONE
         init(C::B_PREADY, 4, C::DKV ? 8 : 4);   // (of four: the warps of a group)
         init(C::B_SREAD, 1, 8);
         init(C::B_FINAL, 1, 1);
@@ -1443,8 +1455,8 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
         ptx::setmaxnreg_dec<C::REGS_LOAD>();
         if (placed) {
             const CUtensorMap* const maps[4] = {&o0, &o1, &o2, &o3};
-            if (warp == 0) jvp_load_ring<MODE, DP, 0>(p, k, &s0, &s1, maps, lane);
-            else if (warp == 2) jvp_load_ring<MODE, DP, 1>(p, k, &s2, &s3, maps, lane);
+            if (warp == 0) jvp_load_ring<MODE, DP, HZ, 0>(p, k, &s0, &s1, maps, lane);
+            else if (warp == 2) jvp_load_ring<MODE, DP, HZ, 1>(p, k, &s2, &s3, maps, lane);
             else if (warp == 1) jvp_issue<MODE, DP, HZ>(p, k);
             else if constexpr (C::FOLD) jvp_fold<MODE, DP>(p, k, lane);
         }

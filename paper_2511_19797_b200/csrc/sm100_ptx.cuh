@@ -214,17 +214,6 @@ __host__ __device__ constexpr uint32_t desc_hi_nosw(uint32_t sbo_bytes) { return
 __device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes) {
     return ((saddr & 0x3FFFFu) >> 4) | (((lbo_bytes >> 4) & 0x3FFFu) << 16);
 }
-template <uint32_t ACC>
-__device__ __forceinline__ void mma_ts_p(uint32_t el, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .pred e;\n\t.reg .b64 b;\n\t"
-        "setp.ne.b32 e, %0, 0;\n\t"
-        "setp.ne.b32 p, %6, 0;\n\t"
-        "mov.b64 b, {%3, %4};\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%1], [%2], b, %5, p;\n\t}"
-        ::"r"(el), "r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "n"(ACC)
-        : "memory");
-}
 __device__ __forceinline__ void mma_ts_acc(uint32_t el, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t.reg .pred e;\n\t.reg .b64 b;\n\t"
@@ -245,6 +234,17 @@ __device__ __forceinline__ void mma_ss_p(uint32_t el, uint32_t d_tmem, uint32_t 
         "mov.b64 b, {%4, %5};\n\t"
         "@e tcgen05.mma.cta_group::1.kind::f16 [%1], a, b, %6, p;\n\t}"
         ::"r"(el), "r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "n"(ACC)
+        : "memory");
+}
+__device__ __forceinline__ void mma_ss_acc(uint32_t el, uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .pred e;\n\t.reg .b64 a;\n\t.reg .b64 b;\n\t"
+        "setp.ne.b32 e, %0, 0;\n\t"
+        "setp.ne.b32 p, %7, 0;\n\t"
+        "mov.b64 a, {%2, %3};\n\t"
+        "mov.b64 b, {%4, %5};\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%1], a, b, %6, p;\n\t}"
+        ::"r"(el), "r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 __device__ __forceinline__ void mma_commit_p(uint32_t el, uint32_t bar) {

@@ -269,6 +269,8 @@ static int launch_pass(const Shape& s, const Operand (&own)[4], const Operand (&
         prm.own[t] = own[t].ptr;
         prm.strm[t] = strm[t].ptr;
     }
+    if (HZ) prm.own[1] = nullptr;             // tangents of the owner side: not loaded
+    if (HZ && C::DKV) prm.own[3] = nullptr;
     // one CTA per SM (each needs the whole tensor memory and most of the shared memory of one); the work
     // items go round-robin over them
     prm.row_tiles = (prm.o.rows + JVP_ROWS - 1) / JVP_ROWS;
