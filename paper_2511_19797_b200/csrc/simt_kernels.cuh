@@ -159,84 +159,6 @@ simt_fwd_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __res
     }
 }
 
-// ------------------------------------------------------------------------------------------------
-// Backward pre-pass (App. C "Step 1", reduced by the identities Sigma_1 = rowsum(dtO*O),
-// Sigma_2 = rowsum(dtO*tO) and the standard-attention row term rowsum(dO*O)):
-//   sig1[row] = sum_c Hc*O        cvec[row] = sum_c G*O + Hc*tO        lse2[row] = lse[row] * log2(e)
-// Pure streaming work (four tensors read once), so it is laid out for the memory system: every lane
-// loads 16 bytes per tensor, a row is shared by the smallest power-of-two group of lanes that covers
-// its d * sizeof(T) / 16 chunks, and a warp has the loads of ROWSUM_UNROLL row groups in flight
-// before it touches the first.
-constexpr int ROWSUM_THREADS = 256;
-constexpr int ROWSUM_UNROLL = 2;
-
-__device__ __forceinline__ void dot_chunk(const uint4& a, const uint4& b, float& acc, float) {
-    const float* x = reinterpret_cast<const float*>(&a);
-    const float* y = reinterpret_cast<const float*>(&b);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) acc = fmaf(x[i], y[i], acc);
-}
-__device__ __forceinline__ void dot_chunk(const uint4& a, const uint4& b, float& acc, __nv_bfloat16) {
-    const __nv_bfloat162* x = reinterpret_cast<const __nv_bfloat162*>(&a);
-    const __nv_bfloat162* y = reinterpret_cast<const __nv_bfloat162*>(&b);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float2 xf = __bfloat1622float2(x[i]), yf = __bfloat1622float2(y[i]);
-        acc = fmaf(xf.x, yf.x, acc);
-        acc = fmaf(xf.y, yf.y, acc);
-    }
-}
-
-// `gs` = lanes per row = chunks per row `cpr`; rows per warp = 32 / gs (the lanes left over idle).
-template <typename T>
-__global__ void __launch_bounds__(ROWSUM_THREADS)
-bwd_rowsums_kernel(const T* __restrict__ G, const T* __restrict__ Hc, const T* __restrict__ O,
-                   const T* __restrict__ tO, const float* __restrict__ lse, float* __restrict__ sig1,
-                   float* __restrict__ cvec, float* __restrict__ lse2, long long rows, Geom qg, int H, int d, int cpr,
-                   int gs, float sign) {
-    constexpr int VEC = 16 / (int)sizeof(T);
-    const int lane = threadIdx.x & 31;
-    const int rpw = 32 / gs;                  // rows per warp and step
-    const int sub = lane / gs, c = lane - sub * gs;
-    const long long warp_id = (long long)blockIdx.x * (ROWSUM_THREADS / 32) + (threadIdx.x >> 5);
-    const long long row0 = warp_id * (ROWSUM_UNROLL * rpw) + sub;
-    uint4 g[ROWSUM_UNROLL], h[ROWSUM_UNROLL], o[ROWSUM_UNROLL], t[ROWSUM_UNROLL];
-    bool act[ROWSUM_UNROLL];
-#pragma unroll
-    for (int u = 0; u < ROWSUM_UNROLL; ++u) {
-        const long long row = row0 + (long long)u * rpw;
-        act[u] = row < rows && c < cpr && sub < rpw;
-        g[u] = h[u] = t[u] = make_uint4(0, 0, 0, 0);  // a null G or Hc (absent cotangent) counts as zeros
-        if (act[u]) {
-            // the statistics are packed (B, H, M); the tensors have strides (H == 0 marks the packed layout: no division)
-            size_t off = (size_t)row * d + (size_t)c * VEC;
-            if (H > 0) {
-                const unsigned bh = (unsigned)row / (unsigned)qg.rows;   // rows fit 31 bits
-                off = qg.head_off((int)bh, H) + (size_t)((unsigned)row - bh * (unsigned)qg.rows) * (size_t)qg.rs + (size_t)c * VEC;
-            }
-            o[u] = __ldg(reinterpret_cast<const uint4*>(O + off));
-            if (G) g[u] = __ldg(reinterpret_cast<const uint4*>(G + off));
-            if (Hc) {
-                h[u] = __ldg(reinterpret_cast<const uint4*>(Hc + off));
-                t[u] = __ldg(reinterpret_cast<const uint4*>(tO + off));
-            }
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < ROWSUM_UNROLL; ++u) {
-        const long long row = row0 + (long long)u * rpw;
-        float s1 = 0.f, cc = 0.f;
-        if (act[u]) {
-            dot_chunk(h[u], o[u], s1, T());
-            dot_chunk(g[u], o[u], cc, T());
-            dot_chunk(h[u], t[u], cc, T());
-        }
-        s1 = lane_group_sum(s1, gs, lane);
-        cc = lane_group_sum(cc, gs, lane);
-        if (c == 0 && sub < rpw && row < rows) { sig1[row] = sign * s1; cvec[row] = sign * cc; lse2[row] = sign * (lse[row] * 1.4426950408889634f); }
-    }
-}
-
 // Writes zeros to every row of a tensor with strides (the gradients that are identically zero when a cotangent is
 // absent); 16 bytes per thread.
 __global__ void __launch_bounds__(256)

@@ -14,6 +14,7 @@
 
 #include "jvp_sm100.cuh"
 #include "qk_rmsnorm.cuh"
+#include "rowsums.cuh"
 #include "simt_kernels.cuh"
 
 namespace tvm_attn {
@@ -186,15 +187,15 @@ static bool q_packed(const Shape& s) {
 template <typename T>
 static int launch_rowsums(const Shape& s, const void* G, const void* Hc, const void* O, const void* tO, const float* lse,
                           float* sig1, float* cvec, float* lse2, float sign, cudaStream_t st) {
-    const long long rows = s.BH * s.M;
-    const int cpr = s.d * (int)sizeof(T) / 16;  // 16-byte chunks per row (d % 8 == 0)
-    const int gs = cpr;                          // lanes per row
-    if (gs > 32) return TVM_ATTN_UNSUPPORTED;   // d <= 128 keeps a row within one warp
-    const long long rows_per_block = (long long)(ROWSUM_THREADS / 32) * ROWSUM_UNROLL * (32 / gs);
-    const unsigned grid = (unsigned)((rows + rows_per_block - 1) / rows_per_block);
+    const long long rows = s.BH * s.M;           // fit 31 bits
+    const int cpr = s.d * (int)sizeof(T) / 16;   // 16-byte chunks per row (d % 8 == 0)
+    if (cpr > 32) return TVM_ATTN_UNSUPPORTED;   // d <= 128
+    const int C = rms_split(cpr, 4), P = cpr / C;
+    const long long rows_per_block = (ROWSUM_THREADS / 32) * (32 / P), blocks = (rows + rows_per_block - 1) / rows_per_block;
+    const auto kern = C == 4 ? bwd_rowsums_kernel<T, 4> : C == 3 ? bwd_rowsums_kernel<T, 3> : C == 2 ? bwd_rowsums_kernel<T, 2> : bwd_rowsums_kernel<T, 1>;
     g_prof.before(st);
-    bwd_rowsums_kernel<T><<<grid, ROWSUM_THREADS, 0, st>>>((const T*)G, (const T*)Hc, (const T*)O, (const T*)tO, lse, sig1,
-                                                           cvec, lse2, rows, s.q, q_packed(s) ? 0 : s.H, s.d, cpr, gs, sign);
+    kern<<<(unsigned)(blocks < ROWSUM_BLOCKS ? blocks : ROWSUM_BLOCKS), ROWSUM_THREADS, 0, st>>>(
+        (const T*)G, (const T*)Hc, (const T*)O, (const T*)tO, lse, sig1, cvec, lse2, (unsigned)rows, s.q, q_packed(s) ? 0 : s.H, s.d, P, sign);
     g_prof.after(st);
     g_launches += 1;
     return cuda_status(cudaGetLastError());

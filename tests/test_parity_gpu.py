@@ -71,6 +71,17 @@ def test_wide_head_dims_with_several_items_per_block(B, H, N, d, peaky):
     assert_within(errs, BF16_FWD, BF16_BWD, BF16_STATS)
 
 
+# row sums of the backward: every split of a row over lanes and chunks, rows that do not fill a warp
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("N,d", [(1, 8), (37, 24), (33, 40), (11, 48), (41, 96), (7, 104), (19, 120)])
+def test_row_sums_of_every_split(N, d, dtype):
+    errs, _, _ = run_case(inputs.custom(1, 3, N, d, seed=700 + d), dtype=dtype)
+    if dtype == torch.float32:
+        assert_within(errs, FP32_TOL, FP32_TOL)
+    else:
+        assert_within(errs, BF16_FWD, BF16_BWD, BF16_STATS)
+
+
 # key and value gradients of one pass: edges of its query tiles (48 rows at d = 72 and 80, else 64) and of the 128 keys of an item
 @pytest.mark.parametrize("absent", [None, "dtO", "dO"])
 @pytest.mark.parametrize("N,d", [(1, 72), (47, 72), (48, 80), (49, 72), (97, 80), (145, 72), (33, 64), (64, 64), (127, 48), (193, 16)])
