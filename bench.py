@@ -37,8 +37,9 @@ BWD_KERNELS = {"narrow": {"bwd_rowsums": (0, 4), "bwd_dkv": (12, 12), "bwd_dq": 
                "wide": {"bwd_rowsums": (0, 4), "bwd_dv": (6, 8), "bwd_dk": (9, 10), "bwd_dq": (9, 10)},
                "detach": {"bwd_rowsums": (0, 2), "bwd_dkv": (4, 6), "bwd_dq": (3, 5)}}
 BWD_CREDITED_GEMMS = 15
-# dram__bytes_read.sum + dram__bytes_write.sum per launch from an ncu capture of the present kernels (None where there is none)
-NCU_TRAFFIC_BYTES = {}
+# dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu capture summarised in
+# profiles/jvp_fwd_bwd_kernels_dit512.md (that workload and the full variant only; None for anything else)
+NCU_TRAFFIC_BYTES = {"dit512": {"fwd": 279.8e6, "bwd_dkv": 420.8e6, "bwd_dq": 360.3e6}}
 
 
 def load_peaks():
@@ -426,7 +427,7 @@ def main():
     step_tensor_frac = (f_fwd + f_bwd) / (ms_step * 1e-3) / 1e12 / peak
     step_hbm_frac = step_bytes / (ms_step * 1e-3) / 1e9 / peaks["hbm_gbs"]
     fwd_hbm_frac = kernel_tensors["fwd"] * tensor_bytes / (ms_fwd / args.steps * 1e-3) / 1e9 / peaks["hbm_gbs"]
-    traffic = NCU_TRAFFIC_BYTES.get(args.workload)
+    traffic = None if detach else NCU_TRAFFIC_BYTES.get(args.workload)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "bf16",
