@@ -138,13 +138,14 @@ long long integer(PyObject* o) {
     if (v == -1 && PyErr_Occurred()) throw python_error();
     return v;
 }
-// The n entries of a sequence as optional tensors.
-void entries(PyObject* o, int n, at::Tensor* to) {
-    PyObject* s = PySequence_Fast(o, "`out` must be a sequence of tensors");
+// The n entries of `out` as optional tensors.  Returns the list or tuple that they were read from: an iterator has nothing
+// left to give after that, so results are made from what is returned here, never from `o` again.
+THPObjectPtr entries(PyObject* o, int n, at::Tensor* to) {
+    THPObjectPtr s(PySequence_Fast(o, "`out` must be a sequence of tensors"));
     if (!s) throw python_error();
-    const THPObjectPtr hold(s);
-    if (PySequence_Fast_GET_SIZE(s) != n) throw ValueError("`out` must hold one entry per output");
-    for (int i = 0; i < n; ++i) to[i] = optional_tensor(PySequence_Fast_GET_ITEM(s, i));
+    if (PySequence_Fast_GET_SIZE(s.get()) != n) throw ValueError("`out` must hold one entry per output");
+    for (int i = 0; i < n; ++i) to[i] = optional_tensor(PySequence_Fast_GET_ITEM(s.get(), i));
+    return s;
 }
 
 // fwd(Q, K, V, tQ, tK, tV, scale, flags, out | None, stream | None)
@@ -153,7 +154,8 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const at::Tensor &Q = tensor(a[0]), &K = tensor(a[1]), &V = tensor(a[2]), &tQ = tensor(a[3]), &tK = tensor(a[4]), &tV = tensor(a[5]);
         const bool given = a[8] != Py_None;
         at::Tensor o[4];
-        if (given) entries(a[8], 4, o);
+        THPObjectPtr outs;
+        if (given) outs = entries(a[8], 4, o);
         const at::Tensor* qs[] = {&tQ, &o[0], &o[1]};
         const at::Tensor* ks[] = {&V, &tK, &tV};
         check_side(Q, qs, 3);
@@ -171,7 +173,7 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
                          nullptr, 0, st);
         });
         if (rc != TVM_ATTN_OK) return PyLong_FromLong(rc);
-        return given ? PySequence_Tuple(a[8]) : tuple_of(o, 4);
+        return given ? PySequence_Tuple(outs.get()) : tuple_of(o, 4);
     });
 }
 
@@ -185,7 +187,8 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const tvm_attn_params p = params(Q, K, number(a[12]), integer(a[13]));
         const bool given = a[14] != Py_None, noalloc = a[17] == Py_True;
         at::Tensor o[6];
-        if (given) entries(a[14], 6, o);
+        THPObjectPtr outs;
+        if (given) outs = entries(a[14], 6, o);
         else if (noalloc) throw ValueError("`out` must hold the six gradients");
         const at::Tensor* qs[] = {&tQ, &O, &tO, &dO, &dtO, &o[0], &o[3]};
         const at::Tensor* ks[] = {&V, &tK, &tV, &o[1], &o[2], &o[4], &o[5]};
@@ -208,7 +211,7 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
                          ptr(dtO), ptr(o[0]), ptr(o[1]), ptr(o[2]), ptr(o[3]), ptr(o[4]), ptr(o[5]), ptr(ws), (size_t)ws.numel(), st);
         });
         if (rc != TVM_ATTN_OK) return PyLong_FromLong(rc);
-        return given ? (noalloc ? PySequence_Tuple(a[14]) : same(a[14])) : tuple_of(o, 6);
+        return given ? (noalloc ? PySequence_Tuple(outs.get()) : same(a[14])) : tuple_of(o, 6);
     });
 }
 

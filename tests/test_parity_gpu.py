@@ -416,3 +416,18 @@ def test_detached_backward_needs_no_tangent_gradient_buffers():
     with pytest.raises(binding.TvmAttnError) as e:        # dtO given: its gradients need somewhere to go
         binding.tvm_attn_jvp_bwd(*args, x["dO"], x["dtO"], out=three)
     assert e.value.code == -1
+
+
+def test_forward_outputs_given_by_an_iterator_are_returned():
+    """`out` of the forward may be anything that yields the four tensors, also once only; they come back as a tuple."""
+    wl = inputs.custom(1, 2, 130, 72, seed=23)
+    x = [v.to(torch.bfloat16).cuda() for v in list(inputs.make_inputs(wl).values())[:6]]
+    want = binding.tvm_attn_jvp_fwd(*x)
+    given = [torch.zeros_like(t) for t in want]
+    for out in (iter(given), (t for t in given), list(given), tuple(given)):
+        got = binding.tvm_attn_jvp_fwd(*x, out=out)
+        binding.tvm_attn_check_status()
+        assert isinstance(got, tuple) and len(got) == 4
+        for a, b, c in zip(got, given, want):
+            assert a is b and torch.equal(a, c)
+            a.zero_()
