@@ -139,8 +139,13 @@ long long integer(PyObject* o) {
     return v;
 }
 // The n entries of `out` as optional tensors.  Returns the list or tuple that they were read from: an iterator has nothing
-// left to give after that, so results are made from what is returned here, never from `o` again.
-THPObjectPtr entries(PyObject* o, int n, at::Tensor* to) {
+// left to give after that, so results are made from what is returned here, never from `o` again.  `indexable`: the caller
+// gets `o` itself back, so an iterator is refused.
+THPObjectPtr entries(PyObject* o, int n, at::Tensor* to, bool indexable) {
+    if (indexable && !PySequence_Check(o) && !PyMapping_Check(o)) {   // (a tensor of stacked outputs is a mapping)
+        PyErr_Format(PyExc_TypeError, "'%.200s' object is not subscriptable: `out` must be a sequence of tensors", Py_TYPE(o)->tp_name);
+        throw python_error();
+    }
     THPObjectPtr s(PySequence_Fast(o, "`out` must be a sequence of tensors"));
     if (!s) throw python_error();
     if (PySequence_Fast_GET_SIZE(s.get()) != n) throw ValueError("`out` must hold one entry per output");
@@ -155,7 +160,7 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const bool given = a[8] != Py_None;
         at::Tensor o[4];
         THPObjectPtr outs;
-        if (given) outs = entries(a[8], 4, o);
+        if (given) outs = entries(a[8], 4, o, false);
         const at::Tensor* qs[] = {&tQ, &o[0], &o[1]};
         const at::Tensor* ks[] = {&V, &tK, &tV};
         check_side(Q, qs, 3);
@@ -188,7 +193,7 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const bool given = a[14] != Py_None, noalloc = a[17] == Py_True;
         at::Tensor o[6];
         THPObjectPtr outs;
-        if (given) outs = entries(a[14], 6, o);
+        if (given) outs = entries(a[14], 6, o, true);
         else if (noalloc) throw ValueError("`out` must hold the six gradients");
         const at::Tensor* qs[] = {&tQ, &O, &tO, &dO, &dtO, &o[0], &o[3]};
         const at::Tensor* ks[] = {&V, &tK, &tV, &o[1], &o[2], &o[4], &o[5]};

@@ -87,3 +87,17 @@ def test_binding_refuses_cpu_tensors():
     x = torch.zeros(1, 1, 8, 8, dtype=torch.bfloat16)
     with pytest.raises(ValueError):
         binding.tvm_attn_jvp_fwd(x, x, x, x, x, x)
+
+
+@pytest.mark.parametrize("noalloc", [False, True])
+def test_backward_refuses_outputs_it_could_not_give_back(noalloc):
+    """The backward returns `out` as it was given: an iterator, empty once its tensors have been read, is refused."""
+    import torch
+    x = torch.zeros(1, 1, 8, 8, dtype=torch.bfloat16)
+    stats = torch.zeros(1, 1, 8)
+    call = binding.tvm_attn_jvp_bwd_noalloc if noalloc else binding.tvm_attn_jvp_bwd
+    with pytest.raises(TypeError, match="not subscriptable"):
+        call(x, x, x, x, x, x, x, x, stats, stats, x, x, out=iter([x] * 6))
+    for out in ([x] * 6, torch.stack([x] * 6)):
+        with pytest.raises(ValueError, match="CUDA"):       # read, and refused for its CPU tensors
+            call(x, x, x, x, x, x, x, x, stats, stats, x, x, out=out)
