@@ -69,7 +69,11 @@ constexpr int JVP_BC = 64;      // stream rows per tile (DKV at padded head dim 
 // Forward, how far the row reference m may lag behind the running maximum (log2 units), and for WIDE head dims how far the
 // centre c of the tangent weights may be from T at the arg-max key before it moves.
 constexpr float JVP_LAZY_LOG2 = 3.0f, JVP_LAZY_LOG2_WIDE = 8.0f, JVP_CENTRE_WIDE = 3.0f;
-constexpr uint64_t JVP_WAIT_LIMIT_NS = 200ull * 1000ull * 1000ull;
+// How long a wait may take: for what is due within a few tiles, and what every tile of an item adds to it where an item's end
+// is waited for (the epilogue).  The slowest tile measured takes 2.7 us (DKV, 2950 cycles at 1.1 GHz); an item of 400 thousand
+// tiles, 128 queries against 25.6 million keys at d = 8, takes 0.24 s.  A tile that hangs is reported after the first limit
+// all the same, by the roles that work on it.
+constexpr uint64_t JVP_WAIT_LIMIT_NS = 200ull * 1000ull * 1000ull, JVP_TILE_LIMIT_NS = 20ull * 1000ull;
 // Registers per thread at launch; setmaxnreg moves them between the four warpgroups (JvpCfg::REGS_*) within what the block
 // was launched with: the host refuses to launch a build whose kernels have fewer.
 constexpr int JVP_REGS = 128;
@@ -223,6 +227,10 @@ struct JvpBlock {
     __device__ __forceinline__ uint32_t bar(int i) const { return base + MISC + 8u * static_cast<uint32_t>(i); }
     __device__ __forceinline__ bool wait(int i, int phase) const {
         return ptx::mbar_wait_warp_s(bar(i), phase & 1, base + ABORT, JVP_WAIT_LIMIT_NS);
+    }
+    // For what comes at the end of an item the caller has just begun to wait for.
+    __device__ __forceinline__ bool wait_item(int i, int phase) const {
+        return ptx::mbar_wait_warp_s(bar(i), phase & 1, base + ABORT, JVP_WAIT_LIMIT_NS + static_cast<uint64_t>(p.T) * JVP_TILE_LIMIT_NS);
     }
     __device__ __forceinline__ bool wait2(int i, int pi, int j, int pj) const {
         if (ptx::mbar_test2_warp(bar(i), pi & 1, bar(j), pj & 1)) return true;
@@ -1308,7 +1316,7 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
         if (C::XT && item + (int)gridDim.x < p.items) {
             load_x(item + gridDim.x, 0, v0);                       // in flight during the wait
             if (MODE != PASS_FWD) load_x(item + gridDim.x, 1, v1);   // (the forward has no registers for the second)
-            if (!k.wait(C::B_XFREE, it)) return;
+            if (!k.wait_item(C::B_XFREE, it)) return;
             ptx::tc_fence_after_sync();
             store_x(0, v0);
             if (MODE == PASS_FWD) load_x(item + gridDim.x, 1, v0);
@@ -1322,7 +1330,7 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
         const bool ok_even = row0 + (row & ~1) < p.o.rows, ok_odd = row0 + (row | 1) < p.o.rows;
         float f0 = p.out_scale, mun = 0.f;
         if constexpr (MODE == PASS_FWD) {   // O = O~/l, tO = R/l - (mu - c) O
-            if (!k.wait(C::B_ROWSTAT, it)) return;
+            if (!k.wait_item(C::B_ROWSTAT, it)) return;
             const int last = (it * p.T + p.T - 1) & 1;   // the group whose reference is the accumulators'
             const float4 f = k.row_sums(last * JVP_ROWS + row), o = k.row_sums((last ^ 1) * JVP_ROWS + row);
             const float scale = ptx::ex2(o.z - f.z);     // (a group without a tile: m = -inf, factor 0)
@@ -1335,7 +1343,7 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
                 p.mu_out[at] = f.w + mun;
             }
         }
-        if (!k.wait(C::B_FINAL, it)) return;
+        if (!k.wait_item(C::B_FINAL, it)) return;
         ptx::tc_fence_after_sync();
 #pragma unroll 1
         for (int i = 0; i < C::KS * (C::NACC / 2); ++i) {

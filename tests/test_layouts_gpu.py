@@ -171,3 +171,27 @@ def test_strides_that_cannot_be_read_are_refused():
     with pytest.raises(binding.TvmAttnError) as e:
         binding.tvm_attn_jvp_fwd(x, k, k, x, k, k)
     assert e.value.code == -2 and big.M == 32
+
+
+def test_an_item_of_many_tiles_is_not_taken_for_one_that_hangs():
+    """Half a million key tiles against one item of 128 queries: the kernels' epilogues wait for 0.3 s (forward) before the
+    first accumulators come to them, longer than a tile may take.  All keys but the last 1024 have scores 1000 / sqrt(8) below
+    the others', so that their weights are exactly zero (in fp32 as in fp64) and the oracle needs the 1024 only."""
+    M, N, real, d = 128, 32_000_000, 1024, 8
+    gen = torch.Generator(device="cuda").manual_seed(31)
+    draw = lambda rows, std=1.0: (std * torch.randn(1, 1, rows, d, generator=gen, device="cuda")).to(torch.bfloat16)
+    Q, tQ, dO, dtO = draw(M), draw(M, 0.5), draw(M), draw(M)
+    K, V, tK, tV = draw(N), draw(N), draw(N, 0.5), draw(N, 0.5)
+    Q[..., 0] = 1.0
+    K[..., :N - real, 0] = -1000.0
+    K[..., N - real:, 0] = 0.0
+    got = _gpu({"Q": Q, "K": K, "V": V, "tQ": tQ, "tK": tK, "tV": tV, "dO": dO, "dtO": dtO})   # (checks the status)
+    cut = lambda t: t[:, :, N - real:]
+    ref = _oracle({k: v.cpu() for k, v in dict(Q=Q, K=cut(K), V=cut(V), tQ=tQ, tK=cut(tK), tV=cut(tV), dO=dO, dtO=dtO).items()}, d)
+    errs = {}
+    for k, r in ref.items():
+        if k in ("dK", "dV", "dtK", "dtV"):
+            assert not got[k][:, :, :N - real].any(), k
+            got[k] = cut(got[k])
+        errs[k] = rel_err(got[k].float().cpu().numpy(), r)
+    assert_within(errs, 1e-2, 2e-2, 1e-4)
