@@ -103,9 +103,10 @@ def _load_native():
     """The native half of the binding, bound to the library's entry points.  Raises if it is not built."""
     global _native
     lib = load()
-    if not os.path.exists(_build.BINDING_PATH):
-        raise FileNotFoundError("%s is missing: run paper_2511_19797_b200/build.py first" % _build.BINDING_PATH)
-    spec = importlib.util.spec_from_file_location("_tvm_binding", _build.BINDING_PATH)
+    path = _build.binding_path()
+    if not os.path.exists(path):
+        raise FileNotFoundError("%s is missing: run paper_2511_19797_b200/build.py first (it is built for one PyTorch)" % path)
+    spec = importlib.util.spec_from_file_location("_tvm_binding", path)
     native = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(native)
     native.bind(*[ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in _BOUND])

@@ -1,7 +1,9 @@
 """Builds the CUDA library in-tree with nvcc for sm_100a (cross-compiles without a GPU), and the native half of its
 Python binding with g++ against the installed PyTorch."""
 import os
+import re
 import subprocess
+import sys
 import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -10,7 +12,6 @@ CSRC = os.path.join(_HERE, "csrc")
 LIB_DIR = os.path.join(_HERE, "_lib")
 LIB_PATH = os.path.join(LIB_DIR, "libtvm_attn.so")
 SOURCES = ["tvm_attn_api.cu"]
-BINDING_PATH = os.path.join(LIB_DIR, "_tvm_binding.so")
 BINDING_SOURCE = os.path.join(CSRC, "torch_binding.cpp")
 
 
@@ -29,6 +30,14 @@ def nvcc_command(out_path, extra=()):
             *extra, "-o", out_path, *[os.path.join(CSRC, s) for s in SOURCES]]
 
 
+def binding_path():
+    """Where the binding's native half lies.  It uses PyTorch's C++ interface, which changes from one build of PyTorch to the
+    next, and CPython's: each pair has a file of its own, so that another PyTorch never loads an object made for this one."""
+    import torch
+    tag = "%s-%s-%s" % (torch.__version__, (torch.version.git_version or "")[:8], sys.implementation.cache_tag)
+    return os.path.join(LIB_DIR, "_tvm_binding-%s.so" % re.sub(r"[^A-Za-z0-9.+-]", "_", tag))
+
+
 def binding_command(out_path):
     import torch
     root = os.path.dirname(torch.__file__)
@@ -41,12 +50,13 @@ def binding_command(out_path):
 
 
 def build_binding(force=False):
-    """Compiles _tvm_binding.so if it is missing or older than its source; returns its path."""
+    """Compiles the binding's native half if there is none for this PyTorch or it is older than its source; returns its path."""
+    path = binding_path()
     header = os.path.join(_ROOT, "include", "tvm_attn.h")
-    if not force and os.path.exists(BINDING_PATH) and os.path.getmtime(BINDING_PATH) >= max(os.path.getmtime(f) for f in (BINDING_SOURCE, header)):
-        return BINDING_PATH
-    _run(binding_command, BINDING_PATH)
-    return BINDING_PATH
+    if not force and os.path.exists(path) and os.path.getmtime(path) >= max(os.path.getmtime(f) for f in (BINDING_SOURCE, header)):
+        return path
+    _run(binding_command, path)
+    return path
 
 
 def _run(command, path, *args):
@@ -76,5 +86,4 @@ def build(force=False, verbose=False, out_path=None):
 
 
 if __name__ == "__main__":
-    import sys
     print(build(force=True, verbose="-v" in sys.argv))

@@ -101,3 +101,16 @@ def test_backward_refuses_outputs_it_could_not_give_back(noalloc):
     for out in ([x] * 6, torch.stack([x] * 6)):
         with pytest.raises(ValueError, match="CUDA"):       # read, and refused for its CPU tensors
             call(x, x, x, x, x, x, x, x, stats, stats, x, x, out=out)
+
+
+def test_native_module_of_another_pytorch_is_not_loaded(lib, monkeypatch):
+    """The native half uses PyTorch's C++ interface: under another PyTorch it is built again, and until then it is missing."""
+    import torch
+    built = build.build_binding()
+    commands = []
+    monkeypatch.setattr(build, "_run", lambda command, path, *args: commands.append(path))
+    assert build.build_binding() == built and not commands
+    monkeypatch.setattr(torch, "__version__", "99.0.0")
+    assert build.build_binding() != built and len(commands) == 1
+    with pytest.raises(FileNotFoundError):
+        binding._load_native()
