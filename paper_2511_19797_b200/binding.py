@@ -52,8 +52,11 @@ def library_path():
 
 
 def load(build_if_missing=False):
-    """Loads libtvm_attn.so (built in-tree by build.py).  Raises if it is not there."""
+    """Loads libtvm_attn.so (built in-tree by build.py).  Raises if it is not there; with build_if_missing it is built
+    first, as is the native half of this binding, which the tensor functions load on their first call."""
     global _lib
+    if build_if_missing and not os.path.exists(_build.binding_path()):
+        _build.build_binding()
     if _lib is not None:
         return _lib
     path = library_path()

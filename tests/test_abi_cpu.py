@@ -114,3 +114,15 @@ def test_native_module_of_another_pytorch_is_not_loaded(lib, monkeypatch):
     assert build.build_binding() != built and len(commands) == 1
     with pytest.raises(FileNotFoundError):
         binding._load_native()
+
+
+@pytest.mark.parametrize("loaded", [False, True])
+def test_load_builds_the_native_module_that_is_missing(lib, monkeypatch, tmp_path, loaded):
+    monkeypatch.setattr(binding, "_lib", lib if loaded else None)
+    monkeypatch.setattr(build, "binding_path", lambda: str(tmp_path / "native.so"))
+    commands = []
+    monkeypatch.setattr(build, "_run", lambda command, path, *args: commands.append(path))
+    binding.load()
+    assert not commands
+    binding.load(build_if_missing=True)
+    assert commands == [str(tmp_path / "native.so")]
