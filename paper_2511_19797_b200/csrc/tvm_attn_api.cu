@@ -48,7 +48,12 @@ static unsigned long long context_id() {
     if (!get_current || !get_id) return 0;
     CUcontext ctx = nullptr;
     if (get_current(&ctx) != CUDA_SUCCESS) return 0;
-    if (!ctx && (cudaFree(nullptr) != cudaSuccess || get_current(&ctx) != CUDA_SUCCESS || !ctx)) return 0;
+    if (!ctx) {
+        // A thread's first CUDA call: the device it is on becomes current.  Not by cudaFree(nullptr), which invalidates the stream
+        // captures under way, of other threads too.
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess || get_current(&ctx) != CUDA_SUCCESS || !ctx) return 0;
+    }
     unsigned long long id = 0;
     return get_id(ctx, &id) == CUDA_SUCCESS ? id : 0;
 }

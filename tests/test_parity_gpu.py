@@ -431,3 +431,34 @@ def test_forward_outputs_given_by_an_iterator_are_returned():
         for a, b, c in zip(got, given, want):
             assert a is b and torch.equal(a, c)
             a.zero_()
+
+
+def test_first_call_of_a_thread_may_be_captured():
+    """A call being recorded may be the first CUDA call of its thread (the device's kernels having been loaded before)."""
+    wl = inputs.custom(2, 4, 200, 72, seed=25)
+    x = {k: v.to(torch.bfloat16).cuda() for k, v in inputs.make_inputs(wl).items()}
+    six = [x[k] for k in inputs.NAMES[:6]]
+    fw = binding.tvm_attn_jvp_fwd(*six)
+    want = tuple(fw) + tuple(binding.tvm_attn_jvp_bwd(*six, *fw, x["dO"], x["dtO"]))
+    binding.tvm_attn_check_status()
+    outs = [torch.zeros_like(t) for t in want]
+    ws = torch.empty(binding.tvm_attn_jvp_workspace_bytes(*x["Q"].shape), dtype=torch.uint8, device="cuda")
+    stream, graph, errors = torch.cuda.Stream(), torch.cuda.CUDAGraph(), []
+
+    def call():
+        try:
+            binding.tvm_attn_jvp_fwd(*six, out=outs[:4], stream=stream)
+            binding.tvm_attn_jvp_bwd(*six, *outs[:4], x["dO"], x["dtO"], out=outs[4:], workspace=ws, stream=stream)
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=stream):
+        thread = threading.Thread(target=call)
+        thread.start()
+        thread.join()
+    assert not errors, errors
+    graph.replay()
+    binding.tvm_attn_check_status()
+    for a, b in zip(outs, want):
+        assert torch.equal(a, b)
