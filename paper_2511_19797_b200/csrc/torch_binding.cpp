@@ -13,6 +13,7 @@
 
 #include <ATen/ATen.h>
 #include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDACachingAllocator.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
@@ -89,9 +90,17 @@ at::Tensor packed(at::IntArrayRef sizes, at::ScalarType type, const at::Device& 
     return at::Tensor(at::detail::empty_cuda(sizes, type, dev, std::nullopt));
 }
 
-void* stream_of(PyObject* o, const at::Device& dev) {
-    if (o != Py_None) return PyLong_AsVoidPtr(o);
-    return (void*)c10::cuda::getCurrentCUDAStream(dev.index()).stream();
+// The stream of a call: the caller's, or PyTorch's current one.
+c10::cuda::CUDAStream stream_of(PyObject* o, const at::Device& dev) {
+    if (o == Py_None) return c10::cuda::getCurrentCUDAStream(dev.index());
+    return c10::cuda::getStreamFromExternal((cudaStream_t)PyLong_AsVoidPtr(o), dev.index());
+}
+// Memory allocated here belongs to the current stream.  Where the call runs on another, the allocator has to know: freed, by this
+// module (the workspace) or by the caller, it is not given out again before that stream is done with it.  (On the stream it
+// belongs to this is no more than a comparison.)
+void used_on(const at::Tensor* ts, int n, c10::cuda::CUDAStream st) {
+    for (int i = 0; i < n; ++i)
+        if (ts[i].defined()) c10::cuda::CUDACachingAllocator::recordStream(ts[i].storage().data_ptr(), st);
 }
 
 PyObject* tuple_of(at::Tensor* ts, int n) {
@@ -172,10 +181,11 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
             o[3] = packed(Q.sizes().slice(0, 3), at::kFloat, Q.device());
         }
         const c10::cuda::CUDAGuard guard(Q.device());
-        void* st = stream_of(a[9], Q.device());
+        const c10::cuda::CUDAStream st = stream_of(a[9], Q.device());
+        if (!given) used_on(o, 4, st);
         const int rc = without_gil([&] {
             return p_fwd(&p, ptr(Q), ptr(K), ptr(V), ptr(tQ), ptr(tK), ptr(tV), ptr(o[0]), ptr(o[1]), (float*)ptr(o[2]), (float*)ptr(o[3]),
-                         nullptr, 0, st);
+                         nullptr, 0, st.stream());
         });
         if (rc != TVM_ATTN_OK) return PyLong_FromLong(rc);
         return given ? PySequence_Tuple(outs.get()) : tuple_of(o, 4);
@@ -202,18 +212,21 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (!given)
             for (int i = 0; i < 6; ++i) o[i] = like(i % 3 == 0 ? Q : K);
         at::Tensor ws = noalloc ? at::Tensor() : optional_tensor(a[15]);
-        if (!noalloc && !ws.defined()) {
+        const bool own_ws = !noalloc && !ws.defined();
+        if (own_ws) {
             const int64_t need = (int64_t)p_ws(&p, 1);
             ws = packed({need > 16 ? need : 16}, at::kByte, Q.device());
         }
         const c10::cuda::CUDAGuard guard(Q.device());
-        void* st = stream_of(a[16], Q.device());
+        const c10::cuda::CUDAStream st = stream_of(a[16], Q.device());
+        if (!given) used_on(o, 6, st);
+        if (own_ws) used_on(&ws, 1, st);
         const int rc = without_gil([&] {
             if (noalloc)
                 return p_bwd_noalloc(&p, ptr(Q), ptr(K), ptr(V), ptr(tQ), ptr(tK), ptr(tV), ptr(O), ptr(tO), (float*)ptr(lse), (float*)ptr(mu),
-                                     ptr(dO), ptr(dtO), ptr(o[0]), ptr(o[1]), ptr(o[2]), ptr(o[3]), ptr(o[4]), ptr(o[5]), st);
+                                     ptr(dO), ptr(dtO), ptr(o[0]), ptr(o[1]), ptr(o[2]), ptr(o[3]), ptr(o[4]), ptr(o[5]), st.stream());
             return p_bwd(&p, ptr(Q), ptr(K), ptr(V), ptr(tQ), ptr(tK), ptr(tV), ptr(O), ptr(tO), (float*)ptr(lse), (float*)ptr(mu), ptr(dO),
-                         ptr(dtO), ptr(o[0]), ptr(o[1]), ptr(o[2]), ptr(o[3]), ptr(o[4]), ptr(o[5]), ptr(ws), (size_t)ws.numel(), st);
+                         ptr(dtO), ptr(o[0]), ptr(o[1]), ptr(o[2]), ptr(o[3]), ptr(o[4]), ptr(o[5]), ptr(ws), (size_t)ws.numel(), st.stream());
         });
         if (rc != TVM_ATTN_OK) return PyLong_FromLong(rc);
         return given ? (noalloc ? PySequence_Tuple(outs.get()) : same(a[14])) : tuple_of(o, 6);
@@ -238,9 +251,10 @@ PyObject* norm_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         at::Tensor o[4] = {like(Q), like(Q), like(K), like(K)};
         const c10::cuda::CUDAGuard guard(Q.device());
         const float eps = (float)number(a[6]);
-        void* st = stream_of(a[7], Q.device());
+        const c10::cuda::CUDAStream st = stream_of(a[7], Q.device());
+        used_on(o, 4, st);
         const int rc = without_gil([&] {
-            return p_norm_fwd(&p, eps, ptr(Q), ptr(tQ), ptr(K), ptr(tK), (float*)ptr(gQ), (float*)ptr(gK), ptr(o[0]), ptr(o[1]), ptr(o[2]), ptr(o[3]), st);
+            return p_norm_fwd(&p, eps, ptr(Q), ptr(tQ), ptr(K), ptr(tK), (float*)ptr(gQ), (float*)ptr(gK), ptr(o[0]), ptr(o[1]), ptr(o[2]), ptr(o[3]), st.stream());
         });
         return rc != TVM_ATTN_OK ? PyLong_FromLong(rc) : tuple_of(o, 4);
     });
@@ -258,17 +272,20 @@ PyObject* norm_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         check_scale(gK, Q);
         const tvm_attn_params p = params(Q, K, 0.0, 0);
         at::Tensor ws = optional_tensor(a[11]);
-        if (!ws.defined()) {
+        const bool own_ws = !ws.defined();
+        if (own_ws) {
             const int64_t need = (int64_t)p_norm_ws(&p);
             ws = packed({need > 16 ? need : 16}, at::kByte, Q.device());
         }
         at::Tensor o[6] = {like(Q), like(Q), like(K), like(K), like(gQ), like(gK)};
         const c10::cuda::CUDAGuard guard(Q.device());
         const float eps = (float)number(a[10]);
-        void* st = stream_of(a[12], Q.device());
+        const c10::cuda::CUDAStream st = stream_of(a[12], Q.device());
+        used_on(o, 6, st);
+        if (own_ws) used_on(&ws, 1, st);
         const int rc = without_gil([&] {
             return p_norm_bwd(&p, eps, ptr(Q), ptr(tQ), ptr(K), ptr(tK), (float*)ptr(gQ), (float*)ptr(gK), ptr(dQn), ptr(dtQn), ptr(dKn), ptr(dtKn),
-                              ptr(o[0]), ptr(o[1]), ptr(o[2]), ptr(o[3]), (float*)ptr(o[4]), (float*)ptr(o[5]), ptr(ws), (size_t)ws.numel(), st);
+                              ptr(o[0]), ptr(o[1]), ptr(o[2]), ptr(o[3]), (float*)ptr(o[4]), (float*)ptr(o[5]), ptr(ws), (size_t)ws.numel(), st.stream());
         });
         return rc != TVM_ATTN_OK ? PyLong_FromLong(rc) : tuple_of(o, 6);
     });

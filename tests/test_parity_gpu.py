@@ -462,3 +462,42 @@ def test_first_call_of_a_thread_may_be_captured():
     binding.tvm_attn_check_status()
     for a, b in zip(outs, want):
         assert torch.equal(a, b)
+
+
+def test_memory_of_a_call_is_kept_for_the_stream_it_runs_on():
+    """What a call allocates belongs to the current stream.  Given another stream, that is still busy when the call returns, its
+    workspace and outputs, once freed, are held back (active, no longer allocated) until that stream is done."""
+    wl = inputs.custom(2, 4, 320, 72, seed=27)
+    x = {k: v.to(torch.bfloat16).cuda() for k, v in inputs.make_inputs(wl).items()}
+    six, g, side = [x[k] for k in inputs.NAMES[:6]], torch.ones(72, device="cuda"), torch.cuda.Stream()
+    fw = binding.tvm_attn_jvp_fwd(*six)
+    norm = (x["Q"], x["tQ"], x["K"], x["tK"], g, g)
+    calls = {"fwd": lambda **kw: binding.tvm_attn_jvp_fwd(*six, **kw),
+             "bwd": lambda **kw: binding.tvm_attn_jvp_bwd(*six, *fw, x["dO"], x["dtO"], **kw),
+             "norm_fwd": lambda **kw: binding.tvm_qk_rmsnorm_jvp_fwd(*norm, **kw),
+             "norm_bwd": lambda **kw: binding.tvm_qk_rmsnorm_jvp_bwd(*norm, x["dO"], x["dtO"], x["V"], x["tV"], **kw)}
+
+    def held_back():
+        stats = torch.cuda.memory_stats()
+        return stats["active_bytes.all.current"] - stats["allocated_bytes.all.current"]
+
+    for name, call in calls.items():
+        want = [t.clone() for t in call()]
+        workspace = {"bwd": binding.tvm_attn_jvp_workspace_bytes(*x["Q"].shape), "norm_bwd": 4 * 72}.get(name, 0)   # at least
+        torch.cuda.synchronize()
+        before = held_back()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(200_000_000)            # a tenth of a second
+        got = call(stream=side)
+        assert held_back() - before >= workspace and (workspace == 0 or held_back() > before), name
+        out_bytes = sum(t.numel() * t.element_size() for t in got)
+        side.synchronize()
+        binding.tvm_attn_check_status()
+        for a, b in zip(got, want):
+            assert torch.equal(a, b), name
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(200_000_000)
+        before = held_back()
+        del got, a
+        assert held_back() - before >= out_bytes, name
+        side.synchronize()
