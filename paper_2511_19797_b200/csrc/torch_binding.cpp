@@ -64,7 +64,7 @@ void side_strides(const at::Tensor& t, int64_t (&st)[3]) {
 }
 
 // Parameters from a query-side tensor q (B, H, M, d) and a key-side tensor k (B, H, N, d).
-tvm_attn_params params(const at::Tensor& q, const at::Tensor& k, double scale, long long flags) {
+tvm_attn_params params(const at::Tensor& q, const at::Tensor& k, double scale, uint32_t flags) {
     if (q.dim() != 4) throw ValueError("expected (B, H, rows, d) tensors");
     tvm_attn_params p;
     std::memset(&p, 0, sizeof p);
@@ -78,7 +78,7 @@ tvm_attn_params params(const at::Tensor& q, const at::Tensor& k, double scale, l
     p.B = (int32_t)B; p.H = (int32_t)H; p.N = (int32_t)N; p.d = (int32_t)d;
     p.M = M == N ? 0 : (int32_t)M;
     p.scale = (float)scale;
-    p.flags = (uint32_t)flags;
+    p.flags = flags;
     side_strides(q, p.q_strides);
     side_strides(k, p.k_strides);
     return p;
@@ -137,15 +137,16 @@ int without_gil(F&& f) {
     return rc;
 }
 
+// What float(o) and int(o) give, the latter's low 32 bits as flags.
 double number(PyObject* o) {
-    const double v = PyFloat_AsDouble(o);
-    if (v == -1.0 && PyErr_Occurred()) throw python_error();
-    return v;
+    THPObjectPtr f(PyNumber_Float(o));
+    if (!f) throw python_error();
+    return PyFloat_AS_DOUBLE(f.get());
 }
-long long integer(PyObject* o) {
-    const long long v = PyLong_AsLongLong(o);
-    if (v == -1 && PyErr_Occurred()) throw python_error();
-    return v;
+uint32_t flag_bits(PyObject* o) {
+    THPObjectPtr i(PyNumber_Long(o));
+    if (!i) throw python_error();
+    return (uint32_t)PyLong_AsUnsignedLongLongMask(i.get());
 }
 // The n entries of `out` as optional tensors.  Returns the list or tuple that they were read from: an iterator has nothing
 // left to give after that, so results are made from what is returned here, never from `o` again.  `indexable`: the caller
@@ -174,7 +175,7 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const at::Tensor* ks[] = {&V, &tK, &tV};
         check_side(Q, qs, 3);
         check_side(K, ks, 3);
-        const tvm_attn_params p = params(Q, K, number(a[6]), integer(a[7]));
+        const tvm_attn_params p = params(Q, K, number(a[6]), flag_bits(a[7]));
         if (!given) {
             o[0] = like(Q); o[1] = like(Q);
             o[2] = packed(Q.sizes().slice(0, 3), at::kFloat, Q.device());
@@ -199,7 +200,7 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const at::Tensor &Q = tensor(a[0]), &K = tensor(a[1]), &V = tensor(a[2]), &tQ = tensor(a[3]), &tK = tensor(a[4]), &tV = tensor(a[5]);
         const at::Tensor &O = tensor(a[6]), &tO = tensor(a[7]), &lse = tensor(a[8]), &mu = tensor(a[9]);
         const at::Tensor dO = optional_tensor(a[10]), dtO = optional_tensor(a[11]);
-        const tvm_attn_params p = params(Q, K, number(a[12]), integer(a[13]));
+        const tvm_attn_params p = params(Q, K, number(a[12]), flag_bits(a[13]));
         const bool given = a[14] != Py_None, noalloc = a[17] == Py_True;
         at::Tensor o[6];
         THPObjectPtr outs;

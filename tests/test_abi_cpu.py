@@ -126,3 +126,17 @@ def test_load_builds_the_native_module_that_is_missing(lib, monkeypatch, tmp_pat
     assert not commands
     binding.load(build_if_missing=True)
     assert commands == [str(tmp_path / "native.so")]
+
+
+def test_scale_and_flags_are_converted_as_numbers():
+    """scale and flags are what float() and int() make of them; what these refuse is refused."""
+    import torch
+    x = torch.zeros(1, 1, 8, 8, dtype=torch.bfloat16)
+    args = (x, x, x, x, x, x, x, x, torch.zeros(1, 1, 8), torch.zeros(1, 1, 8), x, x)
+    for scale, flags in ((1, 1.0), ("0.5", "1"), (torch.tensor(0.5), torch.tensor(1)), (True, -1)):
+        with pytest.raises(ValueError, match="CUDA"):       # past the conversions, to the tensors
+            binding.tvm_attn_jvp_bwd(*args, scale=scale, flags=flags)
+    for bad in ({"scale": "half"}, {"flags": "one"}, {"scale": None}, {"flags": None}):
+        with pytest.raises((TypeError, ValueError)) as e:
+            binding.tvm_attn_jvp_bwd(*args, **bad)
+        assert "CUDA" not in str(e.value)
