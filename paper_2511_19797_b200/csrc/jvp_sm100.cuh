@@ -103,6 +103,7 @@ struct JvpParams {
     // bit 1 = G (dO).  An absent tensor is never loaded; where an MMA still reads its tile, the tile is zeroed once,
     // and the MMAs whose result would be exactly zero are not issued.  out0 may be null when Hc is absent.
     int absent;
+    uint64_t item_wait_ns;     // how long the end of an item may be waited for
 };
 
 template <int MODE, int DP>
@@ -230,7 +231,7 @@ struct JvpBlock {
     }
     // For what comes at the end of an item the caller has just begun to wait for.
     __device__ __forceinline__ bool wait_item(int i, int phase) const {
-        return ptx::mbar_wait_warp_s(bar(i), phase & 1, base + ABORT, JVP_WAIT_LIMIT_NS + static_cast<uint64_t>(p.T) * JVP_TILE_LIMIT_NS);
+        return ptx::mbar_wait_warp_s(bar(i), phase & 1, base + ABORT, p.item_wait_ns);
     }
     __device__ __forceinline__ bool wait2(int i, int pi, int j, int pj) const {
         if (ptx::mbar_test2_warp(bar(i), pi & 1, bar(j), pj & 1)) return true;

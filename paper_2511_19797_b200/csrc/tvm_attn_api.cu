@@ -282,6 +282,7 @@ static int launch_pass(const Shape& s, const Operand (&own)[4], const Operand (&
     prm.row_tiles = (prm.o.rows + JVP_ROWS - 1) / JVP_ROWS;
     prm.items = (int)(s.BH * prm.row_tiles);
     prm.T = (prm.s.rows + C::BC - 1) / C::BC;
+    prm.item_wait_ns = JVP_WAIT_LIMIT_NS + (uint64_t)prm.T * JVP_TILE_LIMIT_NS;
     g_prof.before(st);
     // DK and DQ read nothing that the pass before them writes (all passes depend on the row-sums pre-pass only, which has
     // completed before the first of them starts), so their CTAs may fill the SMs that the last, partial wave of the pass
