@@ -124,8 +124,8 @@ struct JvpCfg {
     static_assert(WIDE || (MODE != PASS_DV && MODE != PASS_DK), "DV and DK on their own: only where DKV does not fit");
     static_assert(!WIDE || !DKV, "DKV: four accumulators do not fit");
     static constexpr bool E_MN = DKV;                      // the E ring is read MN-major too: swizzled atoms like the L ring's
-    // Owner operands.  The pair of the score MMAs on the tile's critical chain (FWD, DV: the only pair; DK, DQ: the second)
-    // lies in tensor memory as bf16 A operands: an MMA with A in shared memory moves 4 KB of A per k-step through the
+    // Owner operands.  The pair of the score MMAs on the tile's critical chain (FWD: the only pair; DQ: the second) lies in
+    // tensor memory as bf16 A operands: an MMA with A in shared memory moves 4 KB of A per k-step through the
     // shared-memory port.  WIDE, DKV: tensor memory has no room, everything is in shared memory.
     static constexpr bool XT = !WIDE && !DKV;
     static constexpr int NOWN = 2 * NPAIR - (XT ? 2 : 0);   // owner tensors in shared memory
@@ -269,11 +269,11 @@ __device__ __forceinline__ void jvp_load_owners(const JvpParams& p, const JvpBlo
         const uint32_t full = k.bar(C::B_OWN + SET);
         uint32_t tx = 0;
 #pragma unroll
-        for (int t = T0; t < T1; ++t) tx += p.own[t] ? C::OWN_ATOM * (C::WIDE ? 2 : 1) : 0;   // null: absent, or not read
+        for (int t = T0; t < T1; ++t) tx += p.own[t] ? C::OWN_ATOM * (C::WIDE ? 2 : 1) : 0;   // null: not read (HZ)
         ptx::mbar_arrive_expect_tx(full, tx);
 #pragma unroll
         for (int t = T0; t < T1; ++t) {
-            if (!p.own[t]) continue;   // (its tile is zeroed once)
+            if (!p.own[t]) continue;
             const uint32_t dst = k.own_tile(t);
             ptx::tma_load_4d(dst, maps[t], full, 0, row0, ch, cb);
             ptx::tma_load_4d(dst + H64, maps[t], full, 0, row0 + 64, ch, cb);
@@ -329,9 +329,9 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
     const uint32_t ring_base = k.base + (RING == 0 ? k.E : k.L);
     const __nv_bfloat16* base0 = p.strm[2 * RING];
     const __nv_bfloat16* base1 = p.strm[2 * RING + 1];
-    // The ring that streams the cotangents (Hc, G): L in DV, E in DK and DKV; an absent one (null) is not loaded, nor, with HZ,
+    // The ring that streams the cotangents (Hc, G) where one of them may be absent (null): that one is not loaded, nor, with HZ,
     // are the tangents.
-    constexpr bool COT = (MODE == PASS_DV && RING == 1) || ((MODE == PASS_DK || C::DKV) && RING == 0);
+    constexpr bool COT = C::DKV && RING == 0;
     const bool has0 = COT ? !HZ && base0 : true, has1 = COT ? HZ || base1 : !HZ;
     const uint32_t tx_bytes = ((has0 ? 1 : 0) + (has1 ? 1 : 0)) * ATOM * (C::WIDE ? 2 : 1);
     // Chunk 0 of row `lane` behind the first atoms: compact blocks in the E ring, a second swizzled atom in the L ring.
@@ -631,19 +631,17 @@ struct JvpIssue {
         if (k.fold_step()) fold_step(el, col, k, fold, T, I_S);
     }
     // Half of acc0 += A0 B0, acc1 += A1 B0 + A0 B1 (k-steps U0, U0 + 1 of four; the operand of a k-step lies at the columns of
-    // the scores it replaces); the terms of an absent tensor are left out.  acc = 0: the accumulators are overwritten.
+    // the scores it replaces); terms that are exactly zero are left out.  acc = 0: the accumulators are overwritten.
     template <int U0>
     static __device__ __forceinline__ void outputs(uint32_t el, uint32_t a0, uint32_t a1, uint32_t lo, uint32_t acc) {
         constexpr uint32_t c0 = C::COL_ACC0, c1 = C::COL_ACC1;
-        constexpr bool DV = MODE == PASS_DV, B0 = !HZ && !(DV && (ABS & ABSENT_HC)), A0 = !HZ && !(!DV && (ABS & ABSENT_HC)), B1 = !(DV && (ABS & ABSENT_G));
-        // (DV: Hc is B0, G is B1; DK, DQ with Hc absent: A0 = W is exactly zero)
-        constexpr bool T0 = A0 && B0, T1 = !DV ? true : B0, T2 = DV ? B1 : A0;   // A0 B0, A1 B0, A0 B1
+        constexpr bool A0 = !HZ && !(ABS & ABSENT_HC);   // (DQ with Hc absent: A0 = W is exactly zero)
 #pragma unroll UNROLL
         for (int u = U0; u < U0 + 2; ++u) {
             const uint32_t b0 = lo + l_n(0, 0) + 128u * u, b1 = lo + l_n(1, 0) + 128u * u, o = 16u * u, first = U0 > 0 || u > 0 ? 1u : acc;
-            if (T0) ptx::mma_ts_acc(el, c0, a0 + o, b0, HI_SW, I_O, first);
-            if (T1) ptx::mma_ts_acc(el, c1, a1 + o, b0, HI_SW, I_O, first);
-            if (T2) ptx::mma_ts_acc(el, c1, a0 + o, b1, HI_SW, I_O, T1 ? 1u : first);
+            if (A0) ptx::mma_ts_acc(el, c0, a0 + o, b0, HI_SW, I_O, first);
+            ptx::mma_ts_acc(el, c1, a1 + o, b0, HI_SW, I_O, first);
+            if (A0) ptx::mma_ts_acc(el, c1, a0 + o, b1, HI_SW, I_O, 1u);
         }
     }
     // DKV: acc[C] += A0 B0, acc[C + 1] += A1 B0 + A0 B1 (T0, T1, T2: which of the three there are).
@@ -732,10 +730,10 @@ __device__ __forceinline__ void jvp_issue_dkv(const JvpParams& p, const JvpBlock
 
 // FWD, DV: two score buffers taken in turn, operands written over the scores; pipe order S(0), S(1), out(0), S(2), out(1), ...:
 // S(n + 1) overwrites what out(n - 1) reads, and the pipe keeps the order.
-template <int MODE, int DP, bool HZ, int ABS>
+template <int MODE, int DP>
 __device__ __forceinline__ void jvp_issue_one_pair(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
     using C = JvpCfg<MODE, DP>;
-    using I = JvpIssue<MODE, DP, HZ, ABS>;
+    using I = JvpIssue<MODE, DP, false, 0>;
     constexpr int RDY = C::XT ? C::B_XRDY : C::B_OWN, FREE = C::XT ? C::B_XFREE : C::B_OWNFREE;
     const JvpBlock<MODE, DP> k = shared.pinned();
     const int T = jvp_pin(p.T), items = jvp_pin(p.items);
@@ -759,8 +757,7 @@ __device__ __forceinline__ void jvp_issue_one_pair(const JvpParams& p, const Jvp
                 k.tile_fence();
                 const uint32_t el = ptx::elect_one();
                 const uint32_t col = C::COL_SCORE + (n & 1) * 2 * C::BC;
-                if (HZ) I::template single<false, C::XT, 0>(el, col, k, x0, e.lo, e.fold);
-                else I::template pair<false, C::XT, true>(el, col, k, x0, x1, e.lo, e.fold, k.bar(C::B_SFULL + (n & 3)));
+                I::template pair<false, C::XT, true>(el, col, k, x0, x1, e.lo, e.fold, k.bar(C::B_SFULL + (n & 3)));
                 ptx::mma_commit_p(el, k.bar(C::B_EDONE + (n & 3)));
                 if (j + 2 == T || (T == 1 && j == 0)) ptx::mma_commit_p(el, k.bar(FREE));   // the item's last scores
                 e.template next<C::SE, I::E_STEP, I::F_STEP>();
@@ -796,8 +793,7 @@ __device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const Jv
     const uint32_t x0 = ptx::desc_lo(k.own_tile(0), 16), x1 = ptx::desc_lo(k.own_tile(1), 16);
     const uint32_t x2 = C::XT ? C::COL_X0 : ptx::desc_lo(k.own_tile(2), 16), x3 = C::XT ? C::COL_X1 : ptx::desc_lo(k.own_tile(3), 16);
     constexpr uint32_t cS = C::COL_SCORE, cD = C::COL_SCORE + 2 * C::BC, cX = C::COL_SCORE + 3 * C::BC;
-    // X3 Y2^T is zero when either factor is an absent cotangent: DK has Y2 = Hc, DQ has X3 = G
-    constexpr bool X3 = !(ABS & (MODE == PASS_DK ? ABSENT_HC : ABSENT_G));
+    constexpr bool X3 = !(ABS & ABSENT_G);   // DQ: X3 Y2^T = G V^T is zero with G absent
     JvpSlot e = I::e_slot(k), l = I::l_slot(k);
     uint32_t lo = l.lo;        // L stage of the outputs' tile
     int n = 0;                 // next tile whose scores are issued
@@ -836,8 +832,8 @@ __device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const Jv
                 if (!e_ready && !k.wait(C::B_EFULL + e.s, e.ph)) return;
                 k.tile_fence();
                 const uint32_t el = ptx::elect_one();
-                // HZ: X = G V^T alone: DK: X2 Y3^T (V, and G the stage's second tensor); DQ: X3 Y2^T (G, and V its first)
-                if (HZ) I::template single<false, C::XT, MODE == PASS_DK ? 1 : 0>(el, cX, k, MODE == PASS_DK ? x2 : x3, e.lo, e.fold);
+                // HZ (DQ): X = G V^T alone: X3 and the stage's first tensor
+                if (HZ) I::template single<false, C::XT, 0>(el, cX, k, x3, e.lo, e.fold);
                 else I::template pair<false, C::XT, X3>(el, cD, k, x2, x3, e.lo, e.fold, 0);
                 ptx::mma_commit_p(el, k.bar(C::B_XFULL + (n & 3)));
                 if (j + 2 == T) ptx::mma_commit_p(el, k.bar(C::XT ? C::B_XFREE : C::B_OWNFREE));
@@ -848,16 +844,17 @@ __device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const Jv
     }
 }
 
-// Which cotangent is absent is decided here, once.
+// Which cotangent is absent is decided here, once (WIDE head dims take both).
 template <int MODE, int DP, bool HZ, int ABS>
 __device__ __forceinline__ void jvp_issue_abs(const JvpParams& p, const JvpBlock<MODE, DP>& k) {
     if constexpr (MODE == PASS_DKV) jvp_issue_dkv<MODE, DP, HZ, ABS>(p, k);
-    else if constexpr (JvpCfg<MODE, DP>::NPAIR == 1) jvp_issue_one_pair<MODE, DP, HZ, ABS>(p, k);
+    else if constexpr (JvpCfg<MODE, DP>::NPAIR == 1) jvp_issue_one_pair<MODE, DP>(p, k);
     else jvp_issue_two_pairs<MODE, DP, HZ, ABS>(p, k);
 }
 template <int MODE, int DP, bool HZ>
 __device__ __forceinline__ void jvp_issue(const JvpParams& p, const JvpBlock<MODE, DP>& k) {
-    if (MODE == PASS_FWD || HZ || p.absent == 0) jvp_issue_abs<MODE, DP, HZ, 0>(p, k);
+    if constexpr (MODE == PASS_FWD || HZ || JvpCfg<MODE, DP>::WIDE) jvp_issue_abs<MODE, DP, HZ, 0>(p, k);
+    else if (p.absent == 0) jvp_issue_abs<MODE, DP, HZ, 0>(p, k);
     else if (p.absent == ABSENT_HC) jvp_issue_abs<MODE, DP, HZ, ABSENT_HC>(p, k);
     else jvp_issue_abs<MODE, DP, HZ, ABSENT_G>(p, k);
 }
@@ -1035,7 +1032,7 @@ __device__ __forceinline__ void jvp_elem_fwd(const JvpParams& p, const JvpBlock<
 }
 
 // DV: P, P Nn from (S, Sd), written over them.
-template <int DP, bool HZ>
+template <int DP>
 __device__ __forceinline__ void jvp_elem_dv(const JvpParams& p, const JvpBlock<PASS_DV, DP>& k, int grp, int q, int lane) {
     using C = JvpCfg<PASS_DV, DP>;
     constexpr int BC = C::BC, HC = BC / 2;
@@ -1050,7 +1047,7 @@ __device__ __forceinline__ void jvp_elem_dv(const JvpParams& p, const JvpBlock<P
         ptx::tc_fence_after_sync();
         uint32_t s[HC], t[HC];
         ptx::tmem_ld32(sb, s);
-        if (!HZ) ptx::tmem_ld32(sb + BC, t);
+        ptx::tmem_ld32(sb + BC, t);
         ptx::tmem_wait_ld();
         const float* st = k.stats(g % C::SL) + grp * HC;
 #pragma unroll
@@ -1059,10 +1056,8 @@ __device__ __forceinline__ void jvp_elem_dv(const JvpParams& p, const JvpBlock<P
 #pragma unroll
             for (int c = 0; c < 16; c += 4) {
                 const int cc = 16 * u + c;
-                ulonglong2 l4;
-                [[maybe_unused]] ulonglong2 m4;
-                l4 = *reinterpret_cast<const ulonglong2*>(st + cc);
-                if (!HZ) m4 = *reinterpret_cast<const ulonglong2*>(st + BC + cc);
+                const ulonglong2 l4 = *reinterpret_cast<const ulonglong2*>(st + cc);
+                const ulonglong2 m4 = *reinterpret_cast<const ulonglong2*>(st + BC + cc);
 #pragma unroll
                 for (int e = 0; e < 4; e += 2) {
                     const uint64_t s2 = ptx::pack2u(s[cc + e], s[cc + e + 1]);
@@ -1070,17 +1065,15 @@ __device__ __forceinline__ void jvp_elem_dv(const JvpParams& p, const JvpBlock<P
                     ptx::unpack2(ptx::fma2(s2, c2c2, e ? l4.y : l4.x), x0, x1);
                     const float p0 = ptx::ex2(x0), p1 = ptx::ex2(x1);
                     pa0[(c + e) >> 1] = ptx::pack_bf16(p0, p1);
-                    if (!HZ) {
-                        const uint64_t t2 = ptx::pack2u(t[cc + e], t[cc + e + 1]);
-                        const uint64_t n2 = ptx::fma2(t2, aa, ptx::neg2(e ? m4.y : m4.x));
-                        float q0, q1;
-                        ptx::unpack2(ptx::mul2(ptx::pack2(p0, p1), n2), q0, q1);
-                        pa1[(c + e) >> 1] = ptx::pack_bf16(q0, q1);
-                    }
+                    const uint64_t t2 = ptx::pack2u(t[cc + e], t[cc + e + 1]);
+                    const uint64_t n2 = ptx::fma2(t2, aa, ptx::neg2(e ? m4.y : m4.x));
+                    float q0, q1;
+                    ptx::unpack2(ptx::mul2(ptx::pack2(p0, p1), n2), q0, q1);
+                    pa1[(c + e) >> 1] = ptx::pack_bf16(q0, q1);
                 }
             }
             ptx::tmem_st8(sb + 16 * u, pa0);
-            if (!HZ) ptx::tmem_st8(sb + BC + 16 * u, pa1);
+            ptx::tmem_st8(sb + BC + 16 * u, pa1);
         }
         ptx::tmem_wait_st();
         k.arrive(C::B_PREADY + 2 * b + grp, lane);
@@ -1135,7 +1128,7 @@ __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const Jvp
                 for (int c = 0; c < HC; c += 4) {
                     [[maybe_unused]] ulonglong2 l4, m4;
                     if (COL) l4 = *reinterpret_cast<const ulonglong2*>(st + c);
-                    if (COL && !HZ) m4 = *reinterpret_cast<const ulonglong2*>(st + BC + c);
+                    if (COL) m4 = *reinterpret_cast<const ulonglong2*>(st + BC + c);
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         const int i = c / 2 + e;
@@ -1163,7 +1156,7 @@ __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const Jvp
 #pragma unroll
                 for (int c = 0; c < 16; c += 4) {
                     [[maybe_unused]] ulonglong2 s4, c4;
-                    if (COL && !HZ) s4 = *reinterpret_cast<const ulonglong2*>(st + 2 * BC + 16 * u + c);
+                    if (COL) s4 = *reinterpret_cast<const ulonglong2*>(st + 2 * BC + 16 * u + c);
                     if (COL) c4 = *reinterpret_cast<const ulonglong2*>(st + 3 * BC + 16 * u + c);
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
@@ -1439,7 +1432,7 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
             }
         }
     }
-    if (!HZ && (MODE == PASS_DK || C::DKV) && p.absent) {
+    if (!HZ && C::DKV && p.absent) {
         // both cotangent tiles of an E stage are read by one MMA: the never-loaded one must read as zero
         const int t = (p.absent & ABSENT_HC) ? 0 : 1;
         uint8_t* e = jvp_smem + C::NOWN * C::OWN_BYTES;
@@ -1454,10 +1447,6 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
     if (C::FOLD)
         for (int i = threadIdx.x; i < 2 * JVP_ROWS; i += JVP_THREADS)
             *reinterpret_cast<uint4*>(jvp_smem + k.ONES + i * 16) = i < JVP_ROWS ? make_uint4(JVP_ONES0, JVP_ONES1, 0, 0) : zero;
-    if (!HZ && MODE == PASS_DQ && !C::XT && p.absent)   // an absent cotangent is an owner tile of zeros
-        for (int t = 2; t < 4; ++t)
-            if (!p.own[t])
-                for (int i = threadIdx.x; i < C::OWN_BYTES / 16; i += JVP_THREADS) *reinterpret_cast<uint4*>(jvp_smem + t * C::OWN_BYTES + i * 16) = zero;
     ptx::fence_proxy_async_smem();
     if (warp == 1) {
         ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
@@ -1492,7 +1481,7 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
             const int grp = (warp - 4) >> 2, q = warp & 3;
             if constexpr (MODE == PASS_FWD) jvp_elem_fwd<DP>(p, k, grp, q, lane);
             else if constexpr (MODE == PASS_DKV) jvp_elem_dkv<DP, HZ>(p, k, grp, q, lane);
-            else if constexpr (MODE == PASS_DV) jvp_elem_dv<DP, HZ>(p, k, grp, q, lane);
+            else if constexpr (MODE == PASS_DV) jvp_elem_dv<DP>(p, k, grp, q, lane);
             else jvp_elem_two_pairs<MODE, DP, HZ>(p, k, grp, q, lane);
         }
     } else {

@@ -152,13 +152,6 @@ __device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// 32 lanes x 8 consecutive 32-bit columns.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr)
-                 : "memory");
-}
 // 16 lanes (from a multiple of 16) x 16 columns: thread t has r[0, 1] = columns 2 (t % 4), 2 (t % 4) + 1 of lane t / 4, r[2, 3] the
 // same of lane 8 + t / 4, r[4..7] the same 8 columns further on.
 __device__ __forceinline__ void tmem_ld16_256x2(uint32_t taddr, uint32_t* r) {
