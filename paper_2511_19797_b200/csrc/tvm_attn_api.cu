@@ -534,6 +534,9 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
         if (x && !aligned16(x)) return TVM_ATTN_INVALID_ARG;
     if (dtO && (!dtQ || !dtK || !dtV)) return TVM_ATTN_INVALID_ARG;
     const int absent = (dtO ? 0 : ABSENT_HC) | (dO ? 0 : ABSENT_G);
+    // DKV takes its statistics divided by the scale, which overflows where that is next to nothing (lse / 1e-36 does at 340):
+    // such a call, all of whose weights are equal, goes to the CUDA-core kernels.
+    if (s.alpha < 1e-36f && pass_exists(PASS_DKV, s.dp)) s.simt = true;
     if ((absent || !s.plain) && !s.simt && s.dp > 80) return TVM_ATTN_UNSUPPORTED;  // head dims above 80: both cotangents, packed self-attention
     const size_t rows = (size_t)s.BH * (size_t)s.M;   // query rows: what the workspace and the statistics are sized by
     if (workspace_bytes < 3 * sizeof(float) * rows) return TVM_ATTN_WORKSPACE_TOO_SMALL;

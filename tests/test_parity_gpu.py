@@ -501,3 +501,11 @@ def test_memory_of_a_call_is_kept_for_the_stream_it_runs_on():
         del got, a
         assert held_back() - before >= out_bytes, name
         side.synchronize()
+
+
+@pytest.mark.parametrize("scale", [1.2e-38, 3e-37, 2e-36])
+@pytest.mark.parametrize("d,absent", [(64, None), (72, "dtO"), (40, "dO"), (96, None)])
+def test_scales_next_to_nothing(scale, d, absent):
+    """Statistics that the kernels divide by the softmax scale stay finite whatever scale is accepted."""
+    errs, _, _ = run_case(inputs.custom(1, 3, 150, d, seed=90 + d), scale=scale, absent=absent)
+    assert_within(errs, BF16_FWD, BF16_BWD, BF16_STATS)
