@@ -224,11 +224,12 @@ def test_longest_sequence_on_sampled_query_rows():
     assert_within(errs, BF16_FWD, BF16_BWD, BF16_STATS)
 
 
-def test_gradients_are_complete_for_work_enqueued_behind_the_call():
-    """The three tensor-core passes of one backward call overlap (the later ones start while the earlier ones
+@pytest.mark.parametrize("d", [72, 104])                 # two and three tensor-core passes
+def test_gradients_are_complete_for_work_enqueued_behind_the_call(d):
+    """The tensor-core passes of one backward call overlap (the later ones start while the earlier ones
     drain).  Work enqueued on the same stream right after the call, with no host synchronisation in between,
     must still see all six gradients complete."""
-    wl = inputs.custom(4, 37, 320, 72, seed=77)          # one wave is not enough: the passes do overlap
+    wl = inputs.custom(4, 37, 320, d, seed=77)           # one wave is not enough: the passes do overlap
     x = {k: v.to(torch.bfloat16).cuda() for k, v in inputs.make_inputs(wl).items()}
     O, tO, lse, mu = binding.tvm_attn_jvp_fwd(x["Q"], x["K"], x["V"], x["tQ"], x["tK"], x["tV"])
     args = (x["Q"], x["K"], x["V"], x["tQ"], x["tK"], x["tV"], O, tO, lse, mu, x["dO"], x["dtO"])
