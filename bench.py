@@ -39,7 +39,7 @@ BWD_KERNELS = {"narrow": {"bwd_rowsums": (0, 4), "bwd_dkv": (12, 12), "bwd_dq": 
 BWD_CREDITED_GEMMS = 15
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu capture summarised in
 # profiles/jvp_fwd_bwd_kernels_dit512.md (that workload and the full variant only; None for anything else)
-NCU_TRAFFIC_BYTES = {"dit512": {"fwd": 279.8e6, "bwd_dkv": 420.8e6, "bwd_dq": 360.3e6}}
+NCU_TRAFFIC_BYTES = {"dit512": {"fwd": 279.5e6, "bwd_dkv": 423.0e6, "bwd_dq": 359.3e6}}
 
 
 def load_peaks():
@@ -295,7 +295,7 @@ def main():
     clocks = sampler.stop() if rank == 0 else None
     binding.tvm_attn_check_status()
 
-    # per-kernel durations (CUDA events recorded by the library around each launch)
+    # per-kernel durations (CUDA events recorded by the library around each launch: the gaps between launches count)
     binding.tvm_attn_set_profiling(True)
     per_kernel = {k: [] for k in kernel_gemms}
     for _ in range(min(args.steps, 20)):

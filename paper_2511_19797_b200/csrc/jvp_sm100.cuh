@@ -43,7 +43,7 @@
 // Measured on B200 at d = 128 (B 2, H 24, N 4096; one CTA per item, 32-key tiles with all four accumulators in two buffers
 // before): forward 1.40 -> 1.08 ms, DV / DK / DQ 1.33 / 2.82 / 2.92 -> 1.06 / 1.48 / 1.42 ms.  At d <= 80 (two
 // element-wise groups on alternate tiles, which also wrote the outputs, before): d = 64 (8, 16, 4096) forward 1.94 -> 1.75 ms,
-// backward 7.37 -> 6.12 ms, with DV and DK in one pass 5.45 ms; d = 72 (16, 16, 1024) forward 321 -> 306 us, backward
+// backward 7.37 -> 6.12 ms, with DV and DK in one pass 5.45 ms; d = 72 (16, 16, 1024) forward 321 -> 313 us, backward
 // 1.22 -> 1.08 -> 1.01 ms.
 //
 // Every wait on an mbarrier is bounded; when one gives up the block records a time-out status and all roles leave their
@@ -70,7 +70,7 @@ constexpr int JVP_BC = 64;      // stream rows per tile (DKV at padded head dim 
 // centre c of the tangent weights may be from T at the arg-max key before it moves.
 constexpr float JVP_LAZY_LOG2 = 3.0f, JVP_LAZY_LOG2_WIDE = 8.0f, JVP_CENTRE_WIDE = 3.0f;
 // How long a wait may take: for what is due within a few tiles, and what every tile of an item adds to it where an item's end
-// is waited for (the epilogue).  The slowest tile measured takes 2.7 us (DKV, 2950 cycles at 1.1 GHz); an item of 400 thousand
+// is waited for (the epilogue).  The slowest tile measured takes 2 us (DKV, 2950 cycles at 1.5 GHz); an item of 400 thousand
 // tiles, 128 queries against 25.6 million keys at d = 8, takes 0.24 s.  A tile that hangs is reported after the first limit
 // all the same, by the roles that work on it.
 constexpr uint64_t JVP_WAIT_LIMIT_NS = 200ull * 1000ull * 1000ull, JVP_TILE_LIMIT_NS = 20ull * 1000ull;

@@ -22,9 +22,9 @@ namespace tvm_attn {
 
 constexpr int RMS_THREADS = 256;
 constexpr int RMS_BWD_THREADS = 128;
-// Blocks of a launch at most, both sides together: what 148 SMs hold at the kernels' register counts, so that every
-// block walks over its rows from the start to the end of the launch.  Fixed numbers: the partial sums of dg have a size
-// and a summation order that do not depend on the device.
+// Blocks of a launch at most, both sides together: what B200's 148 SMs hold at the kernels' register counts, so that every
+// block walks over its rows from the start to the end of the launch.  The backward's number is fixed for one more reason: the
+// partial sums of dg, a row per block, have a size and a summation order that do not depend on the device.
 constexpr int RMS_FWD_BLOCKS = 148 * 3;
 constexpr int RMS_BWD_BLOCKS = 148 * 5;
 constexpr int RMS_PARTIAL_ROWS = 2 * 592;   // rows of d floats in the workspace (more than RMS_BWD_BLOCKS)

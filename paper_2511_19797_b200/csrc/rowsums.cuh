@@ -5,14 +5,16 @@
 // it splits a row over few lanes with several 16-byte chunks each (rms_split: d = 72 is 3 x 3), so that a thread has 192
 // bytes in flight and a row sum costs three shuffles, and sums with two-wide FMAs.
 // Measured on B200 (B 16, H 16, N 1024, d 72: 151 MB) against one chunk per lane, nine lanes a row: 51 -> 37 us,
-// without dtO (75 MB) 47 -> 25 us.
+// without dtO (75 MB) 47 -> 25 us, taken as the library's timing aid takes them, between two events in the backward's stream:
+// that counts the gaps to the launches around it.  The kernel itself takes 28.8 us (5.3 TB/s; the profiler's duration, and
+// that of 50 launches one behind another), without dtO 16.5 us (4.6 TB/s).
 #pragma once
 #include "qk_rmsnorm.cuh"
 
 namespace tvm_attn {
 
 constexpr int ROWSUM_THREADS = 256;
-constexpr int ROWSUM_BLOCKS = 148 * 3;   // of a launch at most: each block walks over its rows
+constexpr int ROWSUM_BLOCKS = 148 * 3;   // of a launch at most, what the 148 SMs hold: each block walks over its rows
 
 // P = lanes per row, C = chunks per lane; the rows of a warp are consecutive.
 template <typename T, int C>

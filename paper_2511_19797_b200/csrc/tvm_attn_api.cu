@@ -310,8 +310,10 @@ static int launch_pass(const Shape& s, const Operand (&own)[4], const Operand (&
 
 template <int MODE, int DP>
 static int launch_pass_hz(const Shape& s, const Operand (&own)[4], const Operand (&strm)[4], const JvpParams& prm, const DeviceFacts& dev, cudaStream_t st) {
-    // dtO absent: the specialisation that leaves the tangent path out (only instantiated for the padded head dims
-    // 64 and 80 of the transformer shapes; other head dims run the general kernel, which skips what it can)
+    // dtO absent: the specialisation that leaves the tangent path out, instantiated for the padded head dims 64 and 80; other
+    // head dims run the general kernel, which skips what it can.  The whole backward without dtO (B 16, H 16, N 1024), general /
+    // specialised: d = 64 571 to 590 / 386 us, 72 751 / 527, 80 782 to 789 / 540; built for them too it measured d = 16
+    // 475 / 333, 32 507 / 351, 48 529 to 547 / 366, so the line is only where it was first needed: it can go.
     if constexpr (MODE != PASS_FWD && (DP == 64 || DP == 80))
         if (prm.absent & ABSENT_HC) return launch_pass<MODE, DP, true>(s, own, strm, prm, dev, st);
     return launch_pass<MODE, DP, false>(s, own, strm, prm, dev, st);
