@@ -256,13 +256,22 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
 }
 
 // The same with the abort flag given by its shared-memory address (one register instead of two where a role has none to
-// spare).
+// spare), and as one small loop: a kernel has some 30 of these waits, its roles share an instruction cache, and a wait that
+// jumps over the code for the rare cases costs its warp 130 to 400 cycles where this one costs 85.  (Kernels of 60 instead of
+// 170 KB; d = 72 (16, 16, 1024): forward 279 -> 249 us, DKV 490 -> 463.)  The clock is read every 256 polls.
 __device__ __forceinline__ bool mbar_wait_warp_s(uint32_t bar, uint32_t parity, uint32_t abort_addr, uint64_t limit_ns) {
-    bool ok = mbar_try_wait(bar, parity);
-    for (int it = 0; it < 256 && !ok; ++it) ok = mbar_try_wait(bar, parity);
-    if (__builtin_expect(__all_sync(0xffffffffu, ok), 1)) return true;
-    if (!ok) ok = mbar_wait(bar, parity, static_cast<volatile int*>(__cvta_shared_to_generic(abort_addr)), limit_ns);
-    return __all_sync(0xffffffffu, ok);
+    uint64_t t0 = 0;
+#pragma unroll 1
+    for (uint32_t it = 1;; ++it) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if (it & 255u) continue;
+        volatile int* abort_flag = static_cast<volatile int*>(__cvta_shared_to_generic(abort_addr));
+        const uint64_t t = globaltimer_ns();
+        if (t0 == 0) t0 = t;
+        const bool late = t - t0 > limit_ns;
+        if (late) *abort_flag = 1;
+        if (__any_sync(0xffffffffu, late || *abort_flag)) return false;
+    }
 }
 // Non-blocking test of two mbarrier phases at once; warp-uniform result.
 __device__ __forceinline__ bool mbar_test2_warp(uint32_t b0, uint32_t p0, uint32_t b1, uint32_t p1) {
