@@ -156,7 +156,7 @@ struct JvpCfg {
     static_assert(!XT || DP + DP / 2 <= 128, "operands do not fit behind their accumulators");
     static_assert(COL_SCORE + 4 * BC <= 512, "TMEM over-subscribed");
     // registers per thread: warpgroup 0, element-wise warps, epilogue warps (which hold an owner row, 4 registers a chunk)
-    static constexpr int REGS_LOAD = MODE == PASS_FWD ? 56 : 96, REGS_ELEM = MODE == PASS_FWD ? 184 : 152, REGS_EPI = MODE == PASS_FWD ? 88 : 112;
+    static constexpr int REGS_LOAD = MODE == PASS_FWD ? 56 : 96, REGS_ELEM = MODE == PASS_FWD ? 168 : 152, REGS_EPI = MODE == PASS_FWD ? 120 : 112;
     static_assert(REGS_LOAD + 2 * REGS_ELEM + REGS_EPI <= 4 * JVP_REGS, "more registers than the block has");
     // barriers
     static constexpr int B_EFULL = 0;
@@ -180,9 +180,9 @@ struct JvpCfg {
     // operands written: + half of the tile (DK, DQ), + 2 (g & 1) + half (FWD, DV), + pair (DKV)
     static constexpr int B_PREADY = B_OUTDONE + 4;
     static constexpr int B_SREAD = B_PREADY + 4;                       // DK, DQ: S, Sd read
-    static constexpr int B_FINAL = B_SREAD + 1;                        // the item's last output MMAs complete
-    static constexpr int B_ACCFREE = B_FINAL + 1;                      // the epilogue has read the accumulators
-    static constexpr int B_TURN = B_ACCFREE + 1;                       // FWD: + lane quadrant: row state of the tile decided
+    static constexpr int B_FINAL = B_SREAD + 1;                        // + pair of accumulators: the item's last output MMAs complete
+    static constexpr int B_ACCFREE = B_FINAL + NACC / 2;               // the epilogue has read the accumulators
+    static constexpr int B_TURN = B_ACCFREE + NACC / 2;                       // FWD: + lane quadrant: row state of the tile decided
     static constexpr int B_ROWSTAT = B_TURN + 4;                       // FWD: the item's row sums written
     static constexpr int B_DRAIN = B_ROWSTAT + 1;                      // used once, while winding down after a time-out
     static constexpr int NBARS = B_DRAIN + 1;
@@ -200,6 +200,11 @@ struct JvpCfg {
 __device__ __forceinline__ int jvp_pin(int v) {
     asm volatile("" : "+r"(v));
     return v;
+}
+
+// Items of this block.
+__device__ __forceinline__ int jvp_item_count(const JvpParams& p) {
+    return (int)blockIdx.x < p.items ? (p.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
 }
 
 // The value is computed here and not behind the next wait: the compiler moves arithmetic down to where its result is used,
@@ -543,7 +548,8 @@ __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE
 //
 // The tensor pipe takes about four MMAs ahead, 130 to 250 cycles of work; whatever the issuing warp does between two
 // batches beyond that leaves the pipe idle.  A wait for a barrier that has completed costs it 85 cycles, a commit 60, a
-// dependent scalar instruction ten.  So: ring positions are carried along as descriptors (every descriptor of a batch is
+// dependent scalar instruction ten, and an MMA 70 instead of 25 where the lane that issues it was elected in front of a branch
+// or a wait: each batch elects its own.  So: ring positions are carried along as descriptors (every descriptor of a batch is
 // the carried one plus a constant), barriers of the rings are tested ahead, in front of the batch before, what depends on
 // the item stays out of the tile's path, and which cotangent is absent (ABS) is a template parameter.
 struct JvpSlot {   // a ring's next tile: stage, phase, low descriptor halves of the stage and of its statistics
@@ -674,64 +680,85 @@ struct JvpIssue {
 // the next stage of the ring, and one completion for outputs and scores.  (Operands handed over in halves, a wait per barrier
 // and four commits: d = 72 (16, 16, 1024) 1034 -> 994 us for the backward, without dtO 656 -> 544.)  What bounds a tile now
 // is the pipe with two operands in shared memory, whose port the loads share: 2950 cycles, 2490 with nothing to load or compute.
+// The tiles run on through the items: the next item's first scores go in front of this one's last outputs, and each pair of
+// accumulators is handed to and from the epilogue on its own.  (d = 72, DKV and DQ, (64, 16, 256): the backward 345 -> 334 us.)
 template <int MODE, int DP, bool HZ, int ABS>
 __device__ __forceinline__ void jvp_issue_dkv(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
     using C = JvpCfg<MODE, DP>;
     using I = JvpIssue<MODE, DP, HZ, ABS>;
     constexpr int BC = C::BC;
     const JvpBlock<MODE, DP> k = shared.pinned();
-    const int T = jvp_pin(p.T), items = jvp_pin(p.items);
+    const int T = jvp_pin(p.T);
     const uint32_t x0 = ptx::desc_lo(k.own_tile(0), 16), x1 = ptx::desc_lo(k.own_tile(1), 16);
     const uint32_t x2 = ptx::desc_lo(k.own_tile(2), 16), x3 = ptx::desc_lo(k.own_tile(3), 16);
     constexpr uint32_t cS = C::COL_SCORE, cT = cS + BC, cD = cS + 2 * BC, cX = cS + 3 * BC;
     constexpr bool H = !HZ && !(ABS & ABSENT_HC), G = !(ABS & ABSENT_G);
     JvpSlot e = I::e_slot(k), l = I::l_slot(k);   // next tile of the scores
     uint32_t elo = e.lo, llo = l.lo;              // stages of the outputs' tile
-    int n = 0, it = 0;                            // next tile whose scores are issued
-    for (int item = blockIdx.x; item < items; item += gridDim.x, ++it) {
-        if (!k.wait(C::B_OWN, it)) return;
-        bool ready = false;                       // what the next batch waits for was seen complete
-        for (int j = -1; j < T; ++j) {
-            const bool out = j >= 0, score = j + 1 < T;
-            const uint32_t acc = j > 0 ? 1u : 0u;
-            // dtV += P^T Hc, dV += (P Nn)^T Hc + P^T G | (S, Sd) of the next tile
-            if (!ready && !(score ? k.wait2(C::B_PREADY, n - 1, C::B_LFULL + l.s, l.ph) : k.wait(C::B_PREADY, n - 1))) return;
-            if (j == 0 && it > 0 && !k.wait(C::B_ACCFREE, it - 1)) return;    // the first tile overwrites the accumulators
-            k.tile_fence();
-            uint32_t el = ptx::elect_one();
-            if (out) I::template dkv_outputs<H, H, G, 0>(el, cS, cT, elo, acc);
-            if (score) {
-                ready = ptx::mbar_test2_warp(k.bar(C::B_PREADY + 1), (n - 1) & 1, k.bar(C::B_EFULL + e.s), e.ph);
-                if (HZ) I::template single<true, false, 0>(el, cS, k, x0, l.lo, l.fold);
-                else I::template pair<true, false, true>(el, cS, k, x0, x1, l.lo, l.fold, 0);
-                ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
-                if (j + 2 == T) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE));
-                l.template next<C::SL, I::L_STEP, I::F_STEP>();
-            } else {
-                ready = false;
+    const int last = jvp_item_count(p) * T;
+    int sj = 0, si = 0, oj = -1, oi = 0;          // tile within its item and item: of the scores, of the outputs (one tile behind)
+    bool ready = false;                           // what the next batch waits for was seen complete
+    for (int n = 0; n <= last; ++n) {
+        const bool out = n > 0, score = n < last;
+        const uint32_t acc = oj > 0 ? 1u : 0u;
+        // dtV += P^T Hc, dV += (P Nn)^T Hc + P^T G | (S, Sd) of the next tile
+        if (!ready && !(score ? k.wait2(C::B_PREADY, n - 1, C::B_LFULL + l.s, l.ph) : k.wait(C::B_PREADY, n - 1))) return;
+        if (oj == 0 && oi > 0 && !k.wait(C::B_ACCFREE, oi - 1)) return;    // the first tile overwrites the accumulators
+        k.tile_fence();
+        if (out) {
+            const uint32_t el = ptx::elect_one();
+            I::template dkv_outputs<H, H, G, 0>(el, cS, cT, elo, acc);
+            if (oj == T - 1) ptx::mma_commit_p(el, k.bar(C::B_FINAL));
+        }
+        if (score) {
+            if (sj == 0) {
+                if (!k.wait(C::B_OWN, si)) return;
+                k.tile_fence();
             }
-            // dtK += W^T Q, dK += dA^T Q + W^T tQ | (D, X) of the next tile
-            if (!ready && !(score ? k.wait2(C::B_PREADY + 1, n - 1, C::B_EFULL + e.s, e.ph) : k.wait(C::B_PREADY + 1, n - 1))) return;
-            if (!out && !k.wait(C::B_OWN + 1, it)) return;
-            k.tile_fence();
-            el = ptx::elect_one();
-            if (out) {
-                I::template dkv_outputs<H, true, H, 2>(el, cD, cX, llo, acc);
-                elo = elo + I::E_STEP == e.lo0 + C::SE * I::E_STEP ? e.lo0 : elo + I::E_STEP;
-                llo = llo + I::L_STEP == l.lo0 + C::SL * I::L_STEP ? l.lo0 : llo + I::L_STEP;
+            ready = ptx::mbar_test2_warp(k.bar(C::B_PREADY + 1), (n - 1) & 1, k.bar(C::B_EFULL + e.s), e.ph);
+            const uint32_t el = ptx::elect_one();
+            if (HZ) I::template single<true, false, 0>(el, cS, k, x0, l.lo, l.fold);
+            else I::template pair<true, false, true>(el, cS, k, x0, x1, l.lo, l.fold, 0);
+            ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
+            if (sj == T - 1) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE));
+            l.template next<C::SL, I::L_STEP, I::F_STEP>();
+        } else {
+            ready = false;
+        }
+        // dtK += W^T Q, dK += dA^T Q + W^T tQ | (D, X) of the next tile
+        if (!ready && !(score ? k.wait2(C::B_PREADY + 1, n - 1, C::B_EFULL + e.s, e.ph) : k.wait(C::B_PREADY + 1, n - 1))) return;
+        if (oj == 0 && oi > 0 && !k.wait(C::B_ACCFREE + 1, oi - 1)) return;
+        k.tile_fence();
+        if (out) {
+            const uint32_t el = ptx::elect_one();
+            I::template dkv_outputs<H, true, H, 2>(el, cD, cX, llo, acc);
+            elo = elo + I::E_STEP == e.lo0 + C::SE * I::E_STEP ? e.lo0 : elo + I::E_STEP;
+            llo = llo + I::L_STEP == l.lo0 + C::SL * I::L_STEP ? l.lo0 : llo + I::L_STEP;
+            if (oj == T - 1) {
+                ptx::mma_commit_p(el, k.bar(C::B_FINAL + 1));
+                oj = -1;
+                ++oi;
             }
-            if (score) {
-                // (the stage of the tile after the next one, where there is one)
-                ready = j + 2 < T && ptx::mbar_test2_warp(k.bar(C::B_PREADY), n & 1, k.bar(C::B_LFULL + l.s), l.ph);
-                if (HZ) I::template single<false, false, 1>(el, cX, k, x2, e.lo, e.fold);   // X = V G^T alone
-                else I::template pair<false, false, H>(el, cD, k, x2, x3, e.lo, e.fold, 0);  // (tV Hc^T is zero with Hc absent)
-                ptx::mma_commit_p(el, k.bar(C::B_XFULL + (n & 3)));
-                if (j + 2 == T) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE + 1));
-                e.template next<C::SE, I::E_STEP, I::F_STEP>();
-                ++n;
-            } else {
-                ptx::mma_commit_p(el, k.bar(C::B_FINAL));
+        }
+        ++oj;
+        if (score) {
+            if (sj == 0) {
+                if (!k.wait(C::B_OWN + 1, si)) return;
+                k.tile_fence();
             }
+            // (the stage of the tile after the next one, where there is one)
+            ready = n + 1 < last && ptx::mbar_test2_warp(k.bar(C::B_PREADY), n & 1, k.bar(C::B_LFULL + l.s), l.ph);
+            const uint32_t el = ptx::elect_one();
+            if (HZ) I::template single<false, false, 1>(el, cX, k, x2, e.lo, e.fold);   // X = V G^T alone
+            else I::template pair<false, false, H>(el, cD, k, x2, x3, e.lo, e.fold, 0);  // (tV Hc^T is zero with Hc absent)
+            ptx::mma_commit_p(el, k.bar(C::B_XFULL + (n & 3)));
+            if (sj == T - 1) {
+                ptx::mma_commit_p(el, k.bar(C::B_OWNFREE + 1));
+                sj = -1;
+                ++si;
+            }
+            ++sj;
+            e.template next<C::SE, I::E_STEP, I::F_STEP>();
         }
     }
 }
@@ -754,7 +781,6 @@ __device__ __forceinline__ void jvp_issue_one_pair(const JvpParams& p, const Jvp
     for (int item = blockIdx.x; item < items; item += gridDim.x, ++it) {
         const bool more = item + (int)gridDim.x < items;
         if (!opened && !k.wait(RDY, it)) return;
-        if (it > 0 && !k.wait(C::B_ACCFREE, it - 1)) return;   // the first tile overwrites the accumulators
         for (int j = opened ? 0 : -1; j < T; ++j) {
             // The scores of the next tile go in front of this tile's outputs.  Where they open an item they do if its owner
             // operands are there already, else they follow when the loop gets there.
@@ -775,6 +801,9 @@ __device__ __forceinline__ void jvp_issue_one_pair(const JvpParams& p, const Jvp
             if (j < 0) continue;
             const int b = g & 1;
             if (!k.wait2(C::B_PREADY + 2 * b, g >> 1, C::B_LFULL + l.s, l.ph)) return;
+            // The first tile overwrites the accumulators.  (Waited for here and not before the item's first scores, and operands loaded
+            // ahead: an item's end costs 2000 cycles instead of 5500.  d = 72: (64, 16, 256) 111 -> 106 us.)
+            if (j == 0 && it > 0 && !k.wait(C::B_ACCFREE, it - 1)) return;
             k.tile_fence();
             const uint32_t a0 = C::COL_SCORE + b * 2 * C::BC;
             I::template outputs<0>(ptx::elect_one(), a0, a0 + C::BC, l.lo, j > 0 ? 1u : 0u);
@@ -797,57 +826,68 @@ __device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const Jv
     using C = JvpCfg<MODE, DP>;
     using I = JvpIssue<MODE, DP, HZ, ABS>;
     const JvpBlock<MODE, DP> k = shared.pinned();
-    const int T = jvp_pin(p.T), items = jvp_pin(p.items);
+    const int T = jvp_pin(p.T);
     const uint32_t x0 = ptx::desc_lo(k.own_tile(0), 16), x1 = ptx::desc_lo(k.own_tile(1), 16);
     const uint32_t x2 = C::XT ? C::COL_X0 : ptx::desc_lo(k.own_tile(2), 16), x3 = C::XT ? C::COL_X1 : ptx::desc_lo(k.own_tile(3), 16);
     constexpr uint32_t cS = C::COL_SCORE, cD = C::COL_SCORE + 2 * C::BC, cX = C::COL_SCORE + 3 * C::BC;
     constexpr bool X3 = !(ABS & ABSENT_G);   // DQ: X3 Y2^T = G V^T is zero with G absent
     JvpSlot e = I::e_slot(k), l = I::l_slot(k);
     uint32_t lo = l.lo;        // L stage of the outputs' tile
-    int n = 0;                 // next tile whose scores are issued
-    bool e_ready = false;
-    int it = 0;
-    for (int item = blockIdx.x; item < items; item += gridDim.x, ++it) {
-        if (!k.wait(C::B_OWN, it)) return;
-        for (int j = -1; j < T; ++j) {
-            if (j + 1 < T) {   // (S, Sd) of the next tile
-                if (!k.wait2(C::B_SREAD, n - 1, C::B_LFULL + l.s, l.ph)) return;   // (a fresh barrier passes for n = 0)
-                k.tile_fence();
-                const uint32_t el = ptx::elect_one();
-                if (HZ) I::template single<true, false, 0>(el, cS, k, x0, l.lo, l.fold);
-                else I::template pair<true, false, true>(el, cS, k, x0, x1, l.lo, l.fold, 0);
-                ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
-                if (C::XT && j + 2 == T) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE));
-                l.template next<C::SL, I::L_STEP, I::F_STEP>();
+    const int last = jvp_item_count(p) * T;
+    int sj = 0, si = 0, oj = -1, oi = 0;   // tile within its item and item: of the scores, of the outputs (one tile behind)
+    for (int n = 0; n <= last; ++n) {
+        const bool score = n < last;
+        auto scores = [&]() {   // (S, Sd) of the next tile
+            if (!k.wait2(C::B_SREAD, n - 1, C::B_LFULL + l.s, l.ph)) return false;   // (a fresh barrier passes for n = 0)
+            if (sj == 0 && !k.wait(C::B_OWN, si)) return false;
+            k.tile_fence();
+            const uint32_t el = ptx::elect_one();
+            if (HZ) I::template single<true, false, 0>(el, cS, k, x0, l.lo, l.fold);
+            else I::template pair<true, false, true>(el, cS, k, x0, x1, l.lo, l.fold, 0);
+            ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
+            if (C::XT && sj == T - 1) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE));
+            l.template next<C::SL, I::L_STEP, I::F_STEP>();
+            return true;
+        };
+        // Where an item opens with owner tiles that the item before has used to its end (WIDE), its outputs go first.
+        const bool first = C::XT || sj > 0;
+        if (score && first && !scores()) return;
+        const bool e_ready = ptx::mbar_test_warp(k.bar(C::B_EFULL + e.s), e.ph);
+        if (n > 0) {       // outputs
+            if (!k.wait(C::B_PREADY, n - 1)) return;
+            if (oj == 0 && oi > 0 && !k.wait(C::B_ACCFREE, oi - 1)) return;    // the first tile overwrites the accumulators
+            ptx::tc_fence_after_sync();
+            I::template outputs<0>(ptx::elect_one(), cD, cX, lo, oj > 0 ? 1u : 0u);
+            if (!k.wait(C::B_PREADY + 1, n - 1)) return;
+            ptx::tc_fence_after_sync();
+            const uint32_t el = ptx::elect_one();
+            I::template outputs<2>(el, cD, cX, lo, 1u);
+            ptx::mma_commit_p(el, k.bar(C::B_OUTDONE + ((n - 1) & 3)));
+            if (oj == T - 1) {
+                ptx::mma_commit_p(el, k.bar(C::B_FINAL));
+                oj = -1;
+                ++oi;
             }
-            e_ready = ptx::mbar_test_warp(k.bar(C::B_EFULL + e.s), e.ph);
-            if (j >= 0) {      // outputs
-                if (!k.wait(C::B_PREADY, n - 1)) return;
-                if (j == 0 && !k.wait(C::B_ACCFREE, it - 1)) return;    // the first tile overwrites the accumulators
-                ptx::tc_fence_after_sync();
-                I::template outputs<0>(ptx::elect_one(), cD, cX, lo, j > 0 ? 1u : 0u);
-                if (!k.wait(C::B_PREADY + 1, n - 1)) return;
-                ptx::tc_fence_after_sync();
-                const uint32_t el = ptx::elect_one();
-                I::template outputs<2>(el, cD, cX, lo, 1u);
-                ptx::mma_commit_p(el, k.bar(C::B_OUTDONE + ((n - 1) & 3)));
-                if (j == T - 1) ptx::mma_commit_p(el, k.bar(C::B_FINAL));
-                lo = lo + I::L_STEP == l.lo0 + C::SL * I::L_STEP ? l.lo0 : lo + I::L_STEP;
-            } else if (C::XT && !k.wait(C::B_XRDY, it)) {
-                return;
+            lo = lo + I::L_STEP == l.lo0 + C::SL * I::L_STEP ? l.lo0 : lo + I::L_STEP;
+        }
+        ++oj;
+        if (score && !first && !scores()) return;
+        if (score) {       // (D, X) of the next tile
+            if (!e_ready && !k.wait(C::B_EFULL + e.s, e.ph)) return;
+            if (C::XT && sj == 0 && !k.wait(C::B_XRDY, si)) return;
+            k.tile_fence();
+            const uint32_t el = ptx::elect_one();
+            // HZ (DQ): X = G V^T alone: X3 and the stage's first tensor
+            if (HZ) I::template single<false, C::XT, 0>(el, cX, k, x3, e.lo, e.fold);
+            else I::template pair<false, C::XT, X3>(el, cD, k, x2, x3, e.lo, e.fold, 0);
+            ptx::mma_commit_p(el, k.bar(C::B_XFULL + (n & 3)));
+            if (sj == T - 1) {
+                ptx::mma_commit_p(el, k.bar(C::XT ? C::B_XFREE : C::B_OWNFREE));
+                sj = -1;
+                ++si;
             }
-            if (j + 1 < T) {   // (D, X) of the next tile
-                if (!e_ready && !k.wait(C::B_EFULL + e.s, e.ph)) return;
-                k.tile_fence();
-                const uint32_t el = ptx::elect_one();
-                // HZ (DQ): X = G V^T alone: X3 and the stage's first tensor
-                if (HZ) I::template single<false, C::XT, 0>(el, cX, k, x3, e.lo, e.fold);
-                else I::template pair<false, C::XT, X3>(el, cD, k, x2, x3, e.lo, e.fold, 0);
-                ptx::mma_commit_p(el, k.bar(C::B_XFULL + (n & 3)));
-                if (j + 2 == T) ptx::mma_commit_p(el, k.bar(C::XT ? C::B_XFREE : C::B_OWNFREE));
-                e.template next<C::SE, I::E_STEP, I::F_STEP>();
-                ++n;
-            }
+            ++sj;
+            e.template next<C::SE, I::E_STEP, I::F_STEP>();
         }
     }
 }
@@ -1046,8 +1086,8 @@ __device__ __forceinline__ void jvp_elem_dv(const JvpParams& p, const JvpBlock<P
     constexpr int BC = C::BC, HC = BC / 2;
     const uint32_t sb0 = (static_cast<uint32_t>(q * 32) << 16) + C::COL_SCORE + grp * HC;
     const uint64_t c2c2 = ptx::pack2(p.c2, p.c2), aa = ptx::pack2(p.alpha, p.alpha);
-    const int n_it = (int)blockIdx.x < p.items ? (p.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-    for (int g = 0; g < n_it * p.T; ++g) {
+    const int tiles = jvp_item_count(p) * p.T;
+    for (int g = 0; g < tiles; ++g) {
         const int b = g & 1;
         const uint32_t sb = sb0 + b * 2 * BC;
         if (!k.done(C::B_SFULL, g)) return;
@@ -1213,8 +1253,8 @@ __device__ __forceinline__ void jvp_elem_dkv(const JvpParams& p, const JvpBlock<
     constexpr int BC = C::BC, NU = BC / 16;
     const uint32_t sb = (static_cast<uint32_t>(q * 32 + grp * 16) << 16) + C::COL_SCORE;
     const uint64_t c2c2 = ptx::pack2(p.c2, p.c2), aa = ptx::pack2(p.alpha, p.alpha);
-    const int n_it = (int)blockIdx.x < p.items ? (p.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-    for (int g = 0; g < n_it * p.T; ++g) {
+    const int tiles = jvp_item_count(p) * p.T;
+    for (int g = 0; g < tiles; ++g) {
         uint64_t P2[4 * NU], N2[4 * NU];
         uint32_t y[8 * NU], x[8 * NU];   // S, Sd, then D, X
         if (!k.done(C::B_SFULL, g)) return;
@@ -1323,12 +1363,11 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
     for (int item = blockIdx.x; item < p.items; item += gridDim.x, ++it) {
         if (C::XT && item + (int)gridDim.x < p.items) {
             load_x(item + gridDim.x, 0, v0);                       // in flight during the wait
-            if (MODE != PASS_FWD) load_x(item + gridDim.x, 1, v1);   // (the forward has no registers for the second)
+            load_x(item + gridDim.x, 1, v1);
             if (!k.wait_item(C::B_XFREE, it)) return;
             ptx::tc_fence_after_sync();
             store_x(0, v0);
-            if (MODE == PASS_FWD) load_x(item + gridDim.x, 1, v0);
-            store_x(1, MODE != PASS_FWD ? v1 : v0);
+            store_x(1, v1);
             ptx::tmem_wait_st();
             k.arrive(C::B_XRDY, lane);
         }
@@ -1351,34 +1390,51 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
                 p.mu_out[at] = f.w + mun;
             }
         }
-        if (!k.wait_item(C::B_FINAL, it)) return;
-        ptx::tc_fence_after_sync();
 #pragma unroll 1
-        for (int i = 0; i < C::KS * (C::NACC / 2); ++i) {
-            const bool second = C::DKV && i >= C::KS;      // the second pair of accumulators
-            const int ch = second ? i - C::KS : i;
-            const uint32_t at = lanes + 16 * ch + (second ? 2 * C::COL_ACC1 : 0);
-            __nv_bfloat16* const out0 = second ? p.out2 : p.out0;
-            __nv_bfloat16* const out1 = second ? p.out3 : p.out1;
-            if (C::DKV) f0 = second ? p.out_scale : 1.0f;
-            uint32_t x0[16], x1[16], q0[8], q1[8];
-            ptx::tmem_ld16(at + C::COL_ACC0, x0);
-            ptx::tmem_ld16(at + C::COL_ACC1, x1);
-            ptx::tmem_wait_ld();
-            if (i == C::KS * (C::NACC / 2) - 1) k.arrive(C::B_ACCFREE, lane);
+        for (int pair = 0; pair < C::NACC / 2; ++pair) {
+            const uint32_t at = lanes + 2 * pair * C::COL_ACC1;
+            __nv_bfloat16* const out0 = pair ? p.out2 : p.out0;
+            __nv_bfloat16* const out1 = pair ? p.out3 : p.out1;
+            if (C::DKV) f0 = pair ? p.out_scale : 1.0f;
+            auto read = [&](int ch, uint32_t (&q0)[8], uint32_t (&q1)[8]) {   // 16 columns of both accumulators, as bf16
+                uint32_t x0[16], x1[16];
+                ptx::tmem_ld16(at + 16 * ch + C::COL_ACC0, x0);
+                ptx::tmem_ld16(at + 16 * ch + C::COL_ACC1, x1);
+                ptx::tmem_wait_ld();
 #pragma unroll
-            for (int c = 0; c < 16; c += 2) {
-                float a0 = __uint_as_float(x0[c]) * f0, a1 = __uint_as_float(x0[c + 1]) * f0;
-                float b0 = __uint_as_float(x1[c]) * f0, b1 = __uint_as_float(x1[c + 1]) * f0;
-                if (MODE == PASS_FWD) { b0 = fmaf(-mun, a0, b0); b1 = fmaf(-mun, a1, b1); }
-                q0[c >> 1] = ptx::pack_bf16(a0, a1);
-                q1[c >> 1] = ptx::pack_bf16(b0, b1);
+                for (int c = 0; c < 16; c += 2) {
+                    float a0 = __uint_as_float(x0[c]) * f0, a1 = __uint_as_float(x0[c + 1]) * f0;
+                    float b0 = __uint_as_float(x1[c]) * f0, b1 = __uint_as_float(x1[c + 1]) * f0;
+                    if (MODE == PASS_FWD) { b0 = fmaf(-mun, a0, b0); b1 = fmaf(-mun, a1, b1); }
+                    q0[c >> 1] = ptx::pack_bf16(a0, a1);
+                    q1[c >> 1] = ptx::pack_bf16(b0, b1);
+                }
+            };
+            auto store = [&](int ch, const uint32_t (&q0)[8], const uint32_t (&q1)[8]) {
+                if (16 * ch >= p.d) return;
+                const bool has_hi = 16 * ch + 8 < p.d;
+                store_row_pairs(out1 + off + 16 * ch, p.o.rs, lane, ok_even, ok_odd, has_hi, make_uint4(q1[0], q1[1], q1[2], q1[3]), make_uint4(q1[4], q1[5], q1[6], q1[7]));
+                if (out0)   // null with Hc absent: acc0 was never written, its gradient is zero
+                    store_row_pairs(out0 + off + 16 * ch, p.o.rs, lane, ok_even, ok_odd, has_hi, make_uint4(q0[0], q0[1], q0[2], q0[3]), make_uint4(q0[4], q0[5], q0[6], q0[7]));
+            };
+            if (!k.wait_item(C::B_FINAL + pair, it)) return;
+            ptx::tc_fence_after_sync();
+            // The next item's first output MMAs wait for the accumulators: up to d = 80 all of them are read and converted first and
+            // stored behind the arrival (reads and stores in turn held them for 3200 cycles at d = 72).  WIDE: there are not the
+            // registers, and the items are long.
+            constexpr int HOLD = C::WIDE ? 1 : C::KS;
+#pragma unroll 1
+            for (int ch = 0; ch < C::KS - HOLD; ++ch) {
+                uint32_t q0[8], q1[8];
+                read(ch, q0, q1);
+                store(ch, q0, q1);
             }
-            if (16 * ch >= p.d) continue;
-            const bool has_hi = 16 * ch + 8 < p.d;
-            store_row_pairs(out1 + off + 16 * ch, p.o.rs, lane, ok_even, ok_odd, has_hi, make_uint4(q1[0], q1[1], q1[2], q1[3]), make_uint4(q1[4], q1[5], q1[6], q1[7]));
-            if (out0)   // null with Hc absent: acc0 was never written, its gradient is zero
-                store_row_pairs(out0 + off + 16 * ch, p.o.rs, lane, ok_even, ok_odd, has_hi, make_uint4(q0[0], q0[1], q0[2], q0[3]), make_uint4(q0[4], q0[5], q0[6], q0[7]));
+            uint32_t q0[HOLD][8], q1[HOLD][8];
+#pragma unroll
+            for (int i = 0; i < HOLD; ++i) read(C::KS - HOLD + i, q0[i], q1[i]);
+            k.arrive(C::B_ACCFREE + pair, lane);
+#pragma unroll
+            for (int i = 0; i < HOLD; ++i) store(C::KS - HOLD + i, q0[i], q1[i]);
         }
     }
 }
@@ -1419,8 +1475,8 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
         init(C::B_SFULL, 12, 1);       // SFULL, XFULL, OUTDONE
         init(C::B_PREADY, 4, C::DKV ? 8 : 4);   // (of four: the warps of a group)
         init(C::B_SREAD, 1, 8);
-        init(C::B_FINAL, 1, 1);
-        init(C::B_ACCFREE, 1, 4);
+        init(C::B_FINAL, C::NACC / 2, 1);
+        init(C::B_ACCFREE, C::NACC / 2, 4);
         init(C::B_TURN, 4, 1);
         init(C::B_ROWSTAT, 1, 8);
         init(C::B_DRAIN, 1, 1);
