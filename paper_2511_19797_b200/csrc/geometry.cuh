@@ -18,9 +18,6 @@ struct Geom {
     }
 };
 
-// Absent cotangents of a backward call (null dtO = Hc, null dO = G), as bits.
-enum : int { ABSENT_HC = 1, ABSENT_G = 2 };
-
 #ifdef __CUDACC__
 // Rows of 2 d bytes, lane = row, 32 bytes (lo, hi) of its row per lane: written 16 bytes per lane, one warp
 // instruction touches 32 half sectors in 32 cache lines.  This helper pairs the lanes instead: lanes 2 i and

@@ -11,6 +11,8 @@
 //   DK    keys        queries      S^T, Sd^T, D^T = V Hc^T, X^T = tV Hc^T + V G^T        W^T, dA^T               dtK/alpha, dK/alpha   (steps 2, 4)
 //   DKV   keys        queries      as DK                                                  as DV; as DK            as DV; as DK (acc2, acc3)
 //   DQ    queries     keys         S, Sd, D = Hc V^T, X = G V^T + Hc tV^T                 W, dA                   dtQ/alpha, dQ/alpha   (steps 3, 5)
+//   DKV_G keys        queries      S^T, X^T = V G^T                                       P^T, dA^T               dV, dK/alpha
+//   DQ_G  queries     keys         S, X = G V^T                                           (none), dA              (none), dQ/alpha
 //
 //   score pair:  S = X0 Y0^T,  Sd = X1 Y0^T + X0 Y1^T        outputs:  acc0 += A0 B0,  acc1 += A1 B0 + A0 B1
 //
@@ -20,6 +22,9 @@
 // DKV does DV's and DK's work with one computation of the scores, and one exponential, instead of two.  Its four accumulators
 // leave tensor memory for four score blocks of 64 columns at d <= 64 and of 48 at d <= 80; above that DV and DK run on their own.
 //
+// DKV_G and DQ_G are the backward without Hc = dtO (the "detach JVP" setting), where everything that only feeds the tangent path
+// is zero and what remains is the standard attention backward, dA = P (X - c).
+//
 // A work item is 128 owner rows of one head, against which the other side streams in tiles of 64 rows (48).  The grid has
 // one CTA per SM (a CTA needs the whole tensor memory of one); the items go round-robin over the CTAs, and the rings,
 // the score buffers and all barrier phases run on through the items.
@@ -28,7 +33,7 @@
 //   warp 0    loads the owner tiles and the E ring (stream tensors that only the score MMAs read)
 //   warp 1    issues the MMAs
 //   warp 2    loads the L ring (stream tensors the output MMAs read)
-//   warp 3    DKV: puts the per-query statistics into the tiles (FOLD below)
+//   warp 3    DKV, DKV_G: puts the per-query statistics into the tiles (FOLD below)
 //   warps 4-11   element-wise work, two groups of four warps
 //   warps 12-15  epilogue: normalise, convert and store an item's accumulators while the next item is under way
 //
@@ -61,7 +66,7 @@
 
 namespace tvm_attn {
 
-enum : int { PASS_FWD = 0, PASS_DV = 1, PASS_DK = 2, PASS_DQ = 3, PASS_DKV = 4 };
+enum : int { PASS_FWD = 0, PASS_DV = 1, PASS_DK = 2, PASS_DQ = 3, PASS_DKV = 4, PASS_DKV_G = 5, PASS_DQ_G = 6 };
 
 constexpr int JVP_THREADS = 512;
 constexpr int JVP_ROWS = 128;   // owner rows per item
@@ -99,10 +104,9 @@ struct JvpParams {
     const float* nsig1;  // -rowsum(dtO * O)
     const float* ncvec;  // -rowsum(dO * O) - rowsum(dtO * tO)
     int* status;         // device status word; non-zero makes the kernel a no-op
-    // Absent cotangents (a null dO or dtO means zero; Sec. 5.3 "detach JVP" is dtO absent): bit 0 = Hc (dtO),
-    // bit 1 = G (dO).  An absent tensor is never loaded; where an MMA still reads its tile, the tile is zeroed once,
-    // and the MMAs whose result would be exactly zero are not issued.  out0 may be null when Hc is absent.
-    int absent;
+    // G (dO) is absent: null means zero.  It is never loaded; where an MMA still reads its tile, the tile is zeroed once, and the
+    // MMAs whose result would be exactly zero are not issued.
+    int no_g;
     uint64_t item_wait_ns;     // how long the end of an item may be waited for
 };
 
@@ -110,8 +114,9 @@ template <int MODE, int DP>
 struct JvpCfg {
     static_assert(DP % 16 == 0 && DP >= 16 && DP <= 128, "padded head dim must be 16..128");
     static constexpr bool DKV = MODE == PASS_DKV;
-    static constexpr int NPAIR = MODE == PASS_FWD || MODE == PASS_DV ? 1 : 2;  // score pairs
-    static constexpr bool TRANSPOSED = MODE != PASS_FWD && MODE != PASS_DQ;    // owner rows are keys
+    static constexpr bool GONLY = MODE == PASS_DKV_G || MODE == PASS_DQ_G;     // one ring (L) of two tensors, two products instead of pairs
+    static constexpr int NPAIR = MODE == PASS_DK || MODE == PASS_DQ || DKV ? 2 : 1;  // score pairs
+    static constexpr bool TRANSPOSED = MODE != PASS_FWD && MODE != PASS_DQ && MODE != PASS_DQ_G;    // owner rows are keys
     // Stream rows per tile.  Four accumulators of DP columns and four of BC have to fit into 512.
     static constexpr int BC = DKV && DP > 64 ? 48 : JVP_BC, KS = DP / 16;
     static constexpr int NA = DP > 64 ? 2 : 1;             // 64-column swizzle atoms per row
@@ -122,41 +127,43 @@ struct JvpCfg {
     static constexpr bool WIDE = DP > 80;
     static constexpr bool TAIL = NA == 2 && !WIDE;
     static_assert(WIDE || (MODE != PASS_DV && MODE != PASS_DK), "DV and DK on their own: only where DKV does not fit");
-    static_assert(!WIDE || !DKV, "DKV: four accumulators do not fit");
+    static_assert(!WIDE || (!DKV && !GONLY), "DKV: four accumulators do not fit; head dims above 80 take both cotangents");
     static constexpr bool E_MN = DKV;                      // the E ring is read MN-major too: swizzled atoms like the L ring's
-    // Owner operands.  The pair of the score MMAs on the tile's critical chain (FWD: the only pair; DQ: the second) lies in
+    // Owner operands.  The pair of the score MMAs on the tile's critical chain (FWD: the only pair; DQ: the second; DKV_G, DQ_G: both tensors) lies in
     // tensor memory as bf16 A operands: an MMA with A in shared memory moves 4 KB of A per k-step through the
     // shared-memory port.  WIDE, DKV: tensor memory has no room, everything is in shared memory.
     static constexpr bool XT = !WIDE && !DKV;
     static constexpr int NOWN = 2 * NPAIR - (XT ? 2 : 0);   // owner tensors in shared memory
-    // FOLD (DKV): the per-query statistics belong to the columns of the tile, the same for every thread; read from
+    // FOLD (DKV, DKV_G): the per-query statistics belong to the columns of the tile, the same for every thread; read from
     // shared memory they would cost 512 bytes a warp and column.  Instead they are an extra piece of the score MMAs: each
     // is split into three bf16 parts in columns of its own behind the stream row, against ones behind the owner row, so
     // that the accumulators arrive as S - lse/alpha, Sd - mu/alpha, D - Sigma1, X - c.  At d = 72 these columns are the
     // padding up to 80; other head dims take one more k-step of N = 128.
-    static constexpr bool FOLD = DKV;
+    static constexpr bool FOLD = DKV || MODE == PASS_DKV_G;
     static constexpr int OWN_ATOM = JVP_ROWS * 128, ATOM = BC * 128;
     static constexpr int OWN_BYTES = OWN_ATOM * (WIDE ? 2 : 1) + (TAIL ? JVP_ROWS * 32 : 0);   // one owner tensor
     static constexpr int EST_BYTES = E_MN ? ATOM * NA : ATOM * (WIDE ? 2 : 1) + (TAIL ? BC * 32 : 0);   // one E-ring tile
     static constexpr int LST_BYTES = ATOM * NA;                                                // one L-ring tile
-    static constexpr int SE = WIDE ? (NPAIR == 2 ? 1 : 2) : DKV ? (TAIL ? 2 : 3) : TAIL ? 3 : 4;
-    static constexpr int SL = WIDE ? 2 : DKV ? (TAIL ? 3 : 4) : TAIL && NPAIR == 2 ? 3 : 4;
+    static constexpr int SE = GONLY ? 0 : WIDE ? (NPAIR == 2 ? 1 : 2) : DKV ? (TAIL ? 2 : 3) : TAIL ? 3 : 4;
+    static constexpr int SL = GONLY ? 6 : WIDE ? 2 : DKV ? (TAIL ? 3 : 4) : TAIL && NPAIR == 2 ? 3 : 4;
     static constexpr int TILE_BYTES = NOWN * OWN_BYTES + SE * 2 * EST_BYTES + SL * 2 * LST_BYTES;
     // FOLD: statistics of a stage, [Y0 rows, Y1 rows][16 bytes], for the rings the score MMAs read; ones and zeros
     static constexpr int FOLD_BYTES = 2 * BC * 16;
-    static constexpr int FOLD_E = FOLD ? SE : 0, FOLD_L = FOLD && NPAIR == 2 ? SL : 0;
+    static constexpr int FOLD_E = FOLD ? SE : 0, FOLD_L = FOLD ? SL : 0;
     static constexpr int ONES_BYTES = FOLD ? JVP_ROWS * 32 : 0;
     static constexpr int EFULL_COUNT = 1 + (TAIL ? 32 : 0) + (FOLD_E ? 1 : 0);   // TMA issuer, each lane's own copies, warp 3
     static constexpr int LFULL_COUNT = 1 + (TAIL || (TRANSPOSED && !FOLD) ? 32 : 0) + (FOLD_L ? 1 : 0);
     // TMEM columns: accumulators, the owner operands in the gaps behind them,
-    // score accumulators (FWD, DV: two buffers of S | Sd; DK, DQ: one of S | Sd | D | X).
+    // score accumulators (FWD, DV: two buffers of S | Sd; DKV_G, DQ_G: of S | X; DK, DQ: one of S | Sd | D | X).
     static constexpr int NACC = DKV ? 4 : 2;
+    static constexpr bool HAS_ACC0 = MODE != PASS_DQ_G;
     static constexpr int COL_ACC0 = 0, COL_ACC1 = XT ? 128 : DP, COL_SCORE = NACC * COL_ACC1;
     static constexpr int COL_X0 = DP, COL_X1 = COL_ACC1 + DP;
     static_assert(!XT || DP + DP / 2 <= 128, "operands do not fit behind their accumulators");
     static_assert(COL_SCORE + 4 * BC <= 512, "TMEM over-subscribed");
     // registers per thread: warpgroup 0, element-wise warps, epilogue warps (which hold an owner row, 4 registers a chunk)
-    static constexpr int REGS_LOAD = MODE == PASS_FWD ? 56 : 96, REGS_ELEM = MODE == PASS_FWD ? 168 : 152, REGS_EPI = MODE == PASS_FWD ? 120 : 112;
+    static constexpr bool TURNS = MODE == PASS_FWD || GONLY;   // the element-wise groups take tiles in turn: 64 columns a thread
+    static constexpr int REGS_LOAD = GONLY ? 72 : TURNS ? 56 : 96, REGS_ELEM = GONLY ? 160 : TURNS ? 168 : 152, REGS_EPI = TURNS ? 120 : 112;
     static_assert(REGS_LOAD + 2 * REGS_ELEM + REGS_EPI <= 4 * JVP_REGS, "more registers than the block has");
     // barriers
     static constexpr int B_EFULL = 0;
@@ -165,20 +172,23 @@ struct JvpCfg {
     static constexpr int B_OWN = B_LFULL + SL;                         // owner tiles in shared memory loaded
     static constexpr int B_OWNFREE = B_OWN + OWN_SETS;                 // ... free: the score MMAs of the item are complete
     static constexpr int B_XRDY = B_OWNFREE + OWN_SETS;                       // owner operands in tensor memory written
-    static constexpr int B_XFREE = B_XRDY + 1;                         // ... free
+    static constexpr int XSETS = GONLY ? 2 : 1;                        // with barriers of their own
+    static constexpr int B_XFREE = B_XRDY + XSETS;                     // ... free
     // MMAs of tile g complete: + (g & 3), phase g >> 2.  The element-wise groups meet every other tile only and the
     // producers run up to four tiles ahead of or behind the others, so that a parity wait on one barrier, or on a pair,
     // could take another tile's completion for its own.  They also tell the producers that a ring stage is free: a commit
     // costs the issuing warp 60 cycles, and a barrier of its own per ring would be one more per tile.
-    static constexpr int B_SFULL = B_XFREE + 1;                        // S (and Sd, except in FWD) written
-    static constexpr int B_XFULL = B_SFULL + 4;                        // FWD: Sd written; DK, DQ: D, X written
+    static constexpr int B_SFULL = B_XFREE + XSETS;                        // S (and Sd, except in FWD) written
+    static constexpr int B_XFULL = B_SFULL + 4;                        // FWD: Sd written; DK, DQ: D, X written; DKV_G, DQ_G: X written
     static constexpr int B_OUTDONE = B_XFULL + 4;                      // output MMAs complete
     // The stage of a tile is free.  DKV: its output MMAs are in front of the next tile's scores, whose completion implies theirs.
     static constexpr int B_EDONE = DKV || MODE == PASS_DV ? B_SFULL : B_XFULL, EDONE_NEXT = DKV ? 1 : 0;
     static constexpr int B_LDONE = DKV ? B_XFULL : B_OUTDONE, LDONE_NEXT = EDONE_NEXT;
-    static_assert(SE <= 4 && SL <= 4, "a ring deeper than the completion barriers");
-    // operands written: + half of the tile (DK, DQ), + 2 (g & 1) + half (FWD, DV), + pair (DKV)
-    static constexpr int B_PREADY = B_OUTDONE + 4;
+    static constexpr int NOUTDONE = GONLY ? 8 : 4;                     // (DKV_G, DQ_G: the L ring is deeper)
+    static_assert(SE <= 4 && SL <= NOUTDONE, "a ring deeper than the completion barriers");
+    // operands written: + half of the tile (DK, DQ), + 2 (g & 1) + half (FWD, DV), + pair (DKV),
+    // + 2 (g & 1): P written (DKV_G) or S read (DQ_G), + 1: dA written
+    static constexpr int B_PREADY = B_OUTDONE + NOUTDONE;
     static constexpr int B_SREAD = B_PREADY + 4;                       // DK, DQ: S, Sd read
     static constexpr int B_FINAL = B_SREAD + 1;                        // + pair of accumulators: the item's last output MMAs complete
     static constexpr int B_ACCFREE = B_FINAL + NACC / 2;               // the epilogue has read the accumulators
@@ -256,6 +266,13 @@ struct JvpBlock {
         ptx::tc_fence_after_sync();
     }
     __device__ __forceinline__ bool done(int i, int g) const { return wait(i + (g & 3), g >> 2); }   // i: B_SFULL, B_XFULL, B_OUTDONE
+    // Ring R's stage of tile g - S is free.
+    template <int R>
+    __device__ __forceinline__ bool stage_free(int g) const {
+        if (R == 0) return done(C::B_EDONE, g - C::SE + C::EDONE_NEXT);
+        const int t = g - C::SL + C::LDONE_NEXT;
+        return wait(C::B_LDONE + (t & (C::NOUTDONE - 1)), t / C::NOUTDONE);
+    }
     __device__ __forceinline__ uint32_t own_tile(int t) const { return base + t * C::OWN_BYTES; }
     __device__ __forceinline__ const float* stats(int s) const { return static_cast<const float*>(__cvta_shared_to_generic(base + STATS + s * C::NSTAT * C::BC * 4)); }
     __device__ __forceinline__ float4& row_state(int r) const { return *static_cast<float4*>(__cvta_shared_to_generic(base + ROW_STATE + 16 * r)); }
@@ -282,11 +299,10 @@ __device__ __forceinline__ void jvp_load_owners(const JvpParams& p, const JvpBlo
         const uint32_t full = k.bar(C::B_OWN + SET);
         uint32_t tx = 0;
 #pragma unroll
-        for (int t = T0; t < T1; ++t) tx += p.own[t] ? C::OWN_ATOM * (C::WIDE ? 2 : 1) : 0;   // null: not read (HZ)
+        for (int t = T0; t < T1; ++t) tx += C::OWN_ATOM * (C::WIDE ? 2 : 1);
         ptx::mbar_arrive_expect_tx(full, tx);
 #pragma unroll
         for (int t = T0; t < T1; ++t) {
-            if (!p.own[t]) continue;
             const uint32_t dst = k.own_tile(t);
             ptx::tma_load_4d(dst, maps[t], full, 0, row0, ch, cb);
             ptx::tma_load_4d(dst + H64, maps[t], full, 0, row0 + 64, ch, cb);
@@ -305,7 +321,7 @@ __device__ __forceinline__ void jvp_load_owners(const JvpParams& p, const JvpBlo
             const uint32_t tile = k.own_tile(t) + C::OWN_ATOM + lane * 16;
 #pragma unroll
             for (int c = 0; c < KT; ++c) {
-                if (x && c < ntail) {
+                if (c < ntail) {
 #pragma unroll
                     for (int rp = 0; rp < JVP_ROWS / 32; ++rp) {
                         const bool v = lane + 32 * rp < rows_left;
@@ -323,14 +339,14 @@ __device__ __forceinline__ void jvp_load_owners(const JvpParams& p, const JvpBlo
 // is left to its copies (a warp that waits for them itself loads no more than one tile per memory latency).  These loops
 // run next to element-wise warps that leave them few issue slots, and a ring is refilled no faster than they run: what does
 // not depend on the tile is set up before them, and tiles whose rows all exist take a path without predicates.
-template <int MODE, int DP, bool HZ, int RING>
+template <int MODE, int DP, int RING>
 __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock<MODE, DP>& shared, const CUtensorMap* map0, const CUtensorMap* map1,
                                               const CUtensorMap* const (&own_maps)[4], int lane) {
     using C = JvpCfg<MODE, DP>;
     const JvpBlock<MODE, DP> k = shared.pinned();
     const int T = jvp_pin(p.T), rows = jvp_pin(p.s.rows);
     constexpr int BC = C::BC, S = RING == 0 ? C::SE : C::SL, ATOM = C::ATOM;
-    constexpr int b_full = RING == 0 ? C::B_EFULL : C::B_LFULL, b_done = RING == 0 ? C::B_EDONE : C::B_LDONE, next = RING == 0 ? C::EDONE_NEXT : C::LDONE_NEXT;
+    constexpr int b_full = RING == 0 ? C::B_EFULL : C::B_LFULL;
     constexpr uint32_t TB = RING == 0 ? C::EST_BYTES : C::LST_BYTES;
     constexpr bool STATS = RING == 1 && C::TRANSPOSED && !C::FOLD;   // this ring carries the statistics as they are
     constexpr bool OWNERS = RING == 0 && C::NOWN > 0;
@@ -342,10 +358,9 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
     const uint32_t ring_base = k.base + (RING == 0 ? k.E : k.L);
     const __nv_bfloat16* base0 = p.strm[2 * RING];
     const __nv_bfloat16* base1 = p.strm[2 * RING + 1];
-    // The ring that streams the cotangents (Hc, G) where one of them may be absent (null): that one is not loaded, nor, with HZ,
-    // are the tangents.
-    constexpr bool COT = C::DKV && RING == 0;
-    const bool has0 = COT ? !HZ && base0 : true, has1 = COT ? HZ || base1 : !HZ;
+    // The ring that streams the cotangents (Hc, G): G may be absent (null) and is not loaded then.
+    constexpr bool has0 = true;
+    const bool has1 = C::DKV && RING == 0 ? base1 != nullptr : true;
     const uint32_t tx_bytes = ((has0 ? 1 : 0) + (has1 ? 1 : 0)) * ATOM * (C::WIDE ? 2 : 1);
     // Chunk 0 of row `lane` behind the first atoms: compact blocks in the E ring, a second swizzled atom in the L ring.
     [[maybe_unused]] const uint32_t sw = lane & 7;  // rows 32 apart share it
@@ -388,7 +403,7 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
                 }
                 ++owners;
             }
-            if (g >= S) ok = k.done(b_done, g - S + next);   // the MMAs that read the stage's last tile
+            if (g >= S) ok = k.template stage_free<RING>(g);   // the MMAs that read the stage's last tile
             if (!ok) break;
             ++g;
             [[maybe_unused]] const int rows_left = rows - j * BC;  // rows of this tile that exist
@@ -480,7 +495,7 @@ __device__ __forceinline__ void jvp_split3(float a, float b, uint2& pa, uint2& p
     pb = make_uint2(__byte_perm(h, m, 0x7632), l >> 16);
 }
 
-// Warp 3: the statistics of the stream rows lane and lane + 32 of a tile, for the L ring (lse, mu) and the E ring (Sigma1, c),
+// Warp 3: the statistics of the stream rows lane and lane + 32 of a tile, for the L ring (lse, mu) and the E ring (Sigma1, c) (DKV_G: lse, c for the L ring),
 // loaded one tile ahead.
 template <int MODE, int DP>
 __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE, DP>& shared, int lane) {
@@ -497,7 +512,8 @@ __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE
     const Dst dl = own ? Dst{k.base + k.FOLD_L + lane * 16, (uint32_t)C::FOLD_BYTES, BC * 16, 32 * 16}
                                         : Dst{k.base + k.L + 2 * C::ATOM + lane * 128 + ((1 ^ sw) << 4), 2u * C::LST_BYTES, C::ATOM, 32 * 128};
     const float f_lse = 1.0f / p.c2, f_mu = -1.0f / p.alpha;   // to the scale of S and Sd
-    float a[4], b[4];   // (statistic of tensor 0, of tensor 1) of the two rows: lse, mu | Sigma1, c
+    float a[4];                        // (statistic of tensor 0, of tensor 1) of the two rows: lse, mu (DKV_G: lse, c)
+    [[maybe_unused]] float b[4];       // DKV: Sigma1, c
     auto load = [&](int bh, int j) {
         const int left = p.s.rows - j * BC - lane;   // queries beyond M: zero, like their rows of the operands
         const size_t at = (size_t)bh * p.s.rows + (size_t)j * BC + lane;
@@ -505,9 +521,11 @@ __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE
         for (int r = 0; r < 2; ++r) {
             const bool v = left > 32 * r;
             a[2 * r] = v ? __ldg(p.nlse2 + at + 32 * r) : 0.f;
-            a[2 * r + 1] = v ? __ldg(p.mu + at + 32 * r) : 0.f;
-            b[2 * r] = v ? __ldg(p.nsig1 + at + 32 * r) : 0.f;
-            b[2 * r + 1] = v ? __ldg(p.ncvec + at + 32 * r) : 0.f;
+            a[2 * r + 1] = v ? __ldg((C::DKV ? p.mu : p.ncvec) + at + 32 * r) : 0.f;
+            if constexpr (C::DKV) {
+                b[2 * r] = v ? __ldg(p.nsig1 + at + 32 * r) : 0.f;
+                b[2 * r + 1] = v ? __ldg(p.ncvec + at + 32 * r) : 0.f;
+            }
         }
     };
     auto put = [&](const Dst& d, int stage, int full, float x0, float x1, float y0, float y1) {
@@ -530,12 +548,15 @@ __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE
     for (int item = blockIdx.x; item < p.items; item += gridDim.x) {
         const int bh = item / p.row_tiles, next = item + (int)gridDim.x;
         for (int j = 0; j < T; ++j, ++g) {
-            if (g >= C::SL && !k.done(C::B_LDONE, g - C::SL + C::LDONE_NEXT)) return;
-            put(dl, sl, C::B_LFULL, a[0] * f_lse, a[1] * f_mu, a[2] * f_lse, a[3] * f_mu);
+            if (g >= C::SL && !k.template stage_free<1>(g)) return;
+            const float f1 = C::DKV ? f_mu : 1.0f;
+            put(dl, sl, C::B_LFULL, a[0] * f_lse, a[1] * f1, a[2] * f_lse, a[3] * f1);
             if (++sl == C::SL) sl = 0;
-            if (g >= C::SE && !k.done(C::B_EDONE, g - C::SE + C::EDONE_NEXT)) return;
+            if constexpr (C::DKV) {
+            if (g >= C::SE && !k.template stage_free<0>(g)) return;
             put(de, se, C::B_EFULL, b[0], b[1], b[2], b[3]);
             if (++se == C::SE) se = 0;
+            }
             const bool more = j + 1 < T;
             if (more || next < p.items) load(more ? bh : next / p.row_tiles, more ? j + 1 : 0);
         }
@@ -564,7 +585,7 @@ struct JvpSlot {   // a ring's next tile: stage, phase, low descriptor halves of
     }
 };
 
-template <int MODE, int DP, bool HZ, int ABS>
+template <int MODE, int DP, bool NO_G>
 struct JvpIssue {
     using C = JvpCfg<MODE, DP>;
     using Block = JvpBlock<MODE, DP>;
@@ -595,8 +616,8 @@ struct JvpIssue {
     static __host__ __device__ constexpr uint32_t l_n(int t, int u) { return (uint32_t)(t * ATOM + u * 2048) / 16 + lbo(2 * ATOM); }
 
     // Long batches are loops: their code, run once a tile by one warp, else pushes the element-wise loops out of the instruction
-    // cache (head dims above 64: 4 to 8 % of a pass; DKV 3 %).  Short ones (d <= 64, without dtO) pay more for the loops.
-    static constexpr int UNROLL = !HZ && (DP > 64 || C::DKV) ? 1 : 8;
+    // cache (head dims above 64: 4 to 8 % of a pass; DKV 3 %).  Short ones (d <= 64, DKV_G and DQ_G) pay more for the loops.
+    static constexpr int UNROLL = !C::GONLY && (DP > 64 || C::DKV) ? 1 : 8;
     // One k-step with A in tensor memory (ATM: a = its columns) or in shared memory (a = the tile's descriptor).
     template <bool ATM>
     static __device__ __forceinline__ void step(uint32_t el, uint32_t col, uint32_t a, uint32_t ahi, uint32_t b, uint32_t bhi, uint32_t idesc, uint32_t acc) {
@@ -645,30 +666,36 @@ struct JvpIssue {
         if (k.fold_step()) fold_step(el, col, k, fold, T, I_S);
     }
     // Half of acc0 += A0 B0, acc1 += A1 B0 + A0 B1 (k-steps U0, U0 + 1 of four; the operand of a k-step lies at the columns of
-    // the scores it replaces); terms that are exactly zero are left out.  acc = 0: the accumulators are overwritten.
+    // the scores it replaces); acc = 0: the accumulators are overwritten.
     template <int U0>
     static __device__ __forceinline__ void outputs(uint32_t el, uint32_t a0, uint32_t a1, uint32_t lo, uint32_t acc) {
         constexpr uint32_t c0 = C::COL_ACC0, c1 = C::COL_ACC1;
-        constexpr bool A0 = !HZ && !(ABS & ABSENT_HC);   // (DQ with Hc absent: A0 = W is exactly zero)
 #pragma unroll UNROLL
         for (int u = U0; u < U0 + 2; ++u) {
             const uint32_t b0 = lo + l_n(0, 0) + 128u * u, b1 = lo + l_n(1, 0) + 128u * u, o = 16u * u, first = U0 > 0 || u > 0 ? 1u : acc;
-            if (A0) ptx::mma_ts_acc(el, c0, a0 + o, b0, HI_SW, I_O, first);
+            ptx::mma_ts_acc(el, c0, a0 + o, b0, HI_SW, I_O, first);
             ptx::mma_ts_acc(el, c1, a1 + o, b0, HI_SW, I_O, first);
-            if (A0) ptx::mma_ts_acc(el, c1, a0 + o, b1, HI_SW, I_O, 1u);
+            ptx::mma_ts_acc(el, c1, a0 + o, b1, HI_SW, I_O, 1u);
         }
     }
-    // DKV: acc[C] += A0 B0, acc[C + 1] += A1 B0 + A0 B1 (T0, T1, T2: which of the three there are).
-    template <bool T0, bool T1, bool T2, int ACC>
+    // DKV: acc[C] += A0 B0, acc[C + 1] += A1 B0 + A0 B1 (T2: the last of them; without G it is zero).
+    template <bool T2, int ACC>
     static __device__ __forceinline__ void dkv_outputs(uint32_t el, uint32_t a0, uint32_t a1, uint32_t lo, uint32_t acc) {
         constexpr uint32_t c0 = ACC * DP, c1 = c0 + DP;
 #pragma unroll UNROLL
         for (int u = 0; u < BC / 16; ++u) {
             const uint32_t b0 = lo + l_n(0, 0) + 128u * u, b1 = lo + l_n(1, 0) + 128u * u, o = 16u * u, first = u > 0 ? 1u : acc;
-            if (T0) ptx::mma_ts_acc(el, c0, a0 + o, b0, HI_SW, I_O, first);
-            if (T1) ptx::mma_ts_acc(el, c1, a1 + o, b0, HI_SW, I_O, first);
-            if (T2) ptx::mma_ts_acc(el, c1, a0 + o, b1, HI_SW, I_O, T1 ? 1u : first);
+            ptx::mma_ts_acc(el, c0, a0 + o, b0, HI_SW, I_O, first);
+            ptx::mma_ts_acc(el, c1, a1 + o, b0, HI_SW, I_O, first);
+            if (T2) ptx::mma_ts_acc(el, c1, a0 + o, b1, HI_SW, I_O, 1u);
         }
+    }
+    // DKV_G: acc0 += P^T G (ACC 0), acc1 += dA^T Q (ACC 1); DQ_G: acc1 += dA K.
+    template <int ACC>
+    static __device__ __forceinline__ void g_outputs(uint32_t el, uint32_t a, uint32_t lo, uint32_t acc) {
+#pragma unroll
+        for (int u = 0; u < BC / 16; ++u)
+            ptx::mma_ts_acc(el, ACC ? C::COL_ACC1 : C::COL_ACC0, a + 16u * u, lo + l_n(1 - ACC, 0) + 128u * u, HI_SW, I_O, u > 0 ? 1u : acc);
     }
 };
 
@@ -678,21 +705,20 @@ struct JvpIssue {
 // instead of 2250 in two passes, half the exponentials and loads.)  The element-wise warps are done 400 to 800 cycles before
 // their operands' turn, so this warp waits and commits twice per tile and no more: for the operands as a whole, together with
 // the next stage of the ring, and one completion for outputs and scores.  (Operands handed over in halves, a wait per barrier
-// and four commits: d = 72 (16, 16, 1024) 1034 -> 994 us for the backward, without dtO 656 -> 544.)  What bounds a tile now
+// and four commits: d = 72 (16, 16, 1024) 1034 -> 994 us for the backward.)  What bounds a tile now
 // is the pipe with two operands in shared memory, whose port the loads share: 2950 cycles, 2490 with nothing to load or compute.
 // The tiles run on through the items: the next item's first scores go in front of this one's last outputs, and each pair of
 // accumulators is handed to and from the epilogue on its own.  (d = 72, DKV and DQ, (64, 16, 256): the backward 345 -> 334 us.)
-template <int MODE, int DP, bool HZ, int ABS>
+template <int MODE, int DP, bool NO_G>
 __device__ __forceinline__ void jvp_issue_dkv(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
     using C = JvpCfg<MODE, DP>;
-    using I = JvpIssue<MODE, DP, HZ, ABS>;
+    using I = JvpIssue<MODE, DP, NO_G>;
     constexpr int BC = C::BC;
     const JvpBlock<MODE, DP> k = shared.pinned();
     const int T = jvp_pin(p.T);
     const uint32_t x0 = ptx::desc_lo(k.own_tile(0), 16), x1 = ptx::desc_lo(k.own_tile(1), 16);
     const uint32_t x2 = ptx::desc_lo(k.own_tile(2), 16), x3 = ptx::desc_lo(k.own_tile(3), 16);
     constexpr uint32_t cS = C::COL_SCORE, cT = cS + BC, cD = cS + 2 * BC, cX = cS + 3 * BC;
-    constexpr bool H = !HZ && !(ABS & ABSENT_HC), G = !(ABS & ABSENT_G);
     JvpSlot e = I::e_slot(k), l = I::l_slot(k);   // next tile of the scores
     uint32_t elo = e.lo, llo = l.lo;              // stages of the outputs' tile
     const int last = jvp_item_count(p) * T;
@@ -707,7 +733,7 @@ __device__ __forceinline__ void jvp_issue_dkv(const JvpParams& p, const JvpBlock
         k.tile_fence();
         if (out) {
             const uint32_t el = ptx::elect_one();
-            I::template dkv_outputs<H, H, G, 0>(el, cS, cT, elo, acc);
+            I::template dkv_outputs<!NO_G, 0>(el, cS, cT, elo, acc);
             if (oj == T - 1) ptx::mma_commit_p(el, k.bar(C::B_FINAL));
         }
         if (score) {
@@ -717,8 +743,7 @@ __device__ __forceinline__ void jvp_issue_dkv(const JvpParams& p, const JvpBlock
             }
             ready = ptx::mbar_test2_warp(k.bar(C::B_PREADY + 1), (n - 1) & 1, k.bar(C::B_EFULL + e.s), e.ph);
             const uint32_t el = ptx::elect_one();
-            if (HZ) I::template single<true, false, 0>(el, cS, k, x0, l.lo, l.fold);
-            else I::template pair<true, false, true>(el, cS, k, x0, x1, l.lo, l.fold, 0);
+            I::template pair<true, false, true>(el, cS, k, x0, x1, l.lo, l.fold, 0);
             ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
             if (sj == T - 1) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE));
             l.template next<C::SL, I::L_STEP, I::F_STEP>();
@@ -731,7 +756,7 @@ __device__ __forceinline__ void jvp_issue_dkv(const JvpParams& p, const JvpBlock
         k.tile_fence();
         if (out) {
             const uint32_t el = ptx::elect_one();
-            I::template dkv_outputs<H, true, H, 2>(el, cD, cX, llo, acc);
+            I::template dkv_outputs<true, 2>(el, cD, cX, llo, acc);
             elo = elo + I::E_STEP == e.lo0 + C::SE * I::E_STEP ? e.lo0 : elo + I::E_STEP;
             llo = llo + I::L_STEP == l.lo0 + C::SL * I::L_STEP ? l.lo0 : llo + I::L_STEP;
             if (oj == T - 1) {
@@ -749,8 +774,7 @@ __device__ __forceinline__ void jvp_issue_dkv(const JvpParams& p, const JvpBlock
             // (the stage of the tile after the next one, where there is one)
             ready = n + 1 < last && ptx::mbar_test2_warp(k.bar(C::B_PREADY), n & 1, k.bar(C::B_LFULL + l.s), l.ph);
             const uint32_t el = ptx::elect_one();
-            if (HZ) I::template single<false, false, 1>(el, cX, k, x2, e.lo, e.fold);   // X = V G^T alone
-            else I::template pair<false, false, H>(el, cD, k, x2, x3, e.lo, e.fold, 0);  // (tV Hc^T is zero with Hc absent)
+            I::template pair<false, false, true>(el, cD, k, x2, x3, e.lo, e.fold, 0);
             ptx::mma_commit_p(el, k.bar(C::B_XFULL + (n & 3)));
             if (sj == T - 1) {
                 ptx::mma_commit_p(el, k.bar(C::B_OWNFREE + 1));
@@ -768,7 +792,7 @@ __device__ __forceinline__ void jvp_issue_dkv(const JvpParams& p, const JvpBlock
 template <int MODE, int DP>
 __device__ __forceinline__ void jvp_issue_one_pair(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
     using C = JvpCfg<MODE, DP>;
-    using I = JvpIssue<MODE, DP, false, 0>;
+    using I = JvpIssue<MODE, DP, false>;
     constexpr int RDY = C::XT ? C::B_XRDY : C::B_OWN, FREE = C::XT ? C::B_XFREE : C::B_OWNFREE;
     const JvpBlock<MODE, DP> k = shared.pinned();
     const int T = jvp_pin(p.T), items = jvp_pin(p.items);
@@ -821,16 +845,16 @@ __device__ __forceinline__ void jvp_issue_one_pair(const JvpParams& p, const Jvp
 
 // DK, DQ: one buffer of (S, Sd | D, X), the operands W, dA over D, X.  Pipe order: (S, Sd)(n) once (S, Sd)(n - 1) has been read |
 // outputs(n - 1), half by half, as W, dA are written | (D, X)(n), which overwrites them.
-template <int MODE, int DP, bool HZ, int ABS>
+template <int MODE, int DP, bool NO_G>
 __device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
     using C = JvpCfg<MODE, DP>;
-    using I = JvpIssue<MODE, DP, HZ, ABS>;
+    using I = JvpIssue<MODE, DP, NO_G>;
     const JvpBlock<MODE, DP> k = shared.pinned();
     const int T = jvp_pin(p.T);
     const uint32_t x0 = ptx::desc_lo(k.own_tile(0), 16), x1 = ptx::desc_lo(k.own_tile(1), 16);
     const uint32_t x2 = C::XT ? C::COL_X0 : ptx::desc_lo(k.own_tile(2), 16), x3 = C::XT ? C::COL_X1 : ptx::desc_lo(k.own_tile(3), 16);
     constexpr uint32_t cS = C::COL_SCORE, cD = C::COL_SCORE + 2 * C::BC, cX = C::COL_SCORE + 3 * C::BC;
-    constexpr bool X3 = !(ABS & ABSENT_G);   // DQ: X3 Y2^T = G V^T is zero with G absent
+    constexpr bool X3 = !NO_G;   // DQ: X3 Y2^T = G V^T is zero with G absent
     JvpSlot e = I::e_slot(k), l = I::l_slot(k);
     uint32_t lo = l.lo;        // L stage of the outputs' tile
     const int last = jvp_item_count(p) * T;
@@ -842,8 +866,7 @@ __device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const Jv
             if (sj == 0 && !k.wait(C::B_OWN, si)) return false;
             k.tile_fence();
             const uint32_t el = ptx::elect_one();
-            if (HZ) I::template single<true, false, 0>(el, cS, k, x0, l.lo, l.fold);
-            else I::template pair<true, false, true>(el, cS, k, x0, x1, l.lo, l.fold, 0);
+            I::template pair<true, false, true>(el, cS, k, x0, x1, l.lo, l.fold, 0);
             ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
             if (C::XT && sj == T - 1) ptx::mma_commit_p(el, k.bar(C::B_OWNFREE));
             l.template next<C::SL, I::L_STEP, I::F_STEP>();
@@ -877,9 +900,7 @@ __device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const Jv
             if (C::XT && sj == 0 && !k.wait(C::B_XRDY, si)) return;
             k.tile_fence();
             const uint32_t el = ptx::elect_one();
-            // HZ (DQ): X = G V^T alone: X3 and the stage's first tensor
-            if (HZ) I::template single<false, C::XT, 0>(el, cX, k, x3, e.lo, e.fold);
-            else I::template pair<false, C::XT, X3>(el, cD, k, x2, x3, e.lo, e.fold, 0);
+            I::template pair<false, C::XT, X3>(el, cD, k, x2, x3, e.lo, e.fold, 0);
             ptx::mma_commit_p(el, k.bar(C::B_XFULL + (n & 3)));
             if (sj == T - 1) {
                 ptx::mma_commit_p(el, k.bar(C::XT ? C::B_XFREE : C::B_OWNFREE));
@@ -892,19 +913,98 @@ __device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const Jv
     }
 }
 
-// Which cotangent is absent is decided here, once (WIDE head dims take both).
-template <int MODE, int DP, bool HZ, int ABS>
-__device__ __forceinline__ void jvp_issue_abs(const JvpParams& p, const JvpBlock<MODE, DP>& k) {
-    if constexpr (MODE == PASS_DKV) jvp_issue_dkv<MODE, DP, HZ, ABS>(p, k);
-    else if constexpr (JvpCfg<MODE, DP>::NPAIR == 1) jvp_issue_one_pair<MODE, DP>(p, k);
-    else jvp_issue_two_pairs<MODE, DP, HZ, ABS>(p, k);
+// DKV_G, DQ_G: two score buffers taken in turn, operands written over the scores.  Pipe order: dV(n - 2) | S(n) | dK(n - 3) | X(n - 1)
+// (DQ_G: S(n) | dQ(n - 3) | X(n - 1)): while a group works on tile n - 2 the other's n - 3 is complete, and the scores of what
+// either takes next are there before it asks for them.  (d = 72 (16, 16, 1024): 461 us for the two passes as specialisations of DKV
+// and DQ, whose layout has room for tiles of 48, one buffer and owners in shared memory; 305 now.)  One wait a tile, for everything that the tile's batch needs (P(n - 2)
+// written, or S(n - 2) read; dA(n - 3) written; stage n full): with a wait in front of every product this warp was what bounded a
+// tile (DQ_G, d = 72: 1240 cycles, MMAs of 480).
+template <int MODE, int DP>
+__device__ __forceinline__ void jvp_issue_g(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
+    using C = JvpCfg<MODE, DP>;
+    using I = JvpIssue<MODE, DP, false>;
+    constexpr bool KEYS = MODE == PASS_DKV_G;
+    const JvpBlock<MODE, DP> k = shared.pinned();
+    const int T = jvp_pin(p.T), last = jvp_item_count(p) * T;
+    // The epilogue stages an item's owner operands once the item two before is over.  Items of three tiles or more run on into one
+    // another; shorter ones are finished one by one.
+    const int chunk = T > 2 ? last : T;
+    JvpSlot l = I::l_slot(k);
+    uint32_t xlo = 0, xfold = 0, vlo = 0, klo = 0;   // stages of the tiles n - 1, n - 2, n - 3
+    uint32_t first = 0, end = 0;                     // bit i: tile n - i is the first, the last of its item
+    int sj = 0, si = 0, xi = 0, oi = 0;              // tile within its item; items opened by S, by X, by the outputs
+    for (int base = 0; base < last; base += chunk) {
+        for (int m = 0; m < chunk + 3; ++m) {
+            const int n = base + m;
+            const bool score = m < chunk, x = m >= 1 && m <= chunk, v_out = m >= 2 && m < chunk + 2, k_out = m >= 3;
+            const int ba = C::B_PREADY + 2 * (n & 1), bb = C::B_PREADY + 2 * ((n - 1) & 1) + 1, pa = ((n - 2) >> 1) & 1, pb = ((n - 3) >> 1) & 1;
+            if (!(k_out && score && ptx::mbar_test3_warp(k.bar(ba), pa, k.bar(bb), pb, k.bar(C::B_LFULL + l.s), l.ph))) {
+                if (v_out && !k.wait(ba, pa)) return;
+                if (k_out && !k.wait(bb, pb)) return;
+                if (score && !k.wait(C::B_LFULL + l.s, l.ph)) return;
+            }
+            first = first << 1 | (score && sj == 0 ? 1u : 0u);
+            end = end << 1 | (score && sj == T - 1 ? 1u : 0u);
+            const uint32_t col = C::COL_SCORE + (n & 1) * 2 * C::BC, colx = C::COL_SCORE + ((n - 1) & 1) * 2 * C::BC + C::BC;
+            // first output MMAs of an item: they overwrite the accumulators
+            auto acc_free = [&]() { return oi++ == 0 || k.wait(C::B_ACCFREE, oi - 2); };
+            auto part_x = [&]() {
+                if (!KEYS && (first & 8u) && !acc_free()) return false;
+                if ((first & 2u) && !k.wait(C::B_XRDY + 1, xi++)) return false;
+                ptx::tc_fence_after_sync();
+                const uint32_t el = ptx::elect_one();
+                if (k_out) {
+                    I::template g_outputs<1>(el, colx, klo, first & 8u ? 0u : 1u);
+                    ptx::mma_commit_p(el, k.bar(C::B_OUTDONE + ((n - 3) & (C::NOUTDONE - 1))));
+                    if (end & 8u) ptx::mma_commit_p(el, k.bar(C::B_FINAL));
+                }
+                if (x) {
+                    const uint32_t el2 = ptx::elect_one();
+                    I::template single<true, true, 1>(el2, colx, k, C::COL_X1, xlo, xfold);
+                    ptx::mma_commit_p(el2, k.bar(C::B_XFULL + ((n - 1) & 3)));
+                    if (end & 2u) ptx::mma_commit_p(el2, k.bar(C::B_XFREE + 1));
+                }
+                return true;
+            };
+            // the item before is still to be ended
+            const bool swap = KEYS && (first & 4u);
+            if (swap && !part_x()) return;
+            if (KEYS && (first & 4u) && !acc_free()) return;
+            if ((first & 1u) && !k.wait(C::B_XRDY, si++)) return;
+            k.tile_fence();
+            if (KEYS && v_out) I::template g_outputs<0>(ptx::elect_one(), col, vlo, first & 4u ? 0u : 1u);
+            if (score) {
+                const uint32_t el = ptx::elect_one();
+                I::template single<true, true, 0>(el, col, k, C::COL_X0, l.lo, l.fold);
+                ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
+                if (end & 1u) ptx::mma_commit_p(el, k.bar(C::B_XFREE));
+            }
+            if (!swap && !part_x()) return;
+            klo = vlo;
+            vlo = xlo;
+            xlo = l.lo;
+            xfold = l.fold;
+            if (score) {
+                l.template next<C::SL, I::L_STEP, I::F_STEP>();
+                if (++sj == T) sj = 0;
+            }
+        }
+    }
 }
-template <int MODE, int DP, bool HZ>
+
+// Whether G is absent is decided here, once (WIDE head dims take both cotangents; without Hc the passes are DKV_G and DQ_G).
+template <int MODE, int DP, bool NO_G>
+__device__ __forceinline__ void jvp_issue_abs(const JvpParams& p, const JvpBlock<MODE, DP>& k) {
+    if constexpr (JvpCfg<MODE, DP>::GONLY) jvp_issue_g<MODE, DP>(p, k);
+    else if constexpr (MODE == PASS_DKV) jvp_issue_dkv<MODE, DP, NO_G>(p, k);
+    else if constexpr (JvpCfg<MODE, DP>::NPAIR == 1) jvp_issue_one_pair<MODE, DP>(p, k);
+    else jvp_issue_two_pairs<MODE, DP, NO_G>(p, k);
+}
+template <int MODE, int DP>
 __device__ __forceinline__ void jvp_issue(const JvpParams& p, const JvpBlock<MODE, DP>& k) {
-    if constexpr (MODE == PASS_FWD || HZ || JvpCfg<MODE, DP>::WIDE) jvp_issue_abs<MODE, DP, HZ, 0>(p, k);
-    else if (p.absent == 0) jvp_issue_abs<MODE, DP, HZ, 0>(p, k);
-    else if (p.absent == ABSENT_HC) jvp_issue_abs<MODE, DP, HZ, ABSENT_HC>(p, k);
-    else jvp_issue_abs<MODE, DP, HZ, ABSENT_G>(p, k);
+    if constexpr (JvpCfg<MODE, DP>::NPAIR == 1 || JvpCfg<MODE, DP>::WIDE) jvp_issue_abs<MODE, DP, false>(p, k);
+    else if (!p.no_g) jvp_issue_abs<MODE, DP, false>(p, k);
+    else jvp_issue_abs<MODE, DP, true>(p, k);
 }
 
 // ------------------------------------------------------------------------------------------------ element-wise warps
@@ -1130,7 +1230,7 @@ __device__ __forceinline__ void jvp_elem_dv(const JvpParams& p, const JvpBlock<P
 
 // DK, DQ.  Phase A: P and Nn from (S, Sd), kept in registers; phase B: W = P (D - Sigma1), dA = P (X - c) + W Nn, written over
 // D and X.  The statistics belong to the columns (DK) or to this thread's row (DQ).
-template <int MODE, int DP, bool HZ>
+template <int MODE, int DP>
 __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const JvpBlock<MODE, DP>& k, int grp, int q, int lane) {
     using C = JvpCfg<MODE, DP>;
     constexpr int BC = C::BC, HC = BC / 2;
@@ -1163,7 +1263,7 @@ __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const Jvp
             {
                 uint32_t s[HC], t[HC];
                 ptx::tmem_ld32(sb, s);
-                if (!HZ) ptx::tmem_ld32(sb + BC, t);
+                ptx::tmem_ld32(sb + BC, t);
                 ptx::tmem_wait_ld();
                 k.arrive(C::B_SREAD, lane);
                 const int nvalid = p.s.rows - j * BC - grp * HC;
@@ -1184,10 +1284,8 @@ __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const Jvp
                         float x0, x1;
                         ptx::unpack2(ptx::fma2(s2, c2c2, COL ? (e ? l4.y : l4.x) : r_l), x0, x1);
                         P2[i] = ptx::pack2(ptx::ex2(x0), ptx::ex2(x1));
-                        if (!HZ) {
-                            const uint64_t ts = ptx::pack2u(t[2 * i], t[2 * i + 1]);
-                            N2[i] = ptx::fma2(ts, aa, COL ? ptx::neg2(e ? m4.y : m4.x) : r_nm);
-                        }
+                        const uint64_t ts = ptx::pack2u(t[2 * i], t[2 * i + 1]);
+                        N2[i] = ptx::fma2(ts, aa, COL ? ptx::neg2(e ? m4.y : m4.x) : r_nm);
                     }
                 }
             }
@@ -1201,7 +1299,7 @@ __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const Jvp
             if (!k.done(C::B_XFULL, g)) return;
             ptx::tc_fence_after_sync();
             uint32_t dd[HC], xx[HC];
-            if (!HZ) ptx::tmem_ld32(sb + 2 * BC, dd);
+            ptx::tmem_ld32(sb + 2 * BC, dd);
             ptx::tmem_ld32(sb + 3 * BC, xx);
             ptx::tmem_wait_ld();
 #pragma unroll
@@ -1218,22 +1316,17 @@ __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const Jvp
                         uint64_t x2 = ptx::pack2u(xx[2 * gi], xx[2 * gi + 1]);
                         x2 = ptx::add2(x2, COL ? (e ? c4.y : c4.x) : r_c);
                         const uint64_t t2 = ptx::mul2(P2[gi], x2);
-                        float d0, d1;
-                        if (HZ) {
-                            ptx::unpack2(t2, d0, d1);
-                        } else {
-                            uint64_t y2 = ptx::pack2u(dd[2 * gi], dd[2 * gi + 1]);
-                            y2 = ptx::add2(y2, COL ? (e ? s4.y : s4.x) : r_s);
-                            const uint64_t w2 = ptx::mul2(P2[gi], y2);
-                            float w0, w1;
-                            ptx::unpack2(w2, w0, w1);
-                            ptx::unpack2(ptx::fma2(w2, N2[gi], t2), d0, d1);
-                            pa0[i] = ptx::pack_bf16(w0, w1);
-                        }
+                        float d0, d1, w0, w1;
+                        uint64_t y2 = ptx::pack2u(dd[2 * gi], dd[2 * gi + 1]);
+                        y2 = ptx::add2(y2, COL ? (e ? s4.y : s4.x) : r_s);
+                        const uint64_t w2 = ptx::mul2(P2[gi], y2);
+                        ptx::unpack2(w2, w0, w1);
+                        ptx::unpack2(ptx::fma2(w2, N2[gi], t2), d0, d1);
+                        pa0[i] = ptx::pack_bf16(w0, w1);
                         pa1[i] = ptx::pack_bf16(d0, d1);
                     }
                 }
-                if (!HZ) ptx::tmem_st8(sb + 2 * BC + 16 * u, pa0);
+                ptx::tmem_st8(sb + 2 * BC + 16 * u, pa0);
                 ptx::tmem_st8(sb + 3 * BC + 16 * u, pa1);
             }
             ptx::tmem_wait_st();
@@ -1247,7 +1340,7 @@ __device__ __forceinline__ void jvp_elem_two_pairs(const JvpParams& p, const Jvp
 // put together by two warps, whatever the width of the tile.  The statistics are in the scores already, so it does not
 // matter which element of a row a thread holds: 16 lanes x 256 bits are read, and two neighbouring values packed make
 // 16 lanes x 128 bits.
-template <int DP, bool HZ>
+template <int DP>
 __device__ __forceinline__ void jvp_elem_dkv(const JvpParams& p, const JvpBlock<PASS_DKV, DP>& k, int grp, int q, int lane) {
     using C = JvpCfg<PASS_DKV, DP>;
     constexpr int BC = C::BC, NU = BC / 16;
@@ -1262,7 +1355,7 @@ __device__ __forceinline__ void jvp_elem_dkv(const JvpParams& p, const JvpBlock<
 #pragma unroll
         for (int u = 0; u < NU; ++u) {
             ptx::tmem_ld16_256x2(sb + 16 * u, y + 8 * u);
-            if (!HZ) ptx::tmem_ld16_256x2(sb + BC + 16 * u, x + 8 * u);
+            ptx::tmem_ld16_256x2(sb + BC + 16 * u, x + 8 * u);
         }
         ptx::tmem_wait_ld();
 #pragma unroll
@@ -1276,14 +1369,12 @@ __device__ __forceinline__ void jvp_elem_dkv(const JvpParams& p, const JvpBlock<
                 x0 = ptx::ex2(x0); x1 = ptx::ex2(x1);
                 P2[c] = ptx::pack2(x0, x1);
                 a0[i] = ptx::pack_bf16(x0, x1);
-                if (!HZ) {
-                    N2[c] = ptx::mul2(ptx::pack2u(x[2 * c], x[2 * c + 1]), aa);
-                    ptx::unpack2(ptx::mul2(P2[c], N2[c]), x0, x1);
-                    a1[i] = ptx::pack_bf16(x0, x1);
-                }
+                N2[c] = ptx::mul2(ptx::pack2u(x[2 * c], x[2 * c + 1]), aa);
+                ptx::unpack2(ptx::mul2(P2[c], N2[c]), x0, x1);
+                a1[i] = ptx::pack_bf16(x0, x1);
             }
             ptx::tmem_st16_128x2(sb + 16 * u, a0);
-            if (!HZ) ptx::tmem_st16_128x2(sb + BC + 16 * u, a1);
+            ptx::tmem_st16_128x2(sb + BC + 16 * u, a1);
         }
         ptx::tmem_wait_st();
         k.arrive(C::B_PREADY, lane);
@@ -1291,7 +1382,7 @@ __device__ __forceinline__ void jvp_elem_dkv(const JvpParams& p, const JvpBlock<
         ptx::tc_fence_after_sync();
 #pragma unroll
         for (int u = 0; u < NU; ++u) {
-            if (!HZ) ptx::tmem_ld16_256x2(sb + 2 * BC + 16 * u, y + 8 * u);
+            ptx::tmem_ld16_256x2(sb + 2 * BC + 16 * u, y + 8 * u);
             ptx::tmem_ld16_256x2(sb + 3 * BC + 16 * u, x + 8 * u);
         }
         ptx::tmem_wait_ld();
@@ -1303,20 +1394,120 @@ __device__ __forceinline__ void jvp_elem_dkv(const JvpParams& p, const JvpBlock<
                 const int c = 4 * u + i;
                 uint64_t t2 = ptx::mul2(P2[c], ptx::pack2u(x[2 * c], x[2 * c + 1]));
                 float x0, x1;
-                if (!HZ) {
-                    const uint64_t w2 = ptx::mul2(P2[c], ptx::pack2u(y[2 * c], y[2 * c + 1]));
-                    ptx::unpack2(w2, x0, x1);
-                    a0[i] = ptx::pack_bf16(x0, x1);
-                    t2 = ptx::fma2(w2, N2[c], t2);
-                }
+                const uint64_t w2 = ptx::mul2(P2[c], ptx::pack2u(y[2 * c], y[2 * c + 1]));
+                ptx::unpack2(w2, x0, x1);
+                a0[i] = ptx::pack_bf16(x0, x1);
+                t2 = ptx::fma2(w2, N2[c], t2);
                 ptx::unpack2(t2, x0, x1);
                 a1[i] = ptx::pack_bf16(x0, x1);
             }
-            if (!HZ) ptx::tmem_st16_128x2(sb + 2 * BC + 16 * u, a0);
+            ptx::tmem_st16_128x2(sb + 2 * BC + 16 * u, a0);
             ptx::tmem_st16_128x2(sb + 3 * BC + 16 * u, a1);
         }
         ptx::tmem_wait_st();
         k.arrive(C::B_PREADY + 1, lane);
+    }
+}
+
+// DKV_G, DQ_G.  The groups take tiles in turn, a row per thread.  DKV_G: P over S, dA = P X over X (the statistics are in the
+// scores); DQ_G: dA = P (X - c) over X, statistics of this thread's row.
+template <int MODE, int DP>
+__device__ __forceinline__ void jvp_elem_g(const JvpParams& p, const JvpBlock<MODE, DP>& k, int grp, int q, int lane) {
+    using C = JvpCfg<MODE, DP>;
+    constexpr int BC = C::BC;
+    constexpr bool ROW = MODE == PASS_DQ_G;
+    const int row = q * 32 + lane, T = p.T, grid = gridDim.x;
+    const uint32_t sb0 = (static_cast<uint32_t>(q * 32) << 16) + C::COL_SCORE + grp * 2 * BC;
+    const uint64_t c2c2 = ptx::pack2(p.c2, p.c2);
+    [[maybe_unused]] float n_lse2 = -CUDART_INF_F, n_cv = 0.f;
+    [[maybe_unused]] auto load_stats = [&](int item) {
+        const int bh = item / p.row_tiles, r = (item - bh * p.row_tiles) * JVP_ROWS + row;
+        n_lse2 = -CUDART_INF_F; n_cv = 0.f;
+        if (item < p.items && r < p.o.rows) {
+            const size_t at = (size_t)bh * p.o.rows + r;
+            n_lse2 = p.nlse2[at]; n_cv = p.ncvec[at];
+        }
+    };
+    // item and tile within it: of this tile, and of the group's next one, whose row's statistics are loaded ahead
+    int item = blockIdx.x, j = grp;
+    for (; j >= T && item < p.items; j -= T) item += grid;
+    if (ROW) load_stats(item);
+    [[maybe_unused]] uint64_t r_l = ptx::pack2(n_lse2, n_lse2), r_c = ptx::pack2(n_cv, n_cv);
+    for (int g = grp; item < p.items; g += 2) {
+        int item1 = item, j1 = j + 2;
+        for (; j1 >= T && item1 < p.items; j1 -= T) item1 += grid;
+        if (ROW && item1 != item) load_stats(item1);
+        uint64_t P2[BC / 2];
+        if (!k.done(C::B_SFULL, g)) return;
+        ptx::tc_fence_after_sync();
+        {
+            uint32_t s[BC];
+            ptx::tmem_ld32(sb0, s);
+            ptx::tmem_ld32(sb0 + 32, s + 32);
+            ptx::tmem_wait_ld();
+            if (ROW) k.arrive(C::B_PREADY + 2 * grp, lane);
+            const int nvalid = p.s.rows - j * BC;
+            if (ROW && __builtin_expect(nvalid < BC, 0)) {   // keys beyond N: P = 0
+#pragma unroll
+                for (int c = 0; c < BC; ++c)
+                    if (c >= nvalid) s[c] = __float_as_uint(-CUDART_INF_F);   // c2 s = -inf (c2 > 0)
+            }
+#pragma unroll
+            for (int i = 0; i < BC / 2; ++i) {
+                const uint64_t s2 = ptx::pack2u(s[2 * i], s[2 * i + 1]);
+                float x0, x1;
+                ptx::unpack2(ROW ? ptx::fma2(s2, c2c2, r_l) : ptx::mul2(s2, c2c2), x0, x1);
+                P2[i] = ptx::pack2(ptx::ex2(x0), ptx::ex2(x1));
+            }
+        }
+        if (!ROW) {
+#pragma unroll
+            for (int u = 0; u < BC / 16; ++u) {
+                uint32_t pa[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    float x0, x1;
+                    ptx::unpack2(P2[8 * u + i], x0, x1);
+                    pa[i] = ptx::pack_bf16(x0, x1);
+                }
+                ptx::tmem_st8(sb0 + 16 * u, pa);
+            }
+            ptx::tmem_wait_st();
+            k.arrive(C::B_PREADY + 2 * grp, lane);
+        } else {   // the exponentials run while X is on its way
+            uint64_t all = 0ull;
+#pragma unroll
+            for (int i = 0; i < BC / 2; ++i) all ^= P2[i];
+            jvp_force(all);
+        }
+        if (!k.done(C::B_XFULL, g)) return;
+        ptx::tc_fence_after_sync();
+        uint32_t x[BC];
+        ptx::tmem_ld32(sb0 + BC, x);
+        ptx::tmem_ld32(sb0 + BC + 32, x + 32);
+        ptx::tmem_wait_ld();
+#pragma unroll
+        for (int u = 0; u < BC / 16; ++u) {
+            uint32_t pa[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int c = 8 * u + i;
+                uint64_t x2 = ptx::pack2u(x[2 * c], x[2 * c + 1]);
+                if (ROW) x2 = ptx::add2(x2, r_c);
+                float d0, d1;
+                ptx::unpack2(ptx::mul2(P2[c], x2), d0, d1);
+                pa[i] = ptx::pack_bf16(d0, d1);
+            }
+            ptx::tmem_st8(sb0 + BC + 16 * u, pa);
+        }
+        ptx::tmem_wait_st();
+        k.arrive(C::B_PREADY + 2 * grp + 1, lane);
+        if (ROW && item1 != item) {
+            r_l = ptx::pack2(n_lse2, n_lse2);
+            r_c = ptx::pack2(n_cv, n_cv);
+        }
+        item = item1;
+        j = j1;
     }
 }
 
@@ -1339,7 +1530,8 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
         const __nv_bfloat16* src = x + (p.o.head_off(bh, p.H) + (size_t)(row0 + row) * (size_t)p.o.rs);
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
-            v[c] = make_uint4(0, 0, 0, 0);
+            // (FOLD: the columns that pad d to DP are ones against the statistics, where those lie there)
+            v[c] = C::FOLD && C::TAIL && 8 * c >= p.d ? make_uint4(JVP_ONES0, JVP_ONES1, 0, 0) : make_uint4(0, 0, 0, 0);
             if (valid && 8 * c < p.d) v[c] = __ldg(reinterpret_cast<const uint4*>(src + 8 * c));
         }
     };
@@ -1355,9 +1547,13 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
         load_x(blockIdx.x, 0, v0);
         store_x(0, v0);
         load_x(blockIdx.x, 1, v0);
+        if (C::XSETS == 2) {
+            ptx::tmem_wait_st();
+            k.arrive(C::B_XRDY, lane);
+        }
         store_x(1, v0);
         ptx::tmem_wait_st();
-        k.arrive(C::B_XRDY, lane);
+        k.arrive(C::B_XRDY + C::XSETS - 1, lane);
     }
     int it = 0;
     for (int item = blockIdx.x; item < p.items; item += gridDim.x, ++it) {
@@ -1367,15 +1563,21 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
             if (!k.wait_item(C::B_XFREE, it)) return;
             ptx::tc_fence_after_sync();
             store_x(0, v0);
+            if (C::XSETS == 2) {
+                ptx::tmem_wait_st();
+                k.arrive(C::B_XRDY, lane);
+                if (!k.wait_item(C::B_XFREE + 1, it)) return;
+                ptx::tc_fence_after_sync();
+            }
             store_x(1, v1);
             ptx::tmem_wait_st();
-            k.arrive(C::B_XRDY, lane);
+            k.arrive(C::B_XRDY + C::XSETS - 1, lane);
         }
         const int bh = item / p.row_tiles, row0 = (item - bh * p.row_tiles) * JVP_ROWS;
         const size_t off = p.o.head_off(bh, p.H) + (size_t)(row0 + row) * (size_t)p.o.rs;
         // lane pairs write the two rows of the pair one after the other, each as complete 32-byte sectors
         const bool ok_even = row0 + (row & ~1) < p.o.rows, ok_odd = row0 + (row | 1) < p.o.rows;
-        float f0 = p.out_scale, mun = 0.f;
+        float f0 = MODE == PASS_DKV_G ? 1.0f : p.out_scale, mun = 0.f;   // (DKV_G: dV is not scaled)
         if constexpr (MODE == PASS_FWD) {   // O = O~/l, tO = R/l - (mu - c) O
             if (!k.wait_item(C::B_ROWSTAT, it)) return;
             const int last = (it * p.T + p.T - 1) & 1;   // the group whose reference is the accumulators'
@@ -1398,13 +1600,15 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
             if (C::DKV) f0 = pair ? p.out_scale : 1.0f;
             auto read = [&](int ch, uint32_t (&q0)[8], uint32_t (&q1)[8]) {   // 16 columns of both accumulators, as bf16
                 uint32_t x0[16], x1[16];
-                ptx::tmem_ld16(at + 16 * ch + C::COL_ACC0, x0);
+                if (C::HAS_ACC0) ptx::tmem_ld16(at + 16 * ch + C::COL_ACC0, x0);
                 ptx::tmem_ld16(at + 16 * ch + C::COL_ACC1, x1);
                 ptx::tmem_wait_ld();
 #pragma unroll
                 for (int c = 0; c < 16; c += 2) {
-                    float a0 = __uint_as_float(x0[c]) * f0, a1 = __uint_as_float(x0[c + 1]) * f0;
-                    float b0 = __uint_as_float(x1[c]) * f0, b1 = __uint_as_float(x1[c + 1]) * f0;
+                    const float f1 = MODE == PASS_DKV_G ? p.out_scale : f0;
+                    float a0 = 0.f, a1 = 0.f;
+                    if (C::HAS_ACC0) { a0 = __uint_as_float(x0[c]) * f0; a1 = __uint_as_float(x0[c + 1]) * f0; }
+                    float b0 = __uint_as_float(x1[c]) * f1, b1 = __uint_as_float(x1[c + 1]) * f1;
                     if (MODE == PASS_FWD) { b0 = fmaf(-mun, a0, b0); b1 = fmaf(-mun, a1, b1); }
                     q0[c >> 1] = ptx::pack_bf16(a0, a1);
                     q1[c >> 1] = ptx::pack_bf16(b0, b1);
@@ -1414,7 +1618,7 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
                 if (16 * ch >= p.d) return;
                 const bool has_hi = 16 * ch + 8 < p.d;
                 store_row_pairs(out1 + off + 16 * ch, p.o.rs, lane, ok_even, ok_odd, has_hi, make_uint4(q1[0], q1[1], q1[2], q1[3]), make_uint4(q1[4], q1[5], q1[6], q1[7]));
-                if (out0)   // null with Hc absent: acc0 was never written, its gradient is zero
+                if (C::HAS_ACC0)
                     store_row_pairs(out0 + off + 16 * ch, p.o.rs, lane, ok_even, ok_odd, has_hi, make_uint4(q0[0], q0[1], q0[2], q0[3]), make_uint4(q0[4], q0[5], q0[6], q0[7]));
             };
             if (!k.wait_item(C::B_FINAL + pair, it)) return;
@@ -1440,17 +1644,14 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
 }
 
 // ------------------------------------------------------------------------------------------------ the kernel
-// HZ: the cotangent Hc = dtO is absent (the "detach JVP" setting), known at compile time: everything that only feeds the
-// tangent path is left out -- Sd, Nn, D, W and their MMAs -- and what remains is the standard attention backward: P from
-// S, dA = P (G V^T - rowsum(G O)), dV = P^T G, dK = alpha dA^T Q, dQ = alpha dA K.
-template <int MODE, int DP, bool HZ>
+template <int MODE, int DP>
 __global__ void __launch_bounds__(JVP_THREADS, 1)
 jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUtensorMap s1, const __grid_constant__ CUtensorMap s2,
            const __grid_constant__ CUtensorMap s3, const __grid_constant__ CUtensorMap o0, const __grid_constant__ CUtensorMap o1,
            const __grid_constant__ CUtensorMap o2, const __grid_constant__ CUtensorMap o3, const __grid_constant__ JvpParams p) {
     using C = JvpCfg<MODE, DP>;
     constexpr int BC = C::BC;
-    constexpr bool DEPENDENT = MODE == PASS_DK || MODE == PASS_DQ;   // launched as a programmatic dependent of the pass before
+    constexpr bool DEPENDENT = MODE == PASS_DK || MODE == PASS_DQ || MODE == PASS_DQ_G;   // launched as a programmatic dependent of the pass before
     // the next backward pass in the stream, if launched as a programmatic dependent, may start as SMs free up
     if (MODE != PASS_FWD) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (*reinterpret_cast<volatile int*>(p.status) != 0) {  // an earlier kernel timed out
@@ -1470,9 +1671,9 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
         init(C::B_LFULL, C::SL, C::LFULL_COUNT);
         init(C::B_OWN, C::OWN_SETS, C::TAIL ? 33 : 1);
         init(C::B_OWNFREE, C::OWN_SETS, 1);
-        init(C::B_XRDY, 1, 4);
-        init(C::B_XFREE, 1, 1);
-        init(C::B_SFULL, 12, 1);       // SFULL, XFULL, OUTDONE
+        init(C::B_XRDY, C::XSETS, 4);
+        init(C::B_XFREE, C::XSETS, 1);
+        init(C::B_SFULL, 8 + C::NOUTDONE, 1);   // SFULL, XFULL, OUTDONE
         init(C::B_PREADY, 4, C::DKV ? 8 : 4);   // (of four: the warps of a group)
         init(C::B_SREAD, 1, 8);
         init(C::B_FINAL, C::NACC / 2, 1);
@@ -1502,9 +1703,9 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
             }
         }
     }
-    if (!HZ && C::DKV && p.absent) {
+    if (C::DKV && p.no_g) {
         // both cotangent tiles of an E stage are read by one MMA: the never-loaded one must read as zero
-        const int t = (p.absent & ABSENT_HC) ? 0 : 1;
+        constexpr int t = 1;
         uint8_t* e = jvp_smem + C::NOWN * C::OWN_BYTES;
         for (int st = 0; st < C::SE; ++st) {
             uint8_t* stage = e + st * 2 * C::EST_BYTES;
@@ -1535,9 +1736,9 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
         ptx::setmaxnreg_dec<C::REGS_LOAD>();
         if (placed) {
             const CUtensorMap* const maps[4] = {&o0, &o1, &o2, &o3};
-            if (warp == 0) jvp_load_ring<MODE, DP, HZ, 0>(p, k, &s0, &s1, maps, lane);
-            else if (warp == 2) jvp_load_ring<MODE, DP, HZ, 1>(p, k, &s2, &s3, maps, lane);
-            else if (warp == 1) jvp_issue<MODE, DP, HZ>(p, k);
+            if (warp == 1) jvp_issue<MODE, DP>(p, k);
+            else if (warp == 2) jvp_load_ring<MODE, DP, 1>(p, k, &s2, &s3, maps, lane);
+            else if (warp == 0) { if constexpr (!C::GONLY) jvp_load_ring<MODE, DP, 0>(p, k, &s0, &s1, maps, lane); }
             else if constexpr (C::FOLD) jvp_fold<MODE, DP>(p, k, lane);
         }
         if (warp == 1 && *abort_flag && placed) {
@@ -1550,9 +1751,10 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
         if (placed) {
             const int grp = (warp - 4) >> 2, q = warp & 3;
             if constexpr (MODE == PASS_FWD) jvp_elem_fwd<DP>(p, k, grp, q, lane);
-            else if constexpr (MODE == PASS_DKV) jvp_elem_dkv<DP, HZ>(p, k, grp, q, lane);
+            else if constexpr (C::GONLY) jvp_elem_g<MODE, DP>(p, k, grp, q, lane);
+            else if constexpr (MODE == PASS_DKV) jvp_elem_dkv<DP>(p, k, grp, q, lane);
             else if constexpr (MODE == PASS_DV) jvp_elem_dv<DP>(p, k, grp, q, lane);
-            else jvp_elem_two_pairs<MODE, DP, HZ>(p, k, grp, q, lane);
+            else jvp_elem_two_pairs<MODE, DP>(p, k, grp, q, lane);
         }
     } else {
         ptx::setmaxnreg_dec<C::REGS_EPI>();

@@ -288,6 +288,23 @@ __device__ __forceinline__ bool mbar_test2_warp(uint32_t b0, uint32_t p0, uint32
     return __all_sync(0xffffffffu, ok != 0);
 }
 
+// The same of three.
+__device__ __forceinline__ bool mbar_test3_warp(uint32_t b0, uint32_t p0, uint32_t b1, uint32_t p1, uint32_t b2, uint32_t p2) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred a;\n\t.reg .pred b;\n\t.reg .pred c;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 a, [%1], %2;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 b, [%3], %4;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 c, [%5], %6;\n\t"
+        "and.pred a, a, b;\n\t"
+        "and.pred a, a, c;\n\t"
+        "selp.u32 %0, 1, 0, a;\n\t}"
+        : "=r"(ok)
+        : "r"(b0), "r"(p0), "r"(b1), "r"(p1), "r"(b2), "r"(p2)
+        : "memory");
+    return __all_sync(0xffffffffu, ok != 0);
+}
+
 // Non-blocking test of one mbarrier phase; warp-uniform result.
 __device__ __forceinline__ bool mbar_test_warp(uint32_t bar, uint32_t parity) {
     uint32_t ok;

@@ -263,10 +263,10 @@ struct Operand {
     const CUtensorMap* map;
 };
 
-template <int MODE, int DP, bool HZ>
+template <int MODE, int DP>
 static int launch_pass(const Shape& s, const Operand (&own)[4], const Operand (&strm)[4], JvpParams prm, const DeviceFacts& dev, cudaStream_t st) {
     using C = JvpCfg<MODE, DP>;
-    constexpr auto kern = jvp_kernel<MODE, DP, HZ>;
+    constexpr auto kern = jvp_kernel<MODE, DP>;
     if (!prepare_kernel<kern>(dev, C::SMEM_BYTES)) return TVM_ATTN_CUDA_ERROR;
     // DV, DK: keys own, queries stream; FWD, DQ: queries own, keys stream
     prm.o = C::TRANSPOSED ? s.k : s.q;
@@ -275,8 +275,6 @@ static int launch_pass(const Shape& s, const Operand (&own)[4], const Operand (&
         prm.own[t] = own[t].ptr;
         prm.strm[t] = strm[t].ptr;
     }
-    if (HZ) prm.own[1] = nullptr;             // tangents of the owner side: not loaded
-    if (HZ && C::DKV) prm.own[3] = nullptr;
     // one CTA per SM (each needs the whole tensor memory and most of the shared memory of one); the work
     // items go round-robin over them
     prm.row_tiles = (prm.o.rows + JVP_ROWS - 1) / JVP_ROWS;
@@ -299,7 +297,7 @@ static int launch_pass(const Shape& s, const Operand (&own)[4], const Operand (&
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = ((MODE == PASS_DK || MODE == PASS_DQ) && !g_prof.enabled.load(std::memory_order_relaxed)) ? 1 : 0;
+    cfg.numAttrs = ((MODE == PASS_DK || MODE == PASS_DQ || MODE == PASS_DQ_G) && !g_prof.enabled.load(std::memory_order_relaxed)) ? 1 : 0;
     if (cudaLaunchKernelEx(&cfg, kern, *strm[0].map, *strm[1].map, *strm[2].map, *strm[3].map, *own[0].map, *own[1].map, *own[2].map,
                            *own[3].map, prm) != cudaSuccess)
         return cuda_status(cudaGetLastError());
@@ -308,20 +306,11 @@ static int launch_pass(const Shape& s, const Operand (&own)[4], const Operand (&
     return cuda_status(cudaGetLastError());
 }
 
-template <int MODE, int DP>
-static int launch_pass_hz(const Shape& s, const Operand (&own)[4], const Operand (&strm)[4], const JvpParams& prm, const DeviceFacts& dev, cudaStream_t st) {
-    // dtO absent: the specialisation that leaves the tangent path out, instantiated for the padded head dims 64 and 80; other
-    // head dims run the general kernel, which skips what it can.  The whole backward without dtO (B 16, H 16, N 1024), general /
-    // specialised: d = 64 571 to 590 / 386 us, 72 751 / 527, 80 782 to 789 / 540; built for them too it measured d = 16
-    // 475 / 333, 32 507 / 351, 48 529 to 547 / 366, so the line is only where it was first needed: it can go.
-    if constexpr (MODE != PASS_FWD && (DP == 64 || DP == 80))
-        if (prm.absent & ABSENT_HC) return launch_pass<MODE, DP, true>(s, own, strm, prm, dev, st);
-    return launch_pass<MODE, DP, false>(s, own, strm, prm, dev, st);
-}
-
 // The passes there are: FWD and DQ for every head dim; DKV where its four accumulators fit into tensor memory next to the
-// scores, DV and DK where they do not.
-static constexpr bool pass_exists(int mode, int dp) { return mode == PASS_DKV ? dp <= 80 : mode == PASS_DV || mode == PASS_DK ? dp > 80 : true; }
+// scores, DV and DK where they do not; DKV_G and DQ_G, the backward without dtO, up to the same head dim.
+static constexpr bool pass_exists(int mode, int dp) {
+    return mode == PASS_DKV || mode == PASS_DKV_G || mode == PASS_DQ_G ? dp <= 80 : mode == PASS_DV || mode == PASS_DK ? dp > 80 : true;
+}
 
 template <int MODE, int DP = 16>
 static int launch_pass_dp(const Shape& s, const Operand (&own)[4], const Operand (&strm)[4], const JvpParams& prm, const DeviceFacts& dev, cudaStream_t st) {
@@ -329,7 +318,7 @@ static int launch_pass_dp(const Shape& s, const Operand (&own)[4], const Operand
         return TVM_ATTN_UNSUPPORTED;
     } else {
         if constexpr (pass_exists(MODE, DP))
-            if (s.dp == DP) return launch_pass_hz<MODE, DP>(s, own, strm, prm, dev, st);
+            if (s.dp == DP) return launch_pass<MODE, DP>(s, own, strm, prm, dev, st);
         return launch_pass_dp<MODE, DP + 16>(s, own, strm, prm, dev, st);
     }
 }
@@ -535,11 +524,10 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
     for (const void* x : opt)
         if (x && !aligned16(x)) return TVM_ATTN_INVALID_ARG;
     if (dtO && (!dtQ || !dtK || !dtV)) return TVM_ATTN_INVALID_ARG;
-    const int absent = (dtO ? 0 : ABSENT_HC) | (dO ? 0 : ABSENT_G);
     // DKV takes its statistics divided by the scale, which overflows where that is next to nothing (lse / 1e-36 does at 340):
     // such a call, all of whose weights are equal, goes to the CUDA-core kernels.
     if (s.alpha < 1e-36f && pass_exists(PASS_DKV, s.dp)) s.simt = true;
-    if ((absent || !s.plain) && !s.simt && s.dp > 80) return TVM_ATTN_UNSUPPORTED;  // head dims above 80: both cotangents, packed self-attention
+    if ((!dO || !dtO || !s.plain) && !s.simt && s.dp > 80) return TVM_ATTN_UNSUPPORTED;  // head dims above 80: both cotangents, packed self-attention
     const size_t rows = (size_t)s.BH * (size_t)s.M;   // query rows: what the workspace and the statistics are sized by
     if (workspace_bytes < 3 * sizeof(float) * rows) return TVM_ATTN_WORKSPACE_TOO_SMALL;
     float* sig1 = static_cast<float*>(workspace);
@@ -586,7 +574,7 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
     const int short_rows = s.dp == 80 ? JvpCfg<PASS_DKV, 80>::BC : JVP_BC;
     for (int t = 0; t < 4; ++t) {
         x[8 + t] = x[t];
-        if (short_rows == JVP_BC || !in[t]) continue;
+        if (short_rows == JVP_BC || !in[t] || !dtO) continue;
         x[8 + t].map = &maps[8 + t];
         rc = make_tmap(&maps[8 + t], in[t], s, s.q, short_rows);
         if (rc != TVM_ATTN_OK) return rc;
@@ -596,17 +584,27 @@ int tvm_attn_jvp_bwd(const tvm_attn_params* p, const void* Q, const void* K, con
     std::memset(&b, 0, sizeof b);
     b.d = s.d; b.H = s.H;
     b.alpha = s.alpha; b.c2 = s.alpha * 1.4426950408889634f;
-    b.nlse2 = lse2; b.mu = mu; b.nsig1 = sig1; b.ncvec = cvec; b.status = dev->status; b.absent = absent;
+    b.nlse2 = lse2; b.mu = mu; b.nsig1 = sig1; b.ncvec = cvec; b.status = dev->status; b.no_g = !dO;
     auto bf16 = [](void* ptr) { return static_cast<__nv_bfloat16*>(ptr); };
+    if (!dtO) {   // owner keys (K, V), stream queries (Q, G); owner queries (Q, G), stream keys (K, V)
+        b.out0 = bf16(dV);
+        b.out1 = bf16(dK);
+        b.out_scale = s.alpha;
+        rc = launch_pass_dp<PASS_DKV_G>(s, {xK, xV, xK, xV}, {xQ, xG, xQ, xG}, b, *dev, st);
+        if (rc != TVM_ATTN_OK) return rc;
+        b.out0 = nullptr;
+        b.out1 = bf16(dQ);
+        return launch_pass_dp<PASS_DQ_G>(s, {xQ, xG, xQ, xG}, {xK, xV, xK, xV}, b, *dev, st);
+    }
     auto outputs = [&](void* tangent, void* primal, float scale) {
-        b.out0 = dtO ? bf16(tangent) : nullptr;
+        b.out0 = bf16(tangent);
         b.out1 = bf16(primal);
         b.out_scale = scale;
     };
     // dtV = P^T Hc, dV = P^T G + (P*Nn)^T Hc; dtK = alpha W^T Q, dK = alpha (dA^T Q + W^T tQ) : owner keys, stream queries
     if (pass_exists(PASS_DKV, s.dp)) {
         outputs(dtV, dV, s.alpha);
-        b.out2 = dtO ? bf16(dtK) : nullptr;
+        b.out2 = bf16(dtK);
         b.out3 = bf16(dK);
         rc = launch_pass_dp<PASS_DKV>(s, {xK, xtK, xV, xtV}, {x[10], x[11], x[8], x[9]}, b, *dev, st);
     } else {
