@@ -163,7 +163,7 @@ struct JvpCfg {
     static_assert(COL_SCORE + 4 * BC <= 512, "TMEM over-subscribed");
     // registers per thread: warpgroup 0, element-wise warps, epilogue warps (which hold an owner row, 4 registers a chunk)
     static constexpr bool TURNS = MODE == PASS_FWD || GONLY;   // the element-wise groups take tiles in turn: 64 columns a thread
-    static constexpr int REGS_LOAD = GONLY ? 72 : TURNS ? 56 : 96, REGS_ELEM = GONLY ? 160 : TURNS ? 168 : 152, REGS_EPI = TURNS ? 120 : 112;
+    static constexpr int REGS_LOAD = GONLY ? 88 : TURNS ? 56 : DKV && DP <= 48 ? 112 : 96, REGS_ELEM = MODE == PASS_FWD ? 168 : 152, REGS_EPI = TURNS ? 120 : DKV && DP <= 48 ? 96 : 112;
     static_assert(REGS_LOAD + 2 * REGS_ELEM + REGS_EPI <= 4 * JVP_REGS, "more registers than the block has");
     // barriers
     static constexpr int B_EFULL = 0;

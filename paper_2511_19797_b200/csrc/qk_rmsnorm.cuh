@@ -50,6 +50,7 @@ template <typename T>
 struct RmsRaw {
     uint4 q;
     __device__ __forceinline__ void load(const T* p) { q = __ldg(reinterpret_cast<const uint4*>(p)); }
+    __device__ __forceinline__ void zero() { q = make_uint4(0, 0, 0, 0); }
     __device__ __forceinline__ void get(uint64_t (&v)[RmsVec<T>::N / 2]) const { rms_unpack(q, v); }
     // Ends the reuse of an earlier unpacking: the next get() unpacks again (one instruction an element) instead of
     // holding twice the registers across the row sums.
@@ -85,16 +86,22 @@ __device__ __forceinline__ float rms_hsum(uint64_t v) {
     return lo + hi;
 }
 
-// How the cpr 16-byte chunks of a row are split: C chunks on each of cpr / C lanes.  The largest C <= cmax that divides
-// cpr and leaves three lanes or more (48 contiguous bytes per row and instruction; 32 would still be whole sectors,
-// but of rows that start on half of one).
-inline int rms_split(int cpr, int cmax) {
-    for (int c = cmax; c > 1; --c)
-        if (cpr % c == 0 && cpr / c >= 3) return c;
-    return 1;
+// How the cpr 16-byte chunks of a row are split: C chunks on each of P lanes.  The largest C <= cmax that divides cpr and
+// leaves three lanes or more (48 contiguous bytes per row and instruction), or, for d = 32, two; if
+// none does (d = 40, 56, 88, 104), the largest whose last lane has one chunk less: a row's sums and scalars cost a warp as much
+// for one chunk a lane as for three.  One chunk a lane before: backward (16, 16, 1024) d = 32 49.8 -> 40.5 us, 40 68.4 -> 61.6,
+// 56 106.9 -> 72.2; forward 27.1 -> 25.0, 36.8 -> 36.9, 51.8 -> 45.5.
+struct RmsSplit { int C, P; };
+inline RmsSplit rms_split(int cpr, int cmax) {
+    for (int waste = 0; waste < 2; ++waste)
+        for (int c = cmax; c > 1; --c) {
+            const int p = (cpr + c - 1) / c;
+            if (c * p - cpr == waste && (p >= 3 || (p == 2 && cpr == 4))) return {c, p};
+        }
+    return {1, cpr};
 }
 
-// Row groups of a warp in flight in the forward: with one chunk per lane (d = 40, 56, 88, 104) a thread would have two
+// Row groups of a warp in flight in the forward: with one chunk per lane (d = 8, 16, 24) a thread would have two
 // 16-byte loads in flight, and four groups measured 12 % faster than one; with two chunks or more, one group was faster.
 __host__ __device__ constexpr int rms_fwd_groups(int C) { return C == 1 ? 4 : 1; }
 
@@ -122,6 +129,16 @@ struct RmsRows {
     }
 };
 
+// The chunks of a lane; the last one reads as zero where there is none.
+template <typename T, int C>
+__device__ __forceinline__ void rms_load(RmsRaw<T> (&r)[C], const T* p, int P, bool full) {
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+        if (i == C - 1 && !full) r[i].zero();
+        else r[i].load(p + P * i * RmsVec<T>::N);
+    }
+}
+
 template <typename T>
 struct RmsFwdSide {
     const T* x; const T* tx; const float* g; T* y; T* ty;
@@ -130,17 +147,18 @@ struct RmsFwdSide {
 
 // Forward for both sides: blocks 0 .. nbq - 1 walk over the rows of Q, the others over those of K.  P = lanes per row;
 // a warp has U groups of 32 / P rows in flight (few chunks per lane: more groups).
-template <typename T, int C>
+template <typename T, int C, bool RAGGED>
 __global__ void __launch_bounds__(RMS_THREADS, 3)
 qk_rmsnorm_jvp_fwd_kernel(const RmsFwdSide<T> q, const RmsFwdSide<T> k, int nbq, int d, int P, float eps) {
     constexpr int V = RmsVec<T>::N, U = rms_fwd_groups(C);
-    __shared__ __align__(16) float scale[128];   // in shared memory: its 8 C registers a thread are worth a third of the warps
+    __shared__ __align__(16) float scale[144];   // (16 more: where a lane has no last chunk) in shared memory: its 8 C registers a thread are worth a third of the warps
     const bool is_q = (int)blockIdx.x < nbq;
     const RmsFwdSide<T>& a = is_q ? q : k;
     const unsigned block = is_q ? blockIdx.x : blockIdx.x - nbq, nblocks = is_q ? nbq : gridDim.x - nbq;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rpw = 32 / P;
     const int sub = lane / P, c = lane - sub * P, first = sub * P;
-    for (int j = threadIdx.x; j < d; j += RMS_THREADS) scale[j] = a.g[j];
+    const bool full = !RAGGED || (c + P * (C - 1)) * V < d;   // the lane has C chunks of its row (else C - 1)
+    for (int j = threadIdx.x; j < 144; j += RMS_THREADS) scale[j] = j < d ? a.g[j] : 0.f;
     __syncthreads();
     const float inv_d = 1.0f / (float)d;
     const unsigned rows_per_block = (RMS_THREADS / 32) * U * rpw, total = a.rows.total;
@@ -153,10 +171,8 @@ qk_rmsnorm_jvp_fwd_kernel(const RmsFwdSide<T> q, const RmsFwdSide<T> k, int nbq,
             const unsigned row = base + (warp * U + u) * rpw + sub;
             act[u] = sub < rpw && row < total;
             off[u] = act[u] ? a.rows.offset(row) + (size_t)c * V : 0;
-#pragma unroll
-            for (int i = 0; i < C; ++i) xr[u][i].load(a.x + off[u] + P * i * V);
-#pragma unroll
-            for (int i = 0; i < C; ++i) tr[u][i].load(a.tx + off[u] + P * i * V);
+            rms_load(xr[u], a.x + off[u], P, full);
+            rms_load(tr[u], a.tx + off[u], P, full);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -179,6 +195,7 @@ qk_rmsnorm_jvp_fwd_kernel(const RmsFwdSide<T> q, const RmsFwdSide<T> k, int nbq,
                     uint64_t x[V / 2], t[V / 2], g[V / 2], y[V / 2], ty[V / 2];
                     xr[u][i].repack(); tr[u][i].repack();
                     xr[u][i].get(x); tr[u][i].get(t);
+                    if (i == C - 1 && !full) continue;
                     rms_scale(scale + (c + P * i) * V, g);
 #pragma unroll
                     for (int e = 0; e < V / 2; ++e) {
@@ -209,7 +226,7 @@ struct RmsBwdSide {
 // Each block walks over its rows with a fixed stride, every thread keeping the dg terms of its own columns; the
 // block then adds them up in a fixed order and writes one partial row; a second kernel adds the partial rows, again
 // in a fixed order, so dg is bit-reproducible.
-template <typename T, int C>
+template <typename T, int C, bool RAGGED>
 __global__ void __launch_bounds__(RMS_BWD_THREADS, 5)
 qk_rmsnorm_jvp_bwd_kernel(const RmsBwdSide<T> q, const RmsBwdSide<T> k, int nbq, int d, int P, float eps) {
     constexpr int V = RmsVec<T>::N;
@@ -219,8 +236,9 @@ qk_rmsnorm_jvp_bwd_kernel(const RmsBwdSide<T> q, const RmsBwdSide<T> k, int nbq,
     const unsigned block = is_q ? blockIdx.x : blockIdx.x - nbq, nblocks = is_q ? nbq : gridDim.x - nbq;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rpw = 32 / P;
     const int sub = lane / P, c = lane - sub * P, first = sub * P;
-    __shared__ __align__(16) float scale[128];
-    for (int j = threadIdx.x; j < d; j += RMS_BWD_THREADS) scale[j] = a.g[j];
+    const bool full = !RAGGED || (c + P * (C - 1)) * V < d;   // the lane has C chunks of its row (else C - 1)
+    __shared__ __align__(16) float scale[144];   // (16 more: where a lane has no last chunk)
+    for (int j = threadIdx.x; j < 144; j += RMS_BWD_THREADS) scale[j] = j < d ? a.g[j] : 0.f;
     __syncthreads();
     uint64_t dg[C][V / 2];
 #pragma unroll
@@ -234,14 +252,10 @@ qk_rmsnorm_jvp_bwd_kernel(const RmsBwdSide<T> q, const RmsBwdSide<T> k, int nbq,
         const bool act = sub < rpw && row < total;
         const size_t off = act ? a.rows.offset(row) + (size_t)c * V : 0;
         RmsRaw<T> xr[C], tr[C], yr[C], zr[C];   // kept as loaded: a quarter of a thread's registers, not half
-#pragma unroll
-        for (int i = 0; i < C; ++i) xr[i].load(a.x + off + P * i * V);
-#pragma unroll
-        for (int i = 0; i < C; ++i) tr[i].load(a.tx + off + P * i * V);
-#pragma unroll
-        for (int i = 0; i < C; ++i) yr[i].load(a.dy + off + P * i * V);
-#pragma unroll
-        for (int i = 0; i < C; ++i) zr[i].load(a.dty + off + P * i * V);
+        rms_load(xr, a.x + off, P, full);
+        rms_load(tr, a.tx + off, P, full);
+        rms_load(yr, a.dy + off, P, full);
+        rms_load(zr, a.dty + off, P, full);
         uint64_t ss2 = 0ull, s2 = 0ull, ax2 = 0ull, bx2 = 0ull, bt2 = 0ull;
 #pragma unroll
         for (int i = 0; i < C; ++i) {
@@ -275,6 +289,7 @@ qk_rmsnorm_jvp_bwd_kernel(const RmsBwdSide<T> q, const RmsBwdSide<T> k, int nbq,
 #pragma unroll
             for (int i = 0; i < C; ++i) {
                 uint64_t x[V / 2], t[V / 2], gy[V / 2], gt[V / 2], g[V / 2], dx[V / 2], dtx[V / 2];
+                if (i == C - 1 && !full) continue;
                 xr[i].repack(); tr[i].repack(); yr[i].repack(); zr[i].repack();
                 xr[i].get(x); tr[i].get(t); yr[i].get(gy); zr[i].get(gt);
                 rms_scale(scale + (c + P * i) * V, g);
@@ -298,6 +313,7 @@ qk_rmsnorm_jvp_bwd_kernel(const RmsBwdSide<T> q, const RmsBwdSide<T> k, int nbq,
     if (sub < rpw) {
 #pragma unroll
         for (int i = 0; i < C; ++i) {
+            if (i == C - 1 && !full) continue;
             uint64_t* mine = reinterpret_cast<uint64_t*>(part + (warp * rpw + sub) * d + (c + P * i) * V);
 #pragma unroll
             for (int e = 0; e < V / 2; ++e) mine[e] = dg[i][e];

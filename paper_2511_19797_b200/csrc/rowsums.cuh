@@ -17,7 +17,7 @@ constexpr int ROWSUM_THREADS = 256;
 constexpr int ROWSUM_BLOCKS = 148 * 3;   // of a launch at most, what the 148 SMs hold: each block walks over its rows
 
 // P = lanes per row, C = chunks per lane; the rows of a warp are consecutive.
-template <typename T, int C>
+template <typename T, int C, bool RAGGED>
 __global__ void __launch_bounds__(ROWSUM_THREADS, 3)
 bwd_rowsums_kernel(const T* __restrict__ G, const T* __restrict__ Hc, const T* __restrict__ O, const T* __restrict__ tO,
                    const float* __restrict__ lse, float* __restrict__ sig1, float* __restrict__ cvec, float* __restrict__ lse2,
@@ -44,6 +44,7 @@ bwd_rowsums_kernel(const T* __restrict__ G, const T* __restrict__ Hc, const T* _
             off += c * V;
 #pragma unroll
             for (int k = 0; k < C; ++k) {
+                if (RAGGED && k == C - 1 && (c + P * k) * V >= d) continue;   // the lane has a chunk less
                 o[k].load(O + off + k * P * V);
                 if (G) x[k].load(G + off + k * P * V);
                 if (Hc) { y[k].load(Hc + off + k * P * V); t[k].load(tO + off + k * P * V); }

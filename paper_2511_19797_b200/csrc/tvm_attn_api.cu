@@ -195,9 +195,13 @@ static int launch_rowsums(const Shape& s, const void* G, const void* Hc, const v
     const long long rows = s.BH * s.M;           // fit 31 bits
     const int cpr = s.d * (int)sizeof(T) / 16;   // 16-byte chunks per row (d % 8 == 0)
     if (cpr > 32) return TVM_ATTN_UNSUPPORTED;   // d <= 128
-    const int C = rms_split(cpr, 4), P = cpr / C;
+    const int C = rms_split(cpr, 4).C, P = rms_split(cpr, 4).P;
     const long long rows_per_block = (ROWSUM_THREADS / 32) * (32 / P), blocks = (rows + rows_per_block - 1) / rows_per_block;
-    const auto kern = C == 4 ? bwd_rowsums_kernel<T, 4> : C == 3 ? bwd_rowsums_kernel<T, 3> : C == 2 ? bwd_rowsums_kernel<T, 2> : bwd_rowsums_kernel<T, 1>;
+    const auto kern = C * P > cpr ? (C == 4 ? bwd_rowsums_kernel<T, 4, true> : C == 3 ? bwd_rowsums_kernel<T, 3, true> : bwd_rowsums_kernel<T, 2, true>)
+                      : C == 4    ? bwd_rowsums_kernel<T, 4, false>
+                      : C == 3    ? bwd_rowsums_kernel<T, 3, false>
+                      : C == 2    ? bwd_rowsums_kernel<T, 2, false>
+                                  : bwd_rowsums_kernel<T, 1, false>;
     g_prof.before(st);
     kern<<<(unsigned)(blocks < ROWSUM_BLOCKS ? blocks : ROWSUM_BLOCKS), ROWSUM_THREADS, 0, st>>>(
         (const T*)G, (const T*)Hc, (const T*)O, (const T*)tO, lse, sig1, cvec, lse2, (unsigned)rows, s.q, q_packed(s) ? 0 : s.H, s.d, P, sign);
@@ -396,11 +400,11 @@ static void rms_blocks(long long rows_q, long long rows_k, int rows_per_block, i
     *nbk = (int)(most - q < need_k ? most - q : need_k);
 }
 
-template <typename T, int C>
+template <typename T, int C, bool RAGGED = false>
 static int rms_fwd_c(const Shape& s, float eps, const RmsFwdSide<T>& q, const RmsFwdSide<T>& k, int P, cudaStream_t st) {
     int nbq, nbk;
     rms_blocks(q.rows.total, k.rows.total, (RMS_THREADS / 32) * rms_fwd_groups(C) * (32 / P), RMS_FWD_BLOCKS, &nbq, &nbk);
-    qk_rmsnorm_jvp_fwd_kernel<T, C><<<nbq + nbk, RMS_THREADS, 0, st>>>(q, k, nbq, s.d, P, eps);
+    qk_rmsnorm_jvp_fwd_kernel<T, C, RAGGED><<<nbq + nbk, RMS_THREADS, 0, st>>>(q, k, nbq, s.d, P, eps);
     g_launches += 1;
     return cuda_status(cudaGetLastError());
 }
@@ -410,7 +414,11 @@ static int rms_fwd(const Shape& s, float eps, const void* Q, const void* tQ, con
                    const float* gK, void* Qn, void* tQn, void* Kn, void* tKn, cudaStream_t st) {
     const RmsFwdSide<T> q{(const T*)Q, (const T*)tQ, gQ, (T*)Qn, (T*)tQn, rms_rows(s, s.q)};
     const RmsFwdSide<T> k{(const T*)K, (const T*)tK, gK, (T*)Kn, (T*)tKn, rms_rows(s, s.k)};
-    const int cpr = s.d * (int)sizeof(T) / 16, C = rms_split(cpr, 4), P = cpr / C;
+    const int cpr = s.d * (int)sizeof(T) / 16, C = rms_split(cpr, 4).C, P = rms_split(cpr, 4).P;
+    if (C * P > cpr)
+        return C == 2   ? rms_fwd_c<T, 2, true>(s, eps, q, k, P, st)
+               : C == 3 ? rms_fwd_c<T, 3, true>(s, eps, q, k, P, st)
+                        : rms_fwd_c<T, 4, true>(s, eps, q, k, P, st);
     switch (C) {
         case 1: return rms_fwd_c<T, 1>(s, eps, q, k, P, st);
         case 2: return rms_fwd_c<T, 2>(s, eps, q, k, P, st);
@@ -419,12 +427,12 @@ static int rms_fwd(const Shape& s, float eps, const void* Q, const void* tQ, con
     }
 }
 
-template <typename T, int C>
+template <typename T, int C, bool RAGGED = false>
 static int rms_bwd_c(const Shape& s, float eps, RmsBwdSide<T> q, RmsBwdSide<T> k, int P, float* dgQ, float* dgK, cudaStream_t st) {
     int nbq, nbk;
     rms_blocks(q.rows.total, k.rows.total, (RMS_BWD_THREADS / 32) * (32 / P), RMS_BWD_BLOCKS, &nbq, &nbk);
     k.partial = q.partial + (size_t)nbq * s.d;
-    qk_rmsnorm_jvp_bwd_kernel<T, C><<<nbq + nbk, RMS_BWD_THREADS, 0, st>>>(q, k, nbq, s.d, P, eps);
+    qk_rmsnorm_jvp_bwd_kernel<T, C, RAGGED><<<nbq + nbk, RMS_BWD_THREADS, 0, st>>>(q, k, nbq, s.d, P, eps);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return TVM_ATTN_CUDA_ERROR;
     cudaLaunchConfig_t cfg = {};
@@ -447,7 +455,8 @@ static int rms_bwd(const Shape& s, float eps, const void* Q, const void* tQ, con
                    void* dK, void* dtK, float* dgQ, float* dgK, float* partial, cudaStream_t st) {
     const RmsBwdSide<T> q{(const T*)Q, (const T*)tQ, gQ, (const T*)dQn, (const T*)dtQn, (T*)dQ, (T*)dtQ, partial, rms_rows(s, s.q)};
     const RmsBwdSide<T> k{(const T*)K, (const T*)tK, gK, (const T*)dKn, (const T*)dtKn, (T*)dK, (T*)dtK, nullptr, rms_rows(s, s.k)};
-    const int cpr = s.d * (int)sizeof(T) / 16, C = rms_split(cpr, 3), P = cpr / C;
+    const int cpr = s.d * (int)sizeof(T) / 16, C = rms_split(cpr, 3).C, P = rms_split(cpr, 3).P;
+    if (C * P > cpr) return C == 2 ? rms_bwd_c<T, 2, true>(s, eps, q, k, P, dgQ, dgK, st) : rms_bwd_c<T, 3, true>(s, eps, q, k, P, dgQ, dgK, st);
     switch (C) {
         case 1: return rms_bwd_c<T, 1>(s, eps, q, k, P, dgQ, dgK, st);
         case 2: return rms_bwd_c<T, 2>(s, eps, q, k, P, dgQ, dgK, st);
