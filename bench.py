@@ -39,7 +39,7 @@ BWD_KERNELS = {"narrow": {"bwd_rowsums": (0, 4), "bwd_dkv": (12, 12), "bwd_dq": 
 BWD_CREDITED_GEMMS = 15
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu capture summarised in
 # profiles/jvp_fwd_bwd_kernels_dit512.md (that workload and the full variant only; None for anything else)
-NCU_TRAFFIC_BYTES = {"dit512": {"fwd": 279.5e6, "bwd_dkv": 423.0e6, "bwd_dq": 359.3e6}}
+NCU_TRAFFIC_BYTES = {"dit512": {"fwd": 278.7e6, "bwd_dkv": 421.6e6, "bwd_dq": 358.7e6}}
 
 
 def load_peaks():
