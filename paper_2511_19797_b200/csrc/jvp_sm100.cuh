@@ -30,7 +30,7 @@
 // the score buffers and all barrier phases run on through the items.
 //
 // 16 warps in four warpgroups:
-//   warp 0    loads the owner tiles and the E ring (stream tensors that only the score MMAs read)
+//   warp 0    loads the owner tiles and the E ring (stream tensors that only the score MMAs read; none in DKV_G, DQ_G)
 //   warp 1    issues the MMAs
 //   warp 2    loads the L ring (stream tensors the output MMAs read)
 //   warp 3    DKV, DKV_G: puts the per-query statistics into the tiles (FOLD below)
@@ -82,6 +82,10 @@ constexpr uint64_t JVP_WAIT_LIMIT_NS = 200ull * 1000ull * 1000ull, JVP_TILE_LIMI
 // Registers per thread at launch; setmaxnreg moves them between the four warpgroups (JvpCfg::REGS_*) within what the block
 // was launched with: the host refuses to launch a build whose kernels have fewer.
 constexpr int JVP_REGS = 128;
+// DKV_G, DQ_G: what the epilogue does in front of an item's stores, in steps of the issuing warp (a tile each) from the item's end on.
+// Owner operands that are due later than that would hold the stores back.  Nothing in front of them / two steps, us: (64, 16, N)
+// d = 72 N = 192 149 / 138, N = 200 165 / 138, d = 64 N = 192 116 / 110; d = 56 N = 256 117 / 121.
+constexpr int JVP_AHEAD = 2;
 
 struct JvpParams {
     int d, H;
@@ -133,15 +137,23 @@ struct JvpCfg {
     // tensor memory as bf16 A operands: an MMA with A in shared memory moves 4 KB of A per k-step through the
     // shared-memory port.  WIDE, DKV: tensor memory has no room, everything is in shared memory.
     static constexpr bool XT = !WIDE && !DKV;
-    static constexpr int NOWN = 2 * NPAIR - (XT ? 2 : 0);   // owner tensors in shared memory
+    // DKV_G, DQ_G (XS): they come to tensor memory by way of shared memory, where warp 0 puts an item's rows as soon as those of the
+    // item before have left it; loaded by the epilogue, uncoalesced and behind its stores, they are the chain of a short item.
+    // (Without dtO, (64, 16, N), us: d = 64 N = 192 144 -> 110, N = 64 42 -> 41, d = 72 N = 192 171 -> 138, d = 80 N = 192 193 ->
+    // 157, (16, 16, 1024, 72) 370 -> 360.  Rows that do not begin on 32 bytes take the TMA longer: d = 40 N = 64 37 -> 41, d = 56
+    // 39 -> 41.  With 16-byte copies instead, by warp 0 or by the epilogue: N = 64 at d = 64 53.)
+    static constexpr bool XS = GONLY;
+    static constexpr int NOWN = XS ? 2 : 2 * NPAIR - (XT ? 2 : 0);   // owner tensors in shared memory
     // FOLD (DKV, DKV_G): the per-query statistics belong to the columns of the tile, the same for every thread; read from
     // shared memory they would cost 512 bytes a warp and column.  Instead they are an extra piece of the score MMAs: each
     // is split into three bf16 parts in columns of its own behind the stream row, against ones behind the owner row, so
     // that the accumulators arrive as S - lse/alpha, Sd - mu/alpha, D - Sigma1, X - c.  At d = 72 these columns are the
-    // padding up to 80; other head dims take one more k-step of N = 128.
+    // padding up to 80; other head dims take one more k-step.
     static constexpr bool FOLD = DKV || MODE == PASS_DKV_G;
     static constexpr int OWN_ATOM = JVP_ROWS * 128, ATOM = BC * 128;
-    static constexpr int OWN_BYTES = OWN_ATOM * (WIDE ? 2 : 1) + (TAIL ? JVP_ROWS * 32 : 0);   // one owner tensor
+    // One owner tensor.  (XS: the columns from 64 on lie in the L ring, whose second atoms have room, so that the ring keeps its six
+    // stages: with five, DQ_G at d = 72 (16, 16, 1024) takes 160 us instead of 142.)
+    static constexpr int OWN_BYTES = OWN_ATOM * (WIDE ? 2 : 1) + (TAIL && !XS ? JVP_ROWS * 32 : 0);
     static constexpr int EST_BYTES = E_MN ? ATOM * NA : ATOM * (WIDE ? 2 : 1) + (TAIL ? BC * 32 : 0);   // one E-ring tile
     static constexpr int LST_BYTES = ATOM * NA;                                                // one L-ring tile
     static constexpr int SE = GONLY ? 0 : WIDE ? (NPAIR == 2 ? 1 : 2) : DKV ? (TAIL ? 2 : 3) : TAIL ? 3 : 4;
@@ -149,10 +161,12 @@ struct JvpCfg {
     static constexpr int TILE_BYTES = NOWN * OWN_BYTES + SE * 2 * EST_BYTES + SL * 2 * LST_BYTES;
     // FOLD: statistics of a stage, [Y0 rows, Y1 rows][16 bytes], for the rings the score MMAs read; ones and zeros
     static constexpr int FOLD_BYTES = 2 * BC * 16;
-    static constexpr int FOLD_E = FOLD ? SE : 0, FOLD_L = FOLD ? SL : 0;
-    static constexpr int ONES_BYTES = FOLD ? JVP_ROWS * 32 : 0;
+    // (DKV_G with a tail: columns 80 to 95 of the L tiles and of the owner operands instead).
+    static constexpr bool FOLD_TAIL = FOLD && XS && TAIL;
+    static constexpr int FOLD_E = FOLD ? SE : 0, FOLD_L = FOLD && !FOLD_TAIL ? SL : 0;
+    static constexpr int ONES_BYTES = FOLD && !FOLD_TAIL ? JVP_ROWS * 32 : 0;
     static constexpr int EFULL_COUNT = 1 + (TAIL ? 32 : 0) + (FOLD_E ? 1 : 0);   // TMA issuer, each lane's own copies, warp 3
-    static constexpr int LFULL_COUNT = 1 + (TAIL || (TRANSPOSED && !FOLD) ? 32 : 0) + (FOLD_L ? 1 : 0);
+    static constexpr int LFULL_COUNT = 1 + (TAIL || (TRANSPOSED && !FOLD) ? 32 : 0) + (FOLD ? 1 : 0);
     // TMEM columns: accumulators, the owner operands in the gaps behind them,
     // score accumulators (FWD, DV: two buffers of S | Sd; DKV_G, DQ_G: of S | X; DK, DQ: one of S | Sd | D | X).
     static constexpr int NACC = DKV ? 4 : 2;
@@ -161,16 +175,16 @@ struct JvpCfg {
     static constexpr int COL_X0 = DP, COL_X1 = COL_ACC1 + DP;
     static_assert(!XT || DP + DP / 2 <= 128, "operands do not fit behind their accumulators");
     static_assert(COL_SCORE + 4 * BC <= 512, "TMEM over-subscribed");
-    // registers per thread: warpgroup 0, element-wise warps, epilogue warps (which hold an owner row, 4 registers a chunk)
-    static constexpr bool TURNS = MODE == PASS_FWD || GONLY;   // the element-wise groups take tiles in turn: 64 columns a thread
-    static constexpr int REGS_LOAD = GONLY ? 88 : TURNS ? 56 : DKV && DP <= 48 ? 112 : 96, REGS_ELEM = MODE == PASS_FWD ? 168 : 152, REGS_EPI = TURNS ? 120 : DKV && DP <= 48 ? 96 : 112;
+    // Registers per thread: warpgroup 0, element-wise warps (FWD, DKV_G, DQ_G: 64 columns a thread), epilogue warps (which hold an owner
+    // row, 4 registers a chunk, or the columns they have read).
+    static constexpr int REGS_LOAD = MODE == PASS_FWD ? 56 : GONLY ? 80 : DKV && DP <= 48 ? 112 : 96, REGS_ELEM = MODE == PASS_FWD ? 168 : 152, REGS_EPI = MODE == PASS_FWD ? 120 : GONLY ? 128 : DKV && DP <= 48 ? 96 : 112;
     static_assert(REGS_LOAD + 2 * REGS_ELEM + REGS_EPI <= 4 * JVP_REGS, "more registers than the block has");
     // barriers
     static constexpr int B_EFULL = 0;
     static constexpr int B_LFULL = B_EFULL + SE;
-    static constexpr int OWN_SETS = DKV ? 2 : 1;                       // owner tiles with barriers of their own (DKV: K, tK | V, tV)
+    static constexpr int OWN_SETS = DKV || XS ? 2 : 1;                 // owner tiles with barriers of their own (DKV: K, tK | V, tV; XS: one tensor each)
     static constexpr int B_OWN = B_LFULL + SL;                         // owner tiles in shared memory loaded
-    static constexpr int B_OWNFREE = B_OWN + OWN_SETS;                 // ... free: the score MMAs of the item are complete
+    static constexpr int B_OWNFREE = B_OWN + OWN_SETS;                 // ... free: the score MMAs of the item are complete (XS: read by the epilogue)
     static constexpr int B_XRDY = B_OWNFREE + OWN_SETS;                       // owner operands in tensor memory written
     static constexpr int XSETS = GONLY ? 2 : 1;                        // with barriers of their own
     static constexpr int B_XFREE = B_XRDY + XSETS;                     // ... free
@@ -274,6 +288,13 @@ struct JvpBlock {
         return wait(C::B_LDONE + (t & (C::NOUTDONE - 1)), t / C::NOUTDONE);
     }
     __device__ __forceinline__ uint32_t own_tile(int t) const { return base + t * C::OWN_BYTES; }
+    // TAIL: 16-byte chunk c behind column 64 of owner row r: compact blocks behind the tile; XS: chunks of the second atoms of the L
+    // ring's first stage, which have 64 columns where the stream's tail, with the statistics, has 32.
+    __device__ __forceinline__ uint32_t own_tail(int t, int r, int c) const {
+        static_assert(!C::XS || C::ATOM == 64 * 128, "rows 64 on: in the second tensor's atom");
+        if (C::XS) return base + L + 2 * C::ATOM + r * 128 + (((4 + 2 * t + c) ^ (r & 7)) << 4);
+        return own_tile(t) + C::OWN_ATOM + (c * JVP_ROWS + r) * 16;
+    }
     __device__ __forceinline__ const float* stats(int s) const { return static_cast<const float*>(__cvta_shared_to_generic(base + STATS + s * C::NSTAT * C::BC * 4)); }
     __device__ __forceinline__ float4& row_state(int r) const { return *static_cast<float4*>(__cvta_shared_to_generic(base + ROW_STATE + 16 * r)); }
     __device__ __forceinline__ float4& row_sums(int r) const { return *static_cast<float4*>(__cvta_shared_to_generic(base + ROW_SUMS + 16 * r)); }
@@ -295,17 +316,18 @@ __device__ __forceinline__ void jvp_load_owners(const JvpParams& p, const JvpBlo
     constexpr int KT = C::TAIL ? (DP - 64) / 8 : 1, H64 = 64 * 128;
     const int bh = item / p.row_tiles, row0 = (item - bh * p.row_tiles) * JVP_ROWS;
     const int cb = bh / p.H, ch = bh - cb * p.H;
+    const bool upper = !C::XS || p.o.rows - row0 > 64;   // (XS: rows beyond the tensor are not read)
     if (lane == 0) {
         const uint32_t full = k.bar(C::B_OWN + SET);
         uint32_t tx = 0;
 #pragma unroll
-        for (int t = T0; t < T1; ++t) tx += C::OWN_ATOM * (C::WIDE ? 2 : 1);
+        for (int t = T0; t < T1; ++t) tx += upper ? C::OWN_ATOM * (C::WIDE ? 2 : 1) : C::OWN_ATOM / 2;
         ptx::mbar_arrive_expect_tx(full, tx);
 #pragma unroll
         for (int t = T0; t < T1; ++t) {
             const uint32_t dst = k.own_tile(t);
             ptx::tma_load_4d(dst, maps[t], full, 0, row0, ch, cb);
-            ptx::tma_load_4d(dst + H64, maps[t], full, 0, row0 + 64, ch, cb);
+            if (upper) ptx::tma_load_4d(dst + H64, maps[t], full, 0, row0 + 64, ch, cb);
             if (C::WIDE) {
                 ptx::tma_load_4d(dst + C::OWN_ATOM, maps[t], full, 64, row0, ch, cb);
                 ptx::tma_load_4d(dst + C::OWN_ATOM + H64, maps[t], full, 64, row0 + 64, ch, cb);
@@ -318,14 +340,13 @@ __device__ __forceinline__ void jvp_load_owners(const JvpParams& p, const JvpBlo
 #pragma unroll
         for (int t = T0; t < T1; ++t) {
             const __nv_bfloat16* x = p.own[t];
-            const uint32_t tile = k.own_tile(t) + C::OWN_ATOM + lane * 16;
 #pragma unroll
             for (int c = 0; c < KT; ++c) {
                 if (c < ntail) {
 #pragma unroll
                     for (int rp = 0; rp < JVP_ROWS / 32; ++rp) {
                         const bool v = lane + 32 * rp < rows_left;
-                        ptx::cp_async_16(tile + (c * JVP_ROWS + 32 * rp) * 16, v ? x + lane_row + rp * d32 + 8 * c : x, v ? 16u : 0u);
+                        ptx::cp_async_16(k.own_tail(t, lane + 32 * rp, c), v ? x + lane_row + rp * d32 + 8 * c : x, v ? 16u : 0u);
                     }
                 }
             }
@@ -482,6 +503,30 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
     }
 }
 
+// XS: warp 0 loads the owner tiles of one item after the other, one tensor at a time.
+template <int MODE, int DP>
+__device__ __forceinline__ void jvp_stage_owners(const JvpParams& p, const JvpBlock<MODE, DP>& shared, const CUtensorMap* const (&maps)[4], int lane) {
+    using C = JvpCfg<MODE, DP>;
+    const JvpBlock<MODE, DP> k = shared.pinned();
+    int n0 = 0, n1 = 0;   // items whose first, second tensor has been asked for
+    bool ok = true;
+    for (int item = blockIdx.x; item < p.items; item += gridDim.x) {
+        ok = n0 == 0 || k.wait_item(C::B_OWNFREE, n0 - 1);
+        if (!ok) break;
+        jvp_load_owners<MODE, DP, 0>(p, k, maps, item, lane);
+        ++n0;
+        ok = n1 == 0 || k.wait_item(C::B_OWNFREE + 1, n1 - 1);
+        if (!ok) break;
+        jvp_load_owners<MODE, DP, 1>(p, k, maps, item, lane);
+        ++n1;
+    }
+    if (C::TAIL) ptx::cp_async_wait_all();   // nothing of ours stays in flight
+    if (!ok) {                               // nor, after a time-out, a TMA load
+        ptx::mbar_wait_drain(k.bar(C::B_OWN), (n0 - 1) & 1, ptx::DRAIN_LIMIT_NS);
+        if (n1 > 0) ptx::mbar_wait_drain(k.bar(C::B_OWN + 1), (n1 - 1) & 1, ptx::DRAIN_LIMIT_NS);
+    }
+}
+
 // FOLD.  Each statistic is stored as three bf16 parts whose sum is its 24 bits, in the first three of eight columns, against
 // ones in the owner operand.
 constexpr uint32_t JVP_ONES0 = 0x3F803F80u, JVP_ONES1 = 0x00003F80u;   // 1, 1, 1, 0 in bf16
@@ -509,8 +554,8 @@ __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE
     const bool own = k.fold_step();
     const Dst de = own ? Dst{k.base + k.FOLD_E + lane * 16, (uint32_t)C::FOLD_BYTES, BC * 16, 32 * 16}
                        : Dst{k.base + k.E + 2 * C::ATOM + lane * 128 + ((1 ^ sw) << 4), 2u * C::EST_BYTES, C::ATOM, 32 * 128};
-    const Dst dl = own ? Dst{k.base + k.FOLD_L + lane * 16, (uint32_t)C::FOLD_BYTES, BC * 16, 32 * 16}
-                                        : Dst{k.base + k.L + 2 * C::ATOM + lane * 128 + ((1 ^ sw) << 4), 2u * C::LST_BYTES, C::ATOM, 32 * 128};
+    const Dst dl = own && !C::FOLD_TAIL ? Dst{k.base + k.FOLD_L + lane * 16, (uint32_t)C::FOLD_BYTES, BC * 16, 32 * 16}
+                                        : Dst{k.base + k.L + 2 * C::ATOM + lane * 128 + (((own ? 2 : 1) ^ sw) << 4), 2u * C::LST_BYTES, C::ATOM, 32 * 128};
     const float f_lse = 1.0f / p.c2, f_mu = -1.0f / p.alpha;   // to the scale of S and Sd
     float a[4];                        // (statistic of tensor 0, of tensor 1) of the two rows: lse, mu (DKV_G: lse, c)
     [[maybe_unused]] float b[4];       // DKV: Sigma1, c
@@ -663,7 +708,11 @@ struct JvpIssue {
         ksteps<FROM_L, ATM>([&](uint32_t ao, uint32_t ahi, uint32_t bo, uint32_t bhi, uint32_t acc) {
             step<ATM>(el, col, a + ao, ahi, lo + bo + ((uint32_t)(bhi == HI_TAIL ? T * BC * 16 : T * ATOM) >> 4), bhi, I_S, acc);
         });
-        if (k.fold_step()) fold_step(el, col, k, fold, T, I_S);
+        if constexpr (C::FOLD_TAIL) {
+            if (k.fold_step()) step<ATM>(el, col, a + 8u * KS, HI_SW, lo + l_k(KS) + ((uint32_t)(T * ATOM) >> 4), HI_SW, I_S, 1u);
+        } else if (k.fold_step()) {
+            fold_step(el, col, k, fold, T, I_S);
+        }
     }
     // Half of acc0 += A0 B0, acc1 += A1 B0 + A0 B1 (k-steps U0, U0 + 1 of four; the operand of a k-step lies at the columns of
     // the scores it replaces); acc = 0: the accumulators are overwritten.
@@ -915,8 +964,9 @@ __device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const Jv
 
 // DKV_G, DQ_G: two score buffers taken in turn, operands written over the scores.  Pipe order: dV(n - 2) | S(n) | dK(n - 3) | X(n - 1)
 // (DQ_G: S(n) | dQ(n - 3) | X(n - 1)): while a group works on tile n - 2 the other's n - 3 is complete, and the scores of what
-// either takes next are there before it asks for them.  (d = 72 (16, 16, 1024): 461 us for the two passes as specialisations of DKV
-// and DQ, whose layout has room for tiles of 48, one buffer and owners in shared memory; 305 now.)  One wait a tile, for everything that the tile's batch needs (P(n - 2)
+// either takes next are there before it asks for them.  (d = 72 (16, 16, 1024), events around each kernel, below the power cap: 314 +
+// 202 us for the two passes as specialisations of DKV and DQ, whose layout has room for tiles of 48, one buffer and owners in
+// shared memory; 163 + 136 now.)  One wait a tile, for everything that the tile's batch needs (P(n - 2)
 // written, or S(n - 2) read; dA(n - 3) written; stage n full): with a wait in front of every product this warp was what bounded a
 // tile (DQ_G, d = 72: 1240 cycles, MMAs of 480).
 template <int MODE, int DP>
@@ -926,68 +976,62 @@ __device__ __forceinline__ void jvp_issue_g(const JvpParams& p, const JvpBlock<M
     constexpr bool KEYS = MODE == PASS_DKV_G;
     const JvpBlock<MODE, DP> k = shared.pinned();
     const int T = jvp_pin(p.T), last = jvp_item_count(p) * T;
-    // The epilogue stages an item's owner operands once the item two before is over.  Items of three tiles or more run on into one
-    // another; shorter ones are finished one by one.
-    const int chunk = T > 2 ? last : T;
     JvpSlot l = I::l_slot(k);
     uint32_t xlo = 0, xfold = 0, vlo = 0, klo = 0;   // stages of the tiles n - 1, n - 2, n - 3
     uint32_t first = 0, end = 0;                     // bit i: tile n - i is the first, the last of its item
     int sj = 0, si = 0, xi = 0, oi = 0;              // tile within its item; items opened by S, by X, by the outputs
-    for (int base = 0; base < last; base += chunk) {
-        for (int m = 0; m < chunk + 3; ++m) {
-            const int n = base + m;
-            const bool score = m < chunk, x = m >= 1 && m <= chunk, v_out = m >= 2 && m < chunk + 2, k_out = m >= 3;
-            const int ba = C::B_PREADY + 2 * (n & 1), bb = C::B_PREADY + 2 * ((n - 1) & 1) + 1, pa = ((n - 2) >> 1) & 1, pb = ((n - 3) >> 1) & 1;
-            if (!(k_out && score && ptx::mbar_test3_warp(k.bar(ba), pa, k.bar(bb), pb, k.bar(C::B_LFULL + l.s), l.ph))) {
-                if (v_out && !k.wait(ba, pa)) return;
-                if (k_out && !k.wait(bb, pb)) return;
-                if (score && !k.wait(C::B_LFULL + l.s, l.ph)) return;
+    for (int n = 0; n < last + 3; ++n) {
+        const bool score = n < last, x = n >= 1 && n <= last, v_out = n >= 2 && n < last + 2, k_out = n >= 3;
+        const int ba = C::B_PREADY + 2 * (n & 1), bb = C::B_PREADY + 2 * ((n - 1) & 1) + 1, pa = ((n - 2) >> 1) & 1, pb = ((n - 3) >> 1) & 1;
+        if (!(k_out && score && ptx::mbar_test3_warp(k.bar(ba), pa, k.bar(bb), pb, k.bar(C::B_LFULL + l.s), l.ph))) {
+            if (v_out && !k.wait(ba, pa)) return;
+            if (k_out && !k.wait(bb, pb)) return;
+            if (score && !k.wait(C::B_LFULL + l.s, l.ph)) return;
+        }
+        first = first << 1 | (score && sj == 0 ? 1u : 0u);
+        end = end << 1 | (score && sj == T - 1 ? 1u : 0u);
+        const uint32_t col = C::COL_SCORE + (n & 1) * 2 * C::BC, colx = C::COL_SCORE + ((n - 1) & 1) * 2 * C::BC + C::BC;
+        // first output MMAs of an item: they overwrite the accumulators
+        auto acc_free = [&]() { return oi++ == 0 || k.wait(C::B_ACCFREE, oi - 2); };
+        auto part_x = [&]() {
+            if (!KEYS && (first & 8u) && !acc_free()) return false;
+            if ((first & 2u) && !k.wait(C::B_XRDY + 1, xi++)) return false;
+            ptx::tc_fence_after_sync();
+            const uint32_t el = ptx::elect_one();
+            if (k_out) {
+                I::template g_outputs<1>(el, colx, klo, first & 8u ? 0u : 1u);
+                ptx::mma_commit_p(el, k.bar(C::B_OUTDONE + ((n - 3) & (C::NOUTDONE - 1))));
+                if (end & 8u) ptx::mma_commit_p(el, k.bar(C::B_FINAL));
             }
-            first = first << 1 | (score && sj == 0 ? 1u : 0u);
-            end = end << 1 | (score && sj == T - 1 ? 1u : 0u);
-            const uint32_t col = C::COL_SCORE + (n & 1) * 2 * C::BC, colx = C::COL_SCORE + ((n - 1) & 1) * 2 * C::BC + C::BC;
-            // first output MMAs of an item: they overwrite the accumulators
-            auto acc_free = [&]() { return oi++ == 0 || k.wait(C::B_ACCFREE, oi - 2); };
-            auto part_x = [&]() {
-                if (!KEYS && (first & 8u) && !acc_free()) return false;
-                if ((first & 2u) && !k.wait(C::B_XRDY + 1, xi++)) return false;
-                ptx::tc_fence_after_sync();
-                const uint32_t el = ptx::elect_one();
-                if (k_out) {
-                    I::template g_outputs<1>(el, colx, klo, first & 8u ? 0u : 1u);
-                    ptx::mma_commit_p(el, k.bar(C::B_OUTDONE + ((n - 3) & (C::NOUTDONE - 1))));
-                    if (end & 8u) ptx::mma_commit_p(el, k.bar(C::B_FINAL));
-                }
-                if (x) {
-                    const uint32_t el2 = ptx::elect_one();
-                    I::template single<true, true, 1>(el2, colx, k, C::COL_X1, xlo, xfold);
-                    ptx::mma_commit_p(el2, k.bar(C::B_XFULL + ((n - 1) & 3)));
-                    if (end & 2u) ptx::mma_commit_p(el2, k.bar(C::B_XFREE + 1));
-                }
-                return true;
-            };
-            // the item before is still to be ended
-            const bool swap = KEYS && (first & 4u);
-            if (swap && !part_x()) return;
-            if (KEYS && (first & 4u) && !acc_free()) return;
-            if ((first & 1u) && !k.wait(C::B_XRDY, si++)) return;
-            k.tile_fence();
-            if (KEYS && v_out) I::template g_outputs<0>(ptx::elect_one(), col, vlo, first & 4u ? 0u : 1u);
-            if (score) {
-                const uint32_t el = ptx::elect_one();
-                I::template single<true, true, 0>(el, col, k, C::COL_X0, l.lo, l.fold);
-                ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
-                if (end & 1u) ptx::mma_commit_p(el, k.bar(C::B_XFREE));
+            if (x) {
+                const uint32_t el2 = ptx::elect_one();
+                I::template single<true, true, 1>(el2, colx, k, C::COL_X1, xlo, xfold);
+                ptx::mma_commit_p(el2, k.bar(C::B_XFULL + ((n - 1) & 3)));
+                if (end & 2u) ptx::mma_commit_p(el2, k.bar(C::B_XFREE + 1));
             }
-            if (!swap && !part_x()) return;
-            klo = vlo;
-            vlo = xlo;
-            xlo = l.lo;
-            xfold = l.fold;
-            if (score) {
-                l.template next<C::SL, I::L_STEP, I::F_STEP>();
-                if (++sj == T) sj = 0;
-            }
+            return true;
+        };
+        // the item before is still to be ended
+        const bool swap = KEYS && (first & 4u);
+        if (swap && !part_x()) return;
+        if (KEYS && (first & 4u) && !acc_free()) return;
+        if ((first & 1u) && !k.wait(C::B_XRDY, si++)) return;
+        k.tile_fence();
+        if (KEYS && v_out) I::template g_outputs<0>(ptx::elect_one(), col, vlo, first & 4u ? 0u : 1u);
+        if (score) {
+            const uint32_t el = ptx::elect_one();
+            I::template single<true, true, 0>(el, col, k, C::COL_X0, l.lo, l.fold);
+            ptx::mma_commit_p(el, k.bar(C::B_SFULL + (n & 3)));
+            if (end & 1u) ptx::mma_commit_p(el, k.bar(C::B_XFREE));
+        }
+        if (!swap && !part_x()) return;
+        klo = vlo;
+        vlo = xlo;
+        xlo = l.lo;
+        xfold = l.fold;
+        if (score) {
+            l.template next<C::SL, I::L_STEP, I::F_STEP>();
+            if (++sj == T) sj = 0;
         }
     }
 }
@@ -1530,8 +1574,7 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
         const __nv_bfloat16* src = x + (p.o.head_off(bh, p.H) + (size_t)(row0 + row) * (size_t)p.o.rs);
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
-            // (FOLD: the columns that pad d to DP are ones against the statistics, where those lie there)
-            v[c] = C::FOLD && C::TAIL && 8 * c >= p.d ? make_uint4(JVP_ONES0, JVP_ONES1, 0, 0) : make_uint4(0, 0, 0, 0);
+            v[c] = make_uint4(0, 0, 0, 0);
             if (valid && 8 * c < p.d) v[c] = __ldg(reinterpret_cast<const uint4*>(src + 8 * c));
         }
     };
@@ -1543,35 +1586,68 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
         }
     };
     [[maybe_unused]] uint4 v0[NCH], v1[NCH];
-    if (C::XT && (int)blockIdx.x < p.items) {
+    if (C::XT && !C::XS && (int)blockIdx.x < p.items) {
         load_x(blockIdx.x, 0, v0);
         store_x(0, v0);
         load_x(blockIdx.x, 1, v0);
-        if (C::XSETS == 2) {
-            ptx::tmem_wait_st();
-            k.arrive(C::B_XRDY, lane);
-        }
         store_x(1, v0);
         ptx::tmem_wait_st();
-        k.arrive(C::B_XRDY + C::XSETS - 1, lane);
+        k.arrive(C::B_XRDY, lane);
+    }
+    // XS.  Tensor t of the block's item i, from shared memory.
+    [[maybe_unused]] const int n_it = jvp_item_count(p);
+    [[maybe_unused]] auto stage_x = [&](int t, int i) {
+        const bool valid = ((int)blockIdx.x + i * (int)gridDim.x) % p.row_tiles * JVP_ROWS + row < p.o.rows;
+        if (!k.wait_item(C::B_OWN + t, i) || (i > 0 && !k.wait_item(C::B_XFREE + t, i - 1))) return false;
+        ptx::tc_fence_after_sync();
+        const uint32_t tile = k.own_tile(t) + row * 128;
+#pragma unroll
+        for (int c = 0; c < NCH; c += 2) {
+            uint4 v[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                // (FOLD: the columns that pad d to DP are ones against the statistics, where those lie there)
+                v[e] = C::FOLD && C::TAIL && 8 * (c + e) >= p.d ? make_uint4(JVP_ONES0, JVP_ONES1, 0, 0) : make_uint4(0, 0, 0, 0);
+                const uint32_t at = c < 8 ? tile + (((c + e) ^ (row & 7)) << 4) : k.own_tail(t, row, c + e - 8);
+                if (valid && 8 * (c + e) < p.d) v[e] = *static_cast<const uint4*>(__cvta_shared_to_generic(at));
+            }
+            const uint32_t r[8] = {v[0].x, v[0].y, v[0].z, v[0].w, v[1].x, v[1].y, v[1].z, v[1].w};
+            ptx::tmem_st8(lanes + (t ? C::COL_X1 : C::COL_X0) + 4 * c, r);
+        }
+        ptx::tmem_wait_st();
+        k.arrive(C::B_XRDY + t, lane);
+        if (lane == 0) ptx::mbar_arrive(k.bar(C::B_OWNFREE + t));
+        return true;
+    };
+    // What the issuing warp completes is waited for in the order in which it does: an item's last scores S in its step of that tile,
+    // the last X one step later, the last outputs three later.  (Short items: several are opened before one ends.)  Here: the
+    // operands whose predecessors are free before step `step`.
+    [[maybe_unused]] int staged = 0;   // tensors taken to tensor memory, the first and the second in turn
+    [[maybe_unused]] auto stage_until = [&](int step) {
+        while (staged < 2 * n_it && (staged >> 1) * p.T - 1 + (staged & 1) < step) {
+            if (!stage_x(staged & 1, staged >> 1)) return false;
+            ++staged;
+        }
+        return true;
+    };
+    if (C::FOLD_TAIL && k.fold_step()) {   // ones against the statistics, for good
+        const uint32_t ones[8] = {JVP_ONES0, JVP_ONES1, 0, 0, 0, 0, 0, 0};
+        ptx::tmem_st8(lanes + C::COL_X0 + 8 * C::KS, ones);
+        ptx::tmem_st8(lanes + C::COL_X1 + 8 * C::KS, ones);
     }
     int it = 0;
     for (int item = blockIdx.x; item < p.items; item += gridDim.x, ++it) {
-        if (C::XT && item + (int)gridDim.x < p.items) {
+        if constexpr (C::XS) {
+            if (!stage_until((it + 1) * p.T + 2)) return;
+        } else if (C::XT && item + (int)gridDim.x < p.items) {
             load_x(item + gridDim.x, 0, v0);                       // in flight during the wait
             load_x(item + gridDim.x, 1, v1);
             if (!k.wait_item(C::B_XFREE, it)) return;
             ptx::tc_fence_after_sync();
             store_x(0, v0);
-            if (C::XSETS == 2) {
-                ptx::tmem_wait_st();
-                k.arrive(C::B_XRDY, lane);
-                if (!k.wait_item(C::B_XFREE + 1, it)) return;
-                ptx::tc_fence_after_sync();
-            }
             store_x(1, v1);
             ptx::tmem_wait_st();
-            k.arrive(C::B_XRDY + C::XSETS - 1, lane);
+            k.arrive(C::B_XRDY, lane);
         }
         const int bh = item / p.row_tiles, row0 = (item - bh * p.row_tiles) * JVP_ROWS;
         const size_t off = p.o.head_off(bh, p.H) + (size_t)(row0 + row) * (size_t)p.o.rs;
@@ -1637,6 +1713,9 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
 #pragma unroll
             for (int i = 0; i < HOLD; ++i) read(C::KS - HOLD + i, q0[i], q1[i]);
             k.arrive(C::B_ACCFREE + pair, lane);
+            // (what the next two steps wait for goes in front of the stores)
+            if constexpr (C::XS)
+                if (!stage_until((it + 1) * p.T + 2 + min(p.T, JVP_AHEAD))) return;
 #pragma unroll
             for (int i = 0; i < HOLD; ++i) store(C::KS - HOLD + i, q0[i], q1[i]);
         }
@@ -1670,7 +1749,7 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
         init(C::B_EFULL, C::SE, C::EFULL_COUNT);
         init(C::B_LFULL, C::SL, C::LFULL_COUNT);
         init(C::B_OWN, C::OWN_SETS, C::TAIL ? 33 : 1);
-        init(C::B_OWNFREE, C::OWN_SETS, 1);
+        init(C::B_OWNFREE, C::OWN_SETS, C::XS ? 4 : 1);
         init(C::B_XRDY, C::XSETS, 4);
         init(C::B_XFREE, C::XSETS, 1);
         init(C::B_SFULL, 8 + C::NOUTDONE, 1);   // SFULL, XFULL, OUTDONE
@@ -1689,7 +1768,7 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
         // written again.  Owners and E ring: the second chunk block; L ring: chunk 1 of the second atom, which lies at
         // physical chunk 1 ^ (r & 7) of row r.  FOLD: the stages have the statistics there, the first owner tensor of a pair
         // the ones.
-        for (int i = threadIdx.x; i < C::NOWN * JVP_ROWS; i += JVP_THREADS)
+        for (int i = threadIdx.x; i < (C::XS ? 0 : C::NOWN) * JVP_ROWS; i += JVP_THREADS)   // (XS: the epilogue puts them in)
             *reinterpret_cast<uint4*>(jvp_smem + (i / JVP_ROWS) * C::OWN_BYTES + C::OWN_ATOM + (JVP_ROWS + i % JVP_ROWS) * 16) =
                 C::FOLD && !(i / JVP_ROWS & 1) ? make_uint4(JVP_ONES0, JVP_ONES1, 0, 0) : zero;
         if (!C::FOLD) {
@@ -1701,6 +1780,13 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
                 const int t = i / BC, r = i - t * BC;
                 *reinterpret_cast<uint4*>(l + (t >> 1) * 2 * C::LST_BYTES + (2 + (t & 1)) * C::ATOM + r * 128 + ((1 ^ (r & 7)) << 4)) = zero;
             }
+        }
+    }
+    if (C::FOLD_TAIL && k.fold_step()) {   // the other half of the statistics' k-step
+        uint8_t* l = jvp_smem + k.L;
+        for (int i = threadIdx.x; i < C::SL * 2 * BC; i += JVP_THREADS) {
+            const int t = i / BC, r = i - t * BC;
+            *reinterpret_cast<uint4*>(l + (t >> 1) * 2 * C::LST_BYTES + (2 + (t & 1)) * C::ATOM + r * 128 + ((3 ^ (r & 7)) << 4)) = zero;
         }
     }
     if (C::DKV && p.no_g) {
@@ -1715,7 +1801,7 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
             }
         }
     }
-    if (C::FOLD)
+    if (C::ONES_BYTES)
         for (int i = threadIdx.x; i < 2 * JVP_ROWS; i += JVP_THREADS)
             *reinterpret_cast<uint4*>(jvp_smem + k.ONES + i * 16) = i < JVP_ROWS ? make_uint4(JVP_ONES0, JVP_ONES1, 0, 0) : zero;
     ptx::fence_proxy_async_smem();
@@ -1738,7 +1824,10 @@ jvp_kernel(const __grid_constant__ CUtensorMap s0, const __grid_constant__ CUten
             const CUtensorMap* const maps[4] = {&o0, &o1, &o2, &o3};
             if (warp == 1) jvp_issue<MODE, DP>(p, k);
             else if (warp == 2) jvp_load_ring<MODE, DP, 1>(p, k, &s2, &s3, maps, lane);
-            else if (warp == 0) { if constexpr (!C::GONLY) jvp_load_ring<MODE, DP, 0>(p, k, &s0, &s1, maps, lane); }
+            else if (warp == 0) {
+                if constexpr (C::XS) jvp_stage_owners<MODE, DP>(p, k, maps, lane);
+                else jvp_load_ring<MODE, DP, 0>(p, k, &s0, &s1, maps, lane);
+            }
             else if constexpr (C::FOLD) jvp_fold<MODE, DP>(p, k, lane);
         }
         if (warp == 1 && *abort_flag && placed) {

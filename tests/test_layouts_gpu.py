@@ -155,6 +155,26 @@ def test_detached_backward_in_the_token_major_layout():
     assert not outs[3].any() and not outs[4].any() and not outs[5].any()
 
 
+@pytest.mark.parametrize("B,H,M,N,d", [(2, 100, 65, 200, 72), (2, 100, 200, 65, 64), (3, 60, 1, 193, 40), (3, 60, 193, 1, 80), (2, 100, 130, 64, 72),
+                                       (2, 90, 64, 321, 56), (2, 80, 129, 192, 16)])
+@pytest.mark.parametrize("absent", ["dtO", "dO"])
+@pytest.mark.parametrize("layout", ["packed", "token"])
+def test_cross_attention_without_a_cotangent_over_several_items_a_block(B, H, M, N, d, absent, layout):
+    """The two passes of such a call have tile counts of their own: items of one or two tiles in one of them and of three or
+    more in the other, more items than SMs in both."""
+    x = _draw(B, H, M, N, d, seed=300 + M + N, dtype=torch.bfloat16)
+    dev = {k: (_as_bnhd(v.cuda()) if layout == "token" else v.cuda()) for k, v in x.items()}
+    dev[absent] = None
+    got = _gpu(dev)
+    x[absent] = torch.zeros_like(x[absent])
+    ref = _oracle(x, d)
+    errs = {k: rel_err(got[k].float().cpu().numpy(), ref[k]) for k in ref}
+    assert_within(errs, 1e-2, 2e-2, 1e-4)
+    if absent == "dtO":
+        for k in ("dtQ", "dtK", "dtV"):
+            assert not got[k].any(), k
+
+
 def test_strides_that_cannot_be_read_are_refused():
     lib = binding.load()
     import ctypes

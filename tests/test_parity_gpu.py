@@ -389,10 +389,19 @@ def test_absent_cotangent_counts_as_zero(absent, B, H, N, d):
 
 @pytest.mark.parametrize("B,H,N,d", [(3, 110, 1, 16), (3, 110, 64, 72), (2, 160, 65, 32), (2, 100, 129, 80), (2, 90, 192, 56), (2, 80, 193, 40)])
 def test_backward_without_dto_over_items_of_few_tiles(B, H, N, d):
-    """Blocks with two items and more of one to four tiles of 64: up to two tiles the items are finished one by one, longer ones
-    run on into one another, two and three tiles of outputs behind the scores."""
+    """Blocks with two items and more of one to four tiles of 64: the items run on into one another, two and three tiles of
+    outputs behind the scores, so that up to four of them are open at once."""
     heads = [0, 3, 147, 148, 151, B * H - 1]
     errs, _, _ = run_case(inputs.custom(B, H, N, d, seed=700 + N + d), oracle_heads=heads, absent="dtO")
+    assert_within(errs, BF16_FWD, BF16_BWD, BF16_STATS)
+
+
+@pytest.mark.parametrize("B,H,N,d", [(3, 110, 1, 16), (3, 110, 64, 72), (3, 150, 48, 80), (2, 160, 65, 32), (2, 100, 97, 72), (2, 100, 129, 64)])
+@pytest.mark.parametrize("absent", [None, "dO"])
+def test_backward_with_dto_over_items_of_few_tiles(B, H, N, d, absent):
+    """The same of the passes with dtO, whose tiles are of 64 rows or, in one of them at head dims above 64, of 48."""
+    heads = [0, 3, 147, 148, 151, B * H - 1]
+    errs, _, _ = run_case(inputs.custom(B, H, N, d, seed=800 + N + d), oracle_heads=heads, absent=absent)
     assert_within(errs, BF16_FWD, BF16_BWD, BF16_STATS)
 
 
