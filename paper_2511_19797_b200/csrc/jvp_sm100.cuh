@@ -1701,23 +1701,31 @@ __device__ __forceinline__ void jvp_epilogue(const JvpParams& p, const JvpBlock<
             ptx::tc_fence_after_sync();
             // The next item's first output MMAs wait for the accumulators: up to d = 80 all of them are read and converted first and
             // stored behind the arrival (reads and stores in turn held them for 3200 cycles at d = 72).  WIDE: there are not the
-            // registers, and the items are long.
-            constexpr int HOLD = C::WIDE ? 1 : C::KS;
+            // registers, and the items are long.  Forward at d > 48 with one or two tiles an item: the stores are what bounds it, and
+            // spread over the reads they get by faster ((64, 16, 256 x 64), both layouts, us: d = 64 62, 63 -> 58, 59, d = 72 78, 84 ->
+            // 68, 71; 256 x 128 72, 90 -> 69, 85; equal at d = 32; three tiles, 256 x 192, d = 72: 81 -> 84).
+            auto put_out = [&](auto hold) {
+                constexpr int HOLD = decltype(hold)::value;
 #pragma unroll 1
-            for (int ch = 0; ch < C::KS - HOLD; ++ch) {
-                uint32_t q0[8], q1[8];
-                read(ch, q0, q1);
-                store(ch, q0, q1);
-            }
-            uint32_t q0[HOLD][8], q1[HOLD][8];
+                for (int ch = 0; ch < C::KS - HOLD; ++ch) {
+                    uint32_t q0[8], q1[8];
+                    read(ch, q0, q1);
+                    store(ch, q0, q1);
+                }
+                uint32_t q0[HOLD][8], q1[HOLD][8];
 #pragma unroll
-            for (int i = 0; i < HOLD; ++i) read(C::KS - HOLD + i, q0[i], q1[i]);
-            k.arrive(C::B_ACCFREE + pair, lane);
-            // (what the next two steps wait for goes in front of the stores)
-            if constexpr (C::XS)
-                if (!stage_until((it + 1) * p.T + 2 + min(p.T, JVP_AHEAD))) return;
+                for (int i = 0; i < HOLD; ++i) read(C::KS - HOLD + i, q0[i], q1[i]);
+                k.arrive(C::B_ACCFREE + pair, lane);
+                // (what the next two steps wait for goes in front of the stores)
+                if constexpr (C::XS)
+                    if (!stage_until((it + 1) * p.T + 2 + min(p.T, JVP_AHEAD))) return false;
 #pragma unroll
-            for (int i = 0; i < HOLD; ++i) store(C::KS - HOLD + i, q0[i], q1[i]);
+                for (int i = 0; i < HOLD; ++i) store(C::KS - HOLD + i, q0[i], q1[i]);
+                return true;
+            };
+            constexpr bool SPREAD = MODE == PASS_FWD && DP > 48 && !C::WIDE;
+            if (SPREAD && p.T <= 2) put_out(std::integral_constant<int, 1>());
+            else if (!put_out(std::integral_constant<int, C::WIDE ? 1 : C::KS>())) return;
         }
     }
 }
