@@ -176,8 +176,9 @@ struct JvpCfg {
     static_assert(!XT || DP + DP / 2 <= 128, "operands do not fit behind their accumulators");
     static_assert(COL_SCORE + 4 * BC <= 512, "TMEM over-subscribed");
     // Registers per thread: warpgroup 0, element-wise warps (FWD, DKV_G, DQ_G: 64 columns a thread), epilogue warps (which hold an owner
-    // row, 4 registers a chunk, or the columns they have read).
-    static constexpr int REGS_LOAD = MODE == PASS_FWD ? 56 : GONLY ? 80 : DKV && DP <= 48 ? 112 : 96, REGS_ELEM = MODE == PASS_FWD ? 168 : 152, REGS_EPI = MODE == PASS_FWD ? 120 : GONLY ? 128 : DKV && DP <= 48 ? 96 : 112;
+    // row, 4 registers a chunk, or the columns they have read).  Shares with which no pass spills; DKV with 96, 152 and 112 spills at
+    // d <= 48 and takes 1 to 3 % longer there ((64, 16, 256, 32), the backward: 163 us, 158 as here), above it makes no difference.
+    static constexpr int REGS_LOAD = MODE == PASS_FWD ? 56 : GONLY ? 80 : DKV ? 112 : 96, REGS_ELEM = MODE == PASS_FWD ? 168 : DKV ? 144 : 152, REGS_EPI = MODE == PASS_FWD ? 120 : GONLY ? 128 : 112;
     static_assert(REGS_LOAD + 2 * REGS_ELEM + REGS_EPI <= 4 * JVP_REGS, "more registers than the block has");
     // barriers
     static constexpr int B_EFULL = 0;
