@@ -87,22 +87,35 @@ __device__ __forceinline__ float rms_hsum(uint64_t v) {
 }
 
 // How the cpr 16-byte chunks of a row are split: C chunks on each of P lanes.  The largest C <= cmax that divides cpr and
-// leaves three lanes or more (48 contiguous bytes per row and instruction), or, for d = 32, two; if
-// none does (d = 40, 56, 88, 104), the largest whose last lane has one chunk less: a row's sums and scalars cost a warp as much
-// for one chunk a lane as for three.  One chunk a lane before: backward (16, 16, 1024) d = 32 49.8 -> 40.5 us, 40 68.4 -> 61.6,
-// 56 106.9 -> 72.2; forward 27.1 -> 25.0, 36.8 -> 36.9, 51.8 -> 45.5.
+// leaves three lanes or more (48 contiguous bytes per row and instruction), or two with up to three chunks each of rows of whole
+// 32-byte sectors; if none does (bf16 d = 40, 56, 88, 104), the largest whose last lane has one chunk less: a row's sums and
+// scalars cost a warp as much for one chunk a lane as for three.  Measured with bf16 (16, 16, 1024), us: one chunk a lane / as
+// here: backward d = 32 49.4 / 40.0, 40 67.9 / 60.8, 56 106.7 / 74.4, 88 231 / 115; forward d = 32 26.7 / 24.6, 40 36.7 / 36.3,
+// 56 51.3 / 44.8, 88 97 / 73.  Two lanes instead of three or four: d = 48 forward 38.4 -> 36.9, backward 63.1 -> 59.5; with
+// four chunks each, d = 64 forward 45.3 -> 53.2.
 struct RmsSplit { int C, P; };
-inline RmsSplit rms_split(int cpr, int cmax) {
+constexpr RmsSplit rms_split(int cpr, int cmax) {
     for (int waste = 0; waste < 2; ++waste)
         for (int c = cmax; c > 1; --c) {
             const int p = (cpr + c - 1) / c;
-            if (c * p - cpr == waste && (p >= 3 || (p == 2 && cpr == 4))) return {c, p};
+            if (c * p - cpr == waste && (p >= 3 || (p == 2 && c <= 3 && cpr % 2 == 0))) return {c, p};
         }
     return {1, cpr};
 }
 
-// Row groups of a warp in flight in the forward: with one chunk per lane (d = 8, 16, 24) a thread would have two
-// 16-byte loads in flight, and four groups measured 12 % faster than one; with two chunks or more, one group was faster.
+// Whether some head dim has its rows split into C chunks a lane, a last lane with one less among them or not.
+template <typename T>
+constexpr bool rms_split_exists(int cmax, int C, bool ragged) {
+    for (int d = 8; d <= 128; d += 8) {
+        const int cpr = d * (int)sizeof(T) / 16;
+        const RmsSplit s = rms_split(cpr, cmax);
+        if (s.C == C && (s.C * s.P > cpr) == ragged) return true;
+    }
+    return false;
+}
+
+// Row groups of a warp in flight in the forward: with one chunk per lane (d = 8, 16, 24) a thread would have two 16-byte loads in
+// flight.  Four groups against one, (16, 16, 1024): d = 24 20.5 us against 23.9, d = 8 and 16 equal (9.1 and 12.3).
 __host__ __device__ constexpr int rms_fwd_groups(int C) { return C == 1 ? 4 : 1; }
 
 // Sum of v over the P consecutive lanes that share a row, returned to all of them, the same bits on each.

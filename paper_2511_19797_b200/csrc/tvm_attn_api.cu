@@ -189,25 +189,37 @@ static bool q_packed(const Shape& s) {
     return s.q.rs == s.d && s.q.hs == (long long)s.M * s.d && s.q.bs == (long long)s.H * s.M * s.d;
 }
 
+// launch(chunks a lane, whether a last lane has one less, lanes a row) for the split of rows of d elements, the first two as
+// types: the streaming kernels exist for the splits that a head dim has.
+template <typename T, int CMAX, int C = CMAX, typename F>
+static int with_split(int d, const F& launch) {
+    if constexpr (C == 0) {
+        return TVM_ATTN_UNSUPPORTED;
+    } else {
+        const int cpr = d * (int)sizeof(T) / 16;   // 16-byte chunks per row (d % 8 == 0)
+        const RmsSplit split = rms_split(cpr, CMAX);
+        const bool ragged = split.C * split.P > cpr;
+        if constexpr (rms_split_exists<T>(CMAX, C, false))
+            if (split.C == C && !ragged) return launch(std::integral_constant<int, C>(), std::false_type(), split.P);
+        if constexpr (rms_split_exists<T>(CMAX, C, true))
+            if (split.C == C && ragged) return launch(std::integral_constant<int, C>(), std::true_type(), split.P);
+        return with_split<T, CMAX, C - 1>(d, launch);
+    }
+}
+
 template <typename T>
 static int launch_rowsums(const Shape& s, const void* G, const void* Hc, const void* O, const void* tO, const float* lse,
                           float* sig1, float* cvec, float* lse2, float sign, cudaStream_t st) {
     const long long rows = s.BH * s.M;           // fit 31 bits
-    const int cpr = s.d * (int)sizeof(T) / 16;   // 16-byte chunks per row (d % 8 == 0)
-    if (cpr > 32) return TVM_ATTN_UNSUPPORTED;   // d <= 128
-    const int C = rms_split(cpr, 4).C, P = rms_split(cpr, 4).P;
-    const long long rows_per_block = (ROWSUM_THREADS / 32) * (32 / P), blocks = (rows + rows_per_block - 1) / rows_per_block;
-    const auto kern = C * P > cpr ? (C == 4 ? bwd_rowsums_kernel<T, 4, true> : C == 3 ? bwd_rowsums_kernel<T, 3, true> : bwd_rowsums_kernel<T, 2, true>)
-                      : C == 4    ? bwd_rowsums_kernel<T, 4, false>
-                      : C == 3    ? bwd_rowsums_kernel<T, 3, false>
-                      : C == 2    ? bwd_rowsums_kernel<T, 2, false>
-                                  : bwd_rowsums_kernel<T, 1, false>;
-    g_prof.before(st);
-    kern<<<(unsigned)(blocks < ROWSUM_BLOCKS ? blocks : ROWSUM_BLOCKS), ROWSUM_THREADS, 0, st>>>(
-        (const T*)G, (const T*)Hc, (const T*)O, (const T*)tO, lse, sig1, cvec, lse2, (unsigned)rows, s.q, q_packed(s) ? 0 : s.H, s.d, P, sign);
-    g_prof.after(st);
-    g_launches += 1;
-    return cuda_status(cudaGetLastError());
+    return with_split<T, 4>(s.d, [&](auto C, auto ragged, int P) {
+        const long long rows_per_block = (ROWSUM_THREADS / 32) * (32 / P), blocks = (rows + rows_per_block - 1) / rows_per_block;
+        g_prof.before(st);
+        bwd_rowsums_kernel<T, C(), ragged()><<<(unsigned)(blocks < ROWSUM_BLOCKS ? blocks : ROWSUM_BLOCKS), ROWSUM_THREADS, 0, st>>>(
+            (const T*)G, (const T*)Hc, (const T*)O, (const T*)tO, lse, sig1, cvec, lse2, (unsigned)rows, s.q, q_packed(s) ? 0 : s.H, s.d, P, sign);
+        g_prof.after(st);
+        g_launches += 1;
+        return cuda_status(cudaGetLastError());
+    });
 }
 
 template <typename T>
@@ -400,7 +412,7 @@ static void rms_blocks(long long rows_q, long long rows_k, int rows_per_block, i
     *nbk = (int)(most - q < need_k ? most - q : need_k);
 }
 
-template <typename T, int C, bool RAGGED = false>
+template <typename T, int C, bool RAGGED>
 static int rms_fwd_c(const Shape& s, float eps, const RmsFwdSide<T>& q, const RmsFwdSide<T>& k, int P, cudaStream_t st) {
     int nbq, nbk;
     rms_blocks(q.rows.total, k.rows.total, (RMS_THREADS / 32) * rms_fwd_groups(C) * (32 / P), RMS_FWD_BLOCKS, &nbq, &nbk);
@@ -414,20 +426,10 @@ static int rms_fwd(const Shape& s, float eps, const void* Q, const void* tQ, con
                    const float* gK, void* Qn, void* tQn, void* Kn, void* tKn, cudaStream_t st) {
     const RmsFwdSide<T> q{(const T*)Q, (const T*)tQ, gQ, (T*)Qn, (T*)tQn, rms_rows(s, s.q)};
     const RmsFwdSide<T> k{(const T*)K, (const T*)tK, gK, (T*)Kn, (T*)tKn, rms_rows(s, s.k)};
-    const int cpr = s.d * (int)sizeof(T) / 16, C = rms_split(cpr, 4).C, P = rms_split(cpr, 4).P;
-    if (C * P > cpr)
-        return C == 2   ? rms_fwd_c<T, 2, true>(s, eps, q, k, P, st)
-               : C == 3 ? rms_fwd_c<T, 3, true>(s, eps, q, k, P, st)
-                        : rms_fwd_c<T, 4, true>(s, eps, q, k, P, st);
-    switch (C) {
-        case 1: return rms_fwd_c<T, 1>(s, eps, q, k, P, st);
-        case 2: return rms_fwd_c<T, 2>(s, eps, q, k, P, st);
-        case 3: return rms_fwd_c<T, 3>(s, eps, q, k, P, st);
-        default: return rms_fwd_c<T, 4>(s, eps, q, k, P, st);
-    }
+    return with_split<T, 4>(s.d, [&](auto C, auto ragged, int P) { return rms_fwd_c<T, C(), ragged()>(s, eps, q, k, P, st); });
 }
 
-template <typename T, int C, bool RAGGED = false>
+template <typename T, int C, bool RAGGED>
 static int rms_bwd_c(const Shape& s, float eps, RmsBwdSide<T> q, RmsBwdSide<T> k, int P, float* dgQ, float* dgK, cudaStream_t st) {
     int nbq, nbk;
     rms_blocks(q.rows.total, k.rows.total, (RMS_BWD_THREADS / 32) * (32 / P), RMS_BWD_BLOCKS, &nbq, &nbk);
@@ -455,13 +457,7 @@ static int rms_bwd(const Shape& s, float eps, const void* Q, const void* tQ, con
                    void* dK, void* dtK, float* dgQ, float* dgK, float* partial, cudaStream_t st) {
     const RmsBwdSide<T> q{(const T*)Q, (const T*)tQ, gQ, (const T*)dQn, (const T*)dtQn, (T*)dQ, (T*)dtQ, partial, rms_rows(s, s.q)};
     const RmsBwdSide<T> k{(const T*)K, (const T*)tK, gK, (const T*)dKn, (const T*)dtKn, (T*)dK, (T*)dtK, nullptr, rms_rows(s, s.k)};
-    const int cpr = s.d * (int)sizeof(T) / 16, C = rms_split(cpr, 3).C, P = rms_split(cpr, 3).P;
-    if (C * P > cpr) return C == 2 ? rms_bwd_c<T, 2, true>(s, eps, q, k, P, dgQ, dgK, st) : rms_bwd_c<T, 3, true>(s, eps, q, k, P, dgQ, dgK, st);
-    switch (C) {
-        case 1: return rms_bwd_c<T, 1>(s, eps, q, k, P, dgQ, dgK, st);
-        case 2: return rms_bwd_c<T, 2>(s, eps, q, k, P, dgQ, dgK, st);
-        default: return rms_bwd_c<T, 3>(s, eps, q, k, P, dgQ, dgK, st);
-    }
+    return with_split<T, 3>(s.d, [&](auto C, auto ragged, int P) { return rms_bwd_c<T, C(), ragged()>(s, eps, q, k, P, dgQ, dgK, st); });
 }
 
 static bool rms_eps_ok(float eps) { return eps >= 0.0f && std::isfinite(eps); }
