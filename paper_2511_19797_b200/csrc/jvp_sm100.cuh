@@ -380,10 +380,9 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
     const uint32_t ring_base = k.base + (RING == 0 ? k.E : k.L);
     const __nv_bfloat16* base0 = p.strm[2 * RING];
     const __nv_bfloat16* base1 = p.strm[2 * RING + 1];
-    // The ring that streams the cotangents (Hc, G): G may be absent (null) and is not loaded then.
-    constexpr bool has0 = true;
+    // DKV streams the cotangents (Hc, G) in its E ring: G may be absent (null) and is not loaded then.
     const bool has1 = C::DKV && RING == 0 ? base1 != nullptr : true;
-    const uint32_t tx_bytes = ((has0 ? 1 : 0) + (has1 ? 1 : 0)) * ATOM * (C::WIDE ? 2 : 1);
+    const uint32_t tx_bytes = (has1 ? 2 : 1) * ATOM * (C::WIDE ? 2 : 1);
     // Chunk 0 of row `lane` behind the first atoms: compact blocks in the E ring, a second swizzled atom in the L ring.
     [[maybe_unused]] const uint32_t sw = lane & 7;  // rows 32 apart share it
     constexpr bool FLAT = RING == 0 && !C::E_MN;
@@ -431,10 +430,8 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
             [[maybe_unused]] const int rows_left = rows - j * BC;  // rows of this tile that exist
             if (ptx::elect_one()) {
                 ptx::mbar_arrive_expect_tx(full, tx_bytes);
-                if (has0) {
-                    ptx::tma_load_4d(stage, map0, full, 0, j * BC, ch, cb);
-                    if (C::WIDE) ptx::tma_load_4d(stage + 2 * ATOM, map0, full, 64, j * BC, ch, cb);
-                }
+                ptx::tma_load_4d(stage, map0, full, 0, j * BC, ch, cb);
+                if (C::WIDE) ptx::tma_load_4d(stage + 2 * ATOM, map0, full, 64, j * BC, ch, cb);
                 if (has1) {
                     ptx::tma_load_4d(stage + ATOM, map1, full, 0, j * BC, ch, cb);
                     if (C::WIDE) ptx::tma_load_4d(stage + 3 * ATOM, map1, full, 64, j * BC, ch, cb);
@@ -467,14 +464,15 @@ __device__ __forceinline__ void jvp_load_ring(const JvpParams& p, const JvpBlock
                     if (c < ntail) {
                         const uint32_t dst = d0 + (FLAT ? c * 2 * BC * 16 : (c ^ sw) << 4);
                         if (__builtin_expect(rows_left >= BC, 1)) {
-                            if (has0) { ptx::cp_async_16(dst, src0 + 8 * c); if (hi) ptx::cp_async_16(dst + R1, src0 + d32 + 8 * c); }
+                            ptx::cp_async_16(dst, src0 + 8 * c);
+                            if (hi) ptx::cp_async_16(dst + R1, src0 + d32 + 8 * c);
                             if (has1) { ptx::cp_async_16(dst + T1, src1 + 8 * c); if (hi) ptx::cp_async_16(dst + T1 + R1, src1 + d32 + 8 * c); }
                         } else {
 #pragma unroll
                             for (int rp = 0; rp < 2; ++rp) {
                                 const bool v = lane + 32 * rp < rows_left;
                                 if (rp == 1 && !hi) continue;
-                                if (has0) ptx::cp_async_16(dst + rp * R1, v ? src0 + rp * d32 + 8 * c : base0, v ? 16u : 0u);
+                                ptx::cp_async_16(dst + rp * R1, v ? src0 + rp * d32 + 8 * c : base0, v ? 16u : 0u);
                                 if (has1) ptx::cp_async_16(dst + rp * R1 + T1, v ? src1 + rp * d32 + 8 * c : base1, v ? 16u : 0u);
                             }
                         }
@@ -599,9 +597,9 @@ __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE
             put(dl, sl, C::B_LFULL, a[0] * f_lse, a[1] * f1, a[2] * f_lse, a[3] * f1);
             if (++sl == C::SL) sl = 0;
             if constexpr (C::DKV) {
-            if (g >= C::SE && !k.template stage_free<0>(g)) return;
-            put(de, se, C::B_EFULL, b[0], b[1], b[2], b[3]);
-            if (++se == C::SE) se = 0;
+                if (g >= C::SE && !k.template stage_free<0>(g)) return;
+                put(de, se, C::B_EFULL, b[0], b[1], b[2], b[3]);
+                if (++se == C::SE) se = 0;
             }
             const bool more = j + 1 < T;
             if (more || next < p.items) load(more ? bh : next / p.row_tiles, more ? j + 1 : 0);
@@ -618,7 +616,7 @@ __device__ __forceinline__ void jvp_fold(const JvpParams& p, const JvpBlock<MODE
 // dependent scalar instruction ten, and an MMA 70 instead of 25 where the lane that issues it was elected in front of a branch
 // or a wait: each batch elects its own.  So: ring positions are carried along as descriptors (every descriptor of a batch is
 // the carried one plus a constant), barriers of the rings are tested ahead, in front of the batch before, what depends on
-// the item stays out of the tile's path, and which cotangent is absent (ABS) is a template parameter.
+// the item stays out of the tile's path, and whether G is absent (NO_G) is a template parameter.
 struct JvpSlot {   // a ring's next tile: stage, phase, low descriptor halves of the stage and of its statistics
     uint32_t lo, fold, lo0, fold0;
     int s = 0, ph = 0;
@@ -631,7 +629,7 @@ struct JvpSlot {   // a ring's next tile: stage, phase, low descriptor halves of
     }
 };
 
-template <int MODE, int DP, bool NO_G>
+template <int MODE, int DP>
 struct JvpIssue {
     using C = JvpCfg<MODE, DP>;
     using Block = JvpBlock<MODE, DP>;
@@ -762,7 +760,7 @@ struct JvpIssue {
 template <int MODE, int DP, bool NO_G>
 __device__ __forceinline__ void jvp_issue_dkv(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
     using C = JvpCfg<MODE, DP>;
-    using I = JvpIssue<MODE, DP, NO_G>;
+    using I = JvpIssue<MODE, DP>;
     constexpr int BC = C::BC;
     const JvpBlock<MODE, DP> k = shared.pinned();
     const int T = jvp_pin(p.T);
@@ -842,7 +840,7 @@ __device__ __forceinline__ void jvp_issue_dkv(const JvpParams& p, const JvpBlock
 template <int MODE, int DP>
 __device__ __forceinline__ void jvp_issue_one_pair(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
     using C = JvpCfg<MODE, DP>;
-    using I = JvpIssue<MODE, DP, false>;
+    using I = JvpIssue<MODE, DP>;
     constexpr int RDY = C::XT ? C::B_XRDY : C::B_OWN, FREE = C::XT ? C::B_XFREE : C::B_OWNFREE;
     const JvpBlock<MODE, DP> k = shared.pinned();
     const int T = jvp_pin(p.T), items = jvp_pin(p.items);
@@ -898,7 +896,7 @@ __device__ __forceinline__ void jvp_issue_one_pair(const JvpParams& p, const Jvp
 template <int MODE, int DP, bool NO_G>
 __device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
     using C = JvpCfg<MODE, DP>;
-    using I = JvpIssue<MODE, DP, NO_G>;
+    using I = JvpIssue<MODE, DP>;
     const JvpBlock<MODE, DP> k = shared.pinned();
     const int T = jvp_pin(p.T);
     const uint32_t x0 = ptx::desc_lo(k.own_tile(0), 16), x1 = ptx::desc_lo(k.own_tile(1), 16);
@@ -973,7 +971,7 @@ __device__ __forceinline__ void jvp_issue_two_pairs(const JvpParams& p, const Jv
 template <int MODE, int DP>
 __device__ __forceinline__ void jvp_issue_g(const JvpParams& p, const JvpBlock<MODE, DP>& shared) {
     using C = JvpCfg<MODE, DP>;
-    using I = JvpIssue<MODE, DP, false>;
+    using I = JvpIssue<MODE, DP>;
     constexpr bool KEYS = MODE == PASS_DKV_G;
     const JvpBlock<MODE, DP> k = shared.pinned();
     const int T = jvp_pin(p.T), last = jvp_item_count(p) * T;
