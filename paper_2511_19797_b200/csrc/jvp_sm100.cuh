@@ -49,7 +49,8 @@
 // before): forward 1.40 -> 1.08 ms, DV / DK / DQ 1.33 / 2.82 / 2.92 -> 1.06 / 1.48 / 1.42 ms.  At d <= 80 (two
 // element-wise groups on alternate tiles, which also wrote the outputs, before): d = 64 (8, 16, 4096) forward 1.94 -> 1.75 ms,
 // backward 7.37 -> 6.12 ms, with DV and DK in one pass 5.45 ms; d = 72 (16, 16, 1024) forward 321 -> 313 us, backward
-// 1.22 -> 1.08 -> 1.01 ms.
+// 1.22 -> 1.08 -> 1.01 ms; with the waits as one small loop and items that run on into one another (both at the power cap)
+// 284 us and 0.89 ms.
 //
 // Every wait on an mbarrier is bounded; when one gives up the block records a time-out status and all roles leave their
 // loops.
@@ -190,7 +191,7 @@ struct JvpCfg {
     static constexpr int XSETS = GONLY ? 2 : 1;                        // with barriers of their own
     static constexpr int B_XFREE = B_XRDY + XSETS;                     // ... free
     // MMAs of tile g complete: + (g & 3), phase g >> 2.  The element-wise groups meet every other tile only and the
-    // producers run up to four tiles ahead of or behind the others, so that a parity wait on one barrier, or on a pair,
+    // producers run up to four tiles ahead of or behind the others (six in DKV_G, DQ_G), so that a parity wait on one barrier, or on a pair,
     // could take another tile's completion for its own.  They also tell the producers that a ring stage is free: a commit
     // costs the issuing warp 60 cycles, and a barrier of its own per ring would be one more per tile.
     static constexpr int B_SFULL = B_XFREE + XSETS;                        // S (and Sd, except in FWD) written
@@ -1051,11 +1052,12 @@ __device__ __forceinline__ void jvp_issue(const JvpParams& p, const JvpBlock<MOD
 }
 
 // ------------------------------------------------------------------------------------------------ element-wise warps
-// Forward: the two groups take the tiles in turn; a thread has owner row `row` and the 64 columns of the tile.  Backward: all
-// eight warps work on every tile; a thread has the 32 columns of its group's half.  (With one score buffer, or in the
-// backward's shorter DV tile, the tensor pipe waits for how long a tile takes; the forward measured 8 % slower that way,
-// with the row maxima to exchange.)  Reads of tensor memory are issued for many columns at once (a read costs 180 cycles
-// whatever its width) and released with one arrival per warp; the operands are handed over half by half.
+// Forward, DKV_G, DQ_G: the two groups take the tiles in turn; a thread has owner row `row` and the 64 columns of the tile.  The
+// other passes: all eight warps work on every tile; a thread has the 32 columns of its group's half (DKV: of half the rows, all
+// columns).  (With one score buffer, or in the shorter DV tile, the tensor pipe waits for how long a tile takes; the forward, with
+// two, measured 8 % slower that way, with the row maxima to exchange.)  Reads of tensor memory are issued for many columns at once
+// (a read costs 180 cycles whatever its width) and released with one arrival per warp; the operands are handed over half by half
+// (DKV, DKV_G, DQ_G: whole).
 
 // Forward.  The reference m of a row and the centre c of its tangent weights are shared by the two groups: the warp that
 // has a row's tile g decides whether to move them and hands the row state on to the warp that has tile g + 1 (B_TURN), long

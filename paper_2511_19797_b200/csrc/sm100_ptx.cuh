@@ -258,7 +258,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
 // The same with the abort flag given by its shared-memory address (one register instead of two where a role has none to
 // spare), and as one small loop: a kernel has some 30 of these waits, its roles share an instruction cache, and a wait that
 // jumps over the code for the rare cases costs its warp 130 to 400 cycles where this one costs 85.  (Kernels of 60 instead of
-// 170 KB; d = 72 (16, 16, 1024): forward 279 -> 249 us, DKV 490 -> 463.)  The clock is read every 256 polls.
+// 170 KB; at d = 72 the forward took a tenth less time for it and DKV a twentieth.)  The clock is read every 256 polls.
 __device__ __forceinline__ bool mbar_wait_warp_s(uint32_t bar, uint32_t parity, uint32_t abort_addr, uint64_t limit_ns) {
     uint64_t t0 = 0;
 #pragma unroll 1
